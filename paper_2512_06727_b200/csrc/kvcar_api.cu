@@ -80,7 +80,8 @@ struct kvcar_ctx {
     size_t plan_off = 0, enc_off = 0, tmap_off = 0, tcpart_off = 0;  // inside weights
     size_t bt_off = 0, len_off = 0, status_off = 0, part_off = 0, stage_off = 0, enchid_off = 0, kvsplit_off = 0, pfhid_off = 0, abs_off = 0;  // inside workspace
     int max_k_sources = 0;  // most distinct source layers any layer's K heads resolve to
-    bool raw_maps = false;  // every raw bf16 pool has its TMA descriptor (raw-row kernel stages with tensor loads)
+    std::vector<RawSources> raw_src;  // [layer] tensor maps and head places of raw bf16 layers
+    std::vector<char> raw_src_ok;     // [layer] filled (else the raw-row kernel stages with cp.async)
     std::vector<EncPlan> enc_host;  // the device's EncPlan table, host copy (tensor-core prefill builds tensor maps from it)
     int max_chunks = 0, chunk_tokens = 128;
     int max_d = 0, max_m = 0, max_in = 0;
@@ -581,12 +582,25 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
         tc_setup_absorb(c->tc, c->cfg, c->max_k_sources, c->max_m, std::min(g.max_seqs, KVCAR_MAX_BATCH), c->max_chunks,
                         c->ws + c->abs_off, img.data() + slot, c->weights + slot);
     }
-    // descriptors of the raw pools (their three slots are otherwise unused: a raw pool has no decoder)
-    c->raw_maps = g.storage == KVCAR_BF16;
-    for (int i = 0; i < nl * 2 && c->raw_maps; ++i) {
-        if (c->ae[i].set || c->width[i] == 0) continue;
-        c->raw_maps = raw_build_map(img.data() + c->tmap_off + (size_t)i * 3 * 128, c->pool + c->pool_off[i],
-                                    (size_t)g.max_pages * g.page_tokens, (uint64_t)c->width[i]);
+    // tensor maps and head places of the raw layers (kernel parameters of the raw-row kernel)
+    c->raw_src.assign(nl, RawSources{});
+    c->raw_src_ok.assign(nl, 0);
+    for (int l = 0; l < nl && g.storage == KVCAR_BF16; ++l) {
+        RawSources &rs = c->raw_src[l];
+        bool ok = layer_is_raw(c, l);
+        for (int which = 0; which < 2 && ok; ++which) {
+            const WhichPlan &wp = plans[l].w[which];
+            ok = wp.n_src <= RAW_MAX_SRC;
+            for (int s = 0; s < wp.n_src && ok; ++s) {
+                const SourcePlan &sp = wp.src[s];
+                ok = raw_build_map(&rs.map[which][s], sp.pool, (size_t)g.max_pages * g.page_tokens, (uint64_t)sp.width);
+                for (int i = 0; i < sp.n_need; ++i) {
+                    rs.idx[which][sp.kv_head[i]] = (uint8_t)s;
+                    rs.col[which][sp.kv_head[i]] = (uint16_t)(sp.slot[i] * 64);
+                }
+            }
+        }
+        c->raw_src_ok[l] = ok;
     }
     c->tc.pbuf = reinterpret_cast<float *>(c->ws + c->kvsplit_off);
     c->tc.pflags = reinterpret_cast<uint32_t *>(c->ws + c->kvsplit_off +
@@ -845,7 +859,6 @@ static int prepare_decode(kvcar_ctx *c, int32_t layer, const int32_t *seqs, int3
     a.max_chunks = c->max_chunks;
     a.flags = flags;
     a.scale = 1.0f / std::sqrt((float)g.head_dim);
-    a.raw_tmaps = c->raw_maps ? c->weights + c->tmap_off : nullptr;
     sl.n = n_seqs;
     memcpy(sl.id, seqs, (size_t)n_seqs * 4);
     return (max_len + c->chunk_tokens - 1) / c->chunk_tokens;
@@ -864,7 +877,7 @@ static kvcar_status enqueue_decode_tiles(kvcar_ctx *c, int32_t layer, const Deco
         return fail(c, KVCAR_ERR_UNSUPPORTED, std::string("tensor-core kernel cannot run this layer: ") + c->tc.why);
     cudaError_t e;
     if (c->kernel != KVCAR_KERNEL_GENERIC && layer_is_raw(c, layer)) {
-        e = launch_decode_raw(a, sl, g.storage, n_chunks, st);
+        e = launch_decode_raw(a, sl, c->raw_src_ok[layer] ? &c->raw_src[layer] : nullptr, g.storage, n_chunks, st);
     } else if (want_tc) {
         int32_t lens[KVCAR_MAX_BATCH];
         for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];

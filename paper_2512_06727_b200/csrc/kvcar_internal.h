@@ -2,6 +2,7 @@
 // Nothing here is part of the public ABI (see include/kvcar.h).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -81,8 +82,16 @@ struct DecodeArgs {
     int32_t chunk_tokens, max_chunks;
     uint32_t flags;
     float scale;
-    const void *raw_tmaps;  // TMA descriptors of the raw (layer, K|V) pools (descriptor of pool i at + i * 384 bytes),
-                            // or null: the raw-row kernel then stages its rows with cp.async
+};
+
+// Where the heads of a raw layer lie: a tensor map per distinct source pool, and each KV head's source and first column.
+// Passed to the kernel by value: tensor maps in kernel parameters need no acquire by every block that uses them (measured
+// with the maps in global memory and a fence.proxy.tensormap per warp: 1248 against 1022 us for a 12-layer step).
+constexpr int RAW_MAX_SRC = 8;  // layers with more sources stage their rows with cp.async
+struct RawSources {
+    CUtensorMap map[2][RAW_MAX_SRC];
+    uint8_t idx[2][KVCAR_MAX_KV_HEADS];
+    uint16_t col[2][KVCAR_MAX_KV_HEADS];
 };
 
 struct EncodeArgs {
@@ -113,7 +122,9 @@ size_t encode_split_smem(int max_in, int max_m);
 cudaError_t launch_decode_generic(const DecodeArgs &a, const SeqList &seqs, int dtype, int max_d, int max_m,
                                   int grid_chunks, cudaStream_t st);
 // raw K/V layers (no autoencoder), head_dim 64, <= 8 query heads per KV head (kvcar_raw.cu)
-cudaError_t launch_decode_raw(const DecodeArgs &a, const SeqList &seqs, int dtype, int grid_chunks, cudaStream_t st);
+// src: the layer's tensor maps and head places, or null (no maps: rows are then staged with cp.async)
+cudaError_t launch_decode_raw(const DecodeArgs &a, const SeqList &seqs, const RawSources *src, int dtype, int grid_chunks,
+                              cudaStream_t st);
 // TMA descriptor of one raw bf16 pool [rows][width] with a box of 32 rows x 64 columns (one head's slice of one
 // 32-token step), 128-byte swizzle; false if the driver entry point is missing or the shape is refused
 bool raw_build_map(void *dst_host, const void *pool_dev, uint64_t rows, uint64_t width);

@@ -111,6 +111,12 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void *tmap,
         "l"(tmap), "r"(x), "r"(y), "r"(cluster_bar)
         : "memory");
 }
+// A tensor map that lies in global memory was written through other proxies (a copy from the host at bind time): the
+// block that uses it has to acquire it first, or it may meet what the map cache of its SM kept of an earlier map at the
+// same address (an earlier context's, whose pool may be gone).
+__device__ __forceinline__ void tmap_acquire(const void *tmap) {
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(tmap) : "memory");
+}
 // bring one box of a tensor into L2 ahead of its load
 __device__ __forceinline__ void tma_prefetch_2d(const void *tmap, int x, int y) {
     asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(tmap), "r"(x), "r"(y) : "memory");

@@ -64,11 +64,11 @@ struct Row64<float> {
 
 // where KV head h of this layer reads its rows: pool base, row width, first column
 struct HeadSrc {
-    const void *pool;
-    int width, col, src_layer;
+    const void *pool = nullptr;
+    int width = 0, col = 0;
 };
 __device__ __forceinline__ HeadSrc find_head(const WhichPlan &wp, int h) {
-    HeadSrc r{nullptr, 0, 0, 0};
+    HeadSrc r;
     for (int s = 0; s < wp.n_src; ++s) {
         const SourcePlan &sp = wp.src[s];
         for (int i = 0; i < sp.n_need; ++i)
@@ -76,7 +76,6 @@ __device__ __forceinline__ HeadSrc find_head(const WhichPlan &wp, int h) {
                 r.pool = sp.pool;
                 r.width = sp.width;
                 r.col = sp.slot[i] * 64;
-                r.src_layer = sp.src_layer;
             }
     }
     return r;
@@ -252,7 +251,8 @@ __device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
 
 template <bool TMA>
 __global__ void __launch_bounds__(GQ_RW * 32) decode_raw_gq_kernel(const __grid_constant__ DecodeArgs a,
-                                                               const __grid_constant__ SeqList seqs) {
+                                                               const __grid_constant__ SeqList seqs,
+                                                               const __grid_constant__ RawSources src) {
     extern __shared__ __align__(128) uint8_t gq_smem[];
     __shared__ __align__(8) uint64_t step_bar[GQ_RW][2];  // TMA build: bytes of a step buffer pair have landed
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -264,7 +264,14 @@ __global__ void __launch_bounds__(GQ_RW * 32) decode_raw_gq_kernel(const __grid_
     if (t0 >= L) return;
     const int valid = min(RT, L - t0);
     const int group = a.hq / a.hkv;
-    const HeadSrc ks = find_head(a.plan->w[0], h), vs = find_head(a.plan->w[1], h);
+    HeadSrc ks, vs;
+    if (TMA) {  // the parameters say where a head's rows lie; a look-up in the device table would be a chain of loads
+        ks.col = src.col[0][h];
+        vs.col = src.col[1][h];
+    } else {
+        ks = find_head(a.plan->w[0], h);
+        vs = find_head(a.plan->w[1], h);
+    }
     const __nv_bfloat16 *kpool = reinterpret_cast<const __nv_bfloat16 *>(ks.pool) + ks.col;
     const __nv_bfloat16 *vpool = reinterpret_cast<const __nv_bfloat16 *>(vs.pool) + vs.col;
     const int32_t *bt = a.block_table + (int64_t)seq * a.max_pages_per_seq;
@@ -273,10 +280,10 @@ __global__ void __launch_bounds__(GQ_RW * 32) decode_raw_gq_kernel(const __grid_
     const uint32_t sbase = ((smem_addr(gq_smem) + 1023u) & ~1023u) + warp * GQ_WARP_SMEM;
     uint8_t *gbase = gq_smem + (sbase - smem_addr(gq_smem));
     const uint32_t bar0 = smem_addr(&step_bar[warp][0]);
-    const char *kmap = nullptr, *vmap = nullptr;
+    const CUtensorMap *kmap = nullptr, *vmap = nullptr;
     if (TMA) {
-        kmap = reinterpret_cast<const char *>(a.raw_tmaps) + (size_t)(ks.src_layer * 2) * 384;
-        vmap = reinterpret_cast<const char *>(a.raw_tmaps) + (size_t)(vs.src_layer * 2 + 1) * 384;
+        kmap = &src.map[0][src.idx[0][h]];
+        vmap = &src.map[1][src.idx[1][h]];
         if (lane == 0) {
             ptx::mbar_init(bar0, 1);
             ptx::mbar_init(bar0 + 8, 1);
@@ -442,7 +449,8 @@ bool raw_build_map(void *dst_host, const void *pool_dev, uint64_t rows, uint64_t
     return encode_bf16_map(fn, dst_host, pool_dev, rows, width, width, GQ_STEP);
 }
 
-cudaError_t launch_decode_raw(const DecodeArgs &a, const SeqList &seqs, int dtype, int grid_chunks, cudaStream_t st) {
+cudaError_t launch_decode_raw(const DecodeArgs &a, const SeqList &seqs, const RawSources *src, int dtype, int grid_chunks,
+                              cudaStream_t st) {
     dim3 grid(grid_chunks, (a.hkv + RW - 1) / RW, seqs.n);
     if (dtype == KVCAR_BF16) {
         static bool configured[64] = {};  // per device: the attribute belongs to the device's copy of the kernel
@@ -457,10 +465,10 @@ cudaError_t launch_decode_raw(const DecodeArgs &a, const SeqList &seqs, int dtyp
             if (dev >= 0 && dev < 64) configured[dev] = true;
         }
         grid.y = (a.hkv + GQ_RW - 1) / GQ_RW;
-        if (a.raw_tmaps && a.page_tokens % GQ_STEP == 0)
-            decode_raw_gq_kernel<true><<<grid, GQ_RW * 32, smem, st>>>(a, seqs);
+        if (src && a.page_tokens % GQ_STEP == 0)
+            decode_raw_gq_kernel<true><<<grid, GQ_RW * 32, smem, st>>>(a, seqs, *src);
         else
-            decode_raw_gq_kernel<false><<<grid, GQ_RW * 32, smem, st>>>(a, seqs);
+            decode_raw_gq_kernel<false><<<grid, GQ_RW * 32, smem, st>>>(a, seqs, RawSources{});
         return cudaGetLastError();
     }
     if (dtype == KVCAR_F32)

@@ -305,6 +305,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     }
     tc_fence_before();
     __syncthreads();
+    // The tensor maps of every source, before any thread of this block uses one: one map per thread, the barrier below
+    // orders the rest of the block behind it.
+    if (threadIdx.x < 2 * TC_MAX_SRC * 3) {
+        const int w_ = threadIdx.x / (TC_MAX_SRC * 3), s_ = threadIdx.x / 3 % TC_MAX_SRC, k_ = threadIdx.x % 3;
+        if (s_ < P.n_src[w_]) {
+            const TcSrc &sp = P.src[w_][s_];
+            tmap_acquire(k_ == 0 ? sp.tm_pool : k_ == 1 ? sp.tm_w1 : sp.tm_w2);
+        }
+    }
+    if (threadIdx.x == NTHREADS - 1 && lay.tm_wq) tmap_acquire(lay.tm_wq);
+    __syncthreads();
     cluster_sync_all();  // the peer's barriers and job tables exist before anyone signals or issues
     tc_fence_after();
     const uint32_t tmem = tmem_base_slot;
