@@ -11,6 +11,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "kvcar_internal.h"
+#include "kvcar_latent.h"
 #include "kvcar_tc.h"
 
 using namespace kvcar;
@@ -78,7 +79,7 @@ struct kvcar_ctx {
     std::vector<char> quant;                // [layer*2+which]: rows are int8 codes
     size_t pool_bytes = 0, weights_bytes = 0, ws_bytes = 0;
     size_t plan_off = 0, enc_off = 0, tmap_off = 0, tcpart_off = 0;  // inside weights
-    size_t bt_off = 0, len_off = 0, status_off = 0, part_off = 0, stage_off = 0, enchid_off = 0, kvsplit_off = 0, pfhid_off = 0, abs_off = 0;  // inside workspace
+    size_t bt_off = 0, len_off = 0, status_off = 0, part_off = 0, stage_off = 0, enchid_off = 0, kvsplit_off = 0, pfhid_off = 0, lat_off = 0;  // inside workspace
     int max_k_sources = 0;  // most distinct source layers any layer's K heads resolve to
     std::vector<RawSources> raw_src;  // [layer] tensor maps and head places of raw bf16 layers
     std::vector<char> raw_src_ok;     // [layer] filled (else the raw-row kernel stages with cp.async)
@@ -87,6 +88,8 @@ struct kvcar_ctx {
     int max_d = 0, max_m = 0, max_in = 0;
     std::vector<LayerPlan> plans_host;
     TcState tc;
+    LatState lat;
+    bool lat_used = false;  // the last tile launch was the latent kernel's: its merge follows
     float *static_scratch = nullptr;  // device address of the built-in scratch array, looked up at bind time
 
     int64_t launches = 0;
@@ -182,7 +185,11 @@ void compute_layout(kvcar_ctx *c) {
         size_t mats = (size_t)a.in_dim * a.hidden + (size_t)a.hidden * a.latent;  // one half (enc or dec)
         w = align_up(w + 2 * mats * c->elem, 256);                                 // transposed enc + dec
         w = align_up(w + (size_t)(4 * a.hidden + a.latent + a.in_dim) * sizeof(float), 256);  // s,t x2, b2 x2
-        if (g.storage == KVCAR_BF16) w = align_up(w + mats * 2, 256);             // K-major decoder copies
+        if (g.storage == KVCAR_BF16) {
+            w = align_up(w + mats * 2, 256);                                       // K-major decoder copies
+            w = align_up(w + (size_t)a.hidden * a.latent * 2, 256);                // FC1 of the latent-attention kernels
+            w = align_up(w + (size_t)(2 * ((a.hidden + 31) & ~31)) * sizeof(float), 256);
+        }
         w = align_up(w + mats * c->elem, 256);                                     // row-major encoder copies
     }
     c->plan_off = w;
@@ -190,7 +197,7 @@ void compute_layout(kvcar_ctx *c) {
     c->enc_off = w;
     w = align_up(w + (size_t)nl * 2 * sizeof(EncPlan), 256);
     c->tmap_off = w;  // TMA descriptors of the tensor-core kernel: pool, decoder FC1, decoder FC2 per (layer, which)
-    w = align_up(w + (size_t)nl * 2 * 3 * 128 + 128, 256);  // + the descriptor of the absorbed-score operands
+    w = align_up(w + (size_t)nl * 2 * 3 * 128, 256);
     c->tcpart_off = w;  // per-layer job tables of the tensor-core kernel
     w = align_up(w + tc_part_bytes(nl), 256);
     c->weights_bytes = w;
@@ -230,8 +237,8 @@ void compute_layout(kvcar_ctx *c) {
         }
         c->max_k_sources = std::max(c->max_k_sources, n);
     }
-    c->abs_off = s;  // operands of the absorbed K scores (tensor-core kernel, KVCAR_ABSORBED)
-    s = align_up(s + tc_absorb_bytes(g, c->max_k_sources, c->max_m, nb, c->max_chunks), 256);
+    c->lat_off = s;  // operands and partial results of the latent-attention kernels
+    s = align_up(s + lat_ws_bytes(g, c->max_k_sources, c->max_m, nb), 256);
     c->ws_bytes = s;
 }
 
@@ -259,6 +266,21 @@ void fuse_bn(const std::vector<float> &b1, const std::vector<float> &bn, int m, 
         double sc = gamma / std::sqrt(var + (double)eps);
         s[j] = (float)sc;
         t[j] = (float)(((double)b1[j] - mean) * sc + beta);
+    }
+}
+
+// First decoder layer for the latent-attention kernels.  LeakyReLU is positively homogeneous: with s the fused BatchNorm scale,
+// LeakyReLU(s x + t) = |s| LeakyReLU(sign(s) x + t / |s|).  The sign goes into the weight row (exact), t / |s| is the shift
+// that is left to the epilogue, |s| goes to the neighbours of the hidden vector (W4^T q and the weighted sum, both fp32).  A
+// scale too small to divide by leaves the constant LeakyReLU(t).
+void put_signed_fc1(char *dst, float *sabs, float *shift, const float *w, const float *s, const float *t, int m, int d) {
+    __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(dst);
+    for (int j = 0; j < m; ++j) {
+        const bool tiny = std::fabs(s[j]) < 1e-20f;
+        const float sign = tiny ? 0.f : s[j] < 0.f ? -1.f : 1.f;
+        sabs[j] = tiny ? 1.f : std::fabs(s[j]);
+        shift[shift_place(j)] = t[j] / sabs[j];
+        for (int k = 0; k < d; ++k) o[(size_t)j * d + k] = __float2bfloat16_rn(sign * w[(size_t)j * d + k]);
     }
 }
 
@@ -340,7 +362,7 @@ bool layer_is_raw(const kvcar_ctx *c, int layer) {
 
 bool use_tensor_kernel(const kvcar_ctx *c) {
     if (c->kernel == KVCAR_KERNEL_GENERIC) return false;
-    return c->tc.available;
+    return c->tc.available || c->lat.available;
 }
 
 // device address of the library's built-in scratch array on the current device (defined with the array, below)
@@ -479,7 +501,7 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
 
     std::vector<char> img(c->weights_bytes, 0);
     struct Packed {
-        size_t enc_w1t, enc_w2t, dec_w1t, dec_w2t, enc_s, enc_t, enc_b2, dec_s, dec_t, dec_b2, w1k, w2k, enc_w1r, enc_w2r;
+        size_t enc_w1t, enc_w2t, dec_w1t, dec_w2t, enc_s, enc_t, enc_b2, dec_s, dec_t, dec_b2, w1k, w2k, w1n, sabs, enc_w1r, enc_w2r;
     };
     std::vector<Packed> pk(nl * 2);
     size_t w = 0;
@@ -514,6 +536,13 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
             w = align_up(w + (M * D + I * M) * 2, 256);
             put_elems(&img[p.w1k], a.dec_w1.data(), M * D, KVCAR_BF16);
             put_elems(&img[p.w2k], a.dec_w2.data(), I * M, KVCAR_BF16);
+            p.w1n = w;
+            w = align_up(w + M * D * 2, 256);
+            p.sabs = w;  // then the shifts
+            const size_t M32 = (M + 31) & ~(size_t)31;
+            w = align_up(w + 2 * M32 * 4, 256);
+            put_signed_fc1(&img[p.w1n], (float *)&img[p.sabs], (float *)&img[p.sabs] + M32, a.dec_w1.data(),
+                           (const float *)&img[p.dec_s], (const float *)&img[p.dec_t], (int)M, (int)D);
         }
         p.enc_w1r = w;
         p.enc_w2r = p.enc_w1r + M * I * E;
@@ -561,6 +590,9 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
                         if (g.storage == KVCAR_BF16) {
                             sp.w1k = c->weights + pk[idx].w1k;
                             sp.w2k = c->weights + pk[idx].w2k;
+                            sp.w1n = c->weights + pk[idx].w1n;
+                            sp.sabs = (const float *)(c->weights + pk[idx].sabs);
+                            sp.shift = sp.sabs + ((a.hidden + 31) & ~31);
                         }
                     } else {
                         sp.d = sp.in_dim = sp.width;
@@ -577,11 +609,8 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
     // tensor maps and job tables of the tensor-core kernel (fills their regions of the image)
     tc_setup(c->tc, c->cfg, plans, nl, c->weights, c->tmap_off, c->tcpart_off, img.data(),
              (size_t)g.max_pages * g.page_tokens);
-    {
-        const size_t slot = c->tmap_off + (size_t)nl * 2 * 3 * 128;
-        tc_setup_absorb(c->tc, c->cfg, c->max_k_sources, c->max_m, std::min(g.max_seqs, KVCAR_MAX_BATCH), c->max_chunks,
-                        c->ws + c->abs_off, img.data() + slot, c->weights + slot);
-    }
+    lat_setup(c->lat, c->cfg, c->plans_host, (size_t)g.max_pages * g.page_tokens, c->max_k_sources, c->max_m,
+              std::min(g.max_seqs, KVCAR_MAX_BATCH), c->ws + c->lat_off);
     // tensor maps and head places of the raw layers (kernel parameters of the raw-row kernel)
     c->raw_src.assign(nl, RawSources{});
     c->raw_src_ok.assign(nl, 0);
@@ -642,6 +671,8 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
     cudaError_t e = cudaMemcpyAsync(c->weights, img.data(), img.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ws, 0, c->part_off, st);  // tables, lengths, status
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + c->kvsplit_off, 0, tc_split_bytes(g), st);  // hand-over flags
+    if (e == cudaSuccess && c->ws_bytes > c->lat_off)
+        e = cudaMemsetAsync(c->ws + c->lat_off, 0, c->ws_bytes - c->lat_off, st);  // operand rows of padding heads stay zero
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(c, e, "upload of packed weights");
     if (!c->side) {  // for kvcar_step_layer; without them it runs its launches in order on the caller's stream
@@ -687,7 +718,7 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
 
 kvcar_status kvcar_set_kernel(kvcar_ctx *c, int32_t kernel) {
     if (!c || kernel < 0 || kernel > 2) return fail(c, KVCAR_ERR_INVALID_ARG, "unknown kernel family");
-    if (kernel == KVCAR_KERNEL_TENSOR && c->bound && !c->tc.available)
+    if (kernel == KVCAR_KERNEL_TENSOR && c->bound && !c->tc.available && !c->lat.available)
         return fail(c, KVCAR_ERR_UNSUPPORTED, std::string("tensor-core kernel unavailable: ") + c->tc.why);
     c->kernel = kernel;
     return KVCAR_OK;
@@ -869,21 +900,32 @@ static int prepare_decode(kvcar_ctx *c, int32_t layer, const int32_t *seqs, int3
 // step's encoder writes (the exact current token enters in the combine kernel).
 static kvcar_status enqueue_decode_tiles(kvcar_ctx *c, int32_t layer, const DecodeArgs &a, const SeqList &sl,
                                          int n_chunks, cudaStream_t st) {
-    c->tc.last_mode = 0;
+    c->lat_used = false;
     if (n_chunks <= 0) return KVCAR_OK;
     const kvcar_config &g = c->cfg;
+    int n_tiles = 0;
+    for (int i = 0; i < sl.n; ++i) n_tiles += (c->len[sl.id[i]] + 127) / 128;
     const bool want_tc = use_tensor_kernel(c) && tc_layer_supported(c->tc, layer);
-    if (c->kernel == KVCAR_KERNEL_TENSOR && !want_tc)
+    bool want_lat = use_tensor_kernel(c) && lat_layer_supported(c->lat, layer, a.flags);
+    // Few tiles leave most of the latent kernel's clusters without work while the restoring kernel spreads a pair of tiles over
+    // several: at 64 tiles of the GPT-2 shape a 12-layer step takes 712 us here and 688 us there, at 128 tiles 814 and 971; at
+    // 128 tiles of the TinyLLaMA shape 868 and 786, at 256 tiles 1024 and 1118.
+    if (want_lat && want_tc && !(a.flags & KVCAR_ABSORBED) && n_tiles < (c->lat.cfg[layer].max_m > 192 ? 80 : 148)) want_lat = false;
+    if (c->kernel == KVCAR_KERNEL_TENSOR && !want_tc && !want_lat)
         return fail(c, KVCAR_ERR_UNSUPPORTED, std::string("tensor-core kernel cannot run this layer: ") + c->tc.why);
     cudaError_t e;
     if (c->kernel != KVCAR_KERNEL_GENERIC && layer_is_raw(c, layer)) {
         e = launch_decode_raw(a, sl, c->raw_src_ok[layer] ? &c->raw_src[layer] : nullptr, g.storage, n_chunks, st);
+    } else if (want_lat) {
+        int32_t lens[KVCAR_MAX_BATCH];
+        for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
+        e = lat_launch_tiles(c->lat, a, sl, lens, layer, st);
+        c->lat_used = true;
+        ++c->launches;
     } else if (want_tc) {
         int32_t lens[KVCAR_MAX_BATCH];
         for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
-        int n_launches = 1;
-        e = tc_launch_decode(c->tc, a, sl, lens, layer, st, &n_launches);
-        if (e == cudaSuccess) c->launches += n_launches - 1;
+        e = tc_launch_decode(c->tc, a, sl, lens, layer, st);
     } else {
         if (decode_generic_smem(a.hq, a.hd, c->max_d, c->max_m) > 227 * 1024)
             return fail(c, KVCAR_ERR_UNSUPPORTED, "shape needs more shared memory than one SM has");
@@ -894,10 +936,15 @@ static kvcar_status enqueue_decode_tiles(kvcar_ctx *c, int32_t layer, const Deco
     return KVCAR_OK;
 }
 
-static kvcar_status enqueue_combine(kvcar_ctx *c, const DecodeArgs &a, const SeqList &sl, int n_chunks, cudaStream_t st) {
-    // a tile launch in the absorbed V form left U vectors, not weighted values: its own merge kernel reads them
-    cudaError_t e = c->tc.last_mode == 2 ? tc_launch_combine_absorbed(c->tc, a, sl, st)
-                                         : launch_combine(a, sl, c->cfg.storage, n_chunks, st);
+static kvcar_status enqueue_combine(kvcar_ctx *c, int32_t layer, const DecodeArgs &a, const SeqList &sl, int n_chunks, cudaStream_t st) {
+    cudaError_t e;
+    if (c->lat_used) {
+        int32_t lens[KVCAR_MAX_BATCH];
+        for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
+        e = lat_launch_merge(c->lat, a, sl, lens, layer, st);
+    } else {
+        e = launch_combine(a, sl, c->cfg.storage, n_chunks, st);
+    }
     if (e != cudaSuccess) return cuda_fail(c, e, "combine launch");
     ++c->launches;
     return KVCAR_OK;
@@ -928,7 +975,7 @@ kvcar_status kvcar_decode_attention(kvcar_ctx *c, int32_t layer, const int32_t *
     const int n_chunks = prepare_decode(c, layer, seqs, n_seqs, q, out, flags, a, sl);
     s = enqueue_decode_tiles(c, layer, a, sl, n_chunks, st);
     if (s != KVCAR_OK) return s;
-    return enqueue_combine(c, a, sl, n_chunks, st);
+    return enqueue_combine(c, layer, a, sl, n_chunks, st);
 }
 
 kvcar_status kvcar_step_layer(kvcar_ctx *c, int32_t layer, const int32_t *seqs, int32_t n_seqs, const void *k,
@@ -974,7 +1021,7 @@ kvcar_status kvcar_step_layer(kvcar_ctx *c, int32_t layer, const int32_t *seqs, 
         s = enqueue_decode_tiles(c, layer, a, sl, n_chunks, st);
         if (s != KVCAR_OK) return s;
     }
-    return enqueue_combine(c, a, sl, n_chunks, st);
+    return enqueue_combine(c, layer, a, sl, n_chunks, st);
 }
 
 kvcar_status kvcar_step_layer_host(kvcar_ctx *c, int32_t layer, const int32_t *seqs, int32_t n_seqs,
@@ -1146,7 +1193,7 @@ kvcar_status kvcar_layer_kernel(kvcar_ctx *c, int32_t layer, int32_t *kernel) {
     if (c->kernel != KVCAR_KERNEL_GENERIC && layer_is_raw(c, layer))
         *kernel = KVCAR_KERNEL_RAW;
     else
-        *kernel = (use_tensor_kernel(c) && tc_layer_supported(c->tc, layer)) ? KVCAR_KERNEL_TENSOR : KVCAR_KERNEL_GENERIC;
+        *kernel = (use_tensor_kernel(c) && (lat_layer_supported(c->lat, layer, 0) || tc_layer_supported(c->tc, layer))) ? KVCAR_KERNEL_TENSOR : KVCAR_KERNEL_GENERIC;
     return KVCAR_OK;
 }
 

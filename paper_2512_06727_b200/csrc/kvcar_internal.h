@@ -25,6 +25,10 @@ struct SourcePlan {
     const void *w1k;   // K-major bf16 copies for the tensor-core kernel: [m][d]
     const void *w2k;   //                                                  [in_dim][m]
     const float *qparam;  // int8 rows: (scale, zero-point) per pool row, else null
+    // latent-attention kernels (bf16): decoder FC1 [m][d] with the signs of the BatchNorm scale taken into its rows, the
+    // sizes of the scale [m], and the shift over them (in the kernels' own order)
+    const void *w1n;
+    const float *sabs, *shift;
     int32_t width;     // elements per pool row (= d if compressed, = in_dim if raw)
     int32_t d, m, in_dim;
     int32_t compressed;

@@ -1,0 +1,1242 @@
+// Decode attention over latent rows without restored K and V rows (bf16 storage, sm_100a).
+//
+// The decoder of a (layer, K/V) is FC -> BatchNorm -> LeakyReLU -> FC with nothing after the last FC (Sec. "Network
+// Architecture").  With a the activated hidden vector of a cached token,
+//     q . k'   = q . (W4_h a + b4_h)     = a . (W4_h^T q) + q . b4_h
+//     sum p v' = sum p (W4_h a + b4_h)   = W4_h (sum p a) + b4_h sum p
+// so the last layer is applied once per sequence and head (to the query before the tiles, to the weighted sum after
+// them) instead of once per token: at the GPT-2 shape 0.91 instead of 2.66 MFLOP per cached token and layer, and the
+// epilogues that consumed restored rows go away.  W4_h^T q and the probabilities enter their products as two bf16
+// terms (value = high + low, 16 bits and the sign; what is left out is 2^-18 of the value, against the 2^-9 that the
+// bf16 hidden vector itself carries), so nothing is rounded more coarsely than in the form that restores the rows;
+// with KVCAR_ABSORBED (| KVCAR_ABSORBED_V) the caller takes one bf16 term, as that flag says.
+//
+// Three launches per call:
+//   latent_query_kernel   W4_h^T q per (K source, listed sequence, query head) -> bf16 rows, high and low part
+//   decode_latent_kernel  tiles of 128 cached tokens -> per run of tiles: reference maximum, sum, U = sum p a
+//   latent_merge_kernel   runs of a sequence -> W4_h U + b4_h sum, the exact current token, the output row
+//
+// decode_latent_kernel.  A cluster of two CTAs walks two runs of consecutive tiles in step, one run per CTA; every
+// product is one tcgen05.mma.cta_group::2 of M = 256 (both tiles), so a weight slab crosses L2 -> shared memory once
+// per 256 tokens, half into each CTA.  Per tile, K side then V side, per source layer, per chunk of 192 hidden columns:
+//   hidden   H[256 tok x 192] = Z[256 tok x d] . W1[192 x d]^T into one of two accumulators in tensor memory; the hidden
+//            warps add the shift, apply LeakyReLU, round to bf16 and write 64-column slabs into a ring.  The BatchNorm
+//            scale is not theirs: its sign is in W1, its size in W4^T q and in the merge (LeakyReLU is positively
+//            homogeneous).  The accumulator is read in matrix-fragment layout: a lane needs eight shifts instead of 32
+//            (scale and shift fetched per column took 750-900 of a slab's 1 300 cycles) and stores with stmatrix.
+//   K side   S[256 tok x 2R] += slab . (W4^T q rows)^T, over all sources: rows of heads that another source serves are
+//            zero, so the sources simply add up.  Columns R r .. belong to CTA r (its own sequence's queries)
+//   V side   per two slabs: U[256 x 2R] = (slab pair)^T [128 features] . P^T over the tile's 128 tokens.  Each CTA supplies
+//            its own hidden slabs and its own probabilities, so in its accumulator its own R columns are its tile's
+// S and the U blocks share two 64-column accumulators in turn; the output warps turn S into probabilities and keep the
+// running sums of U in registers over a run, rescaled when the reference maximum moves (online softmax), so only one
+// partial result per (CTA, sequence) leaves the SM.
+//
+// What bounds it at the GPT-2 shape (d 384, m 576, 12 heads): the tensor pipe.  A product of M 256 x N x K 16 takes
+// max(53, N / 2) cycles (measured alone, whatever the operands' layout), so a pair of tiles needs 2 x 72 x 96 for the hidden
+// layers, 36 x 53 for S and 40 x 53 for U: 17 900 cycles.  The latents stay in shared memory for all chunks of a side (96 KB),
+// which leaves 64 KB for hidden slabs and 48 KB for weight slabs; 192 columns per chunk because 2 x 192 + 2 x 64 fill
+// tensor memory.
+//
+// Two warps issue products, one the hidden jobs, one S and U: with a single issuing thread the two took turns (6 800
+// cycles per chunk, 2 700 of them pipe time), and each waited for what only the other needed.  A warp of the hidden
+// epilogue takes one slab of a job (three slabs, four lane quarters: twelve warps).
+//
+// Warp roles: 0 loads of latents, query rows and shifts, 1 hidden products (leader CTA) and tensor memory, 2 weight loads,
+// 3 S and U products (leader CTA), 4-15 hidden warps, 16-23 output warps.  All waits are bounded and record a code in the
+// status word.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
+#include "kvcar_latent.h"
+#include "kvcar_ptx.cuh"
+
+namespace kvcar {
+
+using namespace ptx;
+
+namespace {
+
+constexpr int TILE = 128;                 // tokens per CTA tile
+constexpr int SLAB = 16384;               // 128 rows x 64 bf16, 128-byte swizzle
+constexpr int CN = 192;                   // hidden columns per job
+constexpr int CSLABS = CN / 64;
+constexpr int WSTAGE = CN / 2 * 128;      // this CTA's half of a weight slab
+constexpr int TM_OUT = 2 * CN;            // tensor-memory columns: hidden 0, 192; outputs 384, 448
+constexpr int HID_WARP = 4, N_HID = 4 * CSLABS, OUT_WARP = HID_WARP + N_HID, N_OUT = 8, N_WARPS = OUT_WARP + N_OUT;
+constexpr int NTHREADS = 32 * N_WARPS;
+constexpr int READY_BARS = 8;             // hidden jobs between their epilogue and their product: at most as many as slabs
+
+// Query heads padded to NQ.  Up to 16: high and low terms of an operand are rows of one operand.  32: the terms of W4^T q
+// are two operands, and the probabilities have one term (groups of more than two heads, whose restoring form rounds
+// restored K, restored V and the probabilities to bf16: the same class).
+__host__ __device__ constexpr int op_rows(int nq) { return nq <= 16 ? 2 * nq : nq; }  // operand rows of a CTA in S and U
+__host__ __device__ constexpr int wq_rows(int nq) { return 2 * nq; }                  // rows of W4^T q per sequence and source
+__host__ __device__ constexpr int wq_slab(int nq) { return wq_rows(nq) * 128; }       // one 64-column slab of them
+
+struct Params {
+    LatLayer l;
+    CUtensorMap tm_wq;
+    LatSeqs sq;
+    const int32_t *block_table;
+    int32_t *status;
+    float *upart, *ml;
+    int32_t max_pages_per_seq, page_tokens;
+    int32_t hq, m_pad, wq_batch;
+    int32_t nz, nh, nw, nqs, nt, m_t;  // places for latent, hidden, weight and query slabs; shift buffers and their floats
+    int32_t t_resident;                // every source has a shift buffer of its own
+    int32_t two_terms_k, two_terms_v;  // low parts of the query rows / of the probabilities are used
+};
+
+template <int SLEEP_NS = 0>
+__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int32_t *status, volatile int *abort_flag, int code) {
+    if (mbar_try(bar, parity)) return;
+    uint32_t n = 0;
+    uint64_t t0 = 0;
+    while (true) {
+        if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
+        if (mbar_try(bar, parity)) return;
+        if ((++n & 255u) == 0) {
+            const uint64_t now = global_ns();
+            if (t0 == 0) t0 = now;
+            if (now - t0 > (*abort_flag ? 2000000ull : 2000000000ull)) {  // 2 ms after a failure, else 2 s
+                *abort_flag = 1;
+                atomicCAS(status, 0, code);
+                return;
+            }
+        }
+    }
+}
+
+// the tiles of one CTA, in order
+struct TileWalk {
+    int si, chunk, n, left;  // listed sequence, tile inside it, its tiles, tiles left of the run (this one included)
+    __device__ __forceinline__ int first(const LatSeqs &sq, int i) const { return (int)(sq.first[i] & 0xffffffu); }
+    __device__ __forceinline__ void idle() { si = chunk = left = 0; n = 1; }
+    __device__ __forceinline__ void start(const LatSeqs &sq, int t) {
+        idle();
+        if (t >= sq.n_tiles) return;
+        left = min(sq.per, sq.n_tiles - t);
+        int lo = 0, hi = sq.n;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (first(sq, mid) <= t) lo = mid; else hi = mid;
+        }
+        si = lo;
+        chunk = t - first(sq, lo);
+        n = first(sq, lo + 1) - first(sq, lo);
+    }
+    __device__ __forceinline__ int valid(const LatSeqs &sq) const {
+        return left == 0 ? 0 : chunk + 1 < n ? TILE : (int)(sq.first[si] >> 24) + 1;
+    }
+    __device__ __forceinline__ bool ends_run() const { return left == 1 || (left > 0 && chunk + 1 == n); }
+    __device__ __forceinline__ void next(const LatSeqs &sq) {
+        if (left == 0) return;
+        if (--left == 0) {
+            idle();
+            return;
+        }
+        if (++chunk == n) {
+            do {
+                ++si;
+                n = first(sq, si + 1) - first(sq, si);
+            } while (n == 0);
+            chunk = 0;
+        }
+    }
+};
+
+__device__ __forceinline__ float redux_max(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+// N values per lane (N = 6, 8 or 16): afterwards lane L holds the maximum over the warp of value L (L < N); halves the values
+// while it halves the lanes' distance, so about N shuffles instead of 5 N
+template <int N>
+__device__ __forceinline__ float max_over_lanes(const float *v, int lane) {
+    constexpr int P = N <= 8 ? 8 : 16;
+    float x[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) x[i] = i < N ? v[i] : -INFINITY;
+#pragma unroll
+    for (int w = P / 2; w > 0; w >>= 1) {
+        const bool up = (lane & w) != 0;
+#pragma unroll
+        for (int i = 0; i < w; ++i) {
+            const float keep = up ? x[i + w] : x[i], give = up ? x[i] : x[i + w];
+            x[i] = fmaxf(keep, __shfl_xor_sync(0xffffffffu, give, w));
+        }
+    }
+#pragma unroll
+    for (int w = P; w < 32; w <<= 1) x[0] = fmaxf(x[0], __shfl_xor_sync(0xffffffffu, x[0], w));
+    return x[0];
+}
+__device__ __forceinline__ float ex2(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// `bytes` (a multiple of 16, both addresses 16-byte aligned) into this CTA's shared memory, counted on a barrier of it
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+                 "r"(bytes), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void stmatrix_x4(uint32_t addr, const uint32_t *w) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                 : "memory");
+}
+__device__ __forceinline__ void st_smem_u16(uint32_t addr, uint16_t v) {
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(v) : "memory");
+}
+
+// what the warps share besides operands and barriers (everything is dynamic shared memory, so that the operand places
+// start at an aligned address and nothing is lost to padding)
+template <int NQ>
+struct __align__(8) Scratch {
+    uint32_t tmem_slot;
+    int abort_flag;
+    float mrun[2][NQ];    // by tile parity: reference maximum before the tile
+    float red[2][NQ][4];  // by tile parity: maxima of the four lane quarters
+    float lred[NQ][4];    // sums of the four lane quarters at the end of a run
+};
+
+// NQ: query heads padded.  NB: U blocks of 128 hidden features at most; fixes the registers of the running sums.
+template <int NQ, int NB>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
+    decode_latent_kernel(const __grid_constant__ Params a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    constexpr int R = op_rows(NQ), PSLAB = R * 128, QSLAB = wq_slab(NQ);
+
+    const uint32_t rank = blockIdx.x & 1u;
+    const bool leader = rank == 0;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t s_z = smem_u32(smem_raw), s_h = s_z + a.nz * SLAB, s_w = s_h + a.nh * SLAB, s_q = s_w + a.nw * WSTAGE;
+    const uint32_t s_p = s_q + a.nqs * QSLAB, s_t = s_p + 2 * PSLAB, s_bar = s_t + a.nt * a.m_t * 4;
+    const uint32_t w_full = s_bar, w_empty = w_full + 8 * a.nw;
+    const uint32_t z_full = w_empty + 8 * a.nw, z_empty = z_full + 8 * a.nz;
+    const uint32_t q_full = z_empty + 8 * a.nz, q_empty = q_full + 8 * a.nqs;
+    const uint32_t tb_full = q_empty + 8 * a.nqs, tb_empty = tb_full + 8 * a.nt;
+    const uint32_t h_ready = tb_empty + 8 * a.nt, h_free = h_ready + 8 * READY_BARS;
+    const uint32_t t_full = h_free + 8 * a.nh, t_empty = t_full + 16, o_full = t_empty + 16, o_empty = o_full + 16;
+    const uint32_t p_ready = o_empty + 16;
+    Scratch<NQ> &sh = *reinterpret_cast<Scratch<NQ> *>(smem_raw + (p_ready + 8 - s_z));
+    volatile int &abort_flag = sh.abort_flag;
+    // tiles of the cluster's longer run (the leader's); the other CTA idles through the last ones it does not have
+    const int cta0 = (int)(blockIdx.x & ~1u);
+    const int n_it = max(0, min(a.sq.per, a.sq.n_tiles - cta0 * a.sq.per));
+    const int my_first = (int)blockIdx.x * a.sq.per;
+
+    if (threadIdx.x == 0) {
+        sh.abort_flag = 0;
+        for (int i = 0; i < a.nw; ++i) {
+            mbar_init(w_full + 8 * i, 1);
+            mbar_init(w_empty + 8 * i, 1);
+        }
+        for (int i = 0; i < a.nz; ++i) {
+            mbar_init(z_full + 8 * i, 1);
+            mbar_init(z_empty + 8 * i, 1);
+        }
+        for (int i = 0; i < a.nqs; ++i) {
+            mbar_init(q_full + 8 * i, 1);
+            mbar_init(q_empty + 8 * i, 1);
+        }
+        for (int i = 0; i < a.nt; ++i) {
+            mbar_init(tb_full + 8 * i, 1);
+            mbar_init(tb_empty + 8 * i, N_HID);
+        }
+        for (int i = 0; i < a.nh; ++i) mbar_init(h_free + 8 * i, 1);
+        for (int i = 0; i < READY_BARS; ++i) mbar_init(h_ready + 8 * i, 2 * N_HID);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(t_full + 8 * i, 1);
+            mbar_init(t_empty + 8 * i, 2 * N_HID);
+            mbar_init(o_full + 8 * i, 1);
+            mbar_init(o_empty + 8 * i, 2 * N_OUT);
+        }
+        mbar_init(p_ready, 2 * N_OUT);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (threadIdx.x < 2 * NQ) sh.mrun[threadIdx.x / NQ][threadIdx.x % NQ] = -INFINITY;
+    if (warp == 1) {  // all of tensor memory in both CTAs (one CTA per SM by shared memory)
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_slot)), "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();  // both CTAs' barriers exist before either signals the other's
+    tc_fence_after();
+    const uint32_t tmem = sh.tmem_slot;
+
+    if (warp == 0) {
+        // ============================== latents, query rows, shifts ==============================
+        // Three independent streams of loads, each into its own ring; one thread looks at the rings in turn and fills the
+        // one that has a place.
+        if (elect_one()) {
+            auto rows_of = [&](const TileWalk &t, int *r) {  // pool rows of the tile's two 64-token halves
+                r[0] = r[1] = 0;
+                const int v = t.valid(a.sq);
+                for (int h = 0; h < 2; ++h) {
+                    if (v == 0) break;
+                    int tok = t.chunk * TILE + 64 * h;
+                    if (64 * h >= v) tok = t.chunk * TILE;  // no valid token there: re-read the first half
+                    const int page = a.block_table[(int64_t)a.sq.id[t.si] * a.max_pages_per_seq + tok / a.page_tokens];
+                    r[h] = page * a.page_tokens + tok % a.page_tokens;
+                }
+            };
+            struct Pos {
+                int it, side, s, k;
+            };
+            Pos z{0, 0, 0, 0}, q{0, 0, 0, 0}, t{0, 0, 0, 0};
+            uint32_t zslot = 0, zphase = 0, qslot = 0, qphase = 0, tslot = 0, tphase = 0;
+            TileWalk zw, qw;
+            zw.start(a.sq, my_first);
+            qw = zw;
+            int row[2], nrow[2];
+            rows_of(zw, row);
+            const bool low_k = NQ <= 16 || a.two_terms_k;
+            const int t_its = a.t_resident ? min(1, n_it) : n_it;
+            uint32_t idle = 0;
+            uint64_t t0 = 0;
+            while (z.it < n_it || q.it < n_it || t.it < t_its) {
+                bool moved = false;
+                if (z.it < n_it && mbar_test(z_empty + 8 * zslot, zphase ^ 1u)) {
+                    moved = true;
+                    if (leader) mbar_expect_tx(z_full + 8 * zslot, 2 * SLAB);
+                    const CUtensorMap *map = &a.l.pool[z.side][z.s];
+                    const uint32_t fb = map_to_cta(z_full + 8 * zslot, 0), dst = s_z + zslot * SLAB;
+                    tma_load_2d_pair(dst, map, z.k * 64, row[0], fb);
+                    tma_load_2d_pair(dst + SLAB / 2, map, z.k * 64, row[1], fb);
+                    if (++zslot == (uint32_t)a.nz) { zslot = 0; zphase ^= 1u; }
+                    const int ks1 = (a.l.src[z.side][z.s].d + 63) >> 6;
+                    if (++z.k == ks1) {
+                        // the same rows of the next tile: from HBM into L2 while this one is worked on
+                        if (z.side == 0 && z.s == 0) {
+                            zw.next(a.sq);
+                            rows_of(zw, nrow);
+                        }
+                        if (zw.left > 0)
+                            for (int ks = 0; ks < ks1; ++ks) {
+                                tma_prefetch_2d(map, ks * 64, nrow[0]);
+                                if (nrow[1] != nrow[0]) tma_prefetch_2d(map, ks * 64, nrow[1]);
+                            }
+                        z.k = 0;
+                        if (++z.s == a.l.n_src[z.side]) {
+                            z.s = 0;
+                            if (++z.side == 2) {
+                                z.side = 0;
+                                ++z.it;
+                                row[0] = nrow[0];
+                                row[1] = nrow[1];
+                            }
+                        }
+                    }
+                }
+                if (t.it < t_its && mbar_test(tb_empty + 8 * tslot, tphase ^ 1u)) {
+                    moved = true;
+                    const LatSrc &sp = a.l.src[t.side][t.s];
+                    const uint32_t bytes = (uint32_t)((sp.m + 31) & ~31) * 4u;
+                    mbar_expect_tx(tb_full + 8 * tslot, bytes);
+                    bulk_load(s_t + tslot * a.m_t * 4, sp.shift, bytes, tb_full + 8 * tslot);
+                    if (++tslot == (uint32_t)a.nt) { tslot = 0; tphase ^= 1u; }
+                    if (++t.s == a.l.n_src[t.side]) {
+                        t.s = 0;
+                        if (++t.side == 2) {
+                            t.side = 0;
+                            ++t.it;
+                        }
+                    }
+                }
+                if (q.it < n_it && mbar_test(q_empty + 8 * qslot, qphase ^ 1u)) {
+                    moved = true;
+                    const int y = (q.s * a.wq_batch + qw.si) * wq_rows(NQ);
+                    if (leader) mbar_expect_tx(q_full + 8 * qslot, low_k ? 2 * QSLAB : QSLAB);
+                    const uint32_t fb = map_to_cta(q_full + 8 * qslot, 0), dst = s_q + qslot * QSLAB;
+                    tma_load_2d_pair(dst, &a.tm_wq, q.k * 64, y, fb);
+                    if (NQ > 16 && low_k) tma_load_2d_pair(dst + QSLAB / 2, &a.tm_wq, q.k * 64, y + R, fb);
+                    if (++qslot == (uint32_t)a.nqs) { qslot = 0; qphase ^= 1u; }
+                    if (++q.k == (a.l.src[0][q.s].m + 63) >> 6) {
+                        q.k = 0;
+                        if (++q.s == a.l.n_src[0]) {
+                            q.s = 0;
+                            ++q.it;
+                            qw.next(a.sq);
+                        }
+                    }
+                }
+                if (moved) {
+                    t0 = 0;
+                    idle = 0;
+                } else {
+                    __nanosleep(20);
+                    if ((++idle & 255u) == 0) {
+                        const uint64_t now = global_ns();
+                        if (t0 == 0) t0 = now;
+                        if (now - t0 > (abort_flag ? 2000000ull : 2000000000ull)) {
+                            abort_flag = 1;
+                            atomicCAS(a.status, 0, 0x601);
+                            break;
+                        }
+                    }
+                }
+            }
+        }
+    } else if (warp == 2) {
+        // ============================== weight loads ==============================
+        if (elect_one()) {
+            uint32_t slot = 0, phase = 0;
+            for (int it = 0; it < n_it; ++it)
+                for (int side = 0; side < 2; ++side)
+                    for (int s = 0; s < a.l.n_src[side]; ++s) {
+                        const int ks1 = (a.l.src[side][s].d + 63) >> 6, m = a.l.src[side][s].m;
+                        const CUtensorMap *map = &a.l.w1[side][s];
+                        for (int c0 = 0; c0 < m; c0 += CN) {
+                            const int y = c0 + (int)rank * (min(CN, m - c0) >> 1);
+                            for (int ks = 0; ks < ks1; ++ks) {
+                                mbar_wait<32>(w_empty + 8 * slot, phase ^ 1u, a.status, &abort_flag, 0x602);
+                                if (leader) mbar_expect_tx(w_full + 8 * slot, 2 * WSTAGE);
+                                tma_load_2d_pair(s_w + slot * WSTAGE, map, ks * 64, y, map_to_cta(w_full + 8 * slot, 0));
+                                if (++slot == (uint32_t)a.nw) { slot = 0; phase ^= 1u; }
+                            }
+                        }
+                    }
+        }
+    } else if (warp == 1) {
+        // ============================== hidden products (leader CTA) ==============================
+        if (leader && elect_one()) {
+            uint32_t wslot = 0, wphase = 0, zslot = 0, zphase = 0, h = 0;
+            const uint64_t z_desc = make_desc(s_z), w_desc = make_desc(s_w);
+            for (int it = 0; it < n_it; ++it)
+                for (int side = 0; side < 2; ++side)
+                    for (int s = 0; s < a.l.n_src[side]; ++s) {
+                        const int d = a.l.src[side][s].d, m = a.l.src[side][s].m;
+                        const int ks1 = (d + 63) >> 6, nk_last = ((d - 1) & 63) / 16 + 1;
+                        uint32_t zs = 0, zp = 0;
+                        for (int c0 = 0; c0 < m; c0 += CN, ++h) {
+                            const bool first = c0 == 0, last = c0 + CN >= m;
+                            const uint32_t buf = h & 1u, acc = tmem + CN * buf, idesc = make_idesc(256, min(CN, m - c0));
+                            mbar_wait(t_empty + 8 * buf, ((h >> 1) & 1u) ^ 1u, a.status, &abort_flag, 0x607);
+                            tc_fence_after();
+                            zs = zslot;  // the source's latent slabs: places zslot ..
+                            zp = zphase;
+#pragma unroll 1
+                            for (int ks = 0; ks < ks1; ++ks) {
+                                if (first) mbar_wait(z_full + 8 * zs, zp, a.status, &abort_flag, 0x608);
+                                mbar_wait(w_full + 8 * wslot, wphase, a.status, &abort_flag, 0x603);
+                                const uint64_t da = z_desc + zs * (SLAB >> 4), db = w_desc + wslot * (WSTAGE >> 4);
+                                if (ks == 0)
+                                    umma_pair<0>(acc, da, db, idesc);
+                                else
+                                    umma_pair<1>(acc, da, db, idesc);
+                                if (ks + 1 < ks1 || nk_last == 4) {
+                                    umma_pair<1>(acc, da + 2u, db + 2u, idesc);
+                                    umma_pair<1>(acc, da + 4u, db + 4u, idesc);
+                                    umma_pair<1>(acc, da + 6u, db + 6u, idesc);
+                                } else {
+                                    for (int t = 1; t < nk_last; ++t) umma_pair<1>(acc, da + 2u * t, db + 2u * t, idesc);
+                                }
+                                umma_commit_pair(w_empty + 8 * wslot);
+                                if (last) umma_commit_pair(z_empty + 8 * zs);
+                                if (++wslot == (uint32_t)a.nw) { wslot = 0; wphase ^= 1u; }
+                                if (++zs == (uint32_t)a.nz) { zs = 0; zp ^= 1u; }
+                            }
+                            umma_commit_pair(t_full + 8 * buf);
+                        }
+                        zslot = zs;
+                        zphase = zp;
+                    }
+        }
+    } else if (warp == 3) {
+        // ============================== S and U products (leader CTA) ==============================
+        if (leader && elect_one()) {
+            uint32_t qslot = 0, qphase = 0, hslot = 0, h = 0, o = 0;
+            constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(2 * R >> 3) << 17) | (16u << 24);
+            constexpr uint32_t idesc_u = idesc | (1u << 15);  // row operand MN-major
+            const uint64_t h_desc = make_desc(s_h), q_desc = make_desc(s_q), p_desc = make_desc(s_p);
+            const bool two = NQ > 16 && a.two_terms_k;
+            for (int it = 0; it < n_it; ++it) {
+                {  // S
+                    const uint32_t ob = o & 1u, acc = tmem + TM_OUT + 64u * ob;
+                    mbar_wait(o_empty + 8 * ob, ((o >> 1) & 1u) ^ 1u, a.status, &abort_flag, 0x605);
+                    bool begin = true;
+                    for (int s = 0; s < a.l.n_src[0]; ++s) {
+                        const int m = a.l.src[0][s].m, ksm = (m + 63) >> 6, nk_last = ((m - 1) & 63) / 16 + 1;
+#pragma unroll 1
+                        for (int sl = 0, in_job = 0; sl < ksm; ++sl) {
+                            if (in_job == 0) {  // the job's slabs, written by both CTAs
+                                mbar_wait(h_ready + 8 * (h & 7u), (h >> 3) & 1u, a.status, &abort_flag, 0x604);
+                                tc_fence_after();
+                                ++h;
+                            }
+                            if (++in_job == CSLABS) in_job = 0;
+                            mbar_wait(q_full + 8 * qslot, qphase, a.status, &abort_flag, 0x60e);
+                            const uint64_t da = h_desc + hslot * (SLAB >> 4), db = q_desc + qslot * (QSLAB >> 4);
+                            if (begin)
+                                umma_pair<0>(acc, da, db, idesc);
+                            else
+                                umma_pair<1>(acc, da, db, idesc);
+                            begin = false;
+                            const int nk = sl + 1 < ksm ? 4 : nk_last;
+                            if (nk > 1) umma_pair<1>(acc, da + 2u, db + 2u, idesc);
+                            if (nk > 2) umma_pair<1>(acc, da + 4u, db + 4u, idesc);
+                            if (nk > 3) umma_pair<1>(acc, da + 6u, db + 6u, idesc);
+                            if (two) {
+                                const uint64_t dl = db + (QSLAB / 2 >> 4);
+                                umma_pair<1>(acc, da, dl, idesc);
+                                if (nk > 1) umma_pair<1>(acc, da + 2u, dl + 2u, idesc);
+                                if (nk > 2) umma_pair<1>(acc, da + 4u, dl + 4u, idesc);
+                                if (nk > 3) umma_pair<1>(acc, da + 6u, dl + 6u, idesc);
+                            }
+                            umma_commit_pair(h_free + 8 * hslot);
+                            umma_commit_pair(q_empty + 8 * qslot);
+                            if (++hslot == (uint32_t)a.nh) hslot = 0;
+                            if (++qslot == (uint32_t)a.nqs) { qslot = 0; qphase ^= 1u; }
+                        }
+                    }
+                    umma_commit_pair(o_full + 8 * ob);
+                    ++o;
+                }
+                bool p_seen = false;
+                for (int s = 0; s < a.l.n_src[1]; ++s) {  // U
+                    const int ksm = (a.l.src[1][s].m + 63) >> 6;
+                    hslot += hslot & 1u;  // slabs go in pairs: a source starts at an even place
+                    if (hslot == (uint32_t)a.nh) hslot = 0;
+#pragma unroll 1
+                    for (int sl = 0, in_job = 0; sl < ksm; ++sl) {
+                        if (in_job == 0) {
+                            mbar_wait(h_ready + 8 * (h & 7u), (h >> 3) & 1u, a.status, &abort_flag, 0x604);
+                            tc_fence_after();
+                            ++h;
+                        }
+                        if (++in_job == CSLABS) in_job = 0;
+                        const uint32_t hs = hslot;
+                        if (++hslot == (uint32_t)a.nh) hslot = 0;
+                        if (!(sl & 1) && sl + 1 < ksm) continue;
+                        if (!p_seen) {
+                            mbar_wait(p_ready, (uint32_t)it & 1u, a.status, &abort_flag, 0x606);
+                            p_seen = true;
+                        }
+                        const uint32_t ob = o & 1u, accu = tmem + TM_OUT + 64u * ob, h0 = hs & ~1u;
+                        mbar_wait(o_empty + 8 * ob, ((o >> 1) & 1u) ^ 1u, a.status, &abort_flag, 0x605);
+                        tc_fence_after();
+                        // rows = features: two 64-feature atoms a slab apart, 8-token groups 1 KB apart (MN-major)
+                        uint64_t da = h_desc + h0 * (SLAB >> 4);
+                        da = (da & ~((uint64_t)0x3FFF << 16)) | ((uint64_t)(SLAB >> 4) << 16);
+                        umma_pair<0>(accu, da, p_desc, idesc_u);
+#pragma unroll
+                        for (int t = 1; t < TILE / 16; ++t)
+                            umma_pair<1>(accu, da + (uint64_t)(t * (16 * 128 >> 4)),
+                                         p_desc + (uint64_t)((t >> 2) * (PSLAB >> 4) + (t & 3) * 2), idesc_u);
+                        umma_commit_pair(h_free + 8 * h0);
+                        if (hs != h0) umma_commit_pair(h_free + 8 * hs);
+                        umma_commit_pair(o_full + 8 * ob);
+                        ++o;
+                    }
+                }
+            }
+        }
+    } else if (warp < OUT_WARP) {
+        // ============================== hidden warps (both CTAs) ==============================
+        const int my_slab = (warp - HID_WARP) >> 2;   // this warp's slab of a job
+        const uint32_t lane_base = 32u * (warp & 3);  // tensor-memory lane quarter of this warp
+        // where this lane's row of the 8 x 8 blocks goes (row lane % 8 of 8, block lane / 8 of 4; 128-byte swizzle)
+        const uint32_t st_row = (lane_base + (lane & 7)) * 128u;
+        const uint32_t ready_leader = map_to_cta(h_ready, 0), empty_leader = map_to_cta(t_empty, 0);
+        uint32_t hslot = 0, hphase = 0, h = 0, tb = 0, tphase = 0;
+        TileWalk tw;
+        tw.start(a.sq, my_first);
+        for (int it = 0; it < n_it; ++it, tw.next(a.sq)) {
+            const int valid = tw.valid(a.sq);
+            for (int side = 0; side < 2; ++side) {
+                for (int s = 0; s < a.l.n_src[side]; ++s) {
+                    const int m = a.l.src[side][s].m;
+                    const float slope = a.l.src[side][s].slope;
+                    const float2 slope2 = make_float2(slope, slope);
+                    const bool lr_max = slope <= 1.f;
+                    // V side: rows past the tile's end may hold anything, and zero times a stray NaN is not zero
+                    const bool clear = side == 1 && valid < TILE;
+                    if (side == 1) {
+                        hslot += hslot & 1u;
+                        if (hslot == (uint32_t)a.nh) hslot = 0;
+                    }
+                    const float *tbuf = reinterpret_cast<const float *>(smem_raw + (s_t - s_z)) + tb * a.m_t;
+                    if (it == 0 || !a.t_resident) mbar_wait(tb_full + 8 * tb, tphase, a.status, &abort_flag, 0x60f);
+                    for (int c0 = 0; c0 < m; c0 += CN, ++h) {
+                        const int nc = min(CN, m - c0);
+                        const uint32_t buf = h & 1u, acc = tmem + CN * buf + (lane_base << 16);
+                        mbar_wait(t_full + 8 * buf, (h >> 1) & 1u, a.status, &abort_flag, 0x609);
+                        __syncwarp();
+                        tc_fence_after();
+                        // The job's places in the ring.  A warp writes one of them but sees every one free: a phase that it
+                        // skipped would let a later wait on the same place pass one phase early.
+                        uint32_t slot = 0;
+                        bool mine = false;
+                        for (int sl = 0; 64 * sl < nc; ++sl) {
+                            if (sl == my_slab) {
+                                mine = true;
+                                slot = hslot;
+                            }
+                            mbar_wait(h_free + 8 * hslot, ((hphase >> hslot) & 1u) ^ 1u, a.status, &abort_flag, 0x60a);
+                            hphase ^= 1u << hslot;
+                            if (++hslot == (uint32_t)a.nh) hslot = 0;
+                        }
+                        __syncwarp();
+                        if (mine) {
+#pragma unroll
+                            for (int half = 0; half < 2; ++half) {
+                                const int col = 64 * my_slab + 32 * half;
+                                if (col < nc) {
+                                    const float4 *t4 = reinterpret_cast<const float4 *>(tbuf + c0 + col) + 2 * (lane & 3);
+                                    const float4 ta = t4[0], tb4 = t4[1];
+                                    const float2 t[4] = {make_float2(ta.x, ta.y), make_float2(ta.z, ta.w), make_float2(tb4.x, tb4.y),
+                                                         make_float2(tb4.z, tb4.w)};
+                                    uint32_t r[2][16];
+                                    tmem_ld_frag_x4(acc + (uint32_t)col, r[0]);
+                                    tmem_ld_frag_x4(acc + (16u << 16) + (uint32_t)col, r[1]);
+                                    tmem_ld_wait();
+                                    const uint32_t dst = s_h + slot * SLAB + st_row + (uint32_t)(((4 * half + (lane >> 3)) ^ (lane & 7)) << 4);
+#pragma unroll
+                                    for (int i = 0; i < 4; ++i) {  // rows 8 i .. of the warp's 32
+                                        uint32_t w[4];
+#pragma unroll
+                                        for (int j = 0; j < 4; ++j) {
+                                            const float2 x = __fadd2_rn(make_float2(__uint_as_float(r[i >> 1][4 * j + 2 * (i & 1)]),
+                                                                                    __uint_as_float(r[i >> 1][4 * j + 2 * (i & 1) + 1])), t[j]);
+                                            const float2 y = __fmul2_rn(x, slope2);
+                                            // LeakyReLU: the larger of x and slope*x for slope <= 1, the smaller for slope > 1
+                                            w[j] = lr_max ? pack_bf16(fmaxf(x.x, y.x), fmaxf(x.y, y.y))
+                                                          : pack_bf16(fminf(x.x, y.x), fminf(x.y, y.y));
+                                            if (clear && (int)lane_base + 8 * i + (lane >> 2) >= valid) w[j] = 0u;
+                                        }
+                                        stmatrix_x4(dst + 1024u * i, w);
+                                    }
+                                }
+                            }
+                        }
+                        tc_fence_before();
+                        fence_async_smem();
+                        __syncwarp();
+                        if (elect_one()) {
+                            mbar_arrive_remote(empty_leader + 8 * buf);
+                            mbar_arrive_remote(ready_leader + 8 * (h & 7u));
+                        }
+                    }
+                    __syncwarp();
+                    if (!a.t_resident && elect_one()) mbar_arrive_local(tb_empty + 8 * tb);
+                    if (++tb == (uint32_t)a.nt || (a.t_resident && side == 1 && s + 1 == a.l.n_src[1])) { tb = 0; tphase ^= 1u; }
+                }
+            }
+        }
+    } else {
+        // ============================== output warps (both CTAs) ==============================
+        // S: thread = token; U: thread = hidden feature of a block.  The two warps of a lane quarter take half of the
+        // query heads each.
+        constexpr int NT = NQ / 2;
+        const int half = (warp - OUT_WARP) >> 2, quarter = warp & 3;
+        const int row = 32 * quarter + lane;
+        const uint32_t lane_sel = (uint32_t)(32 * quarter) << 16;
+        const uint32_t empty_leader = map_to_cta(o_empty, 0), pready_leader = map_to_cta(p_ready, 0);
+        const uint32_t col = TM_OUT + R * rank + NT * half;
+        const int q0 = NT * half;
+        const bool low_v = a.two_terms_v != 0;
+        float acc[NB][NT], l[NT];
+#pragma unroll
+        for (int q = 0; q < NT; ++q) {
+            l[q] = 0.f;
+#pragma unroll
+            for (int b = 0; b < NB; ++b) acc[b][q] = 0.f;
+        }
+        uint32_t o = 0;
+        auto half_sync = [&]() {  // the four warps of this half
+            if (half == 0)
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+            else
+                asm volatile("bar.sync 2, 128;" ::: "memory");
+        };
+        // this warp's columns of the next output accumulator: one value per query head of its half
+        auto fetch = [&](float *v) {
+            const uint32_t ob = o & 1u, addr = tmem + lane_sel + col + 64u * ob;
+            mbar_wait(o_full + 8 * ob, (o >> 1) & 1u, a.status, &abort_flag, 0x60b);
+            __syncwarp();
+            tc_fence_after();
+            float r[16];
+            tmem_ld8(addr, r);
+            tmem_ld8(NQ <= 16 ? addr + NQ : addr + 8u, r + 8);
+            tmem_ld_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (elect_one()) mbar_arrive_remote(empty_leader + 8 * ob);
+            ++o;
+#pragma unroll
+            for (int q = 0; q < NT; ++q) v[q] = NQ <= 16 ? r[q] + r[8 + q] : r[q];  // the low terms have columns of their own
+        };
+        TileWalk tw;
+        tw.start(a.sq, my_first);
+        for (int it = 0; it < n_it; ++it, tw.next(a.sq)) {
+            const int valid = tw.valid(a.sq), par = it & 1;
+            {
+                float s[NT];
+                fetch(s);
+#pragma unroll
+                for (int q = 0; q < NT; ++q)
+                    if (row >= valid) s[q] = -INFINITY;
+                const float keep = max_over_lanes<NT>(s, lane);
+                if (lane < NT) sh.red[par][q0 + lane][quarter] = keep;
+                half_sync();
+                // reference maxima: one head per lane, then broadcast by shuffles of the few values that follow from them
+                float m_new = 0.f, f = 1.f;
+                if (lane < NT) {
+                    const float *r = sh.red[par][q0 + lane];
+                    const float m_old = sh.mrun[par][q0 + lane];
+                    m_new = fmaxf(m_old, fmaxf(fmaxf(r[0], r[1]), fmaxf(r[2], r[3])));
+                    if (m_new != m_old) f = ex2(m_old - m_new);
+                    if (quarter == 0) sh.mrun[par ^ 1][q0 + lane] = m_new;
+                }
+                if (__any_sync(0xffffffffu, f != 1.f)) {
+#pragma unroll
+                    for (int q = 0; q < NT; ++q) {
+                        const float fq = __shfl_sync(0xffffffffu, f, q);
+                        l[q] *= fq;
+#pragma unroll
+                        for (int b = 0; b < NB; ++b) acc[b][q] *= fq;
+                    }
+                }
+                const uint32_t t6 = row & 63;
+                const uint32_t pbase = s_p + (uint32_t)(row >> 6) * PSLAB + (t6 & 7u) * 2u;
+#pragma unroll
+                for (int q = 0; q < NT; ++q) {
+                    const float mq = __shfl_sync(0xffffffffu, m_new, q);
+                    const float p = valid > 0 ? ex2(s[q] - mq) : 0.f;
+                    l[q] += p;
+                    // operand row q0 + q, token t6 of atom row >> 6 (K-major, 128-byte swizzle)
+                    const uint32_t qr = q0 + q;
+                    const __nv_bfloat16 hi = __float2bfloat16_rn(p);
+                    st_smem_u16(pbase + qr * 128u + (((t6 >> 3) ^ (qr & 7u)) << 4), __bfloat16_as_ushort(hi));
+                    if (NQ <= 16) {
+                        const uint32_t ql = qr + NQ;
+                        const __nv_bfloat16 lo = __float2bfloat16_rn(low_v ? p - __bfloat162float(hi) : 0.f);
+                        st_smem_u16(pbase + ql * 128u + (((t6 >> 3) ^ (ql & 7u)) << 4), __bfloat16_as_ushort(lo));
+                    }
+                }
+                fence_async_smem();
+                __syncwarp();
+                if (elect_one()) mbar_arrive_remote(pready_leader);
+            }
+            for (int s = 0; s < a.l.n_src[1]; ++s) {
+                const int n_blk = (((a.l.src[1][s].m + 63) >> 6) + 1) >> 1;
+                const uint32_t mask = a.l.src[1][s].mask >> q0;
+#pragma unroll
+                for (int b = 0; b < NB; ++b) {
+                    if (b < n_blk) {
+                        float u[NT];
+                        fetch(u);
+#pragma unroll
+                        for (int q = 0; q < NT; ++q)
+                            if ((mask >> q) & 1u) acc[b][q] += u[q];
+                    }
+                }
+            }
+            if (tw.ends_run()) {
+                const int64_t run = (int64_t)blockIdx.x + tw.si;  // block and sequence only ever grow along the runs: unique
+                for (int s = 0; s < a.l.n_src[1]; ++s) {
+                    const int m = a.l.src[1][s].m;
+                    const uint32_t mask = a.l.src[1][s].mask >> q0;
+                    float *u = a.upart + (run * a.hq + q0) * a.m_pad + row;
+#pragma unroll
+                    for (int b = 0; b < NB; ++b)
+#pragma unroll
+                        for (int q = 0; q < NT; ++q)
+                            if (((mask >> q) & 1u) && 128 * b + row < m) u[(int64_t)q * a.m_pad + 128 * b] = acc[b][q];
+                }
+                float keep = 0.f;
+#pragma unroll
+                for (int q = 0; q < NT; ++q) {
+                    float v = l[q];
+#pragma unroll
+                    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+                    if (lane == q) keep = v;
+                    l[q] = 0.f;
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) acc[b][q] = 0.f;
+                }
+                if (lane < NT) sh.lred[q0 + lane][quarter] = keep;
+                half_sync();
+                if (quarter == 0 && lane < NT) {
+                    if (q0 + lane < a.hq) {
+                        const float *r = sh.lred[q0 + lane];
+                        float *ml = a.ml + (run * a.hq + q0 + lane) * 2;
+                        ml[0] = sh.mrun[par ^ 1][q0 + lane];
+                        ml[1] = (r[0] + r[1]) + (r[2] + r[3]);
+                    }
+                    sh.mrun[par ^ 1][q0 + lane] = -INFINITY;
+                }
+            }
+        }
+    }
+    // ---- teardown: nobody leaves while the peer may still signal this CTA ----
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+    }
+}
+
+// ---------------------------------------------------------------------------- W4_h^T q
+// grid = (query heads, blocks of 256 hidden columns, blocks of LQ_SB sequences); thread = two hidden columns, all 64 rows of
+// the head.  The query is scaled by 1/sqrt(head_dim) and by log2(e): the tile kernel's exponentials are powers of two.
+// Bound by the latency of the weight loads at few sequences, so all of them are in flight; everything else comes from the
+// parameters.  Operand rows of sources that do not serve the head are zeroed.
+constexpr int LQ_SB = 8, LQ_THREADS = 128;
+__global__ void __launch_bounds__(LQ_THREADS) latent_query_kernel(const __grid_constant__ LatHeads hp, const __nv_bfloat16 *q,
+                                                                  int n_seqs, int hq, int group, float scale, __nv_bfloat16 *wq,
+                                                                  float *qbias, int nq, int m_pad, int batch, int two_terms) {
+    __shared__ __align__(16) float qs[64][LQ_SB];
+    const int qh = blockIdx.x, si0 = blockIdx.z * LQ_SB, tid = threadIdx.x;
+    const int n_here = min(LQ_SB, n_seqs - si0);
+    const int kvh = qh / group, s = hp.idx[0][kvh], slot = hp.slot[0][kvh];
+    const LatHeads::Src &sp = hp.src[0][s];
+    const int m2 = sp.m >> 1, j = blockIdx.y * LQ_THREADS + tid;
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(sp.w2k) + (int64_t)slot * 64 * m2 + j;
+    uint32_t u[64];
+    float2 sab = make_float2(0.f, 0.f);  // the hidden vector is short of these
+#pragma unroll
+    for (int c = 0; c < 64; ++c) u[c] = j < m2 ? __ldg(w + (int64_t)c * m2) : 0u;
+    if (j < m2) sab = __ldg(reinterpret_cast<const float2 *>(sp.sabs) + j);
+    for (int i = tid; i < 64 * LQ_SB; i += LQ_THREADS) {
+        const int k = i >> 6, c = i & 63;
+        qs[c][k] = k < n_here ? __bfloat162float(q[((int64_t)(si0 + k) * hq + qh) * 64 + c]) * scale : 0.f;
+    }
+    __syncthreads();
+    float x[LQ_SB], y[LQ_SB];
+#pragma unroll
+    for (int i = 0; i < LQ_SB; ++i) x[i] = y[i] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 64; ++c) {
+        const float w0 = __uint_as_float(u[c] << 16), w1 = __uint_as_float(u[c] & 0xffff0000u);
+#pragma unroll
+        for (int i = 0; i < LQ_SB; i += 4) {
+            const float4 q4 = *reinterpret_cast<const float4 *>(&qs[c][i]);
+            x[i] = fmaf(w0, q4.x, x[i]);
+            x[i + 1] = fmaf(w0, q4.y, x[i + 1]);
+            x[i + 2] = fmaf(w0, q4.z, x[i + 2]);
+            x[i + 3] = fmaf(w0, q4.w, x[i + 3]);
+            y[i] = fmaf(w1, q4.x, y[i]);
+            y[i + 1] = fmaf(w1, q4.y, y[i + 1]);
+            y[i + 2] = fmaf(w1, q4.z, y[i + 2]);
+            y[i + 3] = fmaf(w1, q4.w, y[i + 3]);
+        }
+    }
+    const int rows = wq_rows(nq);  // operand rows per (source, sequence): high terms, then low terms
+#pragma unroll
+    for (int i = 0; i < LQ_SB; ++i) {
+        if (i >= n_here) break;
+        x[i] *= sab.x;
+        y[i] *= sab.y;
+        const uint32_t hi = pack_bf16(x[i], y[i]);
+        const uint32_t lo = two_terms ? pack_bf16(x[i] - __uint_as_float(hi << 16), y[i] - __uint_as_float(hi & 0xffff0000u)) : 0u;
+        for (int ss = 0; ss < hp.n_src[0]; ++ss) {
+            if (j >= (hp.src[0][ss].m >> 1)) continue;
+            uint32_t *r = reinterpret_cast<uint32_t *>(wq + (((int64_t)ss * batch + si0 + i) * rows + qh) * m_pad) + j;
+            r[0] = ss == s ? hi : 0u;
+            r[(int64_t)nq * m_pad / 2] = ss == s ? lo : 0u;
+        }
+    }
+    if (blockIdx.y != 0) return;
+    const int warp = tid >> 5, lane = tid & 31;
+    for (int i = warp; i < n_here; i += LQ_THREADS / 32) {
+        float b = qs[lane][i] * sp.b2[slot * 64 + lane] + qs[lane + 32][i] * sp.b2[slot * 64 + lane + 32];
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) b += __shfl_xor_sync(0xffffffffu, b, d);
+        if (lane == 0) qbias[(int64_t)(si0 + i) * hq + qh] = b;
+    }
+}
+
+// ---------------------------------------------------------------------------- merge
+// grid = (query heads, blocks of SB sequences).  The last decoder layer's 64 rows of the head (73 KB at m = 576) are read once
+// per SB sequences: SB = 4 where that still fills the machine, else 1 (at 8 sequences x 12 heads, 4 sequences per block left 24
+// blocks and took 57 us; SB = 1 with 288 threads 15 us, a chain of dependent loads; 8 us with 1024 threads whose registers take
+// the weights before anything else is known).
+constexpr int LM_PRE = 18;  // weight words a lane holds ahead: all of them up to m = 576 at 32 warps
+struct MergeArgs {
+    const float *upart, *ml, *qbias;
+    const __nv_bfloat16 *q;
+    __nv_bfloat16 *out;
+    int32_t hq, group, kv_width, m_pad;
+    float scale;
+    int32_t with_current;
+};
+template <int SB, int LM_THREADS>
+__global__ void __launch_bounds__(LM_THREADS) latent_merge_kernel(const __grid_constant__ LatHeads hp, const __grid_constant__ LatSeqs sq,
+                                                                  const __grid_constant__ MergeArgs a) {
+    extern __shared__ __align__(16) float u[];  // [SB][m_pad], with SB = 1 then the groups' partial sums [LM_THREADS][4]
+    constexpr int LM_WARPS = LM_THREADS / 32;
+    __shared__ float wts[SB][LT_MAX_CTAS];
+    __shared__ float fin[SB][2];  // (sum of the runs, exponent reference) per sequence
+    __shared__ float osum[LM_WARPS][SB][64];
+    const int qh = blockIdx.x, si0 = blockIdx.y * SB, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n_here = min(SB, sq.n - si0);
+    const int kvh = qh / a.group, slot = hp.slot[1][kvh];
+    const LatHeads::Src &sp = hp.src[1][hp.idx[1][kvh]];
+    const int m = sp.m, m_pad = a.m_pad;
+    // lane = two channels of the head, warp = every LM_WARPS-th hidden feature
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(sp.w2t) + slot * 32 + lane;
+    const int64_t pitch = sp.in_dim >> 1;
+    uint32_t pre[SB == 1 ? LM_PRE : 1];
+    if (SB == 1) {
+#pragma unroll
+        for (int k = 0; k < LM_PRE; ++k) {
+            const int j = warp + k * LM_WARPS;
+            pre[k] = j < m ? __ldg(w + j * pitch) : 0u;
+        }
+    }
+    auto first = [&](int i) { return (int)(sq.first[i] & 0xffffffu); };
+    auto runs = [&](int si, int &k0) {  // runs of a sequence: k0 .. k0 + n - 1
+        const int f0 = first(si), f1 = first(si + 1);
+        k0 = f0 / sq.per;
+        return f1 > f0 ? (f1 - 1) / sq.per - k0 + 1 : 0;
+    };
+    if (warp < n_here) {  // one warp per sequence: reference maximum over its runs, their weights, the sum
+        const int si = si0 + warp;
+        int k0;
+        const int n_run = runs(si, k0);
+        const float2 *p = reinterpret_cast<const float2 *>(a.ml) + (int64_t)(k0 + si) * a.hq + qh;
+        float M = -INFINITY, S = 0.f;
+        for (int r = lane; r < n_run; r += 32) M = fmaxf(M, p[(int64_t)r * a.hq].x);
+        M = redux_max(M);
+        for (int r = lane; r < n_run; r += 32) {
+            const float2 v = p[(int64_t)r * a.hq];
+            const float wr = ex2(v.x - M);
+            wts[warp][r] = wr;
+            S += wr * v.y;
+        }
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) S += __shfl_xor_sync(0xffffffffu, S, d);
+        if (lane == 0) {
+            fin[warp][0] = S;
+            fin[warp][1] = n_run > 0 ? M + a.qbias[(int64_t)si * a.hq + qh] : -INFINITY;
+        }
+    }
+    __syncthreads();
+    // thread = (sequence, four hidden features); with one sequence the threads that are left share its runs
+    const int nf = m >> 2;
+    auto add_runs = [&](int i, int f, int r0, int step) {
+        int k0;
+        const int n_run = runs(si0 + i, k0);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float *p = a.upart + ((int64_t)(k0 + si0 + i) * a.hq + qh) * m_pad + f;
+#pragma unroll 8
+        for (int r = r0; r < n_run; r += step) {
+            const float4 v = *reinterpret_cast<const float4 *>(p + (int64_t)r * a.hq * m_pad);
+            const float wr = wts[i][r];
+            acc.x = fmaf(wr, v.x, acc.x);
+            acc.y = fmaf(wr, v.y, acc.y);
+            acc.z = fmaf(wr, v.z, acc.z);
+            acc.w = fmaf(wr, v.w, acc.w);
+        }
+        return acc;
+    };
+    auto put = [&](int i, int f, float4 acc) {
+        const float4 sc = *reinterpret_cast<const float4 *>(sp.sabs + f);  // the hidden vector is short of this factor
+        *reinterpret_cast<float4 *>(u + i * m_pad + f) = make_float4(acc.x * sc.x, acc.y * sc.y, acc.z * sc.z, acc.w * sc.w);
+    };
+    if (SB == 1) {
+        float4 *part = reinterpret_cast<float4 *>(u + m_pad);
+        const int n_grp = max(1, LM_THREADS / nf), grp = tid / nf;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (grp < n_grp) acc = add_runs(0, 4 * (tid % nf), grp, n_grp);
+        part[tid] = acc;
+        __syncthreads();
+        if (tid < nf) {
+            for (int g = 1; g < n_grp; ++g) {
+                const float4 v = part[tid + g * nf];
+                acc.x += v.x;
+                acc.y += v.y;
+                acc.z += v.z;
+                acc.w += v.w;
+            }
+            put(0, 4 * tid, acc);
+        }
+    } else {
+        for (int t = tid; t < SB * nf; t += LM_THREADS) {
+            const int i = t / nf, f = 4 * (t % nf);
+            put(i, f, i < n_here ? add_runs(i, f, 0, 1) : make_float4(0.f, 0.f, 0.f, 0.f));
+        }
+    }
+    __syncthreads();
+    {
+        float x[SB], y[SB];
+#pragma unroll
+        for (int i = 0; i < SB; ++i) x[i] = y[i] = 0.f;
+        auto add = [&](uint32_t v, int j) {
+            const float w0 = __uint_as_float(v << 16), w1 = __uint_as_float(v & 0xffff0000u);
+#pragma unroll
+            for (int i = 0; i < SB; ++i) {
+                const float ui = u[i * m_pad + j];
+                x[i] = fmaf(w0, ui, x[i]);
+                y[i] = fmaf(w1, ui, y[i]);
+            }
+        };
+        if (SB == 1) {
+#pragma unroll
+            for (int k = 0; k < LM_PRE; ++k) {
+                const int j = warp + k * LM_WARPS;
+                if (j < m) add(pre[k], j);
+            }
+        }
+#pragma unroll 16
+        for (int j = warp + (SB == 1 ? LM_PRE * LM_WARPS : 0); j < m; j += LM_WARPS) add(__ldg(w + j * pitch), j);
+#pragma unroll
+        for (int i = 0; i < SB; ++i) *reinterpret_cast<float2 *>(&osum[warp][i][2 * lane]) = make_float2(x[i], y[i]);
+    }
+    __syncthreads();
+    if (warp >= n_here) return;
+    // one warp per sequence: add up, the head's bias, the exact current token
+    const int si = si0 + warp;
+    float o[2] = {0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < LM_WARPS; ++k) {
+        o[0] += osum[k][warp][lane];
+        o[1] += osum[k][warp][lane + 32];
+    }
+    float S = fin[warp][0];
+    const float M = fin[warp][1];
+    o[0] += sp.b2[slot * 64 + lane] * S;
+    o[1] += sp.b2[slot * 64 + lane + 32] * S;
+    if (a.with_current) {
+        const int64_t seq = sq.id[si];
+        const __nv_bfloat16 *kc = reinterpret_cast<const __nv_bfloat16 *>(hp.cur[0][kvh]) + seq * a.kv_width;
+        const __nv_bfloat16 *vc = reinterpret_cast<const __nv_bfloat16 *>(hp.cur[1][kvh]) + seq * a.kv_width;
+        const __nv_bfloat16 *qg = a.q + ((int64_t)si * a.hq + qh) * 64;
+        float sc = __bfloat162float(qg[lane]) * __bfloat162float(kc[lane]) + __bfloat162float(qg[lane + 32]) * __bfloat162float(kc[lane + 32]);
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, d);
+        sc *= a.scale;
+        const float Mn = fmaxf(M, sc);
+        const float c0 = M == -INFINITY ? 0.f : ex2(M - Mn), c1 = ex2(sc - Mn);
+        S = S * c0 + c1;
+        o[0] = o[0] * c0 + __bfloat162float(vc[lane]) * c1;
+        o[1] = o[1] * c0 + __bfloat162float(vc[lane + 32]) * c1;
+    }
+    __nv_bfloat16 *out = a.out + ((int64_t)si * a.hq + qh) * 64;
+    out[lane] = __float2bfloat16_rn(S > 0.f ? o[0] / S : 0.f);
+    out[lane + 32] = __float2bfloat16_rn(S > 0.f ? o[1] / S : 0.f);
+}
+
+using Kernel = void (*)(const Params);
+const Kernel kernels[] = {decode_latent_kernel<12, 2>, decode_latent_kernel<12, 5>, decode_latent_kernel<16, 5>,
+                          decode_latent_kernel<16, 8>, decode_latent_kernel<32, 2>, decode_latent_kernel<32, 3>};
+constexpr int KERNEL_NQ[] = {12, 12, 16, 16, 32, 32}, KERNEL_NB[] = {2, 5, 5, 8, 2, 3};
+constexpr int N_KERNELS = 6;
+
+int smem_bytes(int nq, int nz, int nh, int nw, int nqs, int nt, int m_t) {
+    const int scratch = nq == 12 ? sizeof(Scratch<12>) : nq == 16 ? sizeof(Scratch<16>) : sizeof(Scratch<32>);
+    return (nz + nh) * SLAB + nw * WSTAGE + nqs * wq_slab(nq) + 2 * op_rows(nq) * 128 + nt * m_t * 4 +
+           8 * (2 * (nz + nw + nqs + nt) + nh + READY_BARS + 9) + scratch;
+}
+constexpr int SMEM_MAX = 227 * 1024;
+
+int padded_heads(int hq) { return hq <= 12 ? 12 : hq <= 16 ? 16 : 32; }
+
+void fill_seqs(LatSeqs &q, const SeqList &seqs, const int32_t *lens, int n_sms) {
+    uint32_t t = 0;
+    q.n = seqs.n;
+    for (int i = 0; i < seqs.n; ++i) {
+        q.id[i] = seqs.id[i];
+        q.first[i] = t | (uint32_t)(lens[i] > 0 ? (lens[i] - 1) % TILE : 0) << 24;
+        t += (uint32_t)((lens[i] + TILE - 1) / TILE);
+    }
+    q.first[seqs.n] = t;
+    q.n_tiles = (int32_t)t;
+    const int ctas = std::min(n_sms, LT_MAX_CTAS) & ~1;
+    q.per = std::max(1, ((int)t + ctas - 1) / ctas);
+}
+
+constexpr float LOG2E = 1.4426950408889634f;
+
+}  // namespace
+
+size_t lat_ws_bytes(const kvcar_config &cfg, int max_k_sources, int max_m, int batch) {
+    if (cfg.storage != KVCAR_BF16 || cfg.latent_quant || cfg.head_dim != 64 || cfg.n_q_heads > LT_MAX_Q || max_k_sources <= 0 || max_m <= 0)
+        return 0;
+    const size_t nq = padded_heads(cfg.n_q_heads), m_pad = ((size_t)max_m + 63) / 64 * 64;
+    const size_t wq = (size_t)std::min(max_k_sources, LT_MAX_SRC) * batch * wq_rows((int)nq) * m_pad * 2;
+    const size_t bias = ((size_t)batch * cfg.n_q_heads * 4 + 255) / 256 * 256;
+    const size_t runs = (size_t)LT_MAX_CTAS + batch;
+    return wq + bias + runs * cfg.n_q_heads * (m_pad + 2) * sizeof(float);
+}
+
+void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPlan> &plans, size_t pool_rows,
+               int max_k_sources, int max_m, int batch, char *ws_area) {
+    st.available = false;
+    const int nl = cfg.n_layers;
+    st.layer.assign(nl, LatLayer{});
+    st.heads.assign(nl, LatHeads{});
+    st.cfg.assign(nl, LatLayerCfg{});
+    if (lat_ws_bytes(cfg, max_k_sources, max_m, batch) == 0 || cfg.page_tokens % 64 != 0) return;
+    EncodeTiledFn fn = tensor_map_encoder();
+    if (!fn) return;
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int group = cfg.n_q_heads / cfg.n_kv_heads;
+    st.n_sms = sms;
+    st.nq = padded_heads(cfg.n_q_heads);
+    st.group = group;
+    st.m_pad = (max_m + 63) / 64 * 64;
+    st.batch = batch;
+    const size_t n_src = std::min(max_k_sources, LT_MAX_SRC), n_rows = n_src * batch * wq_rows(st.nq);
+    if (!encode_bf16_map(fn, &st.tm_wq, ws_area, n_rows, st.m_pad, st.m_pad, op_rows(st.nq))) return;
+    char *p = ws_area;
+    st.wq = p;
+    p += n_rows * st.m_pad * 2;
+    st.qbias = reinterpret_cast<float *>(p);
+    p += ((size_t)batch * cfg.n_q_heads * 4 + 255) / 256 * 256;
+    st.upart = reinterpret_cast<float *>(p);
+    p += (size_t)(LT_MAX_CTAS + batch) * cfg.n_q_heads * st.m_pad * sizeof(float);
+    st.ml = reinterpret_cast<float *>(p);
+    for (int l = 0; l < nl; ++l) {
+        LatLayer &ly = st.layer[l];
+        LatHeads &hp = st.heads[l];
+        LatLayerCfg &lc = st.cfg[l];
+        bool ok = true;
+        int ks = 0, lm = 0, lmk = 0, chunks = 0;
+        for (int w = 0; w < 2 && ok; ++w) {
+            const WhichPlan &wp = plans[l].w[w];
+            ok = wp.n_src > 0 && wp.n_src <= LT_MAX_SRC;
+            ly.n_src[w] = hp.n_src[w] = wp.n_src;
+            for (int s = 0; s < wp.n_src && ok; ++s) {
+                const SourcePlan &sp = wp.src[s];
+                ok = sp.compressed && !sp.qparam && sp.d % 16 == 0 && sp.m % 16 == 0 && sp.width == sp.d;
+                if (!ok) break;
+                LatSrc &d = ly.src[w][s];
+                d.shift = sp.shift;
+                d.d = sp.d;
+                d.m = sp.m;
+                d.slope = sp.slope;
+                d.mask = 0;
+                hp.src[w][s] = {sp.w2k, sp.w2t, sp.b2, sp.sabs, sp.m, sp.in_dim};
+                for (int i = 0; i < sp.n_need; ++i) {
+                    const int h = sp.kv_head[i];
+                    for (int g = 0; g < group; ++g) d.mask |= 1u << (h * group + g);
+                    hp.idx[w][h] = (uint8_t)s;
+                    hp.slot[w][h] = (uint8_t)sp.slot[i];
+                    hp.cur[w][h] = reinterpret_cast<const __nv_bfloat16 *>(plans[l].cur[w][h]) + plans[l].cur_head[w][h] * 64;
+                }
+                ok = encode_bf16_map(fn, &ly.pool[w][s], sp.pool, pool_rows, sp.width, sp.width) &&
+                     encode_bf16_map(fn, &ly.w1[w][s], sp.w1n, sp.m, sp.d, sp.d, CN / 2);
+                ks = std::max(ks, (sp.d + 63) / 64);
+                lm = std::max(lm, sp.m);
+                if (w == 0) lmk = std::max(lmk, sp.m);
+                chunks = std::max(chunks, (sp.m + CN - 1) / CN);
+            }
+        }
+        if (!ok) continue;
+        int v = 0;
+        while (v < N_KERNELS && (KERNEL_NQ[v] < st.nq || KERNEL_NB[v] * 128 < lm)) ++v;
+        if (v == N_KERNELS || KERNEL_NQ[v] != st.nq) continue;
+        // Staging places.  A side's latents stay for all its chunks (nz >= their slabs).  One-chunk layers get places for the
+        // other side's latents and six hidden slabs, because their jobs are shorter than the way from S to P; the others four
+        // hidden slabs: a chunk's three and the one its predecessor may leave unpaired.
+        const int m_t = (lm + 31) & ~31, n_all = ly.n_src[0] + ly.n_src[1];
+        int nh = chunks == 1 ? 6 : 4, nz = chunks == 1 ? std::max(4, 2 * ks) : ks, nw = 4, nqs = chunks == 1 ? 3 : 2;
+        int nt = chunks == 1 ? std::min(n_all, 4) : 1;
+        auto fits = [&]() { return smem_bytes(st.nq, nz, nh, nw, nqs, nt, m_t) <= SMEM_MAX; };
+        while (nw > 3 && !fits()) --nw;
+        while (nqs > 2 && !fits()) --nqs;
+        while (nz > ks && !fits()) --nz;
+        while (nw > 2 && !fits()) --nw;
+        if (!fits()) continue;
+        while (nt < n_all && (++nt, fits())) {}
+        if (!fits()) --nt;
+        lc.nz = (uint8_t)nz;
+        lc.nh = (uint8_t)nh;
+        lc.nw = (uint8_t)nw;
+        lc.nqs = (uint8_t)nqs;
+        lc.nt = (uint8_t)nt;
+        lc.m_t = m_t;
+        lc.t_resident = nt >= n_all;
+        lc.smem = std::max(smem_bytes(st.nq, nz, nh, nw, nqs, nt, m_t), 120 * 1024);  // one CTA per SM: each takes all of tensor memory
+        lc.variant = (uint8_t)v;
+        lc.max_m = lm;
+        lc.max_mk = lmk;
+        if (cudaFuncSetAttribute(kernels[v], cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        lc.ok = 1;
+        st.available = true;
+    }
+}
+
+bool lat_layer_supported(const LatState &st, int layer, uint32_t flags) {
+    if (!st.available || !st.cfg[layer].ok) return false;
+    // 17 to 32 query heads: the probabilities are one bf16 term.  The restoring kernel keeps them in fp32 for groups of up to
+    // two heads, so those take this path only where the caller has asked for that rounding.
+    return st.nq <= 16 || st.group > 2 || ((flags & KVCAR_ABSORBED) && (flags & KVCAR_ABSORBED_V));
+}
+
+cudaError_t lat_launch_tiles(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer,
+                             cudaStream_t stream) {
+    const LatLayerCfg &lc = st.cfg[layer];
+    if (seqs.n > st.batch) return cudaErrorInvalidValue;  // the list names a sequence twice
+    Params p;
+    fill_seqs(p.sq, seqs, lens, st.n_sms);
+    if (p.sq.n_tiles == 0) return cudaSuccess;
+    p.l = st.layer[layer];
+    p.tm_wq = st.tm_wq;
+    p.block_table = a.block_table;
+    p.status = a.status;
+    p.upart = st.upart;
+    p.ml = st.ml;
+    p.max_pages_per_seq = a.max_pages_per_seq;
+    p.page_tokens = a.page_tokens;
+    p.hq = a.hq;
+    p.m_pad = st.m_pad;
+    p.wq_batch = st.batch;
+    p.nz = lc.nz;
+    p.nh = lc.nh;
+    p.nw = lc.nw;
+    p.nqs = lc.nqs;
+    p.nt = lc.nt;
+    p.m_t = lc.m_t;
+    p.t_resident = lc.t_resident;
+    p.two_terms_k = (a.flags & KVCAR_ABSORBED) ? 0 : 1;
+    p.two_terms_v = (a.flags & KVCAR_ABSORBED) && (a.flags & KVCAR_ABSORBED_V) ? 0 : 1;
+    latent_query_kernel<<<dim3(a.hq, (lc.max_mk / 2 + LQ_THREADS - 1) / LQ_THREADS, (seqs.n + LQ_SB - 1) / LQ_SB), LQ_THREADS, 0, stream>>>(
+        st.heads[layer], reinterpret_cast<const __nv_bfloat16 *>(a.q), seqs.n, a.hq, st.group, a.scale * LOG2E,
+        reinterpret_cast<__nv_bfloat16 *>(st.wq), st.qbias, st.nq, st.m_pad, st.batch, p.two_terms_k);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const int ctas = (p.sq.n_tiles + p.sq.per - 1) / p.sq.per;
+    kernels[lc.variant]<<<dim3((ctas + 1) & ~1), NTHREADS, lc.smem, stream>>>(p);
+    return cudaGetLastError();
+}
+
+cudaError_t lat_launch_merge(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer,
+                             cudaStream_t stream) {
+    LatSeqs q;
+    fill_seqs(q, seqs, lens, st.n_sms);
+    MergeArgs m;
+    m.upart = st.upart;
+    m.ml = st.ml;
+    m.qbias = st.qbias;
+    m.q = reinterpret_cast<const __nv_bfloat16 *>(a.q);
+    m.out = reinterpret_cast<__nv_bfloat16 *>(a.out);
+    m.hq = a.hq;
+    m.group = st.group;
+    m.kv_width = a.hkv * 64;
+    m.m_pad = st.m_pad;
+    m.scale = a.scale * LOG2E;
+    m.with_current = (a.flags & KVCAR_INCLUDE_CURRENT_EXACT) != 0;
+    if (a.hq * seqs.n > 2 * st.n_sms)
+        latent_merge_kernel<4, 288><<<dim3(a.hq, (seqs.n + 3) / 4), 288, (size_t)4 * st.m_pad * 4, stream>>>(st.heads[layer], q, m);
+    else
+        latent_merge_kernel<1, 1024><<<dim3(a.hq, seqs.n), 1024, (size_t)st.m_pad * 4 + 1024 * 16, stream>>>(st.heads[layer], q, m);
+    return cudaGetLastError();
+}
+
+}  // namespace kvcar

@@ -1,0 +1,93 @@
+// Interface between the host runtime and the latent-attention kernels (kvcar_latent.cu).
+#pragma once
+#include <vector>
+
+#include "kvcar_internal.h"
+
+namespace kvcar {
+
+constexpr int LT_MAX_SRC = 6;     // distinct source layers per K or V of a layer
+constexpr int LT_MAX_Q = 32;      // query heads
+constexpr int LT_MAX_CTAS = 160;  // blocks of a launch at most (one per SM)
+
+// Place of hidden feature f's shift in the padded array: groups of 32 features, in each the order in which the four lanes of a
+// fragment row hold them (features 8 j + 2 c + e of a group at 8 c + 2 j + e).
+inline int shift_place(int f) { return (f & ~31) + ((f & 7) >> 1) * 8 + ((f & 31) >> 3) * 2 + (f & 1); }
+
+// One source layer of K or V as the tile kernel sees it (kernel parameter).
+struct LatSrc {
+    const float *shift;  // fused bias + BatchNorm shift over the size of its scale, in fragment order (see shift_place)
+    int32_t d, m;
+    float slope;
+    uint32_t mask;  // query heads whose K (or V) head is served from this source
+};
+
+// The listed sequences of a call: device ids, and the first tile of each (low 24 bits) with the valid tokens of its
+// last tile minus one in the high 8; first[n] = number of tiles.
+struct LatSeqs {
+    int32_t n, n_tiles, per, pad_;  // per: consecutive tiles of one block
+    int32_t id[KVCAR_MAX_BATCH];
+    uint32_t first[KVCAR_MAX_BATCH + 1];
+};
+
+// What a layer's launches need; built at bind time, kept on the host and passed to the kernels by value (tensor maps in
+// kernel parameters need no acquire, and nothing is found through chains of loads).
+struct LatLayer {
+    CUtensorMap pool[2][LT_MAX_SRC], w1[2][LT_MAX_SRC];
+    int32_t n_src[2];
+    LatSrc src[2][LT_MAX_SRC];
+};
+// The last decoder layer of each source, which source and column slot serves a KV head, the exact current-token rows.
+struct LatHeads {
+    struct Src {
+        const void *w2k, *w2t;  // [in_dim][m] and [m][in_dim], bf16
+        const float *b2, *sabs;
+        int32_t m, in_dim;
+    } src[2][LT_MAX_SRC];
+    int32_t n_src[2];
+    const void *cur[2][LT_MAX_Q];  // by KV head: its 64 columns of the current-token row of sequence 0
+    uint8_t idx[2][LT_MAX_Q], slot[2][LT_MAX_Q];
+};
+
+struct LatLayerCfg {
+    uint8_t ok = 0;
+    uint8_t variant = 0;                              // kernel instantiation
+    uint8_t nz = 0, nh = 0, nw = 0, nqs = 0, nt = 0;  // staging places: latent, hidden, weight, query slabs; shift buffers
+    uint8_t t_resident = 0;                           // every source has a shift buffer of its own
+    int32_t m_t = 0;
+    int32_t smem = 0;
+    int32_t max_mk = 0, max_m = 0;  // widest hidden layer of the K sources, of all
+};
+
+struct LatState {
+    bool available = false;
+    std::vector<LatLayer> layer;
+    std::vector<LatHeads> heads;
+    std::vector<LatLayerCfg> cfg;
+    int n_sms = 148;
+    int nq = 12;      // query heads padded
+    int group = 1;    // query heads per KV head
+    int m_pad = 0;    // row pitch of the vectors below
+    int batch = 0;    // sequences per call at most
+    void *wq = nullptr;      // [source][batch][operand rows][m_pad] bf16: W4_h^T q, high parts then low parts
+    float *qbias = nullptr;  // [batch][hq]: q . b4_h, in the exponent's base-2 units
+    float *upart = nullptr;  // [block + sequence][hq][m_pad]: sum over a run of tiles of p * hidden vector
+    float *ml = nullptr;     // [block + sequence][hq][2]: reference maximum and sum of the run
+    CUtensorMap tm_wq;
+};
+
+// bytes of the operands and partial results inside the workspace (0: the shape does not take this path)
+size_t lat_ws_bytes(const kvcar_config &cfg, int max_k_sources, int max_m, int batch);
+// decide per layer whether the kernels take it, build tensor maps, place the workspace area
+void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPlan> &plans, size_t pool_rows,
+               int max_k_sources, int max_m, int batch, char *ws_area);
+// flags: those of the call (17 to 32 query heads in groups of at most two only with KVCAR_ABSORBED_V, see kvcar_latent.cu)
+bool lat_layer_supported(const LatState &st, int layer, uint32_t flags);
+// the operand kernel and the tile kernel (lens: host copy of the listed sequences' lengths)
+cudaError_t lat_launch_tiles(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer,
+                             cudaStream_t stream);
+// the merge of the runs, the last decoder layer of the V side, the current token
+cudaError_t lat_launch_merge(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer,
+                             cudaStream_t stream);
+
+}  // namespace kvcar
