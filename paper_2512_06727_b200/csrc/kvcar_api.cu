@@ -770,9 +770,53 @@ kvcar_status kvcar_encode_append(kvcar_ctx *c, int32_t layer, const int32_t *seq
     return enqueue_encode(c, layer, seqs, n_seqs, n_tokens, k, v, st);
 }
 
+// what the tensor-core encoder takes
+static bool prefill_fits(const kvcar_ctx *c, int32_t layer, const char **why) {
+    const kvcar_config &g = c->cfg;
+    *why = "the tensor-core encoder takes bf16 storage, bf16 latent rows and 64-wide heads";
+    if (g.storage != KVCAR_BF16 || g.head_dim != 64 || g.latent_quant) return false;
+    *why = "the tensor-core encoder needs an autoencoder for K and for V with widths that are multiples of 16";
+    for (int w = 0; w < 2; ++w) {
+        const AEHost &ae = c->ae[layer * 2 + w];
+        if (!ae.set || ae.hidden % 16 || ae.latent % 16 || ae.hidden > 1024 || ae.latent > 1024) return false;
+    }
+    return true;
+}
+
+// exact: hidden activations as their whole fp32 values (kvcar_encode_append), else rounded to bf16
+static kvcar_status enqueue_prefill(kvcar_ctx *c, int32_t layer, const int32_t *seqs, int32_t n_seqs, int32_t n_tokens,
+                                    const void *k, const void *v, bool exact, cudaStream_t st) {
+    const kvcar_config &g = c->cfg;
+    PrefillTcArgs a{};
+    a.plan_dev = reinterpret_cast<const EncPlan *>(c->weights + c->enc_off) + layer * 2;
+    a.plan_host = c->enc_host.data() + layer * 2;
+    a.block_table = reinterpret_cast<const int32_t *>(c->ws + c->bt_off);
+    a.seq_len = reinterpret_cast<const int32_t *>(c->ws + c->len_off);
+    a.status = reinterpret_cast<int32_t *>(c->ws + c->status_off);
+    a.src[0] = k;
+    a.src[1] = v;
+    a.hid = c->ws + c->pfhid_off;
+    a.max_m = c->max_m;
+    a.max_pages_per_seq = g.max_pages_per_seq;
+    a.page_tokens = g.page_tokens;
+    a.n_tokens = n_tokens;
+    a.kv_width = g.n_kv_heads * g.head_dim;
+    SeqList sl;
+    sl.n = n_seqs;
+    memcpy(sl.id, seqs, (size_t)n_seqs * 4);
+    cudaError_t e = launch_prefill_tc(a, sl, exact, st);
+    if (e != cudaSuccess) return cuda_fail(c, e, "tensor-core encoder launch");
+    const int blk = prefill_tc_block(exact);
+    c->launches += 2 * (((int64_t)n_seqs * n_tokens + blk - 1) / blk);
+    return KVCAR_OK;
+}
+
 // the encoder launches of one layer (arguments checked, pages reserved and tables flushed by the caller)
 static kvcar_status enqueue_encode(kvcar_ctx *c, int32_t layer, const int32_t *seqs, int32_t n_seqs, int32_t n_tokens,
                                    const void *k, const void *v, cudaStream_t st) {
+    const char *why;
+    if (n_tokens > 1 && prefill_fits(c, layer, &why) && (int64_t)n_seqs * n_tokens <= 0x7fffffff)
+        return enqueue_prefill(c, layer, seqs, n_seqs, n_tokens, k, v, true, st);
     EncodeArgs a{};
     a.plan = reinterpret_cast<const EncPlan *>(c->weights + c->enc_off) + layer * 2;
     a.block_table = reinterpret_cast<const int32_t *>(c->ws + c->bt_off);
@@ -813,42 +857,15 @@ kvcar_status kvcar_encode_append_tensor(kvcar_ctx *c, int32_t layer, const int32
         return fail(c, KVCAR_ERR_INVALID_ARG, "bad layer, pointer or token count");
     if (!check_seqs(c, seqs, n_seqs)) return fail(c, KVCAR_ERR_INVALID_ARG, "bad sequence list");
     if (((uintptr_t)k | (uintptr_t)v) & 15) return fail(c, KVCAR_ERR_INVALID_ARG, "k/v must be 16-byte aligned");
-    const kvcar_config &g = c->cfg;
-    if (g.storage != KVCAR_BF16 || g.head_dim != 64 || g.latent_quant)
-        return fail(c, KVCAR_ERR_UNSUPPORTED, "the tensor-core encoder takes bf16 storage, bf16 latent rows and 64-wide heads");
-    for (int w = 0; w < 2; ++w) {
-        const AEHost &ae = c->ae[layer * 2 + w];
-        if (!ae.set || ae.hidden % 16 || ae.latent % 16 || ae.hidden > 1024 || ae.latent > 1024)
-            return fail(c, KVCAR_ERR_UNSUPPORTED,
-                        "the tensor-core encoder needs an autoencoder for K and for V with widths that are multiples of 16");
-    }
+    const char *why;
+    if (!prefill_fits(c, layer, &why)) return fail(c, KVCAR_ERR_UNSUPPORTED, why);
     if ((int64_t)n_seqs * n_tokens > 0x7fffffff) return fail(c, KVCAR_ERR_INVALID_ARG, "too many rows");
     kvcar_status s = reserve_pages(c, seqs, n_seqs, n_tokens);
     if (s != KVCAR_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     s = flush_tables(c, st);
     if (s != KVCAR_OK) return s;
-    PrefillTcArgs a{};
-    a.plan_dev = reinterpret_cast<const EncPlan *>(c->weights + c->enc_off) + layer * 2;
-    a.plan_host = c->enc_host.data() + layer * 2;
-    a.block_table = reinterpret_cast<const int32_t *>(c->ws + c->bt_off);
-    a.seq_len = reinterpret_cast<const int32_t *>(c->ws + c->len_off);
-    a.status = reinterpret_cast<int32_t *>(c->ws + c->status_off);
-    a.src[0] = k;
-    a.src[1] = v;
-    a.hid = c->ws + c->pfhid_off;
-    a.max_m = c->max_m;
-    a.max_pages_per_seq = g.max_pages_per_seq;
-    a.page_tokens = g.page_tokens;
-    a.n_tokens = n_tokens;
-    a.kv_width = g.n_kv_heads * g.head_dim;
-    SeqList sl;
-    sl.n = n_seqs;
-    memcpy(sl.id, seqs, (size_t)n_seqs * 4);
-    cudaError_t e = launch_prefill_tc(a, sl, st);
-    if (e != cudaSuccess) return cuda_fail(c, e, "tensor-core encoder launch");
-    c->launches += 2 * (((int64_t)n_seqs * n_tokens + PREFILL_TC_ROWS - 1) / PREFILL_TC_ROWS);
-    return KVCAR_OK;
+    return enqueue_prefill(c, layer, seqs, n_seqs, n_tokens, k, v, false, st);
 }
 
 kvcar_status kvcar_advance(kvcar_ctx *c, const int32_t *seqs, int32_t n_seqs, int32_t n_tokens, void *stream) {

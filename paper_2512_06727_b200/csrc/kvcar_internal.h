@@ -140,6 +140,9 @@ size_t decode_generic_smem(int hq, int hd, int max_d, int max_m);
 // autoencoder, head_dim 64, hidden and latent widths multiples of 16.  Rows are worked through in blocks of
 // PREFILL_TC_ROWS; `hid` is a bf16 scratch of prefill_tc_scratch_bytes(max hidden width) bytes.
 constexpr int PREFILL_TC_ROWS = 32768;
+constexpr int PREFILL_TC_PLANES = 3;  // bf16 terms of an fp32 hidden activation
+// rows of a block: with exact (fp32) hidden activations the scratch holds three planes per row
+inline int prefill_tc_block(bool exact) { return exact ? PREFILL_TC_ROWS / PREFILL_TC_PLANES / 256 * 256 : PREFILL_TC_ROWS; }
 struct PrefillTcArgs {
     const EncPlan *plan_dev;    // this layer's [K, V] plans on the device
     const EncPlan *plan_host;   // the same two plans, host copy (widths and weight pointers for the tensor maps)
@@ -152,6 +155,7 @@ struct PrefillTcArgs {
     int32_t max_pages_per_seq, page_tokens, n_tokens, kv_width;
 };
 size_t prefill_tc_scratch_bytes(int max_m);
-cudaError_t launch_prefill_tc(const PrefillTcArgs &a, const SeqList &seqs, cudaStream_t st);
+// exact: the hidden activations enter the second product as their whole fp32 values, else rounded to bf16
+cudaError_t launch_prefill_tc(const PrefillTcArgs &a, const SeqList &seqs, bool exact, cudaStream_t st);
 
 }  // namespace kvcar

@@ -10,8 +10,11 @@
 // per 256 rows and a k-step costs each SM 32 KB of loads instead of 48 (the one-CTA form was bound by those loads).
 // Per CTA two TMA producer warps, an MMA warp (the leader's issues) and eight epilogue warps; five operand stages and
 // two accumulator buffers; a pair walks several tiles, its epilogue of one under the products of the next.
-// Unlike the decode-time encoder, the hidden activations pass through bf16 here (they are an operand of the second
-// product), so a latent written by this path may differ from the fp32-hidden one by a few bf16 ulps of its scale.
+// The hidden activations are an operand of the second product.  kvcar_encode_append_tensor rounds them to bf16, so a latent
+// written by it may differ from the decode-time encoder's by a few bf16 ulps of its scale.  kvcar_encode_append keeps them in
+// fp32 (EXACT): stage 1 writes each as three bf16 terms (3 x 8 bits: the whole fp32 value) into three planes of the scratch, and
+// stage 2 contracts over the planes one after the other with the same weights.  That is 1.67 times the products of the rounded
+// form, and at the GPT-2 shape, 8 x 1024 rows and 12 layers, 0.65 ms against 11.5 ms for the CUDA-core kernel it replaces.
 // All waits are bounded and record a code in the status word.
 #include <cuda.h>
 
@@ -46,7 +49,7 @@ struct PfArgs {
     int32_t *status;
     const void *src[2];          // the caller's K and V rows [n_rows_total][kv_width] (stage 1: exact current rows)
     __nv_bfloat16 *hid;          // scratch [2][hid_rows][hid_pitch]
-    int32_t hid_rows, hid_pitch;
+    int32_t hid_rows, hid_pitch;  // rows of one plane
     int32_t max_pages_per_seq, page_tokens;
     int32_t n_tokens, kv_width;
     int32_t row0, n_rows_blk;    // this launch covers rows row0 .. row0 + n_rows_blk - 1 of the call
@@ -75,7 +78,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t
 // (tile t = row pair t / n_ct, column tile t % n_ct: the column tiles of a row pair follow each other, so its rows are
 // re-read from L2) with the stride of the cluster count; the operand ring and the two accumulator buffers run on
 // across tiles, so the producer and the issuer are in the next tile while the epilogue warps drain the last one.
-template <int STAGE>
+template <int STAGE, bool EXACT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
     prefill_fc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_a1,
                       const __grid_constant__ CUtensorMap map_b0, const __grid_constant__ CUtensorMap map_b1,
@@ -96,7 +99,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
     const uint32_t bars = base + PF_STAGES * PF_STAGE_BYTES;  // full[S] (leader's are used), empty[S], acc_full[2], acc_empty[2]
     const uint32_t bar_accf = bars + 16 * PF_STAGES, bar_acce = bar_accf + 16;
     const uint32_t stage_base = bars + 128;  // 128-byte aligned (the stages are 1024-byte multiples)
-    const int n_slabs = (kdim + 63) >> 6;
+    constexpr int PLANES = EXACT ? PREFILL_TC_PLANES : 1;
+    const int plane_slabs = (kdim + 63) >> 6, n_slabs = STAGE == 2 ? PLANES * plane_slabs : plane_slabs;
     const int n_ct = (ndim + PF_N - 1) / PF_N;
     const int n_tiles = ((a.n_rows_blk + 2 * PF_M - 1) / (2 * PF_M)) * n_ct;
 
@@ -133,7 +137,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
                 const int n0 = (t % n_ct) * PF_N, r0 = (t / n_ct) * 2 * PF_M + (int)rank * PF_M;
                 const int nt = min(PF_N, ndim - n0), half = nt >> 1;  // this CTA supplies `half` weight rows
                 const int b_boxes = (half + 63) >> 6;                 // in 64-row boxes; rows past the half are never read
-                for (int ks = 0; ks < n_slabs; ++ks, ++g) {
+                for (int kp = 0; kp < n_slabs; ++kp, ++g) {
+                    const int plane = EXACT && STAGE == 2 ? kp / plane_slabs : 0, ks = kp - plane * plane_slabs;
                     const uint32_t s = g % PF_STAGES, use = g / PF_STAGES;
                     if (use > 0 && !mbar_wait(bars + 8 * (PF_STAGES + s), (use - 1u) & 1u, a.status, 0x401)) {
                         ok = false;
@@ -144,7 +149,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
                     if (leader && rows_side) mbar_expect_tx(bars + 8 * s, 2u * (2u * 8192u + (uint32_t)b_boxes * 8192u));
                     // stage 1: K slab ks of X is stored head ks's 64-wide slice; stage 2: columns 64 ks.. of the scratch
                     const int ax = STAGE == 1 ? pl.heads[ks] * 64 : 64 * ks;
-                    const int ay = STAGE == 1 ? a.row0 + r0 : which * a.hid_rows + r0;
+                    const int ay = STAGE == 1 ? a.row0 + r0 : (which * PLANES + plane) * a.hid_rows + r0;
                     if (rows_side) {
                         tma_load_2d_pair(sa, map_a, ax, ay, full);
                         tma_load_2d_pair(sa + 8192, map_a, ax, ay + 64, full);
@@ -167,7 +172,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
                 // the epilogue warps of both CTAs are done with this buffer's previous tile
                 if (it >= 2 && !mbar_wait(bar_acce + 8 * buf, ((it >> 1) - 1u) & 1u, a.status, 0x404)) break;
                 tc_fence_after();
-                for (int ks = 0; ks < n_slabs; ++ks, ++g) {
+                for (int kp = 0, ks = 0; kp < n_slabs; ++kp, ++g) {
                     const uint32_t s = g % PF_STAGES, use = g / PF_STAGES;
                     if (!mbar_wait(bars + 8 * s, use & 1u, a.status, 0x402)) {
                         ok = false;
@@ -178,11 +183,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
                     const uint64_t da = make_desc(sa), db = make_desc(sb);
                     const int nk = min(4, (kdim - 64 * ks) >> 4);
                     for (int k = 0; k < nk; ++k) {
-                        if (ks | k)
+                        if (kp | k)
                             umma_pair<1>(acc, da + 2u * k, db + 2u * k, idesc);
                         else
                             umma_pair<0>(acc, da + 2u * k, db + 2u * k, idesc);
                     }
+                    if (++ks == plane_slabs) ks = 0;
                     umma_commit_pair(bars + 8 * (PF_STAGES + s));  // the stage is free in both CTAs once these products are done
                 }
                 if (ok) umma_commit_pair(bar_accf + 8 * buf);
@@ -212,7 +218,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
             }
             __nv_bfloat16 *dst;
             if (STAGE == 1) {
-                dst = a.hid + ((int64_t)which * a.hid_rows + r0 + rl) * a.hid_pitch + n0;
+                dst = a.hid + ((int64_t)which * PLANES * a.hid_rows + r0 + rl) * a.hid_pitch + n0;
             } else {
                 const int tok = a.seq_len[seq] + tk;
                 const int64_t prow =
@@ -238,42 +244,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
             // instruction (lane = 8 l_row + chunk).
             const uint32_t stg = stage_base + (uint32_t)(warp - 2) * 4096u;
             const uint64_t dst_bits = reinterpret_cast<uint64_t>(dst);
-            for (int b64 = chalf; 64 * b64 < nt; b64 += 2) {
+            // four columns of the accumulator through the layer's epilogue
+            auto act4 = [&](int c, float *x) {
+                const float4 pa = *reinterpret_cast<const float4 *>(&prm[0][c]);
+                const float sa[4] = {pa.x, pa.y, pa.z, pa.w};
+                if (STAGE == 1) {
+                    const float4 pb = *reinterpret_cast<const float4 *>(&prm[1][c]);
+                    const float sb[4] = {pb.x, pb.y, pb.z, pb.w};
 #pragma unroll
-                for (int hg = 0; hg < 2; ++hg) {
-                    const int g = 2 * b64 + hg;
-                    if (32 * g >= nt) break;  // warp-uniform
-                    float v[32];
-                    tmem_ld32(acc + ((uint32_t)(32 * q) << 16) + 32u * g, v);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int c8 = 0; c8 < 4; ++c8) {
-                        const int c = 32 * g + 8 * c8;
-                        if (c >= nt) break;
-                        float o[8], pa[8], pb[8];
-                        *reinterpret_cast<float4 *>(pa) = *reinterpret_cast<const float4 *>(&prm[0][c]);
-                        *reinterpret_cast<float4 *>(pa + 4) = *reinterpret_cast<const float4 *>(&prm[0][c + 4]);
-                        if (STAGE == 1) {
-                            *reinterpret_cast<float4 *>(pb) = *reinterpret_cast<const float4 *>(&prm[1][c]);
-                            *reinterpret_cast<float4 *>(pb + 4) = *reinterpret_cast<const float4 *>(&prm[1][c + 4]);
-                        }
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const float x = v[8 * c8 + e];
-                            if (STAGE == 1) {
-                                const float y = fmaf(x, pa[e], pb[e]);
-                                o[e] = y > 0.f ? y : y * slope;
-                            } else {
-                                o[e] = x + pa[e];
-                            }
-                        }
-                        const uint32_t chunk = (uint32_t)(4 * hg + c8);  // 16-byte chunk of the row's 128-byte segment
-                        const uint32_t addr = stg + (uint32_t)lane * 128u + ((chunk ^ ((uint32_t)lane & 7u)) << 4);
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(pack_bf16(o[0], o[1])),
-                                     "r"(pack_bf16(o[2], o[3])), "r"(pack_bf16(o[4], o[5])), "r"(pack_bf16(o[6], o[7]))
-                                     : "memory");
+                    for (int e = 0; e < 4; ++e) {
+                        const float y = fmaf(x[e], sa[e], sb[e]);
+                        x[e] = y > 0.f ? y : y * slope;
                     }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) x[e] += sa[e];
                 }
+            };
+            auto stage_chunk = [&](int ch, const uint32_t *w) {  // 16-byte chunk of this lane's row
+                const uint32_t addr = stg + (uint32_t)lane * 128u + (((uint32_t)ch ^ ((uint32_t)lane & 7u)) << 4);
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                             : "memory");
+            };
+            auto store_block = [&](int b64, int64_t off) {
                 __syncwarp();
                 const uint32_t chunk = (uint32_t)lane & 7u;
                 const bool col_ok = 64 * b64 + 8 * (int)chunk < nt;  // widths are multiples of 16: whole chunks
@@ -286,10 +279,55 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
                     const uint32_t addr = stg + (uint32_t)rr * 128u + ((chunk ^ ((uint32_t)rr & 7u)) << 4);
                     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w0), "=r"(w1), "=r"(w2), "=r"(w3) : "r"(addr) : "memory");
                     if (ok_row && col_ok)
-                        *reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(d_row) + 64 * b64 + 8 * (int)chunk) =
+                        *reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(d_row) + off + 64 * b64 + 8 * (int)chunk) =
                             make_uint4(w0, w1, w2, w3);
                 }
                 __syncwarp();  // the staging area is free for the next block
+            };
+            for (int b64 = chalf; 64 * b64 < nt; b64 += 2) {
+                constexpr bool SPLIT = EXACT && STAGE == 1;
+                float v[SPLIT ? 64 : 32];
+#pragma unroll
+                for (int hg = 0; hg < 2; ++hg) {
+                    const int g = 2 * b64 + hg;
+                    if (32 * g >= nt) break;  // warp-uniform
+                    float *vh = v + (SPLIT ? 32 * hg : 0);
+                    tmem_ld32(acc + ((uint32_t)(32 * q) << 16) + 32u * g, vh);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int c8 = 0; c8 < 4; ++c8) {
+                        const int c = 32 * g + 8 * c8;
+                        if (c >= nt) break;
+                        act4(c, vh + 8 * c8);
+                        act4(c + 4, vh + 8 * c8 + 4);
+                        if (!SPLIT) {
+                            const float *x = vh + 8 * c8;
+                            const uint32_t w[4] = {pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7])};
+                            stage_chunk(4 * hg + c8, w);
+                        }
+                    }
+                }
+                if (!SPLIT) {
+                    store_block(b64, 0);
+                } else {
+#pragma unroll
+                    for (int plane = 0; plane < PREFILL_TC_PLANES; ++plane) {
+#pragma unroll
+                        for (int ch = 0; ch < 8; ++ch) {
+                            if (64 * b64 + 8 * ch >= nt) break;
+                            uint32_t w[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                float &x0 = v[(8 * ch + 2 * e) % (SPLIT ? 64 : 32)], &x1 = v[(8 * ch + 2 * e + 1) % (SPLIT ? 64 : 32)];
+                                w[e] = pack_bf16(x0, x1);
+                                x0 -= __uint_as_float(w[e] << 16);  // what this term leaves out goes to the next plane
+                                x1 -= __uint_as_float(w[e] & 0xffff0000u);
+                            }
+                            stage_chunk(ch, w);
+                        }
+                        store_block(b64, (int64_t)plane * a.hid_rows * a.hid_pitch);
+                    }
+                }
             }
             // this warp is done reading the buffer: one arrival of the sixteen the issuer waits for
             tc_fence_before();
@@ -319,15 +357,15 @@ size_t prefill_tc_scratch_bytes(int max_m) {
     return (size_t)2 * PREFILL_TC_ROWS * pitch * sizeof(__nv_bfloat16);
 }
 
-cudaError_t launch_prefill_tc(const PrefillTcArgs &h, const SeqList &seqs, cudaStream_t st) {
+cudaError_t launch_prefill_tc(const PrefillTcArgs &h, const SeqList &seqs, bool exact, cudaStream_t st) {
     static bool configured[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64 || !configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(prefill_fc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(prefill_fc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM);
-        if (e != cudaSuccess) return e;
+        for (auto k : {prefill_fc_kernel<1, false>, prefill_fc_kernel<2, false>, prefill_fc_kernel<1, true>, prefill_fc_kernel<2, true>}) {
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM);
+            if (e != cudaSuccess) return e;
+        }
         if (dev >= 0 && dev < 64) configured[dev] = true;
     }
     const int pitch = (h.max_m + 63) & ~63;
@@ -342,7 +380,8 @@ cudaError_t launch_prefill_tc(const PrefillTcArgs &h, const SeqList &seqs, cudaS
             return cudaErrorInvalidValue;
     }
     const int max_m = std::max(h.plan_host[0].m, h.plan_host[1].m), max_d = std::max(h.plan_host[0].d, h.plan_host[1].d);
-    for (int64_t row0 = 0; row0 < n_rows; row0 += PREFILL_TC_ROWS) {
+    const int blk = prefill_tc_block(exact);
+    for (int64_t row0 = 0; row0 < n_rows; row0 += blk) {
         PfArgs a{};
         a.plan = h.plan_dev;
         a.block_table = h.block_table;
@@ -351,22 +390,24 @@ cudaError_t launch_prefill_tc(const PrefillTcArgs &h, const SeqList &seqs, cudaS
         a.src[0] = h.src[0];
         a.src[1] = h.src[1];
         a.hid = reinterpret_cast<__nv_bfloat16 *>(h.hid);
-        a.hid_rows = PREFILL_TC_ROWS;
+        a.hid_rows = blk;
         a.hid_pitch = pitch;
         a.max_pages_per_seq = h.max_pages_per_seq;
         a.page_tokens = h.page_tokens;
         a.n_tokens = h.n_tokens;
         a.kv_width = h.kv_width;
         a.row0 = (int32_t)row0;
-        a.n_rows_blk = (int32_t)std::min<int64_t>(PREFILL_TC_ROWS, n_rows - row0);
+        a.n_rows_blk = (int32_t)std::min<int64_t>(blk, n_rows - row0);
         // 37 clusters per K or V (every SM pair of the device between them), fewer when there are fewer tiles
         const int row_pairs = (a.n_rows_blk + 2 * PF_M - 1) / (2 * PF_M);
         const unsigned c1 = (unsigned)std::min(37, row_pairs * ((max_m + PF_N - 1) / PF_N));
         const unsigned c2 = (unsigned)std::min(37, row_pairs * ((max_d + PF_N - 1) / PF_N));
-        prefill_fc_kernel<1><<<dim3(2 * c1, 1, 2), PF_THREADS, PF_SMEM, st>>>(ax[0], ax[1], w1[0], w1[1], a, seqs);
+        auto k1 = exact ? prefill_fc_kernel<1, true> : prefill_fc_kernel<1, false>;
+        auto k2 = exact ? prefill_fc_kernel<2, true> : prefill_fc_kernel<2, false>;
+        k1<<<dim3(2 * c1, 1, 2), PF_THREADS, PF_SMEM, st>>>(ax[0], ax[1], w1[0], w1[1], a, seqs);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        prefill_fc_kernel<2><<<dim3(2 * c2, 1, 2), PF_THREADS, PF_SMEM, st>>>(ah[0], ah[1], w2[0], w2[1], a, seqs);
+        k2<<<dim3(2 * c2, 1, 2), PF_THREADS, PF_SMEM, st>>>(ah[0], ah[1], w2[0], w2[1], a, seqs);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

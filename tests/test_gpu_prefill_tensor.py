@@ -56,3 +56,18 @@ def test_tensor_prefill_refuses_what_it_cannot_do():
         p.s.ctx.encode_append_tensor(0, [0], 4, k.data_ptr(), k.data_ptr(), p.s.stream())
     assert e.value.status == 5          # KVCAR_ERR_UNSUPPORTED
     assert p.s.ctx.seq_len(0) == 0
+
+
+@pytest.mark.parametrize("batch,tokens", [(1, 2), (1, 127), (1, 129), (3, 86), (2, 5400)])
+def test_bulk_append_keeps_the_hidden_activations_in_fp32(batch, tokens):
+    """kvcar_encode_append of several tokens (hidden activations as three bf16 terms each on the tensor cores) at the edges
+    of a 128-row tile and of a pair of tiles, and past one block of the scratch (10 752 rows): the rows it writes lie within
+    one bf16 step of the oracle's, the tolerance of the fp32-hidden encoder, not the wider one of rounded activations."""
+    w = synth.scaled(synth.CONFIGS["c3"], n_layers=2 if tokens < 1000 else 1, batch=batch, cached_tokens=0, decode_steps=1,
+                     reuse_frac=0.25)
+    pps = (tokens + 63) // 64
+    p = Pair(w, max_seqs=batch, max_pages=batch * pps, max_pages_per_seq=pps)
+    seqs = list(range(batch))
+    p.open(seqs)
+    p.prefill(seqs, tokens)
+    p.check_latents(seqs)
