@@ -11,6 +11,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "kvcar_internal.h"
+#include "kvcar_fma.h"
 #include "kvcar_latent.h"
 #include "kvcar_tc.h"
 
@@ -79,7 +80,7 @@ struct kvcar_ctx {
     std::vector<char> quant;                // [layer*2+which]: rows are int8 codes
     size_t pool_bytes = 0, weights_bytes = 0, ws_bytes = 0;
     size_t plan_off = 0, enc_off = 0, tmap_off = 0, tcpart_off = 0;  // inside weights
-    size_t bt_off = 0, len_off = 0, status_off = 0, part_off = 0, stage_off = 0, enchid_off = 0, kvsplit_off = 0, pfhid_off = 0, lat_off = 0;  // inside workspace
+    size_t bt_off = 0, len_off = 0, status_off = 0, part_off = 0, stage_off = 0, enchid_off = 0, kvsplit_off = 0, pfhid_off = 0, lat_off = 0, fma_off = 0;  // inside workspace
     int max_k_sources = 0;  // most distinct source layers any layer's K heads resolve to
     std::vector<RawSources> raw_src;  // [layer] tensor maps and head places of raw bf16 layers
     std::vector<char> raw_src_ok;     // [layer] filled (else the raw-row kernel stages with cp.async)
@@ -89,7 +90,8 @@ struct kvcar_ctx {
     std::vector<LayerPlan> plans_host;
     TcState tc;
     LatState lat;
-    bool lat_used = false;  // the last tile launch was the latent kernel's: its merge follows
+    FmaState fma;
+    enum Tiles { TILES_ROWS, TILES_LATENT, TILES_FMA } tiles_by = TILES_ROWS;  // whose partial results the merge finds
     float *static_scratch = nullptr;  // device address of the built-in scratch array, looked up at bind time
 
     int64_t launches = 0;
@@ -131,6 +133,9 @@ int stored_width(const kvcar_ctx *c, int layer, int which) {
     if (a.set) return a.latent;
     return (int)stored_heads(c, layer, which).size() * c->cfg.head_dim;
 }
+
+// bf16 rows of 64-wide heads: the tensor-core kernels take all but a few layers, and those few stay with the generic kernel
+bool fma_is_fallback_only(const kvcar_config &g) { return g.storage == KVCAR_BF16 && !g.latent_quant && g.head_dim == 64; }
 
 void compute_layout(kvcar_ctx *c) {
     const kvcar_config &g = c->cfg;
@@ -239,6 +244,8 @@ void compute_layout(kvcar_ctx *c) {
     }
     c->lat_off = s;  // operands and partial results of the latent-attention kernels
     s = align_up(s + lat_ws_bytes(g, c->max_k_sources, c->max_m, nb), 256);
+    c->fma_off = s;  // the same of the fp32-FMA kernels, where latents are not bf16 rows of 64-wide heads
+    if (!fma_is_fallback_only(g)) s = align_up(s + fma_ws_bytes(g, c->max_k_sources, c->max_m, nb, cap), 256);
     c->ws_bytes = s;
 }
 
@@ -611,6 +618,9 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
              (size_t)g.max_pages * g.page_tokens);
     lat_setup(c->lat, c->cfg, c->plans_host, (size_t)g.max_pages * g.page_tokens, c->max_k_sources, c->max_m,
               std::min(g.max_seqs, KVCAR_MAX_BATCH), c->ws + c->lat_off);
+    if (!fma_is_fallback_only(g))
+        fma_setup(c->fma, c->cfg, c->plans_host, c->max_k_sources, c->max_m, std::min(g.max_seqs, KVCAR_MAX_BATCH),
+                  g.max_pages_per_seq * g.page_tokens, c->ws + c->fma_off);
     // tensor maps and head places of the raw layers (kernel parameters of the raw-row kernel)
     c->raw_src.assign(nl, RawSources{});
     c->raw_src_ok.assign(nl, 0);
@@ -917,7 +927,7 @@ static int prepare_decode(kvcar_ctx *c, int32_t layer, const int32_t *seqs, int3
 // step's encoder writes (the exact current token enters in the combine kernel).
 static kvcar_status enqueue_decode_tiles(kvcar_ctx *c, int32_t layer, const DecodeArgs &a, const SeqList &sl,
                                          int n_chunks, cudaStream_t st) {
-    c->lat_used = false;
+    c->tiles_by = kvcar_ctx::TILES_ROWS;
     if (n_chunks <= 0) return KVCAR_OK;
     const kvcar_config &g = c->cfg;
     int n_tiles = 0;
@@ -937,12 +947,19 @@ static kvcar_status enqueue_decode_tiles(kvcar_ctx *c, int32_t layer, const Deco
         int32_t lens[KVCAR_MAX_BATCH];
         for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
         e = lat_launch_tiles(c->lat, a, sl, lens, layer, st);
-        c->lat_used = true;
+        c->tiles_by = kvcar_ctx::TILES_LATENT;
         ++c->launches;
     } else if (want_tc) {
         int32_t lens[KVCAR_MAX_BATCH];
         for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
         e = tc_launch_decode(c->tc, a, sl, lens, layer, st);
+    } else if (c->kernel == KVCAR_KERNEL_AUTO && fma_layer_supported(c->fma, layer)) {
+        int32_t lens[KVCAR_MAX_BATCH];
+        for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
+        int n = 1;
+        e = fma_launch_tiles(c->fma, g, a, sl, lens, layer, st, &n);
+        c->tiles_by = kvcar_ctx::TILES_FMA;
+        c->launches += n - 1;
     } else {
         if (decode_generic_smem(a.hq, a.hd, c->max_d, c->max_m) > 227 * 1024)
             return fail(c, KVCAR_ERR_UNSUPPORTED, "shape needs more shared memory than one SM has");
@@ -955,10 +972,11 @@ static kvcar_status enqueue_decode_tiles(kvcar_ctx *c, int32_t layer, const Deco
 
 static kvcar_status enqueue_combine(kvcar_ctx *c, int32_t layer, const DecodeArgs &a, const SeqList &sl, int n_chunks, cudaStream_t st) {
     cudaError_t e;
-    if (c->lat_used) {
+    if (c->tiles_by != kvcar_ctx::TILES_ROWS) {
         int32_t lens[KVCAR_MAX_BATCH];
         for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
-        e = lat_launch_merge(c->lat, a, sl, lens, layer, st);
+        e = c->tiles_by == kvcar_ctx::TILES_LATENT ? lat_launch_merge(c->lat, a, sl, lens, layer, st)
+                                                   : fma_launch_merge(c->fma, c->cfg, a, sl, lens, layer, st);
     } else {
         e = launch_combine(a, sl, c->cfg.storage, n_chunks, st);
     }

@@ -473,3 +473,28 @@ def test_absorbed_last_layer_matches_the_oracle(shape):
     p2.prefill([1], 130)
     _check_step(p2.decode_step([0, 1], 0, absorbed=True), "bf16", f"absorbed flag on a small grid, {shape}")
 
+
+
+@pytest.mark.parametrize("case", ["small_tiles", "large_tiles", "groups", "int8_large_tiles"])
+def test_fp32_arithmetic_kernels_at_tile_edges(case):
+    """The fp32-FMA attention kernels (fp32 storage, int8 rows, head widths other than 64): blocks of 32 x 32 with two pieces
+    per partial result, blocks of 64 x 64 where those fill the machine, and calls of more than 1024 partial results, which
+    are worked through in groups of sequences.  Lengths around 32, 64 and 128 tokens, one sequence empty; tolerances of the
+    storage type, as everywhere."""
+    lens = {"small_tiles": (31, 32, 33, 0, 63, 64, 65, 129), "large_tiles": (1473, 1, 1472, 0, 1471),
+            "int8_large_tiles": (1473, 1, 1472, 0, 1471), "groups": (33000, 65, 0, 32900)}[case]
+    if case == "groups":
+        w = synth.scaled(synth.CONFIGS["c3"], n_layers=1, n_q_heads=4, n_kv_heads=2, head_dim=32, latent_full=32,
+                         batch=len(lens), cached_tokens=0, decode_steps=1, reuse_frac=0.0, storage="f32")
+    else:
+        quant = case.startswith("int8")
+        w = synth.scaled(synth.CONFIGS["c2"], n_layers=2, batch=len(lens), cached_tokens=0, decode_steps=1, reuse_frac=0.25,
+                         storage="bf16" if quant else "f32")
+    pps = (max(lens) + 2 + w.page_tokens - 1) // w.page_tokens
+    p = Pair(w, max_seqs=len(lens), max_pages=len(lens) * pps, max_pages_per_seq=pps, latent_quant=case.startswith("int8"))
+    seqs = list(range(len(lens)))
+    p.open(seqs)
+    for s_, n in zip(seqs, lens):
+        if n:
+            p.prefill([s_], n)
+    _check_step(p.decode_step(seqs, 0), w.storage, case)
