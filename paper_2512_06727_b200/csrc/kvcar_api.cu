@@ -91,7 +91,7 @@ struct kvcar_ctx {
     TcState tc;
     LatState lat;
     FmaState fma;
-    enum Tiles { TILES_ROWS, TILES_LATENT, TILES_FMA } tiles_by = TILES_ROWS;  // whose partial results the merge finds
+    bool fma_tiles = false;  // the last tile launch was the fp32-FMA kernels': their merge follows
     float *static_scratch = nullptr;  // device address of the built-in scratch array, looked up at bind time
 
     int64_t launches = 0;
@@ -780,6 +780,33 @@ kvcar_status kvcar_encode_append(kvcar_ctx *c, int32_t layer, const int32_t *seq
     return enqueue_encode(c, layer, seqs, n_seqs, n_tokens, k, v, st);
 }
 
+static EncodeArgs encode_args(const kvcar_ctx *c, int32_t layer, int32_t n_tokens, const void *k, const void *v) {
+    EncodeArgs a{};
+    a.plan = reinterpret_cast<const EncPlan *>(c->weights + c->enc_off) + layer * 2;
+    a.block_table = reinterpret_cast<const int32_t *>(c->ws + c->bt_off);
+    a.seq_len = reinterpret_cast<const int32_t *>(c->ws + c->len_off);
+    a.k = k;
+    a.v = v;
+    a.max_pages_per_seq = c->cfg.max_pages_per_seq;
+    a.page_tokens = c->cfg.page_tokens;
+    a.n_tokens = n_tokens;
+    a.kv_width = c->cfg.n_kv_heads * c->cfg.head_dim;
+    a.hd = c->cfg.head_dim;
+    return a;
+}
+
+// one token per sequence: the fully connected layers one after the other, features spread over all SMs (needs 16-byte loadable
+// weight rows and its row block in shared memory)
+static bool encode_splits(const kvcar_ctx *c, int32_t layer) {
+    const int vl = 16 / c->elem;
+    if (c->cfg.latent_quant || c->cfg.head_dim % vl != 0 || encode_split_smem(c->max_in, c->max_m) > 200 * 1024) return false;
+    for (int w = 0; w < 2; ++w) {
+        const AEHost &ae = c->ae[layer * 2 + w];
+        if (ae.set && (ae.in_dim % vl || ae.hidden % vl)) return false;
+    }
+    return true;
+}
+
 // what the tensor-core encoder takes
 static bool prefill_fits(const kvcar_ctx *c, int32_t layer, const char **why) {
     const kvcar_config &g = c->cfg;
@@ -827,28 +854,11 @@ static kvcar_status enqueue_encode(kvcar_ctx *c, int32_t layer, const int32_t *s
     const char *why;
     if (n_tokens > 1 && prefill_fits(c, layer, &why) && (int64_t)n_seqs * n_tokens <= 0x7fffffff)
         return enqueue_prefill(c, layer, seqs, n_seqs, n_tokens, k, v, true, st);
-    EncodeArgs a{};
-    a.plan = reinterpret_cast<const EncPlan *>(c->weights + c->enc_off) + layer * 2;
-    a.block_table = reinterpret_cast<const int32_t *>(c->ws + c->bt_off);
-    a.seq_len = reinterpret_cast<const int32_t *>(c->ws + c->len_off);
-    a.k = k;
-    a.v = v;
-    a.max_pages_per_seq = c->cfg.max_pages_per_seq;
-    a.page_tokens = c->cfg.page_tokens;
-    a.n_tokens = n_tokens;
-    a.kv_width = c->cfg.n_kv_heads * c->cfg.head_dim;
-    a.hd = c->cfg.head_dim;
+    const EncodeArgs a = encode_args(c, layer, n_tokens, k, v);
     SeqList sl;
     sl.n = n_seqs;
     memcpy(sl.id, seqs, (size_t)n_seqs * 4);
-    // one token per sequence: one launch per fully connected layer, features spread over all SMs
-    // (needs 16-byte loadable weight rows and its row block in shared memory)
-    const int vl = 16 / c->elem;
-    bool split_ok = n_tokens == 1 && !c->cfg.latent_quant && c->cfg.head_dim % vl == 0 && encode_split_smem(c->max_in, c->max_m) <= 200 * 1024;
-    for (int w = 0; w < 2 && split_ok; ++w) {
-        const AEHost &ae = c->ae[layer * 2 + w];
-        if (ae.set && (ae.in_dim % vl || ae.hidden % vl)) split_ok = false;
-    }
+    const bool split_ok = n_tokens == 1 && encode_splits(c, layer);
     const int nb = std::min(c->cfg.max_seqs, KVCAR_MAX_BATCH);
     cudaError_t e = split_ok ? launch_encode_split(a, sl, c->cfg.storage, c->max_in, c->max_m, c->max_d,
                                                    reinterpret_cast<float *>(c->ws + c->enchid_off), nb, st)
@@ -927,28 +937,15 @@ static int prepare_decode(kvcar_ctx *c, int32_t layer, const int32_t *seqs, int3
 // step's encoder writes (the exact current token enters in the combine kernel).
 static kvcar_status enqueue_decode_tiles(kvcar_ctx *c, int32_t layer, const DecodeArgs &a, const SeqList &sl,
                                          int n_chunks, cudaStream_t st) {
-    c->tiles_by = kvcar_ctx::TILES_ROWS;
+    c->fma_tiles = false;
     if (n_chunks <= 0) return KVCAR_OK;
     const kvcar_config &g = c->cfg;
-    int n_tiles = 0;
-    for (int i = 0; i < sl.n; ++i) n_tiles += (c->len[sl.id[i]] + 127) / 128;
     const bool want_tc = use_tensor_kernel(c) && tc_layer_supported(c->tc, layer);
-    bool want_lat = use_tensor_kernel(c) && lat_layer_supported(c->lat, layer, a.flags);
-    // Few tiles leave most of the latent kernel's clusters without work while the restoring kernel spreads a pair of tiles over
-    // several: at 64 tiles of the GPT-2 shape a 12-layer step takes 712 us here and 688 us there, at 128 tiles 814 and 971; at
-    // 128 tiles of the TinyLLaMA shape 868 and 786, at 256 tiles 1024 and 1118.
-    if (want_lat && want_tc && !(a.flags & KVCAR_ABSORBED) && n_tiles < (c->lat.cfg[layer].max_m > 192 ? 80 : 148)) want_lat = false;
-    if (c->kernel == KVCAR_KERNEL_TENSOR && !want_tc && !want_lat)
+    if (c->kernel == KVCAR_KERNEL_TENSOR && !want_tc)
         return fail(c, KVCAR_ERR_UNSUPPORTED, std::string("tensor-core kernel cannot run this layer: ") + c->tc.why);
     cudaError_t e;
     if (c->kernel != KVCAR_KERNEL_GENERIC && layer_is_raw(c, layer)) {
         e = launch_decode_raw(a, sl, c->raw_src_ok[layer] ? &c->raw_src[layer] : nullptr, g.storage, n_chunks, st);
-    } else if (want_lat) {
-        int32_t lens[KVCAR_MAX_BATCH];
-        for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
-        e = lat_launch_tiles(c->lat, a, sl, lens, layer, st);
-        c->tiles_by = kvcar_ctx::TILES_LATENT;
-        ++c->launches;
     } else if (want_tc) {
         int32_t lens[KVCAR_MAX_BATCH];
         for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
@@ -958,7 +955,7 @@ static kvcar_status enqueue_decode_tiles(kvcar_ctx *c, int32_t layer, const Deco
         for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
         int n = 1;
         e = fma_launch_tiles(c->fma, g, a, sl, lens, layer, st, &n);
-        c->tiles_by = kvcar_ctx::TILES_FMA;
+        c->fma_tiles = true;
         c->launches += n - 1;
     } else {
         if (decode_generic_smem(a.hq, a.hd, c->max_d, c->max_m) > 227 * 1024)
@@ -972,16 +969,48 @@ static kvcar_status enqueue_decode_tiles(kvcar_ctx *c, int32_t layer, const Deco
 
 static kvcar_status enqueue_combine(kvcar_ctx *c, int32_t layer, const DecodeArgs &a, const SeqList &sl, int n_chunks, cudaStream_t st) {
     cudaError_t e;
-    if (c->tiles_by != kvcar_ctx::TILES_ROWS) {
+    if (c->fma_tiles) {
         int32_t lens[KVCAR_MAX_BATCH];
         for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
-        e = c->tiles_by == kvcar_ctx::TILES_LATENT ? lat_launch_merge(c->lat, a, sl, lens, layer, st)
-                                                   : fma_launch_merge(c->fma, c->cfg, a, sl, lens, layer, st);
+        e = fma_launch_merge(c->fma, c->cfg, a, sl, lens, layer, st);
     } else {
         e = launch_combine(a, sl, c->cfg.storage, n_chunks, st);
     }
     if (e != cudaSuccess) return cuda_fail(c, e, "combine launch");
     ++c->launches;
+    return KVCAR_OK;
+}
+
+// the latent-attention kernels take this call
+static bool use_latent(const kvcar_ctx *c, int32_t layer, int n_chunks, uint32_t flags) {
+    return n_chunks > 0 && use_tensor_kernel(c) && lat_layer_supported(c->lat, layer, flags);
+}
+// all of such a call; with k and v the encoder of the same step's rows goes along in the same launches
+static kvcar_status enqueue_latent(kvcar_ctx *c, int32_t layer, const DecodeArgs &a, const SeqList &sl, const void *k, const void *v,
+                                   cudaStream_t st) {
+    int32_t lens[KVCAR_MAX_BATCH];
+    for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
+    LatEncode e;
+    const bool carry = k && encode_splits(c, layer) && encode_split_smem(c->max_in, c->max_m) <= LT_ENC_SMEM;
+    if (carry) {
+        e.a = encode_args(c, layer, 1, k, v);
+        e.hid = reinterpret_cast<float *>(c->ws + c->enchid_off);
+        e.pitch = c->max_m;
+        e.max_batch = std::min(c->cfg.max_seqs, KVCAR_MAX_BATCH);
+        e.max_m = e.max_d = 0;
+        for (int w = 0; w < 2; ++w) {
+            e.max_m = std::max(e.max_m, c->ae[layer * 2 + w].hidden);
+            e.max_d = std::max(e.max_d, c->ae[layer * 2 + w].latent);
+        }
+        e.max_in = c->max_in;
+    } else if (k) {
+        kvcar_status s = enqueue_encode(c, layer, sl.id, sl.n, 1, k, v, st);
+        if (s != KVCAR_OK) return s;
+    }
+    int n = 0;
+    cudaError_t err = lat_launch(c->lat, a, sl, lens, layer, carry ? &e : nullptr, st, &n);
+    if (err != cudaSuccess) return cuda_fail(c, err, "decode launch");
+    c->launches += n;
     return KVCAR_OK;
 }
 
@@ -1008,6 +1037,7 @@ kvcar_status kvcar_decode_attention(kvcar_ctx *c, int32_t layer, const int32_t *
     DecodeArgs a;
     SeqList sl;
     const int n_chunks = prepare_decode(c, layer, seqs, n_seqs, q, out, flags, a, sl);
+    if (use_latent(c, layer, n_chunks, flags)) return enqueue_latent(c, layer, a, sl, nullptr, nullptr, st);
     s = enqueue_decode_tiles(c, layer, a, sl, n_chunks, st);
     if (s != KVCAR_OK) return s;
     return enqueue_combine(c, layer, a, sl, n_chunks, st);
@@ -1029,6 +1059,7 @@ kvcar_status kvcar_step_layer(kvcar_ctx *c, int32_t layer, const int32_t *seqs, 
     DecodeArgs a;
     SeqList sl;
     const int n_chunks = prepare_decode(c, layer, seqs, n_seqs, q, out, flags, a, sl);
+    if (use_latent(c, layer, n_chunks, flags)) return enqueue_latent(c, layer, a, sl, k, v, st);
     // The tile kernel does not depend on this step's encoder, so it goes to a side stream that forks here and
     // joins before the combine kernel: the encoder's two short launches overlap it instead of running in front
     // of it.  (The other way round - encoder on the side stream behind the fork event - measured no gain: the

@@ -11,10 +11,14 @@
 // bf16 hidden vector itself carries), so nothing is rounded more coarsely than in the form that restores the rows;
 // with KVCAR_ABSORBED (| KVCAR_ABSORBED_V) the caller takes one bf16 term, as that flag says.
 //
-// Three launches per call:
-//   latent_query_kernel   W4_h^T q per (K source, listed sequence, query head) -> bf16 rows, high and low part
-//   decode_latent_kernel  tiles of 128 cached tokens -> per run of tiles: reference maximum, sum, U = sum p a
-//   latent_merge_kernel   runs of a sequence -> W4_h U + b4_h sum, the exact current token, the output row
+// Three launches per call, four on small grids, one behind the other in the caller's stream as programmatic dependent launches
+// (each starts while its predecessor ends and waits for it only where it needs its results):
+//   latent_front_kernel   W4_h^T q per (K source, listed sequence, query head) -> bf16 rows, high and low part; in a step also
+//                         the first layer of the new rows' encoder
+//   decode_latent_kernel  tiles of 128 cached tokens -> per run of tiles: reference maximum, sum, U = sum p a.  Small grids: one
+//                         launch for the scores and one for U, their clusters side by side (see lat_launch)
+//   latent_back_kernel    runs of a sequence -> W4_h U + b4_h sum, the exact current token, the output row; in a step also the
+//                         second layer of the encoder
 //
 // decode_latent_kernel.  A cluster of two CTAs walks two runs of consecutive tiles in step, one run per CTA; every
 // product is one tcgen05.mma.cta_group::2 of M = 256 (both tiles), so a weight slab crosses L2 -> shared memory once
@@ -49,6 +53,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "kvcar_encode.cuh"
 #include "kvcar_latent.h"
 #include "kvcar_ptx.cuh"
 
@@ -76,8 +81,11 @@ __host__ __device__ constexpr int wq_rows(int nq) { return 2 * nq; }            
 __host__ __device__ constexpr int wq_slab(int nq) { return wq_rows(nq) * 128; }       // one 64-column slab of them
 
 struct Params {
-    LatLayer l;
-    CUtensorMap tm_wq;
+    CUtensorMap pool[2][LT_MAX_SRC], w1[2][LT_MAX_SRC], tm_wq;
+    // MODE_BOTH: list[0] = K, list[1] = V.  MODE_K / MODE_V: list[p] = part p of that side's columns, one cluster per part
+    LatList list[LT_MAX_PARTS];
+    int32_t mode, n_parts, k_parts;  // k_parts: parts of the scores (MODE_V sums them)
+    float *score;
     LatSeqs sq;
     const int32_t *block_table;
     int32_t *status;
@@ -88,6 +96,8 @@ struct Params {
     int32_t t_resident;                // every source has a shift buffer of its own
     int32_t two_terms_k, two_terms_v;  // low parts of the query rows / of the probabilities are used
 };
+
+constexpr int MODE_BOTH = 0, MODE_K = 1, MODE_V = 2;
 
 template <int SLEEP_NS = 0>
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int32_t *status, volatile int *abort_flag, int code) {
@@ -224,10 +234,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     const uint32_t p_ready = o_empty + 16;
     Scratch<NQ> &sh = *reinterpret_cast<Scratch<NQ> *>(smem_raw + (p_ready + 8 - s_z));
     volatile int &abort_flag = sh.abort_flag;
+    // pair of runs, and which part of a side's hidden columns (one part unless the grid is small)
+    const int pair = (int)(blockIdx.x >> 1) / a.n_parts, part = (int)(blockIdx.x >> 1) % a.n_parts;
+    const int side_lo = a.mode == MODE_V ? 1 : 0, side_hi = a.mode == MODE_K ? 1 : 2;
+    auto list_of = [&](int side) -> const LatList & { return a.list[a.mode == MODE_BOTH ? side : part]; };
     // tiles of the cluster's longer run (the leader's); the other CTA idles through the last ones it does not have
-    const int cta0 = (int)(blockIdx.x & ~1u);
-    const int n_it = max(0, min(a.sq.per, a.sq.n_tiles - cta0 * a.sq.per));
-    const int my_first = (int)blockIdx.x * a.sq.per;
+    const int my_run = 2 * pair + (int)rank;
+    const int n_it = max(0, min(a.sq.per, a.sq.n_tiles - 2 * pair * a.sq.per));
+    const int my_first = my_run * a.sq.per;
+    enc::launch_dependents();
 
     if (threadIdx.x == 0) {
         sh.abort_flag = 0;
@@ -289,7 +304,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             struct Pos {
                 int it, side, s, k;
             };
-            Pos z{0, 0, 0, 0}, q{0, 0, 0, 0}, t{0, 0, 0, 0};
+            Pos z{0, side_lo, 0, 0}, q{a.mode == MODE_V ? n_it : 0, 0, 0, 0}, t{0, side_lo, 0, 0};
+            bool waited = false;  // for the launch before, which writes the query rows
             uint32_t zslot = 0, zphase = 0, qslot = 0, qphase = 0, tslot = 0, tphase = 0;
             TileWalk zw, qw;
             zw.start(a.sq, my_first);
@@ -305,15 +321,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                 if (z.it < n_it && mbar_test(z_empty + 8 * zslot, zphase ^ 1u)) {
                     moved = true;
                     if (leader) mbar_expect_tx(z_full + 8 * zslot, 2 * SLAB);
-                    const CUtensorMap *map = &a.l.pool[z.side][z.s];
+                    const LatSrc &zp_ = list_of(z.side).src[z.s];
+                    const CUtensorMap *map = &a.pool[z.side][zp_.map];
                     const uint32_t fb = map_to_cta(z_full + 8 * zslot, 0), dst = s_z + zslot * SLAB;
                     tma_load_2d_pair(dst, map, z.k * 64, row[0], fb);
                     tma_load_2d_pair(dst + SLAB / 2, map, z.k * 64, row[1], fb);
                     if (++zslot == (uint32_t)a.nz) { zslot = 0; zphase ^= 1u; }
-                    const int ks1 = (a.l.src[z.side][z.s].d + 63) >> 6;
+                    const int ks1 = (zp_.d + 63) >> 6;
                     if (++z.k == ks1) {
                         // the same rows of the next tile: from HBM into L2 while this one is worked on
-                        if (z.side == 0 && z.s == 0) {
+                        if (z.side == side_lo && z.s == 0) {
                             zw.next(a.sq);
                             rows_of(zw, nrow);
                         }
@@ -323,10 +340,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                                 if (nrow[1] != nrow[0]) tma_prefetch_2d(map, ks * 64, nrow[1]);
                             }
                         z.k = 0;
-                        if (++z.s == a.l.n_src[z.side]) {
+                        if (++z.s == list_of(z.side).n) {
                             z.s = 0;
-                            if (++z.side == 2) {
-                                z.side = 0;
+                            if (++z.side == side_hi) {
+                                z.side = side_lo;
                                 ++z.it;
                                 row[0] = nrow[0];
                                 row[1] = nrow[1];
@@ -336,30 +353,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                 }
                 if (t.it < t_its && mbar_test(tb_empty + 8 * tslot, tphase ^ 1u)) {
                     moved = true;
-                    const LatSrc &sp = a.l.src[t.side][t.s];
+                    const LatSrc &sp = list_of(t.side).src[t.s];
                     const uint32_t bytes = (uint32_t)((sp.m + 31) & ~31) * 4u;
                     mbar_expect_tx(tb_full + 8 * tslot, bytes);
                     bulk_load(s_t + tslot * a.m_t * 4, sp.shift, bytes, tb_full + 8 * tslot);
                     if (++tslot == (uint32_t)a.nt) { tslot = 0; tphase ^= 1u; }
-                    if (++t.s == a.l.n_src[t.side]) {
+                    if (++t.s == list_of(t.side).n) {
                         t.s = 0;
-                        if (++t.side == 2) {
-                            t.side = 0;
+                        if (++t.side == side_hi) {
+                            t.side = side_lo;
                             ++t.it;
                         }
                     }
                 }
-                if (q.it < n_it && mbar_test(q_empty + 8 * qslot, qphase ^ 1u)) {
+                if (!waited && a.mode != MODE_V && (!moved || z.it > 0 || z.side > side_lo)) {
+                    enc::grid_dependency_wait();
+                    waited = moved = true;
+                }
+                if (waited && q.it < n_it && mbar_test(q_empty + 8 * qslot, qphase ^ 1u)) {
                     moved = true;
-                    const int y = (q.s * a.wq_batch + qw.si) * wq_rows(NQ);
+                    const LatSrc &sp = list_of(0).src[q.s];
+                    const int y = (sp.map * a.wq_batch + qw.si) * wq_rows(NQ), x = sp.c0 + q.k * 64;
                     if (leader) mbar_expect_tx(q_full + 8 * qslot, low_k ? 2 * QSLAB : QSLAB);
                     const uint32_t fb = map_to_cta(q_full + 8 * qslot, 0), dst = s_q + qslot * QSLAB;
-                    tma_load_2d_pair(dst, &a.tm_wq, q.k * 64, y, fb);
-                    if (NQ > 16 && low_k) tma_load_2d_pair(dst + QSLAB / 2, &a.tm_wq, q.k * 64, y + R, fb);
+                    tma_load_2d_pair(dst, &a.tm_wq, x, y, fb);
+                    if (NQ > 16 && low_k) tma_load_2d_pair(dst + QSLAB / 2, &a.tm_wq, x, y + R, fb);
                     if (++qslot == (uint32_t)a.nqs) { qslot = 0; qphase ^= 1u; }
-                    if (++q.k == (a.l.src[0][q.s].m + 63) >> 6) {
+                    if (++q.k == (sp.m + 63) >> 6) {
                         q.k = 0;
-                        if (++q.s == a.l.n_src[0]) {
+                        if (++q.s == list_of(0).n) {
                             q.s = 0;
                             ++q.it;
                             qw.next(a.sq);
@@ -382,18 +404,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                     }
                 }
             }
+            if (!waited) enc::grid_dependency_wait();  // every block sees the launches before complete: those after rely on it
         }
     } else if (warp == 2) {
         // ============================== weight loads ==============================
         if (elect_one()) {
             uint32_t slot = 0, phase = 0;
             for (int it = 0; it < n_it; ++it)
-                for (int side = 0; side < 2; ++side)
-                    for (int s = 0; s < a.l.n_src[side]; ++s) {
-                        const int ks1 = (a.l.src[side][s].d + 63) >> 6, m = a.l.src[side][s].m;
-                        const CUtensorMap *map = &a.l.w1[side][s];
+                for (int side = side_lo; side < side_hi; ++side)
+                    for (int s = 0; s < list_of(side).n; ++s) {
+                        const LatSrc &sp = list_of(side).src[s];
+                        const int ks1 = (sp.d + 63) >> 6, m = sp.m;
+                        const CUtensorMap *map = &a.w1[side][sp.map];
                         for (int c0 = 0; c0 < m; c0 += CN) {
-                            const int y = c0 + (int)rank * (min(CN, m - c0) >> 1);
+                            const int y = sp.c0 + c0 + (int)rank * (min(CN, m - c0) >> 1);
                             for (int ks = 0; ks < ks1; ++ks) {
                                 mbar_wait<32>(w_empty + 8 * slot, phase ^ 1u, a.status, &abort_flag, 0x602);
                                 if (leader) mbar_expect_tx(w_full + 8 * slot, 2 * WSTAGE);
@@ -409,9 +433,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             uint32_t wslot = 0, wphase = 0, zslot = 0, zphase = 0, h = 0;
             const uint64_t z_desc = make_desc(s_z), w_desc = make_desc(s_w);
             for (int it = 0; it < n_it; ++it)
-                for (int side = 0; side < 2; ++side)
-                    for (int s = 0; s < a.l.n_src[side]; ++s) {
-                        const int d = a.l.src[side][s].d, m = a.l.src[side][s].m;
+                for (int side = side_lo; side < side_hi; ++side)
+                    for (int s = 0; s < list_of(side).n; ++s) {
+                        const int d = list_of(side).src[s].d, m = list_of(side).src[s].m;
                         const int ks1 = (d + 63) >> 6, nk_last = ((d - 1) & 63) / 16 + 1;
                         uint32_t zs = 0, zp = 0;
                         for (int c0 = 0; c0 < m; c0 += CN, ++h) {
@@ -457,12 +481,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             const uint64_t h_desc = make_desc(s_h), q_desc = make_desc(s_q), p_desc = make_desc(s_p);
             const bool two = NQ > 16 && a.two_terms_k;
             for (int it = 0; it < n_it; ++it) {
-                {  // S
+                if (side_lo == 0) {  // S
                     const uint32_t ob = o & 1u, acc = tmem + TM_OUT + 64u * ob;
                     mbar_wait(o_empty + 8 * ob, ((o >> 1) & 1u) ^ 1u, a.status, &abort_flag, 0x605);
                     bool begin = true;
-                    for (int s = 0; s < a.l.n_src[0]; ++s) {
-                        const int m = a.l.src[0][s].m, ksm = (m + 63) >> 6, nk_last = ((m - 1) & 63) / 16 + 1;
+                    for (int s = 0; s < list_of(0).n; ++s) {
+                        const int m = list_of(0).src[s].m, ksm = (m + 63) >> 6, nk_last = ((m - 1) & 63) / 16 + 1;
 #pragma unroll 1
                         for (int sl = 0, in_job = 0; sl < ksm; ++sl) {
                             if (in_job == 0) {  // the job's slabs, written by both CTAs
@@ -499,8 +523,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                     ++o;
                 }
                 bool p_seen = false;
-                for (int s = 0; s < a.l.n_src[1]; ++s) {  // U
-                    const int ksm = (a.l.src[1][s].m + 63) >> 6;
+                for (int s = 0; s < (side_hi == 2 ? list_of(1).n : 0); ++s) {  // U
+                    const int ksm = (list_of(1).src[s].m + 63) >> 6;
                     hslot += hslot & 1u;  // slabs go in pairs: a source starts at an even place
                     if (hslot == (uint32_t)a.nh) hslot = 0;
 #pragma unroll 1
@@ -549,10 +573,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         tw.start(a.sq, my_first);
         for (int it = 0; it < n_it; ++it, tw.next(a.sq)) {
             const int valid = tw.valid(a.sq);
-            for (int side = 0; side < 2; ++side) {
-                for (int s = 0; s < a.l.n_src[side]; ++s) {
-                    const int m = a.l.src[side][s].m;
-                    const float slope = a.l.src[side][s].slope;
+            for (int side = side_lo; side < side_hi; ++side) {
+                const int n_src = list_of(side).n;
+                for (int s = 0; s < n_src; ++s) {
+                    const int m = list_of(side).src[s].m;
+                    const float slope = list_of(side).src[s].slope;
                     const float2 slope2 = make_float2(slope, slope);
                     const bool lr_max = slope <= 1.f;
                     // V side: rows past the tile's end may hold anything, and zero times a stray NaN is not zero
@@ -625,7 +650,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                     }
                     __syncwarp();
                     if (!a.t_resident && elect_one()) mbar_arrive_local(tb_empty + 8 * tb);
-                    if (++tb == (uint32_t)a.nt || (a.t_resident && side == 1 && s + 1 == a.l.n_src[1])) { tb = 0; tphase ^= 1u; }
+                    if (++tb == (uint32_t)a.nt || (a.t_resident && side + 1 == side_hi && s + 1 == n_src)) { tb = 0; tphase ^= 1u; }
                 }
             }
         }
@@ -676,9 +701,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         tw.start(a.sq, my_first);
         for (int it = 0; it < n_it; ++it, tw.next(a.sq)) {
             const int valid = tw.valid(a.sq), par = it & 1;
-            {
-                float s[NT];
+            float s[NT];
+            if (a.mode != MODE_V) {
                 fetch(s);
+            } else {
+                if (it == 0) enc::grid_dependency_wait();  // the launch before holds the scores
+#pragma unroll
+                for (int q = 0; q < NT; ++q) s[q] = 0.f;
+                for (int p = 0; p < a.k_parts; ++p) {
+                    const float *sp = a.score + ((int64_t)((pair * a.k_parts + p) * 2 + (int)rank) * NQ + q0) * TILE + row;
+#pragma unroll
+                    for (int q = 0; q < NT; ++q) s[q] += sp[q * TILE];
+                }
+            }
+            if (a.mode == MODE_K) {  // one cluster's part of the sums over the hidden columns
+                float *sp = a.score + ((int64_t)blockIdx.x * NQ + q0) * TILE + row;
+#pragma unroll
+                for (int q = 0; q < NT; ++q) sp[q * TILE] = s[q];
+                continue;
+            }
+            {
 #pragma unroll
                 for (int q = 0; q < NT; ++q)
                     if (row >= valid) s[q] = -INFINITY;
@@ -724,9 +766,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                 __syncwarp();
                 if (elect_one()) mbar_arrive_remote(pready_leader);
             }
-            for (int s = 0; s < a.l.n_src[1]; ++s) {
-                const int n_blk = (((a.l.src[1][s].m + 63) >> 6) + 1) >> 1;
-                const uint32_t mask = a.l.src[1][s].mask >> q0;
+            for (int si = 0; si < list_of(1).n; ++si) {
+                const int n_blk = (((list_of(1).src[si].m + 63) >> 6) + 1) >> 1;
+                const uint32_t mask = list_of(1).src[si].mask >> q0;
 #pragma unroll
                 for (int b = 0; b < NB; ++b) {
                     if (b < n_blk) {
@@ -739,11 +781,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                 }
             }
             if (tw.ends_run()) {
-                const int64_t run = (int64_t)blockIdx.x + tw.si;  // block and sequence only ever grow along the runs: unique
-                for (int s = 0; s < a.l.n_src[1]; ++s) {
-                    const int m = a.l.src[1][s].m;
-                    const uint32_t mask = a.l.src[1][s].mask >> q0;
-                    float *u = a.upart + (run * a.hq + q0) * a.m_pad + row;
+                const int64_t run = (int64_t)my_run + tw.si;  // run and sequence only ever grow along the runs: unique
+                for (int si = 0; si < list_of(1).n; ++si) {
+                    const int m = list_of(1).src[si].m;
+                    const uint32_t mask = list_of(1).src[si].mask >> q0;
+                    float *u = a.upart + (run * a.hq + q0) * a.m_pad + list_of(1).src[si].c0 + row;
 #pragma unroll
                     for (int b = 0; b < NB; ++b)
 #pragma unroll
@@ -764,7 +806,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                 if (lane < NT) sh.lred[q0 + lane][quarter] = keep;
                 half_sync();
                 if (quarter == 0 && lane < NT) {
-                    if (q0 + lane < a.hq) {
+                    if (q0 + lane < a.hq && part == 0) {
                         const float *r = sh.lred[q0 + lane];
                         float *ml = a.ml + (run * a.hq + q0 + lane) * 2;
                         ml[0] = sh.mrun[par ^ 1][q0 + lane];
@@ -786,82 +828,102 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     }
 }
 
-// ---------------------------------------------------------------------------- W4_h^T q
-// grid = (query heads, blocks of 256 hidden columns, blocks of LQ_SB sequences); thread = two hidden columns, all 64 rows of
-// the head.  The query is scaled by 1/sqrt(head_dim) and by log2(e): the tile kernel's exponentials are powers of two.
-// Bound by the latency of the weight loads at few sequences, so all of them are in flight; everything else comes from the
-// parameters.  Operand rows of sources that do not serve the head are zeroed.
-constexpr int LQ_SB = 8, LQ_THREADS = 128;
-__global__ void __launch_bounds__(LQ_THREADS) latent_query_kernel(const __grid_constant__ LatHeads hp, const __nv_bfloat16 *q,
-                                                                  int n_seqs, int hq, int group, float scale, __nv_bfloat16 *wq,
-                                                                  float *qbias, int nq, int m_pad, int batch, int two_terms) {
+// ---------------------------------------------------------------------------- front
+// Encoder blocks first (where the call carries the encoder), then the query blocks: (query head, 256 hidden columns, 8 sequences),
+// thread = two hidden columns and four of the sequences, all 64 rows of the head.  The query is scaled by 1/sqrt(head_dim) and by
+// log2(e): the tile kernel's exponentials are powers of two.  Bound by the latency of the weight loads at few sequences, so all
+// of them are in flight before the wait for the preceding kernels; everything else comes from the parameters.  Operand rows of
+// sources that do not serve the head are zeroed.
+constexpr int LQ_SB = 8, LQ_COLS = 256, LF_THREADS = 256;
+struct QueryArgs {
+    const __nv_bfloat16 *q;
+    __nv_bfloat16 *wq;
+    float *qbias;
+    int32_t n_seqs, hq, group, nq, m_pad, batch, two_terms;
+    int32_t col_blocks;
+    float scale;
+};
+__device__ __forceinline__ void query_block(const LatHeads &hp, const QueryArgs &a, int b) {
     __shared__ __align__(16) float qs[64][LQ_SB];
-    const int qh = blockIdx.x, si0 = blockIdx.z * LQ_SB, tid = threadIdx.x;
-    const int n_here = min(LQ_SB, n_seqs - si0);
-    const int kvh = qh / group, s = hp.idx[0][kvh], slot = hp.slot[0][kvh];
+    const int qh = b % a.hq, cb = b / a.hq % a.col_blocks, si0 = b / a.hq / a.col_blocks * LQ_SB, tid = threadIdx.x;
+    const int n_here = min(LQ_SB, a.n_seqs - si0), i0 = 4 * (tid >> 7);
+    const int kvh = qh / a.group, s = hp.idx[0][kvh], slot = hp.slot[0][kvh];
     const LatHeads::Src &sp = hp.src[0][s];
-    const int m2 = sp.m >> 1, j = blockIdx.y * LQ_THREADS + tid;
+    const int m2 = sp.m >> 1, j = cb * (LQ_COLS / 2) + (tid & 127);
     const uint32_t *w = reinterpret_cast<const uint32_t *>(sp.w2k) + (int64_t)slot * 64 * m2 + j;
     uint32_t u[64];
     float2 sab = make_float2(0.f, 0.f);  // the hidden vector is short of these
 #pragma unroll
     for (int c = 0; c < 64; ++c) u[c] = j < m2 ? __ldg(w + (int64_t)c * m2) : 0u;
     if (j < m2) sab = __ldg(reinterpret_cast<const float2 *>(sp.sabs) + j);
-    for (int i = tid; i < 64 * LQ_SB; i += LQ_THREADS) {
+    enc::grid_dependency_wait();
+    enc::launch_dependents();
+    for (int i = tid; i < 64 * LQ_SB; i += LF_THREADS) {
         const int k = i >> 6, c = i & 63;
-        qs[c][k] = k < n_here ? __bfloat162float(q[((int64_t)(si0 + k) * hq + qh) * 64 + c]) * scale : 0.f;
+        qs[c][k] = k < n_here ? __bfloat162float(a.q[((int64_t)(si0 + k) * a.hq + qh) * 64 + c]) * a.scale : 0.f;
     }
     __syncthreads();
-    float x[LQ_SB], y[LQ_SB];
-#pragma unroll
-    for (int i = 0; i < LQ_SB; ++i) x[i] = y[i] = 0.f;
+    float x[4] = {0.f, 0.f, 0.f, 0.f}, y[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int c = 0; c < 64; ++c) {
         const float w0 = __uint_as_float(u[c] << 16), w1 = __uint_as_float(u[c] & 0xffff0000u);
-#pragma unroll
-        for (int i = 0; i < LQ_SB; i += 4) {
-            const float4 q4 = *reinterpret_cast<const float4 *>(&qs[c][i]);
-            x[i] = fmaf(w0, q4.x, x[i]);
-            x[i + 1] = fmaf(w0, q4.y, x[i + 1]);
-            x[i + 2] = fmaf(w0, q4.z, x[i + 2]);
-            x[i + 3] = fmaf(w0, q4.w, x[i + 3]);
-            y[i] = fmaf(w1, q4.x, y[i]);
-            y[i + 1] = fmaf(w1, q4.y, y[i + 1]);
-            y[i + 2] = fmaf(w1, q4.z, y[i + 2]);
-            y[i + 3] = fmaf(w1, q4.w, y[i + 3]);
-        }
+        const float4 q4 = *reinterpret_cast<const float4 *>(&qs[c][i0]);
+        x[0] = fmaf(w0, q4.x, x[0]);
+        x[1] = fmaf(w0, q4.y, x[1]);
+        x[2] = fmaf(w0, q4.z, x[2]);
+        x[3] = fmaf(w0, q4.w, x[3]);
+        y[0] = fmaf(w1, q4.x, y[0]);
+        y[1] = fmaf(w1, q4.y, y[1]);
+        y[2] = fmaf(w1, q4.z, y[2]);
+        y[3] = fmaf(w1, q4.w, y[3]);
     }
-    const int rows = wq_rows(nq);  // operand rows per (source, sequence): high terms, then low terms
+    const int rows = wq_rows(a.nq);  // operand rows per (source, sequence): high terms, then low terms
 #pragma unroll
-    for (int i = 0; i < LQ_SB; ++i) {
-        if (i >= n_here) break;
+    for (int i = 0; i < 4; ++i) {
+        if (i0 + i >= n_here) break;
         x[i] *= sab.x;
         y[i] *= sab.y;
         const uint32_t hi = pack_bf16(x[i], y[i]);
-        const uint32_t lo = two_terms ? pack_bf16(x[i] - __uint_as_float(hi << 16), y[i] - __uint_as_float(hi & 0xffff0000u)) : 0u;
+        const uint32_t lo = a.two_terms ? pack_bf16(x[i] - __uint_as_float(hi << 16), y[i] - __uint_as_float(hi & 0xffff0000u)) : 0u;
         for (int ss = 0; ss < hp.n_src[0]; ++ss) {
             if (j >= (hp.src[0][ss].m >> 1)) continue;
-            uint32_t *r = reinterpret_cast<uint32_t *>(wq + (((int64_t)ss * batch + si0 + i) * rows + qh) * m_pad) + j;
+            uint32_t *r = reinterpret_cast<uint32_t *>(a.wq + (((int64_t)ss * a.batch + si0 + i0 + i) * rows + qh) * a.m_pad) + j;
             r[0] = ss == s ? hi : 0u;
-            r[(int64_t)nq * m_pad / 2] = ss == s ? lo : 0u;
+            r[(int64_t)a.nq * a.m_pad / 2] = ss == s ? lo : 0u;
         }
     }
-    if (blockIdx.y != 0) return;
+    if (cb != 0) return;
     const int warp = tid >> 5, lane = tid & 31;
-    for (int i = warp; i < n_here; i += LQ_THREADS / 32) {
-        float b = qs[lane][i] * sp.b2[slot * 64 + lane] + qs[lane + 32][i] * sp.b2[slot * 64 + lane + 32];
+    if (warp < n_here) {
+        float bias = qs[lane][warp] * sp.b2[slot * 64 + lane] + qs[lane + 32][warp] * sp.b2[slot * 64 + lane + 32];
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) b += __shfl_xor_sync(0xffffffffu, b, d);
-        if (lane == 0) qbias[(int64_t)(si0 + i) * hq + qh] = b;
+        for (int d = 16; d > 0; d >>= 1) bias += __shfl_xor_sync(0xffffffffu, bias, d);
+        if (lane == 0) a.qbias[(int64_t)(si0 + warp) * a.hq + qh] = bias;
     }
 }
 
-// ---------------------------------------------------------------------------- merge
-// grid = (query heads, blocks of SB sequences).  The last decoder layer's 64 rows of the head (73 KB at m = 576) are read once
+// n_enc = encoder blocks (0: none): nbx x nby x 2
+struct EncodeGrid {
+    int32_t n_enc, nbx, nby;
+};
+__global__ void __launch_bounds__(LF_THREADS) latent_front_kernel(const __grid_constant__ LatHeads hp, const __grid_constant__ QueryArgs a,
+                                                                  const __grid_constant__ LatEncode e, const __grid_constant__ SeqList seqs,
+                                                                  const __grid_constant__ EncodeGrid g) {
+    extern __shared__ __align__(16) float xs[];
+    const int b = blockIdx.x;
+    if (b < g.n_enc)
+        enc::encode_fc_block<__nv_bfloat16, 1, false>(e.a, seqs.id, seqs.n, e.hid, e.pitch, e.max_batch, xs, b % g.nbx, b / g.nbx % g.nby,
+                                                      b / g.nbx / g.nby, g.nbx);
+    else
+        query_block(hp, a, b - g.n_enc);
+}
+
+// ---------------------------------------------------------------------------- back
+// Encoder blocks first, then the merge: (query head, SB sequences).  The last decoder layer's 64 rows of the head (73 KB at m = 576) are read once
 // per SB sequences: SB = 4 where that still fills the machine, else 1 (at 8 sequences x 12 heads, 4 sequences per block left 24
-// blocks and took 57 us; SB = 1 with 288 threads 15 us, a chain of dependent loads; 8 us with 1024 threads whose registers take
-// the weights before anything else is known).
-constexpr int LM_PRE = 18;  // weight words a lane holds ahead: all of them up to m = 576 at 32 warps
+// blocks and took 57 us; SB = 1 with 288 threads 15 us, a chain of dependent loads; 8 us with threads whose registers take the
+// weights before anything else is known).
+constexpr int LM_PRE = 36;  // weight words a lane holds ahead: all of them up to m = 576 at 16 warps
 struct MergeArgs {
     const float *upart, *ml, *qbias;
     const __nv_bfloat16 *q;
@@ -871,14 +933,13 @@ struct MergeArgs {
     int32_t with_current;
 };
 template <int SB, int LM_THREADS>
-__global__ void __launch_bounds__(LM_THREADS) latent_merge_kernel(const __grid_constant__ LatHeads hp, const __grid_constant__ LatSeqs sq,
-                                                                  const __grid_constant__ MergeArgs a) {
-    extern __shared__ __align__(16) float u[];  // [SB][m_pad], with SB = 1 then the groups' partial sums [LM_THREADS][4]
+__device__ __forceinline__ void merge_block(const LatHeads &hp, const LatSeqs &sq, const MergeArgs &a, float *u, int b) {
+    // u: [SB][m_pad], with SB = 1 then the groups' partial sums [LM_THREADS][4]
     constexpr int LM_WARPS = LM_THREADS / 32;
     __shared__ float wts[SB][LT_MAX_CTAS];
     __shared__ float fin[SB][2];  // (sum of the runs, exponent reference) per sequence
     __shared__ float osum[LM_WARPS][SB][64];
-    const int qh = blockIdx.x, si0 = blockIdx.y * SB, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int qh = b % a.hq, si0 = b / a.hq * SB, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_here = min(SB, sq.n - si0);
     const int kvh = qh / a.group, slot = hp.slot[1][kvh];
     const LatHeads::Src &sp = hp.src[1][hp.idx[1][kvh]];
@@ -894,6 +955,8 @@ __global__ void __launch_bounds__(LM_THREADS) latent_merge_kernel(const __grid_c
             pre[k] = j < m ? __ldg(w + j * pitch) : 0u;
         }
     }
+    enc::grid_dependency_wait();
+    enc::launch_dependents();
     auto first = [&](int i) { return (int)(sq.first[i] & 0xffffffu); };
     auto runs = [&](int si, int &k0) {  // runs of a sequence: k0 .. k0 + n - 1
         const int f0 = first(si), f1 = first(si + 1);
@@ -1027,6 +1090,19 @@ __global__ void __launch_bounds__(LM_THREADS) latent_merge_kernel(const __grid_c
     out[lane + 32] = __float2bfloat16_rn(S > 0.f ? o[1] / S : 0.f);
 }
 
+template <int SB, int THREADS>
+__global__ void __launch_bounds__(THREADS) latent_back_kernel(const __grid_constant__ LatHeads hp, const __grid_constant__ LatSeqs sq,
+                                                              const __grid_constant__ MergeArgs a, const __grid_constant__ LatEncode e,
+                                                              const __grid_constant__ EncodeGrid g) {
+    extern __shared__ __align__(16) float sm[];
+    const int b = blockIdx.x;
+    if (b < g.n_enc)
+        enc::encode_fc_block<__nv_bfloat16, 2, false>(e.a, sq.id, sq.n, e.hid, e.pitch, e.max_batch, sm, b % g.nbx, b / g.nbx % g.nby,
+                                                      b / g.nbx / g.nby, g.nbx);
+    else
+        merge_block<SB, THREADS>(hp, sq, a, sm, b - g.n_enc);
+}
+
 using Kernel = void (*)(const Params);
 const Kernel kernels[] = {decode_latent_kernel<12, 2>, decode_latent_kernel<12, 5>, decode_latent_kernel<16, 5>,
                           decode_latent_kernel<16, 8>, decode_latent_kernel<32, 2>, decode_latent_kernel<32, 3>};
@@ -1067,7 +1143,7 @@ size_t lat_ws_bytes(const kvcar_config &cfg, int max_k_sources, int max_m, int b
     const size_t wq = (size_t)std::min(max_k_sources, LT_MAX_SRC) * batch * wq_rows((int)nq) * m_pad * 2;
     const size_t bias = ((size_t)batch * cfg.n_q_heads * 4 + 255) / 256 * 256;
     const size_t runs = (size_t)LT_MAX_CTAS + batch;
-    return wq + bias + runs * cfg.n_q_heads * (m_pad + 2) * sizeof(float);
+    return wq + bias + runs * cfg.n_q_heads * (m_pad + 2) * sizeof(float) + (size_t)LT_MAX_CTAS * nq * TILE * sizeof(float);
 }
 
 void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPlan> &plans, size_t pool_rows,
@@ -1084,6 +1160,9 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int group = cfg.n_q_heads / cfg.n_kv_heads;
     st.n_sms = sms;
+    for (auto k : {latent_back_kernel<4, 256>, latent_back_kernel<1, 512>})
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, LT_ENC_SMEM) != cudaSuccess) return;
+    if (cudaFuncSetAttribute(latent_front_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LT_ENC_SMEM) != cudaSuccess) return;
     st.nq = padded_heads(cfg.n_q_heads);
     st.group = group;
     st.m_pad = (max_m + 63) / 64 * 64;
@@ -1098,6 +1177,8 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
     st.upart = reinterpret_cast<float *>(p);
     p += (size_t)(LT_MAX_CTAS + batch) * cfg.n_q_heads * st.m_pad * sizeof(float);
     st.ml = reinterpret_cast<float *>(p);
+    p += (size_t)(LT_MAX_CTAS + batch) * cfg.n_q_heads * 2 * sizeof(float);
+    st.score = reinterpret_cast<float *>(p);
     for (int l = 0; l < nl; ++l) {
         LatLayer &ly = st.layer[l];
         LatHeads &hp = st.heads[l];
@@ -1107,13 +1188,15 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
         for (int w = 0; w < 2 && ok; ++w) {
             const WhichPlan &wp = plans[l].w[w];
             ok = wp.n_src > 0 && wp.n_src <= LT_MAX_SRC;
-            ly.n_src[w] = hp.n_src[w] = wp.n_src;
+            ly.list[w].n = hp.n_src[w] = wp.n_src;
             for (int s = 0; s < wp.n_src && ok; ++s) {
                 const SourcePlan &sp = wp.src[s];
                 ok = sp.compressed && !sp.qparam && sp.d % 16 == 0 && sp.m % 16 == 0 && sp.width == sp.d;
                 if (!ok) break;
-                LatSrc &d = ly.src[w][s];
+                LatSrc &d = ly.list[w].src[s];
                 d.shift = sp.shift;
+                d.c0 = 0;
+                d.map = s;
                 d.d = sp.d;
                 d.m = sp.m;
                 d.slope = sp.slope;
@@ -1141,7 +1224,7 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
         // Staging places.  A side's latents stay for all its chunks (nz >= their slabs).  One-chunk layers get places for the
         // other side's latents and six hidden slabs, because their jobs are shorter than the way from S to P; the others four
         // hidden slabs: a chunk's three and the one its predecessor may leave unpaired.
-        const int m_t = (lm + 31) & ~31, n_all = ly.n_src[0] + ly.n_src[1];
+        const int m_t = (lm + 31) & ~31, n_all = ly.list[0].n + ly.list[1].n;
         int nh = chunks == 1 ? 6 : 4, nz = chunks == 1 ? std::max(4, 2 * ks) : ks, nw = 4, nqs = chunks == 1 ? 3 : 2;
         int nt = chunks == 1 ? std::min(n_all, 4) : 1;
         auto fits = [&]() { return smem_bytes(st.nq, nz, nh, nw, nqs, nt, m_t) <= SMEM_MAX; };
@@ -1179,19 +1262,104 @@ bool lat_layer_supported(const LatState &st, int layer, uint32_t flags) {
     return st.nq <= 16 || st.group > 2 || ((flags & KVCAR_ABSORBED) && (flags & KVCAR_ABSORBED_V));
 }
 
-cudaError_t lat_launch_tiles(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer,
-                             cudaStream_t stream) {
+namespace {
+
+// the launch attribute of a programmatic dependent launch
+template <typename... Formal, typename... Args>
+cudaError_t launch_pdl(void (*k)(Formal...), dim3 grid, int threads, size_t smem, cudaStream_t st, const Args &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
+// A side's hidden columns in `n` parts of whole 192-column chunks, of about the same number of products each; a part holds one
+// range of columns per source at most (the ranges of a source follow one another).  False where a part would be empty.
+bool split_side(const LatList &all, int n, LatList *out) {
+    int total = 0, done = 0;
+    for (int s = 0; s < all.n; ++s) total += (all.src[s].d + 63) / 64 * ((all.src[s].m + 63) / 64);
+    for (int p = 0; p < n; ++p) out[p].n = 0;
+    for (int s = 0; s < all.n; ++s)
+        for (int c0 = 0; c0 < all.src[s].m; c0 += CN) {
+            const int w = std::min(CN, all.src[s].m - c0), cost = (all.src[s].d + 63) / 64 * ((w + 63) / 64);
+            LatList &l = out[std::min(n - 1, (int)((int64_t)(2 * done + cost) * n / (2 * total)))];  // by the chunk's middle
+            done += cost;
+            if (l.n > 0 && l.src[l.n - 1].map == all.src[s].map) {
+                l.src[l.n - 1].m += w;
+                continue;
+            }
+            LatSrc &u = l.src[l.n++];
+            u = all.src[s];
+            u.shift += c0;
+            u.c0 = c0;
+            u.m = w;
+        }
+    for (int p = 0; p < n; ++p)
+        if (out[p].n == 0) return false;
+    return true;
+}
+int count_chunks(const LatList &l) {
+    int n = 0;
+    for (int s = 0; s < l.n; ++s) n += (l.src[s].m + CN - 1) / CN;
+    return n;
+}
+
+}  // namespace
+
+cudaError_t lat_launch(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer, const LatEncode *enc_in,
+                       cudaStream_t stream, int *n_launches) {
     const LatLayerCfg &lc = st.cfg[layer];
     if (seqs.n > st.batch) return cudaErrorInvalidValue;  // the list names a sequence twice
+    const LatLayer &ly = st.layer[layer];
     Params p;
     fill_seqs(p.sq, seqs, lens, st.n_sms);
-    if (p.sq.n_tiles == 0) return cudaSuccess;
-    p.l = st.layer[layer];
+    const bool two_k = !(a.flags & KVCAR_ABSORBED), two_v = !((a.flags & KVCAR_ABSORBED) && (a.flags & KVCAR_ABSORBED_V));
+    LatEncode e{};
+    if (enc_in) e = *enc_in;
+    EncodeGrid g{0, 1, 1};
+    // ---- front
+    QueryArgs qa;
+    qa.q = reinterpret_cast<const __nv_bfloat16 *>(a.q);
+    qa.wq = reinterpret_cast<__nv_bfloat16 *>(st.wq);
+    qa.qbias = st.qbias;
+    qa.n_seqs = seqs.n;
+    qa.hq = a.hq;
+    qa.group = st.group;
+    qa.nq = st.nq;
+    qa.m_pad = st.m_pad;
+    qa.batch = st.batch;
+    qa.two_terms = two_k;
+    qa.col_blocks = (lc.max_mk + LQ_COLS - 1) / LQ_COLS;
+    qa.scale = a.scale * LOG2E;
+    size_t smem = 0;
+    if (enc_in) {
+        g.nbx = (std::max(e.max_m, 1) + LF_THREADS / 32 - 1) / (LF_THREADS / 32);
+        g.nby = (seqs.n + enc::RB - 1) / enc::RB;
+        g.n_enc = g.nbx * g.nby * 2;
+        smem = (size_t)enc::RB * e.max_in * sizeof(float);
+    }
+    cudaError_t err = launch_pdl(latent_front_kernel, dim3(g.n_enc + a.hq * qa.col_blocks * ((seqs.n + LQ_SB - 1) / LQ_SB)), LF_THREADS,
+                                 smem, stream, st.heads[layer], qa, e, seqs, g);
+    if (err != cudaSuccess) return err;
+    // ---- tiles
+    for (int w = 0; w < 2; ++w)
+        for (int s = 0; s < ly.list[w].n; ++s) {
+            p.pool[w][s] = ly.pool[w][s];
+            p.w1[w][s] = ly.w1[w][s];
+        }
     p.tm_wq = st.tm_wq;
     p.block_table = a.block_table;
     p.status = a.status;
     p.upart = st.upart;
     p.ml = st.ml;
+    p.score = st.score;
     p.max_pages_per_seq = a.max_pages_per_seq;
     p.page_tokens = a.page_tokens;
     p.hq = a.hq;
@@ -1204,39 +1372,59 @@ cudaError_t lat_launch_tiles(LatState &st, const DecodeArgs &a, const SeqList &s
     p.nt = lc.nt;
     p.m_t = lc.m_t;
     p.t_resident = lc.t_resident;
-    p.two_terms_k = (a.flags & KVCAR_ABSORBED) ? 0 : 1;
-    p.two_terms_v = (a.flags & KVCAR_ABSORBED) && (a.flags & KVCAR_ABSORBED_V) ? 0 : 1;
-    latent_query_kernel<<<dim3(a.hq, (lc.max_mk / 2 + LQ_THREADS - 1) / LQ_THREADS, (seqs.n + LQ_SB - 1) / LQ_SB), LQ_THREADS, 0, stream>>>(
-        st.heads[layer], reinterpret_cast<const __nv_bfloat16 *>(a.q), seqs.n, a.hq, st.group, a.scale * LOG2E,
-        reinterpret_cast<__nv_bfloat16 *>(st.wq), st.qbias, st.nq, st.m_pad, st.batch, p.two_terms_k);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const int ctas = (p.sq.n_tiles + p.sq.per - 1) / p.sq.per;
-    kernels[lc.variant]<<<dim3((ctas + 1) & ~1), NTHREADS, lc.smem, stream>>>(p);
-    return cudaGetLastError();
-}
-
-cudaError_t lat_launch_merge(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer,
-                             cudaStream_t stream) {
-    LatSeqs q;
-    fill_seqs(q, seqs, lens, st.n_sms);
+    p.two_terms_k = two_k;
+    p.two_terms_v = two_v;
+    const int pairs = (((p.sq.n_tiles + p.sq.per - 1) / p.sq.per) + 1) / 2, slots = st.n_sms / 2;
+    // Small grids.  Where two clusters per pair of tiles fit on the machine, K and V are two launches and a side's hidden columns
+    // are spread over as many clusters as there is room for.  The V launch starts beside the K launch (all of whose blocks run by
+    // then), does its hidden layer meanwhile and waits for the K launch only before it sums the parts of the scores.  12-layer step
+    // of the GPT-2 shape at 1 / 8 x 1024 tokens: 371 / 649 us, 625 / 712 us with one cluster per pair.
+    int kp = std::min({(slots / pairs + 1) / 2, count_chunks(ly.list[0]), LT_MAX_PARTS});
+    int vp = std::min({slots / pairs - kp, count_chunks(ly.list[1]), LT_MAX_PARTS});
+    *n_launches = 3;
+    if (p.sq.per == 1 && kp >= 1 && vp >= 1) {
+        p.mode = MODE_K;
+        while (!split_side(ly.list[0], kp, p.list)) --kp;
+        p.n_parts = p.k_parts = kp;
+        err = launch_pdl(kernels[lc.variant], dim3(2 * pairs * kp), NTHREADS, lc.smem, stream, p);
+        if (err != cudaSuccess) return err;
+        p.mode = MODE_V;
+        while (!split_side(ly.list[1], vp, p.list)) --vp;
+        p.n_parts = vp;
+        err = launch_pdl(kernels[lc.variant], dim3(2 * pairs * vp), NTHREADS, lc.smem, stream, p);
+        *n_launches = 4;
+    } else {
+        p.mode = MODE_BOTH;
+        p.n_parts = p.k_parts = 1;
+        p.list[0] = ly.list[0];
+        p.list[1] = ly.list[1];
+        err = launch_pdl(kernels[lc.variant], dim3(2 * pairs), NTHREADS, lc.smem, stream, p);
+    }
+    if (err != cudaSuccess) return err;
+    // ---- back
     MergeArgs m;
     m.upart = st.upart;
     m.ml = st.ml;
     m.qbias = st.qbias;
-    m.q = reinterpret_cast<const __nv_bfloat16 *>(a.q);
+    m.q = qa.q;
     m.out = reinterpret_cast<__nv_bfloat16 *>(a.out);
     m.hq = a.hq;
     m.group = st.group;
     m.kv_width = a.hkv * 64;
     m.m_pad = st.m_pad;
-    m.scale = a.scale * LOG2E;
+    m.scale = qa.scale;
     m.with_current = (a.flags & KVCAR_INCLUDE_CURRENT_EXACT) != 0;
-    if (a.hq * seqs.n > 2 * st.n_sms)
-        latent_merge_kernel<4, 288><<<dim3(a.hq, (seqs.n + 3) / 4), 288, (size_t)4 * st.m_pad * 4, stream>>>(st.heads[layer], q, m);
-    else
-        latent_merge_kernel<1, 1024><<<dim3(a.hq, seqs.n), 1024, (size_t)st.m_pad * 4 + 1024 * 16, stream>>>(st.heads[layer], q, m);
-    return cudaGetLastError();
+    const bool wide = a.hq * seqs.n > st.n_sms;
+    const int threads = wide ? 256 : 512, sb = wide ? 4 : 1;
+    smem = (size_t)sb * st.m_pad * 4 + (wide ? 0 : threads * 16);
+    if (enc_in) {
+        g.nbx = (std::max(e.max_d, 1) + threads / 32 - 1) / (threads / 32);
+        g.n_enc = g.nbx * g.nby * 2;
+        smem = std::max(smem, (size_t)enc::RB * e.pitch * sizeof(float));
+    }
+    const dim3 grid(g.n_enc + a.hq * ((seqs.n + sb - 1) / sb));
+    return wide ? launch_pdl(latent_back_kernel<4, 256>, grid, threads, smem, stream, st.heads[layer], p.sq, m, e, g)
+                : launch_pdl(latent_back_kernel<1, 512>, grid, threads, smem, stream, st.heads[layer], p.sq, m, e, g);
 }
 
 }  // namespace kvcar

@@ -8,18 +8,25 @@ namespace kvcar {
 
 constexpr int LT_MAX_SRC = 6;     // distinct source layers per K or V of a layer
 constexpr int LT_MAX_Q = 32;      // query heads
+constexpr int LT_ENC_SMEM = 160 * 1024;  // what the encoder's input rows may take in the launches that carry it
 constexpr int LT_MAX_CTAS = 160;  // blocks of a launch at most (one per SM)
 
 // Place of hidden feature f's shift in the padded array: groups of 32 features, in each the order in which the four lanes of a
 // fragment row hold them (features 8 j + 2 c + e of a group at 8 c + 2 j + e).
 inline int shift_place(int f) { return (f & ~31) + ((f & 7) >> 1) * 8 + ((f & 31) >> 3) * 2 + (f & 1); }
 
-// One source layer of K or V as the tile kernel sees it (kernel parameter).
+// Hidden columns c0 .. c0 + m - 1 of one source layer of K or V as the tile kernel sees them (kernel parameter).
 struct LatSrc {
-    const float *shift;  // fused bias + BatchNorm shift over the size of its scale, in fragment order (see shift_place)
-    int32_t d, m;
+    const float *shift;  // fused bias + BatchNorm shift over the size of its scale, from c0, in fragment order (see shift_place)
+    int32_t d, m, c0;
+    int32_t map;    // which of the layer's tensor maps
     float slope;
     uint32_t mask;  // query heads whose K (or V) head is served from this source
+};
+constexpr int LT_MAX_PARTS = 8;  // clusters that share the K (or the V) side of a pair of tiles
+struct LatList {
+    int32_t n;
+    LatSrc src[LT_MAX_SRC];
 };
 
 // The listed sequences of a call: device ids, and the first tile of each (low 24 bits) with the valid tokens of its
@@ -34,8 +41,7 @@ struct LatSeqs {
 // kernel parameters need no acquire, and nothing is found through chains of loads).
 struct LatLayer {
     CUtensorMap pool[2][LT_MAX_SRC], w1[2][LT_MAX_SRC];
-    int32_t n_src[2];
-    LatSrc src[2][LT_MAX_SRC];
+    LatList list[2];  // K, V: every source whole
 };
 // The last decoder layer of each source, which source and column slot serves a KV head, the exact current-token rows.
 struct LatHeads {
@@ -73,6 +79,7 @@ struct LatState {
     float *qbias = nullptr;  // [batch][hq]: q . b4_h, in the exponent's base-2 units
     float *upart = nullptr;  // [block + sequence][hq][m_pad]: sum over a run of tiles of p * hidden vector
     float *ml = nullptr;     // [block + sequence][hq][2]: reference maximum and sum of the run
+    float *score = nullptr;  // [block][heads padded][128]: parts of the scores (small grids)
     CUtensorMap tm_wq;
 };
 
@@ -83,11 +90,14 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
                int max_k_sources, int max_m, int batch, char *ws_area);
 // flags: those of the call (17 to 32 query heads in groups of at most two only with KVCAR_ABSORBED_V, see kvcar_latent.cu)
 bool lat_layer_supported(const LatState &st, int layer, uint32_t flags);
-// the operand kernel and the tile kernel (lens: host copy of the listed sequences' lengths)
-cudaError_t lat_launch_tiles(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer,
-                             cudaStream_t stream);
-// the merge of the runs, the last decoder layer of the V side, the current token
-cudaError_t lat_launch_merge(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer,
-                             cudaStream_t stream);
+// The encoder of the same step's new rows, carried by the first and the last launch (null: none).
+struct LatEncode {
+    EncodeArgs a;
+    float *hid;
+    int32_t pitch, max_batch, max_m, max_d, max_in;
+};
+// All launches of one call on `stream`.  lens: host copy of the listed sequences' lengths, not all zero.
+cudaError_t lat_launch(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer, const LatEncode *enc,
+                       cudaStream_t stream, int *n_launches);
 
 }  // namespace kvcar
