@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(NW * 32)
     encode_fc_kernel(const __grid_constant__ EncodeArgs a, const __grid_constant__ SeqList seqs, float *hid, int hid_pitch,
                      int max_batch) {
     extern __shared__ __align__(16) float xs[];  // [RB][n_in]
-    encode_fc_block<T, STAGE, true>(a, seqs.id, seqs.n, hid, hid_pitch, max_batch, xs, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x);
+    encode_fc_block<T, STAGE, true, 1>(a, seqs.id, seqs.n, hid, hid_pitch, max_batch, xs, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x);
 }
 
 template <typename T, int STAGE>

@@ -41,30 +41,38 @@ struct Vec16<__nv_bfloat16> {
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// acc[r] += sum over this lane's share of w[0..n) * x[r][0..n); `pre` holds the lane's first vector already
-template <typename T>
-__device__ __forceinline__ void lane_dots(const T *wrow, const uint4 &pre, const float *x, int n, int lane, float *acc) {
+// acc[f][r] += sum over this lane's share of w_f[0..n) * x[r][0..n); `pre` holds the lane's first vector of each row already
+template <typename T, int NF>
+__device__ __forceinline__ void lane_dots(const T *wrow, const uint4 *pre, const float *x, int n, int lane, float (*acc)[RB]) {
     constexpr int VL = Vec16<T>::N;
-    uint4 cur = pre;
+    uint4 cur[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) cur[f] = pre[f];
     for (int k0 = lane * VL; k0 < n; k0 += 32 * VL) {
         const int kn = k0 + 32 * VL;
-        uint4 nxt = cur;
-        if (kn < n) nxt = Vec16<T>::load(wrow + kn);
-        float w[VL];
-        Vec16<T>::unpack(cur, w);
+        uint4 nxt[NF];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) nxt[f] = kn < n ? Vec16<T>::load(wrow + (int64_t)f * n + kn) : cur[f];
+        float w[NF][VL];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) Vec16<T>::unpack(cur[f], w[f]);
 #pragma unroll
         for (int r = 0; r < RB; ++r) {
             const float4 *xr = reinterpret_cast<const float4 *>(x + r * n + k0);
 #pragma unroll
             for (int i = 0; i < VL / 4; ++i) {
                 const float4 xv = xr[i];
-                acc[r] = fmaf(w[4 * i + 0], xv.x, acc[r]);
-                acc[r] = fmaf(w[4 * i + 1], xv.y, acc[r]);
-                acc[r] = fmaf(w[4 * i + 2], xv.z, acc[r]);
-                acc[r] = fmaf(w[4 * i + 3], xv.w, acc[r]);
+#pragma unroll
+                for (int f = 0; f < NF; ++f) {
+                    acc[f][r] = fmaf(w[f][4 * i + 0], xv.x, acc[f][r]);
+                    acc[f][r] = fmaf(w[f][4 * i + 1], xv.y, acc[f][r]);
+                    acc[f][r] = fmaf(w[f][4 * i + 2], xv.z, acc[f][r]);
+                    acc[f][r] = fmaf(w[f][4 * i + 3], xv.w, acc[f][r]);
+                }
             }
         }
-        cur = nxt;
+#pragma unroll
+        for (int f = 0; f < NF; ++f) cur[f] = nxt[f];
     }
 }
 
@@ -103,35 +111,38 @@ __device__ __forceinline__ int row_of_lane(int lane) {
 }
 
 // STAGE 1: hidden = LeakyReLU(BN(W1 x + b1)) -> scratch.  STAGE 2: latent = W2 hidden + b2 -> cache rows.
-// Block (bx, by, which) of ceil(features / warps) x ceil(rows / RB) x 2 [K, V]; xs: [RB][n_in] floats of shared memory, 16-byte
+// A warp takes NF features: a row's values are read from shared memory once per NF weights, and those reads bound the block when
+// many row blocks share a launch (256 rows of the GPT-2 shape: see latent_front_kernel).
+// Block (bx, by, which) of ceil(features / (warps x NF)) x ceil(rows / RB) x 2 [K, V]; xs: [RB][n_in] floats of shared memory, 16-byte
 // aligned.  Weights are requested before the wait for the preceding kernels of the stream.  EARLY: dependent launches may start
 // before that wait.
-template <typename T, int STAGE, bool EARLY>
+template <typename T, int STAGE, bool EARLY, int NF>
 __device__ __forceinline__ void encode_fc_block(const EncodeArgs &a, const int32_t *seq_ids, int n_seqs, float *hid, int hid_pitch,
                                                 int max_batch, float *xs, int bx, int by, int which, int nbx) {
-    const int NW = blockDim.x >> 5;  // warps (= output features) of a block
+    const int NW = (blockDim.x >> 5) * NF;  // output features of a block
     const EncPlan &pl = a.plan[which];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_rows = n_seqs, r0 = by * RB;
     const int in_dim = pl.in_dim, m = pl.m, d = pl.d;
     const int n_in = STAGE == 1 ? in_dim : m, n_out = STAGE == 1 ? m : d;
-    const int j = bx * NW + warp;  // this warp's output feature
+    const int j = bx * NW + warp * NF;  // this warp's first output feature
     const T *src = reinterpret_cast<const T *>(which == 0 ? a.k : a.v);
     const bool compressed = pl.compressed != 0;
 
     // weights do not depend on anything earlier in the stream: start fetching them right away
     constexpr int VL = Vec16<T>::N;
     const T *wrow = reinterpret_cast<const T *>(STAGE == 1 ? pl.w1r : pl.w2r) + (int64_t)j * n_in;
-    uint4 pre = make_uint4(0, 0, 0, 0);
-    const bool active = compressed && j < n_out;
-    float p0 = 0.f, p1 = 0.f;  // stage 1: fused BatchNorm scale, shift; stage 2: bias
-    if (active) {
-        if (lane * VL < n_in) pre = Vec16<T>::load(wrow + lane * VL);
-        if (STAGE == 1) {
-            p0 = pl.s1[j];
-            p1 = pl.t1[j];
-        } else {
-            p0 = pl.b2[j];
+    uint4 pre[NF];
+    float p0[NF], p1[NF];  // stage 1: fused BatchNorm scale, shift; stage 2: bias
+    const bool active = compressed && j < n_out;  // n_out is a multiple of NF where NF > 1
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        pre[f] = make_uint4(0, 0, 0, 0);
+        p0[f] = p1[f] = 0.f;
+        if (active) {
+            if (lane * VL < n_in) pre[f] = Vec16<T>::load(wrow + (int64_t)f * n_in + lane * VL);
+            p0[f] = STAGE == 1 ? pl.s1[j + f] : pl.b2[j + f];
+            if (STAGE == 1) p1[f] = pl.t1[j + f];
         }
     }
     if (EARLY) launch_dependents();
@@ -215,18 +226,25 @@ __device__ __forceinline__ void encode_fc_block(const EncodeArgs &a, const int32
     }
     __syncthreads();
     if (!active) return;
-    float acc[RB];
+    float acc[NF][RB];
 #pragma unroll
-    for (int r = 0; r < RB; ++r) acc[r] = 0.f;
-    lane_dots<T>(wrow, pre, xs, n_in, lane, acc);
-    const float sum = reduce_rows(acc, lane);
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+        for (int r = 0; r < RB; ++r) acc[f][r] = 0.f;
+    lane_dots<T, NF>(wrow, pre, xs, n_in, lane, acc);
+    float sum[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) sum[f] = reduce_rows(acc[f], lane);
     if ((lane & 1) || my_row >= rows_here) return;
-    if (STAGE == 1) {
-        float hv = fmaf(sum, p0, p1);
-        hv = hv > 0.f ? hv : hv * pl.slope;
-        hid[((int64_t)which * max_batch + r0 + my_row) * hid_pitch + j] = hv;
-    } else {
-        Vec16<T>::store(reinterpret_cast<T *>(pl.pool) + prow * pl.width + j, sum + p0);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        if (STAGE == 1) {
+            float hv = fmaf(sum[f], p0[f], p1[f]);
+            hv = hv > 0.f ? hv : hv * pl.slope;
+            hid[((int64_t)which * max_batch + r0 + my_row) * hid_pitch + j + f] = hv;
+        } else {
+            Vec16<T>::store(reinterpret_cast<T *>(pl.pool) + prow * pl.width + j + f, sum[f] + p0[f]);
+        }
     }
 }
 

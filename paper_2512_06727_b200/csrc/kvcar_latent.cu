@@ -906,13 +906,14 @@ __device__ __forceinline__ void query_block(const LatHeads &hp, const QueryArgs 
 struct EncodeGrid {
     int32_t n_enc, nbx, nby;
 };
+template <int NF>
 __global__ void __launch_bounds__(LF_THREADS) latent_front_kernel(const __grid_constant__ LatHeads hp, const __grid_constant__ QueryArgs a,
                                                                   const __grid_constant__ LatEncode e, const __grid_constant__ SeqList seqs,
                                                                   const __grid_constant__ EncodeGrid g) {
     extern __shared__ __align__(16) float xs[];
     const int b = blockIdx.x;
     if (b < g.n_enc)
-        enc::encode_fc_block<__nv_bfloat16, 1, false>(e.a, seqs.id, seqs.n, e.hid, e.pitch, e.max_batch, xs, b % g.nbx, b / g.nbx % g.nby,
+        enc::encode_fc_block<__nv_bfloat16, 1, false, NF>(e.a, seqs.id, seqs.n, e.hid, e.pitch, e.max_batch, xs, b % g.nbx, b / g.nbx % g.nby,
                                                       b / g.nbx / g.nby, g.nbx);
     else
         query_block(hp, a, b - g.n_enc);
@@ -1090,14 +1091,14 @@ __device__ __forceinline__ void merge_block(const LatHeads &hp, const LatSeqs &s
     out[lane + 32] = __float2bfloat16_rn(S > 0.f ? o[1] / S : 0.f);
 }
 
-template <int SB, int THREADS>
+template <int SB, int THREADS, int NF>
 __global__ void __launch_bounds__(THREADS) latent_back_kernel(const __grid_constant__ LatHeads hp, const __grid_constant__ LatSeqs sq,
                                                               const __grid_constant__ MergeArgs a, const __grid_constant__ LatEncode e,
                                                               const __grid_constant__ EncodeGrid g) {
     extern __shared__ __align__(16) float sm[];
     const int b = blockIdx.x;
     if (b < g.n_enc)
-        enc::encode_fc_block<__nv_bfloat16, 2, false>(e.a, sq.id, sq.n, e.hid, e.pitch, e.max_batch, sm, b % g.nbx, b / g.nbx % g.nby,
+        enc::encode_fc_block<__nv_bfloat16, 2, false, NF>(e.a, sq.id, sq.n, e.hid, e.pitch, e.max_batch, sm, b % g.nbx, b / g.nbx % g.nby,
                                                       b / g.nbx / g.nby, g.nbx);
     else
         merge_block<SB, THREADS>(hp, sq, a, sm, b - g.n_enc);
@@ -1160,9 +1161,10 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int group = cfg.n_q_heads / cfg.n_kv_heads;
     st.n_sms = sms;
-    for (auto k : {latent_back_kernel<4, 256>, latent_back_kernel<1, 512>})
+    for (auto k : {latent_back_kernel<4, 256, 1>, latent_back_kernel<4, 256, 2>, latent_back_kernel<1, 512, 1>})
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, LT_ENC_SMEM) != cudaSuccess) return;
-    if (cudaFuncSetAttribute(latent_front_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LT_ENC_SMEM) != cudaSuccess) return;
+    for (auto k : {latent_front_kernel<1>, latent_front_kernel<2>})
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, LT_ENC_SMEM) != cudaSuccess) return;
     st.nq = padded_heads(cfg.n_q_heads);
     st.group = group;
     st.m_pad = (max_m + 63) / 64 * 64;
@@ -1338,14 +1340,18 @@ cudaError_t lat_launch(LatState &st, const DecodeArgs &a, const SeqList &seqs, c
     qa.two_terms = two_k;
     qa.col_blocks = (lc.max_mk + LQ_COLS - 1) / LQ_COLS;
     qa.scale = a.scale * LOG2E;
+    // Features per warp of the encoder: one spreads a few rows' weights over the most warps, two read the rows half as often from
+    // shared memory.  12-layer step of the GPT-2 shape over 256 cached tokens: 64 sequences 954 us with one, 817 with two; 256
+    // sequences 3093, 2686 (four: 902, 3069, the registers leave one block per SM).
+    const int nf = seqs.n >= 64 ? 2 : 1;
     size_t smem = 0;
     if (enc_in) {
-        g.nbx = (std::max(e.max_m, 1) + LF_THREADS / 32 - 1) / (LF_THREADS / 32);
+        g.nbx = (std::max(e.max_m, 1) + LF_THREADS / 32 * nf - 1) / (LF_THREADS / 32 * nf);
         g.nby = (seqs.n + enc::RB - 1) / enc::RB;
         g.n_enc = g.nbx * g.nby * 2;
         smem = (size_t)enc::RB * e.max_in * sizeof(float);
     }
-    cudaError_t err = launch_pdl(latent_front_kernel, dim3(g.n_enc + a.hq * qa.col_blocks * ((seqs.n + LQ_SB - 1) / LQ_SB)), LF_THREADS,
+    cudaError_t err = launch_pdl(nf == 2 ? latent_front_kernel<2> : latent_front_kernel<1>, dim3(g.n_enc + a.hq * qa.col_blocks * ((seqs.n + LQ_SB - 1) / LQ_SB)), LF_THREADS,
                                  smem, stream, st.heads[layer], qa, e, seqs, g);
     if (err != cudaSuccess) return err;
     // ---- tiles
@@ -1418,13 +1424,14 @@ cudaError_t lat_launch(LatState &st, const DecodeArgs &a, const SeqList &seqs, c
     const int threads = wide ? 256 : 512, sb = wide ? 4 : 1;
     smem = (size_t)sb * st.m_pad * 4 + (wide ? 0 : threads * 16);
     if (enc_in) {
-        g.nbx = (std::max(e.max_d, 1) + threads / 32 - 1) / (threads / 32);
+        const int per = threads / 32 * (wide ? nf : 1);
+        g.nbx = (std::max(e.max_d, 1) + per - 1) / per;
         g.n_enc = g.nbx * g.nby * 2;
         smem = std::max(smem, (size_t)enc::RB * e.pitch * sizeof(float));
     }
     const dim3 grid(g.n_enc + a.hq * ((seqs.n + sb - 1) / sb));
-    return wide ? launch_pdl(latent_back_kernel<4, 256>, grid, threads, smem, stream, st.heads[layer], p.sq, m, e, g)
-                : launch_pdl(latent_back_kernel<1, 512>, grid, threads, smem, stream, st.heads[layer], p.sq, m, e, g);
+    return wide ? launch_pdl(nf == 2 ? latent_back_kernel<4, 256, 2> : latent_back_kernel<4, 256, 1>, grid, threads, smem, stream, st.heads[layer], p.sq, m, e, g)
+                : launch_pdl(latent_back_kernel<1, 512, 1>, grid, threads, smem, stream, st.heads[layer], p.sq, m, e, g);
 }
 
 }  // namespace kvcar
