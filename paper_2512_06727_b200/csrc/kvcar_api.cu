@@ -223,8 +223,8 @@ void compute_layout(kvcar_ctx *c) {
     s = align_up(s + (size_t)nb * c->max_chunks * g.n_q_heads * (g.head_dim + 2) * sizeof(float), 256);
     c->stage_off = s;
     s = align_up(s + (size_t)nb * (2 * W + 2 * g.n_q_heads * g.head_dim) * c->elem + 4 * 256, 256);
-    c->enchid_off = s;  // hidden activations between the two decode-time encoder launches
-    s = align_up(s + (size_t)2 * nb * c->max_m * sizeof(float), 256);
+    c->enchid_off = s;  // hidden activations between the decode-time encoder's launches; int8 rows: then the fp32 latents
+    s = align_up(s + (size_t)2 * nb * (c->max_m + (g.latent_quant ? c->max_d : 0)) * sizeof(float), 256);
     c->kvsplit_off = s;  // probabilities handed from K clusters to V clusters (tensor-core kernel, small grids)
     s = align_up(s + tc_split_bytes(g), 256);
     c->pfhid_off = s;  // bf16 hidden activations between the two launches of the tensor-core prefill
@@ -792,6 +792,10 @@ static EncodeArgs encode_args(const kvcar_ctx *c, int32_t layer, int32_t n_token
     a.n_tokens = n_tokens;
     a.kv_width = c->cfg.n_kv_heads * c->cfg.head_dim;
     a.hd = c->cfg.head_dim;
+    if (c->cfg.latent_quant && n_tokens == 1) {
+        a.z = reinterpret_cast<float *>(c->ws + c->enchid_off) + (size_t)2 * std::min(c->cfg.max_seqs, KVCAR_MAX_BATCH) * c->max_m;
+        a.z_pitch = c->max_d;
+    }
     return a;
 }
 
@@ -799,7 +803,7 @@ static EncodeArgs encode_args(const kvcar_ctx *c, int32_t layer, int32_t n_token
 // weight rows and its row block in shared memory)
 static bool encode_splits(const kvcar_ctx *c, int32_t layer) {
     const int vl = 16 / c->elem;
-    if (c->cfg.latent_quant || c->cfg.head_dim % vl != 0 || encode_split_smem(c->max_in, c->max_m) > 200 * 1024) return false;
+    if (c->cfg.head_dim % vl != 0 || encode_split_smem(c->max_in, c->max_m) > 200 * 1024) return false;
     for (int w = 0; w < 2; ++w) {
         const AEHost &ae = c->ae[layer * 2 + w];
         if (ae.set && (ae.in_dim % vl || ae.hidden % vl)) return false;
@@ -864,7 +868,7 @@ static kvcar_status enqueue_encode(kvcar_ctx *c, int32_t layer, const int32_t *s
                                                    reinterpret_cast<float *>(c->ws + c->enchid_off), nb, st)
                              : launch_encode_generic(a, sl, c->cfg.storage, c->max_in, c->max_m, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "encode launch");
-    c->launches += split_ok ? 2 : 1;
+    c->launches += split_ok ? (c->cfg.latent_quant ? 3 : 2) : 1;
     return KVCAR_OK;
 }
 

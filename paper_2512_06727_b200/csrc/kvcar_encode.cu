@@ -50,7 +50,59 @@ cudaError_t launch_stage(const EncodeArgs &a, const SeqList &seqs, float *hid, i
     return cudaLaunchKernelEx(&cfg, encode_fc_kernel<T, STAGE>, a, seqs, hid, hid_pitch, max_batch);
 }
 
+// Eq. 4 per cached row, as the tail of encode_generic_kernel: scale = 255/(max-min), zero-point = -round(scale*min) - 128,
+// code = round(scale*x + zero-point) kept inside int8.  grid = ceil(2 * rows / 8), one warp per (K or V, row).
+__global__ void __launch_bounds__(256) encode_quant_kernel(const __grid_constant__ EncodeArgs a, const __grid_constant__ SeqList seqs,
+                                                           int max_batch) {
+    grid_dependency_wait();
+    launch_dependents();
+    const int item = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int which = item / seqs.n, r = item % seqs.n;
+    if (which > 1) return;
+    const EncPlan &pl = a.plan[which];
+    if (!pl.qparam) return;
+    const float *z = a.z + ((int64_t)which * max_batch + r) * a.z_pitch;
+    const int seq = seqs.id[r], t = a.seq_len[seq], d = pl.d;
+    const int page = a.block_table[(int64_t)seq * a.max_pages_per_seq + t / a.page_tokens];
+    const int64_t row = (int64_t)page * a.page_tokens + t % a.page_tokens;
+    float lo = INFINITY, hi = -INFINITY;
+    for (int j = lane; j < d; j += 32) {
+        lo = fminf(lo, z[j]);
+        hi = fmaxf(hi, z[j]);
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    float scale = 1.f, zp = -lo;  // a row of equal values has no range: code 0 with zero-point -x restores it exactly
+    if (hi > lo) {
+        scale = 255.f / (hi - lo);
+        zp = -rintf(scale * lo) - 128.f;
+    }
+    int8_t *codes = reinterpret_cast<int8_t *>(pl.pool) + row * pl.width;
+    for (int j = lane; j < d; j += 32)
+        codes[j] = (int8_t)(int)(hi > lo ? fminf(fmaxf(rintf(fmaf(scale, z[j], zp)), -128.f), 127.f) : 0.f);
+    if (lane == 0) {
+        pl.qparam[row * 2] = scale;
+        pl.qparam[row * 2 + 1] = zp;
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_encode_quant(const EncodeArgs &a, const SeqList &seqs, int max_batch, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((2 * seqs.n + 7) / 8);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, encode_quant_kernel, a, seqs, max_batch);
+}
 
 size_t encode_split_smem(int max_in, int max_m) { return (size_t)RB * std::max(max_in, max_m) * sizeof(float); }
 
@@ -65,6 +117,7 @@ cudaError_t launch_encode_split(const EncodeArgs &a, const SeqList &seqs, int dt
         e = launch_stage<__nv_bfloat16, 1>(a, seqs, hid, max_m, max_batch, n_hidden, max_in, st);
         if (e == cudaSuccess && max_m > 0)
             e = launch_stage<__nv_bfloat16, 2>(a, seqs, hid, max_m, max_batch, max_d, max_m, st);
+        if (e == cudaSuccess && a.z) e = launch_encode_quant(a, seqs, max_batch, st);
     }
     return e;
 }

@@ -243,7 +243,10 @@ __device__ __forceinline__ void encode_fc_block(const EncodeArgs &a, const int32
             hv = hv > 0.f ? hv : hv * pl.slope;
             hid[((int64_t)which * max_batch + r0 + my_row) * hid_pitch + j + f] = hv;
         } else {
-            Vec16<T>::store(reinterpret_cast<T *>(pl.pool) + prow * pl.width + j + f, sum[f] + p0[f]);
+            if (pl.qparam)
+                a.z[((int64_t)which * max_batch + r0 + my_row) * a.z_pitch + j + f] = sum[f] + p0[f];
+            else
+                Vec16<T>::store(reinterpret_cast<T *>(pl.pool) + prow * pl.width + j + f, sum[f] + p0[f]);
         }
     }
 }

@@ -105,6 +105,8 @@ struct EncodeArgs {
     const void *k, *v;    // [n_seqs][n_tokens][kv_width]
     int32_t max_pages_per_seq, page_tokens;
     int32_t n_tokens, kv_width, hd;
+    float *z;             // int8 rows, one new token per sequence: the fp32 latents [2][max_batch][z_pitch] before their codes
+    int32_t z_pitch;
 };
 
 struct TableUpdates {
@@ -123,6 +125,8 @@ cudaError_t launch_encode_generic(const EncodeArgs &a, const SeqList &seqs, int 
 cudaError_t launch_encode_split(const EncodeArgs &a, const SeqList &seqs, int dtype, int max_in, int max_m, int max_d,
                                 float *hid, int max_batch, cudaStream_t st);
 size_t encode_split_smem(int max_in, int max_m);
+// int8 rows: codes, scale and zero-point of the latents that the second launch left in a.z (launch_encode_split includes it)
+cudaError_t launch_encode_quant(const EncodeArgs &a, const SeqList &seqs, int max_batch, cudaStream_t st);
 cudaError_t launch_decode_generic(const DecodeArgs &a, const SeqList &seqs, int dtype, int max_d, int max_m,
                                   int grid_chunks, cudaStream_t st);
 // raw K/V layers (no autoencoder), head_dim 64, <= 8 query heads per KV head (kvcar_raw.cu)
