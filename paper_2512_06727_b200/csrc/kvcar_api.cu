@@ -81,7 +81,7 @@ struct kvcar_ctx {
     size_t pool_bytes = 0, weights_bytes = 0, ws_bytes = 0;
     size_t plan_off = 0, enc_off = 0, tmap_off = 0, tcpart_off = 0;  // inside weights
     size_t bt_off = 0, len_off = 0, status_off = 0, part_off = 0, stage_off = 0, enchid_off = 0, kvsplit_off = 0, pfhid_off = 0, lat_off = 0, fma_off = 0;  // inside workspace
-    int max_k_sources = 0;  // most distinct source layers any layer's K heads resolve to
+    int max_sources = 0;  // most distinct source layers any layer's K or V heads resolve to
     std::vector<RawSources> raw_src;  // [layer] tensor maps and head places of raw bf16 layers
     std::vector<char> raw_src_ok;     // [layer] filled (else the raw-row kernel stages with cp.async)
     std::vector<EncPlan> enc_host;  // the device's EncPlan table, host copy (tensor-core prefill builds tensor maps from it)
@@ -134,8 +134,8 @@ int stored_width(const kvcar_ctx *c, int layer, int which) {
     return (int)stored_heads(c, layer, which).size() * c->cfg.head_dim;
 }
 
-// bf16 rows of 64-wide heads: the tensor-core kernels take all but a few layers, and those few stay with the generic kernel
-bool fma_is_fallback_only(const kvcar_config &g) { return g.storage == KVCAR_BF16 && !g.latent_quant && g.head_dim == 64; }
+// bf16 storage and 64-wide heads: the tensor-core kernels take all but a few layers, and those few stay with the generic kernel
+bool fma_is_fallback_only(const kvcar_config &g) { return g.storage == KVCAR_BF16 && g.head_dim == 64; }
 
 void compute_layout(kvcar_ctx *c) {
     const kvcar_config &g = c->cfg;
@@ -193,7 +193,7 @@ void compute_layout(kvcar_ctx *c) {
         if (g.storage == KVCAR_BF16) {
             w = align_up(w + mats * 2, 256);                                       // K-major decoder copies
             w = align_up(w + (size_t)a.hidden * a.latent * 2, 256);                // FC1 of the latent-attention kernels
-            w = align_up(w + (size_t)(2 * ((a.hidden + 31) & ~31)) * sizeof(float), 256);
+            w = align_up(w + (size_t)(3 * ((a.hidden + 31) & ~31)) * sizeof(float), 256);
         }
         w = align_up(w + mats * c->elem, 256);                                     // row-major encoder copies
     }
@@ -229,23 +229,24 @@ void compute_layout(kvcar_ctx *c) {
     s = align_up(s + tc_split_bytes(g), 256);
     c->pfhid_off = s;  // bf16 hidden activations between the two launches of the tensor-core prefill
     if (g.storage == KVCAR_BF16 && c->max_m > 0) s = align_up(s + prefill_tc_scratch_bytes(c->max_m), 256);
-    c->max_k_sources = 0;
-    for (int l = 0; l < nl; ++l) {
-        std::vector<char> seen(nl, 0);
-        int n = 0;
-        for (int h = 0; h < g.n_kv_heads; ++h) {
-            const int r = resolve(c, l, h, 0).root_layer;
-            if (!seen[r]) {
-                seen[r] = 1;
-                ++n;
+    c->max_sources = 0;
+    for (int which = 0; which < 2; ++which)
+        for (int l = 0; l < nl; ++l) {
+            std::vector<char> seen(nl, 0);
+            int n = 0;
+            for (int h = 0; h < g.n_kv_heads; ++h) {
+                const int r = resolve(c, l, h, which).root_layer;
+                if (!seen[r]) {
+                    seen[r] = 1;
+                    ++n;
+                }
             }
+            c->max_sources = std::max(c->max_sources, n);
         }
-        c->max_k_sources = std::max(c->max_k_sources, n);
-    }
     c->lat_off = s;  // operands and partial results of the latent-attention kernels
-    s = align_up(s + lat_ws_bytes(g, c->max_k_sources, c->max_m, nb), 256);
+    s = align_up(s + lat_ws_bytes(g, c->max_sources, c->max_m, c->max_d, nb, cap), 256);
     c->fma_off = s;  // the same of the fp32-FMA kernels, where latents are not bf16 rows of 64-wide heads
-    if (!fma_is_fallback_only(g)) s = align_up(s + fma_ws_bytes(g, c->max_k_sources, c->max_m, nb, cap), 256);
+    if (!fma_is_fallback_only(g)) s = align_up(s + fma_ws_bytes(g, c->max_sources, c->max_m, nb, cap), 256);
     c->ws_bytes = s;
 }
 
@@ -280,14 +281,20 @@ void fuse_bn(const std::vector<float> &b1, const std::vector<float> &bn, int m, 
 // LeakyReLU(s x + t) = |s| LeakyReLU(sign(s) x + t / |s|).  The sign goes into the weight row (exact), t / |s| is the shift
 // that is left to the epilogue, |s| goes to the neighbours of the hidden vector (W4^T q and the weighted sum, both fp32).  A
 // scale too small to divide by leaves the constant LeakyReLU(t).
-void put_signed_fc1(char *dst, float *sabs, float *shift, const float *w, const float *s, const float *t, int m, int d) {
+void put_signed_fc1(char *dst, float *sabs, size_t stride, const float *w, const float *s, const float *t, int m, int d) {
     __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(dst);
+    float *shift = sabs + stride, *rowsum = shift + stride;
     for (int j = 0; j < m; ++j) {
         const bool tiny = std::fabs(s[j]) < 1e-20f;
         const float sign = tiny ? 0.f : s[j] < 0.f ? -1.f : 1.f;
         sabs[j] = tiny ? 1.f : std::fabs(s[j]);
         shift[shift_place(j)] = t[j] / sabs[j];
-        for (int k = 0; k < d; ++k) o[(size_t)j * d + k] = __float2bfloat16_rn(sign * w[(size_t)j * d + k]);
+        double sum = 0.0;
+        for (int k = 0; k < d; ++k) {
+            o[(size_t)j * d + k] = __float2bfloat16_rn(sign * w[(size_t)j * d + k]);
+            sum += (double)__bfloat162float(o[(size_t)j * d + k]);
+        }
+        rowsum[shift_place(j)] = (float)sum;
     }
 }
 
@@ -545,10 +552,10 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
             put_elems(&img[p.w2k], a.dec_w2.data(), I * M, KVCAR_BF16);
             p.w1n = w;
             w = align_up(w + M * D * 2, 256);
-            p.sabs = w;  // then the shifts
+            p.sabs = w;  // then the shifts, then the row sums
             const size_t M32 = (M + 31) & ~(size_t)31;
-            w = align_up(w + 2 * M32 * 4, 256);
-            put_signed_fc1(&img[p.w1n], (float *)&img[p.sabs], (float *)&img[p.sabs] + M32, a.dec_w1.data(),
+            w = align_up(w + 3 * M32 * 4, 256);
+            put_signed_fc1(&img[p.w1n], (float *)&img[p.sabs], M32, a.dec_w1.data(),
                            (const float *)&img[p.dec_s], (const float *)&img[p.dec_t], (int)M, (int)D);
         }
         p.enc_w1r = w;
@@ -600,6 +607,7 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
                             sp.w1n = c->weights + pk[idx].w1n;
                             sp.sabs = (const float *)(c->weights + pk[idx].sabs);
                             sp.shift = sp.sabs + ((a.hidden + 31) & ~31);
+                            sp.rowsum = sp.shift + ((a.hidden + 31) & ~31);
                         }
                     } else {
                         sp.d = sp.in_dim = sp.width;
@@ -616,10 +624,10 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
     // tensor maps and job tables of the tensor-core kernel (fills their regions of the image)
     tc_setup(c->tc, c->cfg, plans, nl, c->weights, c->tmap_off, c->tcpart_off, img.data(),
              (size_t)g.max_pages * g.page_tokens);
-    lat_setup(c->lat, c->cfg, c->plans_host, (size_t)g.max_pages * g.page_tokens, c->max_k_sources, c->max_m,
-              std::min(g.max_seqs, KVCAR_MAX_BATCH), c->ws + c->lat_off);
+    lat_setup(c->lat, c->cfg, c->plans_host, (size_t)g.max_pages * g.page_tokens, c->max_sources, c->max_m, c->max_d,
+              std::min(g.max_seqs, KVCAR_MAX_BATCH), g.max_pages_per_seq * g.page_tokens, c->ws + c->lat_off);
     if (!fma_is_fallback_only(g))
-        fma_setup(c->fma, c->cfg, c->plans_host, c->max_k_sources, c->max_m, std::min(g.max_seqs, KVCAR_MAX_BATCH),
+        fma_setup(c->fma, c->cfg, c->plans_host, c->max_sources, c->max_m, std::min(g.max_seqs, KVCAR_MAX_BATCH),
                   g.max_pages_per_seq * g.page_tokens, c->ws + c->fma_off);
     // tensor maps and head places of the raw layers (kernel parameters of the raw-row kernel)
     c->raw_src.assign(nl, RawSources{});
@@ -1015,6 +1023,11 @@ static kvcar_status enqueue_latent(kvcar_ctx *c, int32_t layer, const DecodeArgs
     cudaError_t err = lat_launch(c->lat, a, sl, lens, layer, carry ? &e : nullptr, st, &n);
     if (err != cudaSuccess) return cuda_fail(c, err, "decode launch");
     c->launches += n;
+    if (carry && e.a.z) {  // int8 rows: the last launch left the new rows' latents in fp32
+        err = launch_encode_quant(e.a, sl, e.max_batch, st);
+        if (err != cudaSuccess) return cuda_fail(c, err, "encode launch");
+        ++c->launches;
+    }
     return KVCAR_OK;
 }
 

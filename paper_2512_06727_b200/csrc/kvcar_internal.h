@@ -28,7 +28,7 @@ struct SourcePlan {
     // latent-attention kernels (bf16): decoder FC1 [m][d] with the signs of the BatchNorm scale taken into its rows, the
     // sizes of the scale [m], and the shift over them (in the kernels' own order)
     const void *w1n;
-    const float *sabs, *shift;
+    const float *sabs, *shift, *rowsum;  // rowsum: of w1n's rows, in the order of the shift
     int32_t width;     // elements per pool row (= d if compressed, = in_dim if raw)
     int32_t d, m, in_dim;
     int32_t compressed;

@@ -46,6 +46,12 @@
 // cycles per chunk, 2 700 of them pipe time), and each waited for what only the other needed.  A warp of the hidden
 // epilogue takes one slab of a job (three slabs, four lane quarters: twelve warps).
 //
+// int8 latent rows (Eq. 4: x = (code - zero-point) / scale).  latent_widen_kernel, ahead of the front, writes code - z0 as bf16 rows
+// into the workspace, z0 the zero-point kept to [-128, 128]: whole numbers of at most 256, exact in bf16 (a row whose range holds
+// zero, as latents have it, has z0 = zero-point).  The hidden warps of the Q8 builds then apply 1 / scale per token, and where a row
+// has some of its zero-point left over, that times the weights' row sum: nothing is rounded that the fp32 form does not round.  12-layer step of the GPT-2 shape,
+// 8 x 1024 tokens: 973 us, 6404 us in fp32 on the CUDA cores.
+//
 // Warp roles: 0 loads of latents, query rows and shifts, 1 hidden products (leader CTA) and tensor memory, 2 weight loads,
 // 3 S and U products (leader CTA), 4-15 hidden warps, 16-23 output warps.  All waits are bounded and record a code in the
 // status word.
@@ -94,6 +100,7 @@ struct Params {
     int32_t hq, m_pad, wq_batch;
     int32_t nz, nh, nw, nqs, nt, m_t;  // places for latent, hidden, weight and query slabs; shift buffers and their floats
     int32_t t_resident;                // every source has a shift buffer of its own
+    int32_t wide;                      // latents come from the widened rows of the launch's tiles
     int32_t two_terms_k, two_terms_v;  // low parts of the query rows / of the probabilities are used
 };
 
@@ -214,7 +221,7 @@ struct __align__(8) Scratch {
 };
 
 // NQ: query heads padded.  NB: U blocks of 128 hidden features at most; fixes the registers of the running sums.
-template <int NQ, int NB>
+template <int NQ, int NB, bool Q8>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     decode_latent_kernel(const __grid_constant__ Params a) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -293,8 +300,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             auto rows_of = [&](const TileWalk &t, int *r) {  // pool rows of the tile's two 64-token halves
                 r[0] = r[1] = 0;
                 const int v = t.valid(a.sq);
+                if (Q8) {  // widened rows lie in the order of the launch's tiles
+                    r[0] = v == 0 ? 0 : (t.first(a.sq, t.si) + t.chunk) * TILE;
+                    r[1] = r[0] + (v > 64 ? 64 : 0);
+                }
+#pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    if (v == 0) break;
+                    if (Q8 || v == 0) break;
                     int tok = t.chunk * TILE + 64 * h;
                     if (64 * h >= v) tok = t.chunk * TILE;  // no valid token there: re-read the first half
                     const int page = a.block_table[(int64_t)a.sq.id[t.si] * a.max_pages_per_seq + tok / a.page_tokens];
@@ -586,6 +598,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                         hslot += hslot & 1u;
                         if (hslot == (uint32_t)a.nh) hslot = 0;
                     }
+                    float inv[4] = {1.f, 1.f, 1.f, 1.f}, left[4] = {0.f, 0.f, 0.f, 0.f};  // int8 rows: this lane's four tokens
+                    bool any_left = false;
+                    if (Q8) {
+                        const int r0 = valid == 0 ? 0 : (tw.first(a.sq, tw.si) + tw.chunk) * TILE;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int r = (int)lane_base + 8 * i + (lane >> 2);
+                            if (r < valid) {
+                                const float2 p = list_of(side).src[s].rowp[r0 + r];
+                                inv[i] = p.x;
+                                left[i] = p.y;
+                            }
+                            any_left |= left[i] != 0.f;
+                        }
+                        any_left = __any_sync(0xffffffffu, any_left);
+                    }
                     const float *tbuf = reinterpret_cast<const float *>(smem_raw + (s_t - s_z)) + tb * a.m_t;
                     if (it == 0 || !a.t_resident) mbar_wait(tb_full + 8 * tb, tphase, a.status, &abort_flag, 0x60f);
                     for (int c0 = 0; c0 < m; c0 += CN, ++h) {
@@ -627,8 +655,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                                         uint32_t w[4];
 #pragma unroll
                                         for (int j = 0; j < 4; ++j) {
-                                            const float2 x = __fadd2_rn(make_float2(__uint_as_float(r[i >> 1][4 * j + 2 * (i & 1)]),
-                                                                                    __uint_as_float(r[i >> 1][4 * j + 2 * (i & 1) + 1])), t[j]);
+                                            float2 h2 = make_float2(__uint_as_float(r[i >> 1][4 * j + 2 * (i & 1)]),
+                                                                    __uint_as_float(r[i >> 1][4 * j + 2 * (i & 1) + 1]));
+                                            if (Q8 && any_left) {
+                                                const float2 rs = __ldg(reinterpret_cast<const float2 *>(list_of(side).src[s].rowsum + c0 + col) +
+                                                                        4 * (lane & 3) + j);
+                                                h2 = __ffma2_rn(make_float2(-left[i], -left[i]), rs, h2);
+                                            }
+                                            const float2 x = Q8 ? __ffma2_rn(h2, make_float2(inv[i], inv[i]), t[j]) : __fadd2_rn(h2, t[j]);
                                             const float2 y = __fmul2_rn(x, slope2);
                                             // LeakyReLU: the larger of x and slope*x for slope <= 1, the smaller for slope > 1
                                             w[j] = lr_max ? pack_bf16(fmaxf(x.x, y.x), fmaxf(x.y, y.y))
@@ -1094,19 +1128,66 @@ __device__ __forceinline__ void merge_block(const LatHeads &hp, const LatSeqs &s
 template <int SB, int THREADS, int NF>
 __global__ void __launch_bounds__(THREADS) latent_back_kernel(const __grid_constant__ LatHeads hp, const __grid_constant__ LatSeqs sq,
                                                               const __grid_constant__ MergeArgs a, const __grid_constant__ LatEncode e,
-                                                              const __grid_constant__ EncodeGrid g) {
+                                                              const __grid_constant__ SeqList all, const __grid_constant__ EncodeGrid g) {
     extern __shared__ __align__(16) float sm[];
     const int b = blockIdx.x;
     if (b < g.n_enc)
-        enc::encode_fc_block<__nv_bfloat16, 2, false, NF>(e.a, sq.id, sq.n, e.hid, e.pitch, e.max_batch, sm, b % g.nbx, b / g.nbx % g.nby,
+        enc::encode_fc_block<__nv_bfloat16, 2, false, NF>(e.a, all.id, all.n, e.hid, e.pitch, e.max_batch, sm, b % g.nbx, b / g.nbx % g.nby,
                                                       b / g.nbx / g.nby, g.nbx);
     else
         merge_block<SB, THREADS>(hp, sq, a, sm, b - g.n_enc);
 }
 
+// int8 rows to bf16: grid = (tiles, sources of K and V, 2 pieces of a tile's rows).  Bound by memory: a byte in, two out.
+__global__ void __launch_bounds__(256) latent_widen_kernel(const __grid_constant__ LatCodes c, const __grid_constant__ LatSeqs sq,
+                                                           const int32_t *block_table, int max_pages_per_seq, int page_tokens,
+                                                           __nv_bfloat16 *wide, float2 *rowp, int wide_rows, int pitch) {
+    __shared__ int64_t rows[64];
+    __shared__ int z0[64];
+    const int side = (int)blockIdx.y >= c.n_src[0], s = blockIdx.y - (side ? c.n_src[0] : 0), t = blockIdx.x, tid = threadIdx.x;
+    TileWalk tw;
+    tw.start(sq, t);
+    tw.left = 1;
+    const int valid = min(64, (tw.chunk + 1 < tw.n ? TILE : (int)(sq.first[tw.si] >> 24) + 1) - 64 * (int)blockIdx.z);
+    if (valid <= 0) return;
+    const int64_t out0 = (int64_t)(side * LT_MAX_SRC + s) * wide_rows + t * TILE + 64 * blockIdx.z;
+    enc::grid_dependency_wait();
+    enc::launch_dependents();
+    if (tid < valid) {
+        const int tok = tw.chunk * TILE + 64 * blockIdx.z + tid;
+        const int page = block_table[(int64_t)sq.id[tw.si] * max_pages_per_seq + tok / page_tokens];
+        const int64_t r = (int64_t)page * page_tokens + tok % page_tokens;
+        const float scale = c.qparam[side][s][2 * r], zp = c.qparam[side][s][2 * r + 1];
+        // a row of equal values has any zero-point: its whole part within reach goes into the codes, the rest is left over
+        const float z = rintf(fminf(fmaxf(zp, -128.f), 128.f));
+        rows[tid] = r;
+        z0[tid] = (int)z;
+        rowp[out0 + tid] = make_float2(1.f / scale, zp - z);
+    }
+    __syncthreads();
+    const int d = c.d[side][s], nv = d >> 4;
+    for (int i = tid; i < valid * nv; i += 256) {
+        const int r = i / nv, k = 16 * (i % nv);
+        const int4 v = *reinterpret_cast<const int4 *>(c.codes[side][s] + rows[r] * d + k);
+        const int words[4] = {v.x, v.y, v.z, v.w};
+        uint32_t o[8];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const int b0 = (int8_t)words[w], b1 = (int8_t)(words[w] >> 8), b2 = (int8_t)(words[w] >> 16), b3 = words[w] >> 24;
+            o[2 * w] = pack_bf16((float)(b0 - z0[r]), (float)(b1 - z0[r]));
+            o[2 * w + 1] = pack_bf16((float)(b2 - z0[r]), (float)(b3 - z0[r]));
+        }
+        uint4 *dst = reinterpret_cast<uint4 *>(wide + (out0 + r) * pitch + k);
+        dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+        dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+    }
+}
+
 using Kernel = void (*)(const Params);
-const Kernel kernels[] = {decode_latent_kernel<12, 2>, decode_latent_kernel<12, 5>, decode_latent_kernel<16, 5>,
-                          decode_latent_kernel<16, 8>, decode_latent_kernel<32, 2>, decode_latent_kernel<32, 3>};
+const Kernel kernels[2][6] = {{decode_latent_kernel<12, 2, false>, decode_latent_kernel<12, 5, false>, decode_latent_kernel<16, 5, false>,
+                               decode_latent_kernel<16, 8, false>, decode_latent_kernel<32, 2, false>, decode_latent_kernel<32, 3, false>},
+                              {decode_latent_kernel<12, 2, true>, decode_latent_kernel<12, 5, true>, decode_latent_kernel<16, 5, true>,
+                               decode_latent_kernel<16, 8, true>, decode_latent_kernel<32, 2, true>, decode_latent_kernel<32, 3, true>}};
 constexpr int KERNEL_NQ[] = {12, 12, 16, 16, 32, 32}, KERNEL_NB[] = {2, 5, 5, 8, 2, 3};
 constexpr int N_KERNELS = 6;
 
@@ -1137,24 +1218,31 @@ constexpr float LOG2E = 1.4426950408889634f;
 
 }  // namespace
 
-size_t lat_ws_bytes(const kvcar_config &cfg, int max_k_sources, int max_m, int batch) {
-    if (cfg.storage != KVCAR_BF16 || cfg.latent_quant || cfg.head_dim != 64 || cfg.n_q_heads > LT_MAX_Q || max_k_sources <= 0 || max_m <= 0)
-        return 0;
+static int lat_wide_tiles(int batch, int max_len) {
+    const int per_seq = (max_len + TILE - 1) / TILE;
+    return (int)std::min<int64_t>((int64_t)batch * per_seq, std::max(LT_WIDE_TILES, per_seq));
+}
+
+size_t lat_ws_bytes(const kvcar_config &cfg, int max_sources, int max_m, int max_d, int batch, int max_len) {
+    if (cfg.storage != KVCAR_BF16 || cfg.head_dim != 64 || cfg.n_q_heads > LT_MAX_Q || max_sources <= 0 || max_m <= 0) return 0;
     const size_t nq = padded_heads(cfg.n_q_heads), m_pad = ((size_t)max_m + 63) / 64 * 64;
-    const size_t wq = (size_t)std::min(max_k_sources, LT_MAX_SRC) * batch * wq_rows((int)nq) * m_pad * 2;
+    const size_t wq = (size_t)std::min(max_sources, LT_MAX_SRC) * batch * wq_rows((int)nq) * m_pad * 2;
     const size_t bias = ((size_t)batch * cfg.n_q_heads * 4 + 255) / 256 * 256;
     const size_t runs = (size_t)LT_MAX_CTAS + batch;
-    return wq + bias + runs * cfg.n_q_heads * (m_pad + 2) * sizeof(float) + (size_t)LT_MAX_CTAS * nq * TILE * sizeof(float);
+    size_t n = wq + bias + runs * cfg.n_q_heads * (m_pad + 2) * sizeof(float) + (size_t)LT_MAX_CTAS * nq * TILE * sizeof(float);
+    if (cfg.latent_quant)  // the widened rows start at a multiple of 256 bytes
+        n = (n + 255) / 256 * 256 + (size_t)(LT_MAX_SRC + std::min(max_sources, LT_MAX_SRC)) * lat_wide_tiles(batch, max_len) * TILE * (2 * (size_t)max_d + sizeof(float2));
+    return n;
 }
 
 void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPlan> &plans, size_t pool_rows,
-               int max_k_sources, int max_m, int batch, char *ws_area) {
+               int max_sources, int max_m, int max_d, int batch, int max_len, char *ws_area) {
     st.available = false;
     const int nl = cfg.n_layers;
     st.layer.assign(nl, LatLayer{});
     st.heads.assign(nl, LatHeads{});
     st.cfg.assign(nl, LatLayerCfg{});
-    if (lat_ws_bytes(cfg, max_k_sources, max_m, batch) == 0 || cfg.page_tokens % 64 != 0) return;
+    if (lat_ws_bytes(cfg, max_sources, max_m, max_d, batch, max_len) == 0 || cfg.page_tokens % 64 != 0) return;
     EncodeTiledFn fn = tensor_map_encoder();
     if (!fn) return;
     int dev = 0, sms = 148;
@@ -1169,7 +1257,7 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
     st.group = group;
     st.m_pad = (max_m + 63) / 64 * 64;
     st.batch = batch;
-    const size_t n_src = std::min(max_k_sources, LT_MAX_SRC), n_rows = n_src * batch * wq_rows(st.nq);
+    const size_t n_src = std::min(max_sources, LT_MAX_SRC), n_rows = n_src * batch * wq_rows(st.nq);
     if (!encode_bf16_map(fn, &st.tm_wq, ws_area, n_rows, st.m_pad, st.m_pad, op_rows(st.nq))) return;
     char *p = ws_area;
     st.wq = p;
@@ -1181,6 +1269,15 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
     st.ml = reinterpret_cast<float *>(p);
     p += (size_t)(LT_MAX_CTAS + batch) * cfg.n_q_heads * 2 * sizeof(float);
     st.score = reinterpret_cast<float *>(p);
+    p += (size_t)LT_MAX_CTAS * st.nq * TILE * sizeof(float);
+    p = ws_area + ((size_t)(p - ws_area) + 255) / 256 * 256;
+    st.quant = cfg.latent_quant != 0;
+    st.wide_tiles = lat_wide_tiles(batch, max_len);
+    const size_t wide_rows = (size_t)st.wide_tiles * TILE, regions = LT_MAX_SRC + n_src;
+    st.wide = p;
+    st.rowp = reinterpret_cast<float2 *>(p + regions * wide_rows * 2 * max_d);
+    st.max_d = max_d;
+    st.codes.assign(st.quant ? nl : 0, LatCodes{});
     for (int l = 0; l < nl; ++l) {
         LatLayer &ly = st.layer[l];
         LatHeads &hp = st.heads[l];
@@ -1193,10 +1290,13 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
             ly.list[w].n = hp.n_src[w] = wp.n_src;
             for (int s = 0; s < wp.n_src && ok; ++s) {
                 const SourcePlan &sp = wp.src[s];
-                ok = sp.compressed && !sp.qparam && sp.d % 16 == 0 && sp.m % 16 == 0 && sp.width == sp.d;
+                ok = sp.compressed && (sp.qparam != nullptr) == st.quant && sp.d % 16 == 0 && sp.m % 16 == 0 && sp.width == sp.d;
                 if (!ok) break;
                 LatSrc &d = ly.list[w].src[s];
                 d.shift = sp.shift;
+                d.rowsum = sp.rowsum;
+                const size_t region = (size_t)(w * LT_MAX_SRC + s) * wide_rows;
+                d.rowp = st.rowp + region;
                 d.c0 = 0;
                 d.map = s;
                 d.d = sp.d;
@@ -1211,7 +1311,15 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
                     hp.slot[w][h] = (uint8_t)sp.slot[i];
                     hp.cur[w][h] = reinterpret_cast<const __nv_bfloat16 *>(plans[l].cur[w][h]) + plans[l].cur_head[w][h] * 64;
                 }
-                ok = encode_bf16_map(fn, &ly.pool[w][s], sp.pool, pool_rows, sp.width, sp.width) &&
+                if (st.quant) {
+                    LatCodes &c = st.codes[l];
+                    c.codes[w][s] = reinterpret_cast<const int8_t *>(sp.pool);
+                    c.qparam[w][s] = sp.qparam;
+                    c.d[w][s] = sp.d;
+                    c.n_src[w] = wp.n_src;
+                }
+                ok = (st.quant ? encode_bf16_map(fn, &ly.pool[w][s], reinterpret_cast<__nv_bfloat16 *>(st.wide) + region * max_d, wide_rows, sp.d, max_d)
+                               : encode_bf16_map(fn, &ly.pool[w][s], sp.pool, pool_rows, sp.width, sp.width)) &&
                      encode_bf16_map(fn, &ly.w1[w][s], sp.w1n, sp.m, sp.d, sp.d, CN / 2);
                 ks = std::max(ks, (sp.d + 63) / 64);
                 lm = std::max(lm, sp.m);
@@ -1248,7 +1356,7 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
         lc.variant = (uint8_t)v;
         lc.max_m = lm;
         lc.max_mk = lmk;
-        if (cudaFuncSetAttribute(kernels[v], cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess) {
+        if (cudaFuncSetAttribute(kernels[st.quant][v], cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess) {
             cudaGetLastError();
             continue;
         }
@@ -1300,6 +1408,7 @@ bool split_side(const LatList &all, int n, LatList *out) {
             LatSrc &u = l.src[l.n++];
             u = all.src[s];
             u.shift += c0;
+            u.rowsum += c0;
             u.c0 = c0;
             u.m = w;
         }
@@ -1315,10 +1424,10 @@ int count_chunks(const LatList &l) {
 
 }  // namespace
 
-cudaError_t lat_launch(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer, const LatEncode *enc_in,
-                       cudaStream_t stream, int *n_launches) {
+// `seqs` of a call; `all`: those whose rows the carried encoder takes
+static cudaError_t launch_group(LatState &st, const DecodeArgs &a, const SeqList &seqs, const SeqList &all, const int32_t *lens, int layer,
+                                const LatEncode *enc_in, cudaStream_t stream, int *n_launches) {
     const LatLayerCfg &lc = st.cfg[layer];
-    if (seqs.n > st.batch) return cudaErrorInvalidValue;  // the list names a sequence twice
     const LatLayer &ly = st.layer[layer];
     Params p;
     fill_seqs(p.sq, seqs, lens, st.n_sms);
@@ -1326,6 +1435,14 @@ cudaError_t lat_launch(LatState &st, const DecodeArgs &a, const SeqList &seqs, c
     LatEncode e{};
     if (enc_in) e = *enc_in;
     EncodeGrid g{0, 1, 1};
+    if (st.quant) {
+        const LatCodes &c = st.codes[layer];
+        cudaError_t err = launch_pdl(latent_widen_kernel, dim3(p.sq.n_tiles, c.n_src[0] + c.n_src[1], 2), 256, 0, stream, c, p.sq, a.block_table,
+                                     a.max_pages_per_seq, a.page_tokens, reinterpret_cast<__nv_bfloat16 *>(st.wide), st.rowp,
+                                     st.wide_tiles * TILE, st.max_d);
+        if (err != cudaSuccess) return err;
+        ++*n_launches;
+    }
     // ---- front
     QueryArgs qa;
     qa.q = reinterpret_cast<const __nv_bfloat16 *>(a.q);
@@ -1343,16 +1460,16 @@ cudaError_t lat_launch(LatState &st, const DecodeArgs &a, const SeqList &seqs, c
     // Features per warp of the encoder: one spreads a few rows' weights over the most warps, two read the rows half as often from
     // shared memory.  12-layer step of the GPT-2 shape over 256 cached tokens: 64 sequences 954 us with one, 817 with two; 256
     // sequences 3093, 2686 (four: 902, 3069, the registers leave one block per SM).
-    const int nf = seqs.n >= 64 ? 2 : 1;
+    const int nf = all.n >= 64 ? 2 : 1;
     size_t smem = 0;
     if (enc_in) {
         g.nbx = (std::max(e.max_m, 1) + LF_THREADS / 32 * nf - 1) / (LF_THREADS / 32 * nf);
-        g.nby = (seqs.n + enc::RB - 1) / enc::RB;
+        g.nby = (all.n + enc::RB - 1) / enc::RB;
         g.n_enc = g.nbx * g.nby * 2;
         smem = (size_t)enc::RB * e.max_in * sizeof(float);
     }
     cudaError_t err = launch_pdl(nf == 2 ? latent_front_kernel<2> : latent_front_kernel<1>, dim3(g.n_enc + a.hq * qa.col_blocks * ((seqs.n + LQ_SB - 1) / LQ_SB)), LF_THREADS,
-                                 smem, stream, st.heads[layer], qa, e, seqs, g);
+                                 smem, stream, st.heads[layer], qa, e, all, g);
     if (err != cudaSuccess) return err;
     // ---- tiles
     for (int w = 0; w < 2; ++w)
@@ -1387,24 +1504,24 @@ cudaError_t lat_launch(LatState &st, const DecodeArgs &a, const SeqList &seqs, c
     // of the GPT-2 shape at 1 / 8 x 1024 tokens: 371 / 649 us, 625 / 712 us with one cluster per pair.
     int kp = std::min({(slots / pairs + 1) / 2, count_chunks(ly.list[0]), LT_MAX_PARTS});
     int vp = std::min({slots / pairs - kp, count_chunks(ly.list[1]), LT_MAX_PARTS});
-    *n_launches = 3;
+    *n_launches += 3;
     if (p.sq.per == 1 && kp >= 1 && vp >= 1) {
         p.mode = MODE_K;
         while (!split_side(ly.list[0], kp, p.list)) --kp;
         p.n_parts = p.k_parts = kp;
-        err = launch_pdl(kernels[lc.variant], dim3(2 * pairs * kp), NTHREADS, lc.smem, stream, p);
+        err = launch_pdl(kernels[st.quant][lc.variant], dim3(2 * pairs * kp), NTHREADS, lc.smem, stream, p);
         if (err != cudaSuccess) return err;
         p.mode = MODE_V;
         while (!split_side(ly.list[1], vp, p.list)) --vp;
         p.n_parts = vp;
-        err = launch_pdl(kernels[lc.variant], dim3(2 * pairs * vp), NTHREADS, lc.smem, stream, p);
-        *n_launches = 4;
+        err = launch_pdl(kernels[st.quant][lc.variant], dim3(2 * pairs * vp), NTHREADS, lc.smem, stream, p);
+        ++*n_launches;
     } else {
         p.mode = MODE_BOTH;
         p.n_parts = p.k_parts = 1;
         p.list[0] = ly.list[0];
         p.list[1] = ly.list[1];
-        err = launch_pdl(kernels[lc.variant], dim3(2 * pairs), NTHREADS, lc.smem, stream, p);
+        err = launch_pdl(kernels[st.quant][lc.variant], dim3(2 * pairs), NTHREADS, lc.smem, stream, p);
     }
     if (err != cudaSuccess) return err;
     // ---- back
@@ -1430,8 +1547,34 @@ cudaError_t lat_launch(LatState &st, const DecodeArgs &a, const SeqList &seqs, c
         smem = std::max(smem, (size_t)enc::RB * e.pitch * sizeof(float));
     }
     const dim3 grid(g.n_enc + a.hq * ((seqs.n + sb - 1) / sb));
-    return wide ? launch_pdl(nf == 2 ? latent_back_kernel<4, 256, 2> : latent_back_kernel<4, 256, 1>, grid, threads, smem, stream, st.heads[layer], p.sq, m, e, g)
-                : launch_pdl(latent_back_kernel<1, 512, 1>, grid, threads, smem, stream, st.heads[layer], p.sq, m, e, g);
+    return wide ? launch_pdl(nf == 2 ? latent_back_kernel<4, 256, 2> : latent_back_kernel<4, 256, 1>, grid, threads, smem, stream, st.heads[layer], p.sq, m, e, all, g)
+                : launch_pdl(latent_back_kernel<1, 512, 1>, grid, threads, smem, stream, st.heads[layer], p.sq, m, e, all, g);
+}
+
+cudaError_t lat_launch(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer, const LatEncode *enc,
+                       cudaStream_t stream, int *n_launches) {
+    if (seqs.n > st.batch) return cudaErrorInvalidValue;  // the list names a sequence twice
+    *n_launches = 0;
+    if (!st.quant) return launch_group(st, a, seqs, seqs, lens, layer, enc, stream, n_launches);
+    // int8 rows: as many sequences at a time as the widened rows have room for; the encoder goes with the first
+    for (int i0 = 0; i0 < seqs.n;) {
+        SeqList g;
+        g.n = 0;
+        int tiles = 0, i = i0;
+        for (; i < seqs.n; ++i) {
+            const int n = (lens[i] + TILE - 1) / TILE;
+            if (g.n > 0 && tiles > 0 && tiles + n > st.wide_tiles) break;
+            g.id[g.n++] = seqs.id[i];
+            tiles += n;
+        }
+        DecodeArgs ga = a;
+        ga.q = reinterpret_cast<const __nv_bfloat16 *>(a.q) + (int64_t)i0 * a.hq * 64;
+        ga.out = reinterpret_cast<__nv_bfloat16 *>(a.out) + (int64_t)i0 * a.hq * 64;
+        cudaError_t err = launch_group(st, ga, g, seqs, lens + i0, layer, i0 == 0 ? enc : nullptr, stream, n_launches);
+        if (err != cudaSuccess) return err;
+        i0 = i;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace kvcar

@@ -17,12 +17,15 @@ inline int shift_place(int f) { return (f & ~31) + ((f & 7) >> 1) * 8 + ((f & 31
 
 // Hidden columns c0 .. c0 + m - 1 of one source layer of K or V as the tile kernel sees them (kernel parameter).
 struct LatSrc {
+    const float *rowsum;  // int8 rows: sums of the rows of the signed first layer, from c0, in the same order
+    const float2 *rowp;   // int8 rows: (1/scale, what is left of the zero-point) per widened row
     const float *shift;  // fused bias + BatchNorm shift over the size of its scale, from c0, in fragment order (see shift_place)
     int32_t d, m, c0;
     int32_t map;    // which of the layer's tensor maps
     float slope;
     uint32_t mask;  // query heads whose K (or V) head is served from this source
 };
+constexpr int LT_WIDE_TILES = 296;  // int8 rows: tiles widened at a time (more if one sequence needs more)
 constexpr int LT_MAX_PARTS = 8;  // clusters that share the K (or the V) side of a pair of tiles
 struct LatList {
     int32_t n;
@@ -54,6 +57,13 @@ struct LatHeads {
     const void *cur[2][LT_MAX_Q];  // by KV head: its 64 columns of the current-token row of sequence 0
     uint8_t idx[2][LT_MAX_Q], slot[2][LT_MAX_Q];
 };
+// int8 rows: where a source's codes and its rows' (scale, zero-point) lie, the column sums of its signed first layer
+struct LatCodes {
+    const int8_t *codes[2][LT_MAX_SRC];
+    const float *qparam[2][LT_MAX_SRC];
+    int32_t d[2][LT_MAX_SRC];
+    int32_t n_src[2];
+};
 
 struct LatLayerCfg {
     uint8_t ok = 0;
@@ -69,6 +79,11 @@ struct LatState {
     bool available = false;
     std::vector<LatLayer> layer;
     std::vector<LatHeads> heads;
+    std::vector<LatCodes> codes;  // int8 rows only
+    bool quant = false;
+    int wide_tiles = 0, max_d = 0;
+    void *wide = nullptr;         // int8 rows: [K, V][source][wide_tiles * 128][max_d] bf16
+    float2 *rowp = nullptr;       // [K, V][source][wide_tiles * 128]
     std::vector<LatLayerCfg> cfg;
     int n_sms = 148;
     int nq = 12;      // query heads padded
@@ -84,10 +99,10 @@ struct LatState {
 };
 
 // bytes of the operands and partial results inside the workspace (0: the shape does not take this path)
-size_t lat_ws_bytes(const kvcar_config &cfg, int max_k_sources, int max_m, int batch);
+size_t lat_ws_bytes(const kvcar_config &cfg, int max_sources, int max_m, int max_d, int batch, int max_len);
 // decide per layer whether the kernels take it, build tensor maps, place the workspace area
 void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPlan> &plans, size_t pool_rows,
-               int max_k_sources, int max_m, int batch, char *ws_area);
+               int max_sources, int max_m, int max_d, int batch, int max_len, char *ws_area);
 // flags: those of the call (17 to 32 query heads in groups of at most two only with KVCAR_ABSORBED_V, see kvcar_latent.cu)
 bool lat_layer_supported(const LatState &st, int layer, uint32_t flags);
 // The encoder of the same step's new rows, carried by the first and the last launch (null: none).

@@ -498,3 +498,39 @@ def test_fp32_arithmetic_kernels_at_tile_edges(case):
         if n:
             p.prefill([s_], n)
     _check_step(p.decode_step(seqs, 0), w.storage, case)
+
+
+@pytest.mark.parametrize("case", ["offset_rows", "groups"])
+def test_int8_rows_on_the_tensor_cores_beyond_the_usual(case, monkeypatch):
+    """int8 rows are widened to whole numbers that bf16 holds exactly.  offset_rows: K latents far from zero (their zero-points
+    do not fit the codes, the rest goes through the weights' row sums); a constant on every K latent adds the same to all
+    scores of a head, so the outputs keep their size and the usual tolerance.  groups: more tiles than the widened rows have
+    room for at a time (296), worked through in two groups of sequences, an empty sequence among them."""
+    if case == "offset_rows":
+        real = synth.make_stack_autoencoders
+
+        def shifted(*a, **kw):
+            aes = real(*a, **kw)
+            for (_, which), ae in aes.items():
+                if which == K:
+                    ae["enc_b2"] = ae["enc_b2"] + np.float32(6.0)
+            return aes
+        monkeypatch.setattr(synth, "make_stack_autoencoders", shifted)
+        w = synth.scaled(synth.CONFIGS["c2"], n_layers=2, batch=3, cached_tokens=0, decode_steps=1, reuse_frac=0.25)
+        lens = (200, 129, 64)
+    else:
+        w = synth.scaled(synth.CONFIGS["c3"], n_layers=1, batch=4, cached_tokens=0, decode_steps=1, reuse_frac=0.0)
+        lens = (13000, 0, 12801, 12929)
+    pps = (max(lens) + 2 + w.page_tokens - 1) // w.page_tokens
+    p = Pair(w, max_seqs=len(lens), max_pages=len(lens) * pps, max_pages_per_seq=pps, latent_quant=True)
+    assert all(p.s.ctx.layer_kernel(l) == B.KERNEL_TENSOR for l in range(w.n_layers))
+    seqs = list(range(len(lens)))
+    p.open(seqs)
+    for s_, n in zip(seqs, lens):
+        if n:
+            p.prefill([s_], n)
+    if case == "offset_rows":
+        q = p.s.pool_quant_params(0, 0)[p.o.locate(0, 5)[1]].cpu().numpy()
+        assert q[1] < -129      # the zero-point really is out of the codes' reach
+    for fused in (False, True):
+        _check_step(p.decode_step(seqs, int(fused), fused=fused), "bf16", f"{case} fused={fused}")
