@@ -37,17 +37,8 @@ cudaError_t launch_stage(const EncodeArgs &a, const SeqList &seqs, float *hid, i
     const size_t smem = (size_t)RB * n_in_max * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(encode_fc_kernel<T, STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((n_out_max + NW - 1) / NW, (seqs.n + RB - 1) / RB, 2);
-    cfg.blockDim = dim3(NW * 32);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, encode_fc_kernel<T, STAGE>, a, seqs, hid, hid_pitch, max_batch);
+    return launch_pdl(encode_fc_kernel<T, STAGE>, dim3((n_out_max + NW - 1) / NW, (seqs.n + RB - 1) / RB, 2), NW * 32, smem, st, a, seqs, hid,
+                      hid_pitch, max_batch);
 }
 
 // Eq. 4 per cached row, as the tail of encode_generic_kernel: scale = 255/(max-min), zero-point = -round(scale*min) - 128,
@@ -92,16 +83,7 @@ __global__ void __launch_bounds__(256) encode_quant_kernel(const __grid_constant
 }  // namespace
 
 cudaError_t launch_encode_quant(const EncodeArgs &a, const SeqList &seqs, int max_batch, cudaStream_t st) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((2 * seqs.n + 7) / 8);
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, encode_quant_kernel, a, seqs, max_batch);
+    return launch_pdl(encode_quant_kernel, dim3((2 * seqs.n + 7) / 8), 256, 0, st, a, seqs, max_batch);
 }
 
 size_t encode_split_smem(int max_in, int max_m) { return (size_t)RB * std::max(max_in, max_m) * sizeof(float); }

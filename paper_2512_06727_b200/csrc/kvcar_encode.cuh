@@ -2,6 +2,7 @@
 // feature.  Device code only; shared by the encoder's own launches and by those that carry it beside other work.
 #pragma once
 #include "kvcar_internal.h"
+#include "kvcar_pdl.cuh"
 
 namespace kvcar {
 namespace enc {
@@ -37,9 +38,6 @@ struct Vec16<__nv_bfloat16> {
     static __device__ __forceinline__ float one(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
     static __device__ __forceinline__ void store(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 };
-
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // acc[f][r] += sum over this lane's share of w_f[0..n) * x[r][0..n); `pre` holds the lane's first vector of each row already
 template <typename T, int NF>

@@ -249,7 +249,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     const int my_run = 2 * pair + (int)rank;
     const int n_it = max(0, min(a.sq.per, a.sq.n_tiles - 2 * pair * a.sq.per));
     const int my_first = my_run * a.sq.per;
-    enc::launch_dependents();
+    launch_dependents();
 
     if (threadIdx.x == 0) {
         sh.abort_flag = 0;
@@ -379,7 +379,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                     }
                 }
                 if (!waited && a.mode != MODE_V && (!moved || z.it > 0 || z.side > side_lo)) {
-                    enc::grid_dependency_wait();
+                    grid_dependency_wait();
                     waited = moved = true;
                 }
                 if (waited && q.it < n_it && mbar_test(q_empty + 8 * qslot, qphase ^ 1u)) {
@@ -416,7 +416,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                     }
                 }
             }
-            if (!waited) enc::grid_dependency_wait();  // every block sees the launches before complete: those after rely on it
+            if (!waited) grid_dependency_wait();  // every block sees the launches before complete: those after rely on it
         }
     } else if (warp == 2) {
         // ============================== weight loads ==============================
@@ -739,7 +739,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             if (a.mode != MODE_V) {
                 fetch(s);
             } else {
-                if (it == 0) enc::grid_dependency_wait();  // the launch before holds the scores
+                if (it == 0) grid_dependency_wait();  // the launch before holds the scores
 #pragma unroll
                 for (int q = 0; q < NT; ++q) s[q] = 0.f;
                 for (int p = 0; p < a.k_parts; ++p) {
@@ -890,8 +890,8 @@ __device__ __forceinline__ void query_block(const LatHeads &hp, const QueryArgs 
 #pragma unroll
     for (int c = 0; c < 64; ++c) u[c] = j < m2 ? __ldg(w + (int64_t)c * m2) : 0u;
     if (j < m2) sab = __ldg(reinterpret_cast<const float2 *>(sp.sabs) + j);
-    enc::grid_dependency_wait();
-    enc::launch_dependents();
+    grid_dependency_wait();
+    launch_dependents();
     for (int i = tid; i < 64 * LQ_SB; i += LF_THREADS) {
         const int k = i >> 6, c = i & 63;
         qs[c][k] = k < n_here ? __bfloat162float(a.q[((int64_t)(si0 + k) * a.hq + qh) * 64 + c]) * a.scale : 0.f;
@@ -990,8 +990,8 @@ __device__ __forceinline__ void merge_block(const LatHeads &hp, const LatSeqs &s
             pre[k] = j < m ? __ldg(w + j * pitch) : 0u;
         }
     }
-    enc::grid_dependency_wait();
-    enc::launch_dependents();
+    grid_dependency_wait();
+    launch_dependents();
     auto first = [&](int i) { return (int)(sq.first[i] & 0xffffffu); };
     auto runs = [&](int si, int &k0) {  // runs of a sequence: k0 .. k0 + n - 1
         const int f0 = first(si), f1 = first(si + 1);
@@ -1151,8 +1151,8 @@ __global__ void __launch_bounds__(256) latent_widen_kernel(const __grid_constant
     const int valid = min(64, (tw.chunk + 1 < tw.n ? TILE : (int)(sq.first[tw.si] >> 24) + 1) - 64 * (int)blockIdx.z);
     if (valid <= 0) return;
     const int64_t out0 = (int64_t)(side * LT_MAX_SRC + s) * wide_rows + t * TILE + 64 * blockIdx.z;
-    enc::grid_dependency_wait();
-    enc::launch_dependents();
+    grid_dependency_wait();
+    launch_dependents();
     if (tid < valid) {
         const int tok = tw.chunk * TILE + 64 * blockIdx.z + tid;
         const int page = block_table[(int64_t)sq.id[tw.si] * max_pages_per_seq + tok / page_tokens];
@@ -1373,22 +1373,6 @@ bool lat_layer_supported(const LatState &st, int layer, uint32_t flags) {
 }
 
 namespace {
-
-// the launch attribute of a programmatic dependent launch
-template <typename... Formal, typename... Args>
-cudaError_t launch_pdl(void (*k)(Formal...), dim3 grid, int threads, size_t smem, cudaStream_t st, const Args &...args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, args...);
-}
 
 // A side's hidden columns in `n` parts of whole 192-column chunks, of about the same number of products each; a part holds one
 // range of columns per source at most (the ranges of a source follow one another).  False where a part would be empty.

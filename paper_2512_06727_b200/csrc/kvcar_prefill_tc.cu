@@ -22,6 +22,7 @@
 #include <cstring>
 
 #include "kvcar_internal.h"
+#include "kvcar_pdl.cuh"
 #include "kvcar_ptx.cuh"
 
 namespace kvcar {
@@ -125,6 +126,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
     cluster_sync_all();  // both CTAs' barriers exist before either signals the other's
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    // Dependent launches: barriers and tensor memory are set up while the launch before drains.  (A block of the next one finds
+    // shared memory on an SM only when this one's has left.)
+    grid_dependency_wait();
+    launch_dependents();
 
     if (warp == 0 || warp == 2 + PF_EPI_WARPS) {
         // two producers share a k-step's loads (a tensor load costs its thread ~100 cycles here): warp 0 the row operand,
@@ -404,11 +409,8 @@ cudaError_t launch_prefill_tc(const PrefillTcArgs &h, const SeqList &seqs, bool 
         const unsigned c2 = (unsigned)std::min(37, row_pairs * ((max_d + PF_N - 1) / PF_N));
         auto k1 = exact ? prefill_fc_kernel<1, true> : prefill_fc_kernel<1, false>;
         auto k2 = exact ? prefill_fc_kernel<2, true> : prefill_fc_kernel<2, false>;
-        k1<<<dim3(2 * c1, 1, 2), PF_THREADS, PF_SMEM, st>>>(ax[0], ax[1], w1[0], w1[1], a, seqs);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        k2<<<dim3(2 * c2, 1, 2), PF_THREADS, PF_SMEM, st>>>(ah[0], ah[1], w2[0], w2[1], a, seqs);
-        e = cudaGetLastError();
+        cudaError_t e = launch_pdl(k1, dim3(2 * c1, 1, 2), PF_THREADS, PF_SMEM, st, ax[0], ax[1], w1[0], w1[1], a, seqs);
+        if (e == cudaSuccess) e = launch_pdl(k2, dim3(2 * c2, 1, 2), PF_THREADS, PF_SMEM, st, ah[0], ah[1], w2[0], w2[1], a, seqs);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
