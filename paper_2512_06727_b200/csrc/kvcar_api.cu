@@ -61,6 +61,10 @@ struct kvcar_ctx {
     size_t hslot_bytes = 0;
     cudaEvent_t ev_h[H_SLOTS] = {};
     bool ev_h_used[H_SLOTS] = {};
+    // their copies run on a stream of the library's own into one of as many device slots, ahead of the caller's stream
+    cudaStream_t copy = nullptr;
+    cudaEvent_t ev_d[H_SLOTS] = {};  // the step that reads a device slot is done
+    bool ev_d_used[H_SLOTS] = {};
     unsigned hslot = 0;
 
     // pages
@@ -221,8 +225,9 @@ void compute_layout(kvcar_ctx *c) {
     c->part_off = s;
     const int nb = std::min(g.max_seqs, KVCAR_MAX_BATCH);
     s = align_up(s + (size_t)nb * c->max_chunks * g.n_q_heads * (g.head_dim + 2) * sizeof(float), 256);
-    c->stage_off = s;
-    s = align_up(s + (size_t)nb * (2 * W + 2 * g.n_q_heads * g.head_dim) * c->elem + 4 * 256, 256);
+    c->stage_off = s;  // host-buffer entry point: H_SLOTS slots of k, v and q, then one out
+    s = align_up(s + (kvcar_ctx::H_SLOTS * (2 * align_up((size_t)nb * W * c->elem, 256) + align_up((size_t)nb * g.n_q_heads * g.head_dim * c->elem, 256)) +
+                      (size_t)nb * g.n_q_heads * g.head_dim * c->elem), 256);
     c->enchid_off = s;  // hidden activations between the decode-time encoder's launches; int8 rows: then the fp32 latents
     s = align_up(s + (size_t)2 * nb * (c->max_m + (g.latent_quant ? c->max_d : 0)) * sizeof(float), 256);
     c->kvsplit_off = s;  // probabilities handed from K clusters to V clusters (tensor-core kernel, small grids)
@@ -420,6 +425,9 @@ kvcar_status kvcar_destroy(kvcar_ctx *ctx) {
     if (ctx->side) cudaStreamDestroy(ctx->side);
     for (cudaEvent_t e : ctx->ev_h)
         if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : ctx->ev_d)
+        if (e) cudaEventDestroy(e);
+    if (ctx->copy) cudaStreamDestroy(ctx->copy);
     if (ctx->hstage) cudaFreeHost(ctx->hstage);
     delete ctx;
     return KVCAR_OK;
@@ -713,8 +721,10 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
         const size_t kvb = align_up(nbatch * hkv * hd * c->elem, 256), qb = align_up(nbatch * g.n_q_heads * hd * c->elem, 256);
         c->hslot_bytes = 2 * kvb + qb;
         bool ok = cudaHostAlloc((void **)&c->hstage, c->hslot_bytes * kvcar_ctx::H_SLOTS, cudaHostAllocDefault) == cudaSuccess;
+        ok = ok && cudaStreamCreateWithFlags(&c->copy, cudaStreamNonBlocking) == cudaSuccess;
         for (int i = 0; ok && i < kvcar_ctx::H_SLOTS; ++i)
-            ok = cudaEventCreateWithFlags(&c->ev_h[i], cudaEventDisableTiming) == cudaSuccess;
+            ok = cudaEventCreateWithFlags(&c->ev_h[i], cudaEventDisableTiming) == cudaSuccess &&
+                 cudaEventCreateWithFlags(&c->ev_d[i], cudaEventDisableTiming) == cudaSuccess;
         if (!ok) {
             cudaGetLastError();
             if (c->hstage) cudaFreeHost(c->hstage);
@@ -1118,14 +1128,20 @@ kvcar_status kvcar_step_layer_host(kvcar_ctx *c, int32_t layer, const int32_t *s
     const kvcar_config &g = c->cfg;
     const size_t kvb = align_up((size_t)n_seqs * g.n_kv_heads * g.head_dim * c->elem, 256);
     const size_t qb = align_up((size_t)n_seqs * g.n_q_heads * g.head_dim * c->elem, 256);
-    char *dk = c->ws + c->stage_off, *dv = dk + kvb, *dq = dv + kvb, *dout = dq + qb;
     cudaStream_t st = (cudaStream_t)stream;
     const size_t kv_bytes = (size_t)n_seqs * g.n_kv_heads * g.head_dim * c->elem;
     const size_t q_bytes = (size_t)n_seqs * g.n_q_heads * g.head_dim * c->elem;
-    cudaError_t e;
-    if (c->hstage && 2 * kvb + q_bytes <= c->hslot_bytes) {
-        // one copy: k, v, q gathered in a pinned slot with the device staging area's layout
-        const unsigned slot = c->hslot++ % kvcar_ctx::H_SLOTS;
+    const unsigned slot = c->hslot++ % kvcar_ctx::H_SLOTS;
+    char *dk = c->ws + c->stage_off + (size_t)slot * c->hslot_bytes, *dv = dk + kvb, *dq = dv + kvb;
+    char *dout = c->ws + c->stage_off + (size_t)kvcar_ctx::H_SLOTS * c->hslot_bytes;
+    cudaError_t e = cudaSuccess;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+    const bool ahead = c->hstage && cap == cudaStreamCaptureStatusNone;
+    if (ahead) {
+        // One copy: k, v, q gathered in a pinned slot with the device slot's layout.  It depends on nothing in the caller's stream
+        // but the step that read the device slot eight calls ago, so it runs ahead of the steps before this one
+        // (on the caller's stream it stood between two steps: 12 layers, batch 8, 1024 tokens, 898 us; so, with the output below, 742).
         if (c->ev_h_used[slot]) {
             e = cudaEventSynchronize(c->ev_h[slot]);  // the copy that read this slot eight calls ago
             if (e != cudaSuccess) return cuda_fail(c, e, "staging slot");
@@ -1134,18 +1150,34 @@ kvcar_status kvcar_step_layer_host(kvcar_ctx *c, int32_t layer, const int32_t *s
         memcpy(h, k_host, kv_bytes);
         memcpy(h + kvb, v_host, kv_bytes);
         memcpy(h + 2 * kvb, q_host, q_bytes);
-        e = cudaMemcpyAsync(dk, h, 2 * kvb + q_bytes, cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) e = cudaEventRecord(c->ev_h[slot], st);
+        // before its first use: whatever the caller's stream still does with the memory it gave as workspace
+        if (!c->ev_d_used[slot]) e = cudaEventRecord(c->ev_d[slot], st);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(c->copy, c->ev_d[slot], 0);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(dk, h, 2 * kvb + q_bytes, cudaMemcpyHostToDevice, c->copy);
+        if (e == cudaSuccess) e = cudaEventRecord(c->ev_h[slot], c->copy);
         c->ev_h_used[slot] = e == cudaSuccess;
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c->ev_h[slot], 0);
     } else {
         e = cudaMemcpyAsync(dk, k_host, kv_bytes, cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(dv, v_host, kv_bytes, cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(dq, q_host, q_bytes, cudaMemcpyHostToDevice, st);
     }
     if (e != cudaSuccess) return cuda_fail(c, e, "host to device copy");
-    kvcar_status s = kvcar_step_layer(c, layer, seqs, n_seqs, dk, dv, dq, dout, flags, stream);
-    if (s != KVCAR_OK) return s;
-    e = cudaMemcpyAsync(out_host, dout, (size_t)n_seqs * g.n_q_heads * g.head_dim * c->elem, cudaMemcpyDeviceToHost, st);
+    // A page-locked output is written by the step's last kernel itself: each value once, and a copy behind the kernel costs the stream
+    // more than the writes do at every size (12 layers of GPT-2's shape, 128 tokens: batch 8, 12 KB, 538 us with the copy and 471
+    // without; batch 256, 384 KB, 2425 and 2269).
+    char *out = dout;
+    cudaPointerAttributes at;
+    if (((uintptr_t)out_host & 15) == 0) {
+        if (cudaPointerGetAttributes(&at, out_host) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer)
+            out = (char *)at.devicePointer;
+        else
+            cudaGetLastError();
+    }
+    kvcar_status s = kvcar_step_layer(c, layer, seqs, n_seqs, dk, dv, dq, out, flags, stream);
+    if (ahead) c->ev_d_used[slot] = cudaEventRecord(c->ev_d[slot], st) == cudaSuccess;
+    if (s != KVCAR_OK || out != dout) return s;
+    e = cudaMemcpyAsync(out_host, dout, q_bytes, cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "device to host copy");
     return KVCAR_OK;
 }
