@@ -322,6 +322,42 @@ def test_host_buffer_entry_point_matches_device_entry_points():
         assert_close(ho.float().numpy().astype(np.float64), ref, "bf16", f"host entry layer {l}")
 
 
+@pytest.mark.parametrize("pinned_out", [True, False], ids=["page_locked_out", "pageable_out"])
+def test_host_buffer_steps_equal_device_steps(pinned_out):
+    """Eleven host-buffer steps of two layers, nothing awaited between them and the inputs overwritten after each call (more calls
+    than the library has staging slots), bit for bit against the device entry point on a twin context."""
+    w = synth.scaled(synth.CONFIGS["c3"], n_layers=2, batch=2, reuse_frac=0.25)
+    seqs, steps = [0, 1], 11
+    host, dev = [Pair(w, max_seqs=2, max_pages=8, max_pages_per_seq=4, with_oracle=False) for _ in range(2)]
+    for p in (host, dev):
+        p.open(seqs)
+        p.prefill(seqs, 50)
+    dt = host.s.dtype
+    shape = [(2, w.n_kv_heads, w.head_dim)] * 2 + [(2, w.n_q_heads, w.head_dim)]
+    buf = [torch.empty(s, dtype=dt).pin_memory() for s in shape]
+    out = torch.zeros((steps, 2) + shape[2], dtype=dt)
+    out = out.pin_memory() if pinned_out else out
+    ref = torch.zeros((steps, 2) + shape[2], dtype=dt, device="cuda")
+    gen = torch.Generator().manual_seed(5)
+    for step in range(steps):
+        for l in range(2):
+            x = [torch.randn(s, generator=gen).to(dt) for s in shape]
+            for b, t in zip(buf, x):
+                b.copy_(t)
+            host.s.ctx.step_layer_host(l, seqs, *(b.data_ptr() for b in buf), out[step, l].data_ptr(),
+                                       B.INCLUDE_CURRENT_EXACT, host.s.stream())
+            for b in buf:
+                b.zero_()
+            d = [t.cuda() for t in x]
+            dev.s.ctx.step_layer(l, seqs, *(t.data_ptr() for t in d), ref[step, l].data_ptr(), B.INCLUDE_CURRENT_EXACT,
+                                 dev.s.stream())
+        for p in (host, dev):
+            p.s.ctx.advance(seqs, 1, p.s.stream())
+    host.s.ctx.sync_status(host.s.stream())
+    dev.s.ctx.sync_status(dev.s.stream())
+    assert torch.equal(out, ref.cpu())
+
+
 def test_errors_leave_state_untouched():
     w = synth.scaled(synth.CONFIGS["c3"], n_layers=1, batch=1, reuse_frac=0.0)
     p = Pair(w, max_seqs=2, max_pages=2, max_pages_per_seq=2, with_oracle=False)
