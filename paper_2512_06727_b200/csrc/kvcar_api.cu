@@ -956,9 +956,9 @@ static int prepare_decode(kvcar_ctx *c, int32_t layer, const int32_t *seqs, int3
 
 // The kernel that works through the cached tokens tile by tile (tensor-core, raw or generic) and leaves one partial
 // result per tile.  It reads the cache rows below the sequences' lengths, the tables and q - nothing that this
-// step's encoder writes (the exact current token enters in the combine kernel).
+// step's encoder writes (the exact current token enters in the combine kernel).  Raw layers: `raw_rows` are appended by the same launch.
 static kvcar_status enqueue_decode_tiles(kvcar_ctx *c, int32_t layer, const DecodeArgs &a, const SeqList &sl,
-                                         int n_chunks, cudaStream_t st) {
+                                         int n_chunks, cudaStream_t st, const EncodeArgs *raw_rows = nullptr) {
     c->fma_tiles = false;
     if (n_chunks <= 0) return KVCAR_OK;
     const kvcar_config &g = c->cfg;
@@ -967,7 +967,7 @@ static kvcar_status enqueue_decode_tiles(kvcar_ctx *c, int32_t layer, const Deco
         return fail(c, KVCAR_ERR_UNSUPPORTED, std::string("tensor-core kernel cannot run this layer: ") + c->tc.why);
     cudaError_t e;
     if (c->kernel != KVCAR_KERNEL_GENERIC && layer_is_raw(c, layer)) {
-        e = launch_decode_raw(a, sl, c->raw_src_ok[layer] ? &c->raw_src[layer] : nullptr, g.storage, n_chunks, st);
+        e = launch_decode_raw(a, sl, c->raw_src_ok[layer] ? &c->raw_src[layer] : nullptr, raw_rows, g.storage, n_chunks, st);
     } else if (want_tc) {
         int32_t lens[KVCAR_MAX_BATCH];
         for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
@@ -1087,6 +1087,13 @@ kvcar_status kvcar_step_layer(kvcar_ctx *c, int32_t layer, const int32_t *seqs, 
     SeqList sl;
     const int n_chunks = prepare_decode(c, layer, seqs, n_seqs, q, out, flags, a, sl);
     if (use_latent(c, layer, n_chunks, flags)) return enqueue_latent(c, layer, a, sl, k, v, st);
+    // a raw layer has no encoder: its new rows are copied in the tile kernel's launch
+    if (n_chunks > 0 && c->kernel != KVCAR_KERNEL_GENERIC && layer_is_raw(c, layer) && !c->ae[layer * 2].set && !c->ae[layer * 2 + 1].set) {
+        const EncodeArgs rows = encode_args(c, layer, 1, k, v);
+        s = enqueue_decode_tiles(c, layer, a, sl, n_chunks, st, &rows);
+        if (s != KVCAR_OK) return s;
+        return enqueue_combine(c, layer, a, sl, n_chunks, st);
+    }
     // The tile kernel does not depend on this step's encoder, so it goes to a side stream that forks here and
     // joins before the combine kernel: the encoder's two short launches overlap it instead of running in front
     // of it.  (The other way round - encoder on the side stream behind the fork event - measured no gain: the

@@ -108,6 +108,37 @@ __device__ __forceinline__ int row_of_lane(int lane) {
     return ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
 }
 
+// raw layer: 16 bytes of input row r's stored heads, from stored channel c on, into the row's place in the cache
+template <typename T>
+__device__ __forceinline__ void copy_raw_vec(const EncodeArgs &a, const EncPlan &pl, const T *src, const int32_t *seq_ids, int r, int c) {
+    const int seq = seq_ids[r], t = a.seq_len[seq];
+    const int page = a.block_table[(int64_t)seq * a.max_pages_per_seq + t / a.page_tokens];
+    const int64_t pr = (int64_t)page * a.page_tokens + t % a.page_tokens;
+    *reinterpret_cast<uint4 *>(reinterpret_cast<T *>(pl.pool) + pr * pl.width + c) =
+        Vec16<T>::load(src + (int64_t)r * a.kv_width + pl.heads[c / a.hd] * a.hd + c % a.hd);
+}
+
+// A raw layer's whole append of one token per sequence, K and V: the exact current rows (all heads) and the cache rows.  Thread
+// `tid` of `n_threads` that share the work.
+template <typename T>
+__device__ __forceinline__ void append_raw_rows(const EncodeArgs &a, const int32_t *seq_ids, int n_rows, int tid, int n_threads) {
+    constexpr int VL = Vec16<T>::N;
+    const int wv = a.kv_width / VL;
+    for (int which = 0; which < 2; ++which) {
+        const EncPlan &pl = a.plan[which];
+        const T *src = reinterpret_cast<const T *>(which == 0 ? a.k : a.v);
+        const int nv = pl.in_dim / VL, per_row = wv + nv;
+        for (int idx = tid; idx < n_rows * per_row; idx += n_threads) {
+            const int r = idx / per_row, i = idx % per_row;
+            if (i < wv)
+                reinterpret_cast<uint4 *>(reinterpret_cast<T *>(pl.cur) + (int64_t)seq_ids[r] * a.kv_width)[i] =
+                    reinterpret_cast<const uint4 *>(src + (int64_t)r * a.kv_width)[i];
+            else
+                copy_raw_vec<T>(a, pl, src, seq_ids, r, (i - wv) * VL);
+        }
+    }
+}
+
 // STAGE 1: hidden = LeakyReLU(BN(W1 x + b1)) -> scratch.  STAGE 2: latent = W2 hidden + b2 -> cache rows.
 // A warp takes NF features: a row's values are read from shared memory once per NF weights, and those reads bound the block when
 // many row blocks share a launch (256 rows of the GPT-2 shape: see latent_front_kernel).
@@ -163,17 +194,10 @@ __device__ __forceinline__ void encode_fc_block(const EncodeArgs &a, const int32
                     reinterpret_cast<const uint4 *>(src + (int64_t)r * a.kv_width)[cv];
             }
         }
-        if (!compressed) {  // raw layer: copy the stored heads' slices into the cache rows, 16 bytes at a time
-            T *pool = reinterpret_cast<T *>(pl.pool);
+        if (!compressed) {
             const int nv = in_dim / VL;
-            for (int idx = bx * blockDim.x + threadIdx.x; idx < rows_here * nv; idx += nbx * blockDim.x) {
-                const int rr = idx / nv, c = (idx % nv) * VL, r = r0 + rr;
-                const int seq = seq_ids[r], t = a.seq_len[seq];
-                const int page = a.block_table[(int64_t)seq * a.max_pages_per_seq + t / a.page_tokens];
-                const int64_t pr = (int64_t)page * a.page_tokens + t % a.page_tokens;
-                *reinterpret_cast<uint4 *>(pool + pr * pl.width + c) =
-                    Vec16<T>::load(src + (int64_t)r * a.kv_width + pl.heads[c / a.hd] * a.hd + c % a.hd);
-            }
+            for (int idx = bx * blockDim.x + threadIdx.x; idx < rows_here * nv; idx += nbx * blockDim.x)
+                copy_raw_vec<T>(a, pl, src, seq_ids, r0 + idx / nv, (idx % nv) * VL);
             return;
         }
         if (bx * NW >= n_out) return;

@@ -3,6 +3,7 @@
 // split-KV combine.  They handle every supported shape in both storage types and
 // are the fp32-mode path; the bf16 tensor-core kernel lives in kvcar_tc.cu.
 #include "kvcar_internal.h"
+#include "kvcar_pdl.cuh"
 
 namespace kvcar {
 
@@ -442,6 +443,8 @@ __device__ __forceinline__ float block_reduce(float v, bool is_max, float *red) 
 template <typename T>
 __global__ void __launch_bounds__(32 * CB_WARPS) combine_kernel(const __grid_constant__ DecodeArgs a,
                                                                 const __grid_constant__ SeqList seqs) {
+    grid_dependency_wait();
+    launch_dependents();
     const int qh = blockIdx.x, si = blockIdx.y, c = threadIdx.x, lane = c & 31, warp = c >> 5;
     const int seq = seqs.id[si];
     const int L = a.seq_len[seq];
@@ -528,6 +531,8 @@ __global__ void __launch_bounds__(32 * CB_WARPS) combine_kernel(const __grid_con
 template <typename T>
 __global__ void __launch_bounds__(32 * CB_WARPS) combine_warp_kernel(const __grid_constant__ DecodeArgs a,
                                                                      const __grid_constant__ SeqList seqs) {
+    grid_dependency_wait();
+    launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int hd = a.hd, hq = a.hq;  // hd <= 128
     const int item = blockIdx.x * CB_WARPS + warp;
@@ -673,18 +678,11 @@ cudaError_t launch_combine(const DecodeArgs &a, const SeqList &seqs, int dtype, 
     // Longer sequences: a CTA per row, which walks a row's tiles in parallel.
     if (n_chunks <= 32) {
         const int grid = (a.hq * seqs.n + CB_WARPS - 1) / CB_WARPS;
-        if (dtype == KVCAR_F32)
-            combine_warp_kernel<float><<<grid, 32 * CB_WARPS, 0, st>>>(a, seqs);
-        else
-            combine_warp_kernel<__nv_bfloat16><<<grid, 32 * CB_WARPS, 0, st>>>(a, seqs);
-        return cudaGetLastError();
+        return launch_pdl(dtype == KVCAR_F32 ? combine_warp_kernel<float> : combine_warp_kernel<__nv_bfloat16>, dim3(grid),
+                          32 * CB_WARPS, 0, st, a, seqs);
     }
-    dim3 grid(a.hq, seqs.n);
-    if (dtype == KVCAR_F32)
-        combine_kernel<float><<<grid, 32 * CB_WARPS, 0, st>>>(a, seqs);
-    else
-        combine_kernel<__nv_bfloat16><<<grid, 32 * CB_WARPS, 0, st>>>(a, seqs);
-    return cudaGetLastError();
+    return launch_pdl(dtype == KVCAR_F32 ? combine_kernel<float> : combine_kernel<__nv_bfloat16>, dim3(a.hq, seqs.n), 32 * CB_WARPS,
+                      0, st, a, seqs);
 }
 
 }  // namespace kvcar

@@ -131,8 +131,8 @@ cudaError_t launch_decode_generic(const DecodeArgs &a, const SeqList &seqs, int 
                                   int grid_chunks, cudaStream_t st);
 // raw K/V layers (no autoencoder), head_dim 64, <= 8 query heads per KV head (kvcar_raw.cu)
 // src: the layer's tensor maps and head places, or null (no maps: rows are then staged with cp.async)
-cudaError_t launch_decode_raw(const DecodeArgs &a, const SeqList &seqs, const RawSources *src, int dtype, int grid_chunks,
-                              cudaStream_t st);
+cudaError_t launch_decode_raw(const DecodeArgs &a, const SeqList &seqs, const RawSources *src, const EncodeArgs *enc, int dtype,
+                              int grid_chunks, cudaStream_t st);
 // TMA descriptor of one raw bf16 pool [rows][width] with a box of 32 rows x 64 columns (one head's slice of one
 // 32-token step), 128-byte swizzle; false if the driver entry point is missing or the shape is refused
 bool raw_build_map(void *dst_host, const void *pool_dev, uint64_t rows, uint64_t width);

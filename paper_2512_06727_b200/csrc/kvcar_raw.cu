@@ -14,6 +14,7 @@
 // per step, the row index and the probabilities come from the owning lane through shared memory.
 #include <cuda.h>
 
+#include "kvcar_encode.cuh"
 #include "kvcar_internal.h"
 #include "kvcar_ptx.cuh"
 
@@ -26,28 +27,6 @@ constexpr int RW = 4;    // warps (= KV heads) per CTA
 
 template <typename T>
 struct Row64;
-template <>
-struct Row64<__nv_bfloat16> {
-    // 64 values of one token and head -> fp32
-    static __device__ __forceinline__ void load(const __nv_bfloat16 *p, float *x) {
-        const uint4 *q = reinterpret_cast<const uint4 *>(p);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const uint4 v = __ldg(q + i);
-            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                x[8 * i + 2 * j] = __uint_as_float(u[j] << 16);
-                x[8 * i + 2 * j + 1] = __uint_as_float(u[j] & 0xFFFF0000u);
-            }
-        }
-    }
-    static __device__ __forceinline__ float2 load2(const __nv_bfloat16 *p) {  // two adjacent channels
-        const uint32_t u = __ldg(reinterpret_cast<const uint32_t *>(p));
-        return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u));
-    }
-    static __device__ __forceinline__ float one(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
-};
 template <>
 struct Row64<float> {
     static __device__ __forceinline__ void load(const float *p, float *x) {
@@ -81,13 +60,28 @@ __device__ __forceinline__ HeadSrc find_head(const WhichPlan &wp, int h) {
     return r;
 }
 
-// grid = (tiles, ceil(hkv / RW), n_seqs); block = RW warps; head_dim 64, at most 8 query heads per KV head
+// The step's new rows ride along: layers of the grid from z = n_seqs on copy them (see append_raw_rows) to the row behind each
+// sequence's last, which the tiles do not use, and to the current-token buffers, which the merge behind this launch reads.
+template <typename T>
+__device__ __forceinline__ void append_block(const EncodeArgs &e, const SeqList &seqs) {
+    const int per_z = gridDim.x * gridDim.y;
+    const int block = (blockIdx.z - seqs.n) * per_z + blockIdx.y * gridDim.x + blockIdx.x;
+    enc::append_raw_rows<T>(e, seqs.id, seqs.n, block * blockDim.x + threadIdx.x, (gridDim.z - seqs.n) * per_z * blockDim.x);
+}
+
+// grid = (tiles, ceil(hkv / RW), n_seqs + layers that append); block = RW warps; head_dim 64, at most 8 query heads per KV head
 template <typename T>
 __global__ void __launch_bounds__(RW * 32, 4) decode_raw_kernel(const __grid_constant__ DecodeArgs a,
-                                                             const __grid_constant__ SeqList seqs) {
+                                                             const __grid_constant__ SeqList seqs, const __grid_constant__ EncodeArgs enc) {
     __shared__ __align__(16) float qs[RW][8][64];
     __shared__ __align__(16) float ps[RW][8][32];  // probabilities of the current 32-token group
     __shared__ int64_t rows[RW][32];                // and their cache rows
+    grid_dependency_wait();
+    launch_dependents();
+    if (blockIdx.z >= seqs.n) {
+        append_block<T>(enc, seqs);
+        return;
+    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tile = blockIdx.x, h = blockIdx.y * RW + warp, si = blockIdx.z;
     if (h >= a.hkv) return;
@@ -215,6 +209,11 @@ __global__ void __launch_bounds__(RW * 32, 4) decode_raw_kernel(const __grid_con
 // pool, 128-byte swizzle: the same layout the cp.async build writes by hand) that count their bytes on a barrier
 // of the warp, instead of sixteen 16-byte copies and eight page-table look-ups per lane.  (Requesting
 // the whole tile at once - four buffers per warp - halves the resident warps and measured slower at every size.)
+// The maps' L2 promotion is 128 bytes, one head's slice: at 256 a step that needs only some of the stored heads (the others reused)
+// fetched their neighbours too (517 MB read where 403 are needed, batch 32, 4096 tokens, GPT-2's shape).
+// The new rows' copies ride in this launch and the merge is a dependent launch behind it.  12 layers, us per step, with the copies
+// in a launch of their own on a side stream and 256-byte promotion -> now: batch 32, 4096 tokens 950 -> 849 (87 % of the measured
+// copy bandwidth over the cached rows); batch 8, 1000 tokens 317 -> 158; batch 1, 200 tokens 244 -> 129; batch 128, 300 tokens 414 -> 340.
 constexpr int GQ_STEP = 32;                      // tokens per step
 constexpr int GQ_BUF = GQ_STEP * 64 * 2;         // bytes of one K (or V) step buffer: 32 rows x 128 B
 constexpr int GQ_WARP_SMEM = 4 * GQ_BUF;         // K and V, two steps each
@@ -252,15 +251,41 @@ __device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
 template <bool TMA>
 __global__ void __launch_bounds__(GQ_RW * 32) decode_raw_gq_kernel(const __grid_constant__ DecodeArgs a,
                                                                const __grid_constant__ SeqList seqs,
-                                                               const __grid_constant__ RawSources src) {
+                                                               const __grid_constant__ RawSources src,
+                                                               const __grid_constant__ EncodeArgs enc) {
     extern __shared__ __align__(128) uint8_t gq_smem[];
     __shared__ __align__(8) uint64_t step_bar[GQ_RW][2];  // TMA build: bytes of a step buffer pair have landed
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tile = blockIdx.x, h = blockIdx.y * GQ_RW + warp, si = blockIdx.z;
+    if (si >= seqs.n) {
+        grid_dependency_wait();
+        launch_dependents();
+        append_block<__nv_bfloat16>(enc, seqs);
+        return;
+    }
+    const uint32_t bar0 = smem_addr(&step_bar[warp][0]);
+    if (TMA) {
+        if (lane == 0) {
+            ptx::mbar_init(bar0, 1);
+            ptx::mbar_init(bar0 + 8, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        ptx::fence_async_smem();
+        __syncwarp();
+    }
+    grid_dependency_wait();
+    launch_dependents();
     if (h >= a.hkv) return;
     const int seq = seqs.id[si];
-    const int L = a.seq_len[seq];
+    const int32_t *bt = a.block_table + (int64_t)seq * a.max_pages_per_seq;
     const int t0 = tile * RT;
+    // TMA build, lane i < 4: first row of step i, requested beside the length and before it is known which steps there are
+    int step_row = 0;
+    if (TMA && lane < RT / GQ_STEP) {
+        const int tok = t0 + GQ_STEP * lane, pg = tok / a.page_tokens;
+        if (pg < a.max_pages_per_seq) step_row = bt[pg] * a.page_tokens + tok % a.page_tokens;
+    }
+    const int L = a.seq_len[seq];
     if (t0 >= L) return;
     const int valid = min(RT, L - t0);
     const int group = a.hq / a.hkv;
@@ -274,23 +299,14 @@ __global__ void __launch_bounds__(GQ_RW * 32) decode_raw_gq_kernel(const __grid_
     }
     const __nv_bfloat16 *kpool = reinterpret_cast<const __nv_bfloat16 *>(ks.pool) + ks.col;
     const __nv_bfloat16 *vpool = reinterpret_cast<const __nv_bfloat16 *>(vs.pool) + vs.col;
-    const int32_t *bt = a.block_table + (int64_t)seq * a.max_pages_per_seq;
     // K step buffers 0, 1, then V step buffers 0, 1 (1024-byte aligned: the swizzle pattern of the tensor loads is a
     // function of the address)
     const uint32_t sbase = ((smem_addr(gq_smem) + 1023u) & ~1023u) + warp * GQ_WARP_SMEM;
     uint8_t *gbase = gq_smem + (sbase - smem_addr(gq_smem));
-    const uint32_t bar0 = smem_addr(&step_bar[warp][0]);
     const CUtensorMap *kmap = nullptr, *vmap = nullptr;
     if (TMA) {
         kmap = &src.map[0][src.idx[0][h]];
         vmap = &src.map[1][src.idx[1][h]];
-        if (lane == 0) {
-            ptx::mbar_init(bar0, 1);
-            ptx::mbar_init(bar0 + 8, 1);
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        }
-        ptx::fence_async_smem();
-        __syncwarp();
     }
     const int g = lane >> 2, t = lane & 3;
 
@@ -309,9 +325,8 @@ __global__ void __launch_bounds__(GQ_RW * 32) decode_raw_gq_kernel(const __grid_
     // the tile's first row (their probabilities are zero)
     auto fetch = [&](int step, int buf) {
         if (TMA) {
+            const int row = __shfl_sync(0xffffffffu, step_row, step);  // the step's 32 tokens lie in one page
             if (ptx::elect_one()) {
-                const int tok = t0 + GQ_STEP * step;  // the step's 32 tokens lie in one page
-                const int row = bt[tok / a.page_tokens] * a.page_tokens + tok % a.page_tokens;
                 ptx::mbar_expect_tx(bar0 + 8 * buf, 2 * GQ_BUF);
                 ptx::tma_load_2d(sbase + buf * GQ_BUF, kmap, ks.col, row, bar0 + 8 * buf);
                 ptx::tma_load_2d(sbase + (2 + buf) * GQ_BUF, vmap, vs.col, row, bar0 + 8 * buf);
@@ -446,36 +461,32 @@ __global__ void __launch_bounds__(GQ_RW * 32) decode_raw_gq_kernel(const __grid_
 bool raw_build_map(void *dst_host, const void *pool_dev, uint64_t rows, uint64_t width) {
     static EncodeTiledFn fn = tensor_map_encoder();
     if (!fn || width % 8 != 0) return false;
-    return encode_bf16_map(fn, dst_host, pool_dev, rows, width, width, GQ_STEP);
+    return encode_bf16_map(fn, dst_host, pool_dev, rows, width, width, GQ_STEP, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
 }
 
-cudaError_t launch_decode_raw(const DecodeArgs &a, const SeqList &seqs, const RawSources *src, int dtype, int grid_chunks,
-                              cudaStream_t st) {
-    dim3 grid(grid_chunks, (a.hkv + RW - 1) / RW, seqs.n);
-    if (dtype == KVCAR_BF16) {
-        static bool configured[64] = {};  // per device: the attribute belongs to the device's copy of the kernel
-        int dev = 0;
-        cudaGetDevice(&dev);
-        constexpr int smem = GQ_SMEM + 1024;  // + room to align the step buffers
-        if (dev < 0 || dev >= 64 || !configured[dev]) {
-            cudaError_t e = cudaFuncSetAttribute(decode_raw_gq_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(decode_raw_gq_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (e != cudaSuccess) return e;
-            if (dev >= 0 && dev < 64) configured[dev] = true;
-        }
-        grid.y = (a.hkv + GQ_RW - 1) / GQ_RW;
-        if (src && a.page_tokens % GQ_STEP == 0)
-            decode_raw_gq_kernel<true><<<grid, GQ_RW * 32, smem, st>>>(a, seqs, *src);
-        else
-            decode_raw_gq_kernel<false><<<grid, GQ_RW * 32, smem, st>>>(a, seqs, RawSources{});
-        return cudaGetLastError();
+cudaError_t launch_decode_raw(const DecodeArgs &a, const SeqList &seqs, const RawSources *src, const EncodeArgs *enc, int dtype,
+                              int grid_chunks, cudaStream_t st) {
+    dim3 grid(grid_chunks, (a.hkv + (dtype == KVCAR_BF16 ? GQ_RW : RW) - 1) / (dtype == KVCAR_BF16 ? GQ_RW : RW), seqs.n);
+    const int threads = dtype == KVCAR_BF16 ? GQ_RW * 32 : RW * 32;
+    if (enc) {  // about two 16-byte copies a thread, so that these blocks do not outlast the tiles
+        const int64_t vecs = (int64_t)seqs.n * 2 * 2 * (a.hkv * 64 / (dtype == KVCAR_BF16 ? 8 : 4));
+        const int64_t per_z = (int64_t)grid.x * grid.y * threads * 2;
+        grid.z += (unsigned)((vecs + per_z - 1) / per_z);
     }
-    if (dtype == KVCAR_F32)
-        decode_raw_kernel<float><<<grid, RW * 32, 0, st>>>(a, seqs);
-    else
-        decode_raw_kernel<__nv_bfloat16><<<grid, RW * 32, 0, st>>>(a, seqs);
-    return cudaGetLastError();
+    const EncodeArgs e = enc ? *enc : EncodeArgs{};
+    if (dtype == KVCAR_F32) return launch_pdl(decode_raw_kernel<float>, grid, threads, 0, st, a, seqs, e);
+    static bool configured[64] = {};  // per device: the attribute belongs to the device's copy of the kernel
+    int dev = 0;
+    cudaGetDevice(&dev);
+    constexpr int smem = GQ_SMEM + 1024;  // + room to align the step buffers
+    if (dev < 0 || dev >= 64 || !configured[dev]) {
+        cudaError_t r = cudaFuncSetAttribute(decode_raw_gq_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (r == cudaSuccess) r = cudaFuncSetAttribute(decode_raw_gq_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (r != cudaSuccess) return r;
+        if (dev >= 0 && dev < 64) configured[dev] = true;
+    }
+    if (src && a.page_tokens % GQ_STEP == 0) return launch_pdl(decode_raw_gq_kernel<true>, grid, threads, smem, st, a, seqs, *src, e);
+    return launch_pdl(decode_raw_gq_kernel<false>, grid, threads, smem, st, a, seqs, RawSources{}, e);
 }
 
 }  // namespace kvcar

@@ -166,6 +166,23 @@ def test_uncompressed_twin_with_query_groups(heads):
         _check_step(p.decode_step(seqs, step), "bf16", f"raw group {hq // hkv} step {step}")
 
 
+@pytest.mark.parametrize("storage,page_tokens,batch", [("bf16", 64, 1), ("bf16", 16, 5), ("bf16", 64, 33), ("f32", 64, 5)])
+def test_uncompressed_single_call_steps(storage, page_tokens, batch):
+    """Raw layers through the single call, whose tile launch also appends the rows: pages of less than a 32-token step (plain copies)
+    and more (tensor loads), fp32 rows, lengths on both sides of a step, a tile and a page."""
+    w = synth.scaled(synth.CONFIGS["c2"], n_layers=2, storage=storage, page_tokens=page_tokens, batch=batch, reuse_frac=0.3)
+    seqs = list(range(batch))
+    lens = [(1, 127, 128, 31, 65)[s % 5] for s in seqs]
+    per = (130 + page_tokens) // page_tokens + 1
+    p = Pair(w, max_seqs=batch, max_pages=batch * per, max_pages_per_seq=per, compress=False)
+    p.open(seqs)
+    for s_, n in zip(seqs, lens):
+        p.prefill([s_], n)
+    for step in range(2):
+        _check_step(p.decode_step(seqs, step, fused=True), storage, f"raw {storage} page {page_tokens} batch {batch} step {step}")
+    p.check_latents(seqs)
+
+
 @pytest.mark.parametrize("kernel", KERNELS, ids=lambda k: KNAME[k])
 def test_physical_page_permutation_is_bit_invariant(kernel):
     """The same logical cache laid out on different physical pages must give
