@@ -285,15 +285,18 @@ void fuse_bn(const std::vector<float> &b1, const std::vector<float> &bn, int m, 
 // First decoder layer for the latent-attention kernels.  LeakyReLU is positively homogeneous: with s the fused BatchNorm scale,
 // LeakyReLU(s x + t) = |s| LeakyReLU(sign(s) x + t / |s|).  The sign goes into the weight row (exact), t / |s| is the shift
 // that is left to the epilogue, |s| goes to the neighbours of the hidden vector (W4^T q and the weighted sum, both fp32).  A
-// scale too small to divide by leaves the constant LeakyReLU(t).
-void put_signed_fc1(char *dst, float *sabs, size_t stride, const float *w, const float *s, const float *t, int m, int d) {
+// scale too small to divide by leaves the constant LeakyReLU(t).  A slope above 1 is turned into one below: LeakyReLU(x) is then
+// -slope max(-x, -x / slope), so rows and shift change their sign and -slope goes with |s|; the kernel knows the larger-of form only.
+void put_signed_fc1(char *dst, float *sabs, size_t stride, const float *w, const float *s, const float *t, float slope, int m, int d) {
+    const float flip = slope > 1.f ? -1.f : 1.f, gain = slope > 1.f ? -slope : 1.f;
     __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(dst);
     float *shift = sabs + stride, *rowsum = shift + stride;
     for (int j = 0; j < m; ++j) {
         const bool tiny = std::fabs(s[j]) < 1e-20f;
-        const float sign = tiny ? 0.f : s[j] < 0.f ? -1.f : 1.f;
-        sabs[j] = tiny ? 1.f : std::fabs(s[j]);
-        shift[shift_place(j)] = t[j] / sabs[j];
+        const float sign = tiny ? 0.f : s[j] < 0.f ? -flip : flip;
+        const float size = tiny ? 1.f : std::fabs(s[j]);
+        sabs[j] = gain * size;
+        shift[shift_place(j)] = flip * t[j] / size;
         double sum = 0.0;
         for (int k = 0; k < d; ++k) {
             o[(size_t)j * d + k] = __float2bfloat16_rn(sign * w[(size_t)j * d + k]);
@@ -564,7 +567,7 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
             const size_t M32 = (M + 31) & ~(size_t)31;
             w = align_up(w + 3 * M32 * 4, 256);
             put_signed_fc1(&img[p.w1n], (float *)&img[p.sabs], M32, a.dec_w1.data(),
-                           (const float *)&img[p.dec_s], (const float *)&img[p.dec_t], (int)M, (int)D);
+                           (const float *)&img[p.dec_s], (const float *)&img[p.dec_t], a.slope, (int)M, (int)D);
         }
         p.enc_w1r = w;
         p.enc_w2r = p.enc_w1r + M * I * E;

@@ -22,11 +22,12 @@
 //
 // decode_latent_kernel.  A cluster of two CTAs walks two runs of consecutive tiles in step, one run per CTA; every
 // product is one tcgen05.mma.cta_group::2 of M = 256 (both tiles), so a weight slab crosses L2 -> shared memory once
-// per 256 tokens, half into each CTA.  Per tile, K side then V side, per source layer, per chunk of 192 hidden columns:
+// per 256 tokens, half into each CTA.  Per step the K side of a tile, then the V side of the tile before (so that the way from S to
+// the probabilities is behind the next scores' products), per source layer, per chunk of 192 hidden columns:
 //   hidden   H[256 tok x 192] = Z[256 tok x d] . W1[192 x d]^T into one of two accumulators in tensor memory; the hidden
 //            warps add the shift, apply LeakyReLU, round to bf16 and write 64-column slabs into a ring.  The BatchNorm
 //            scale is not theirs: its sign is in W1, its size in W4^T q and in the merge (LeakyReLU is positively
-//            homogeneous).  The accumulator is read in matrix-fragment layout: a lane needs eight shifts instead of 32
+//            homogeneous; a slope above 1 is turned round on the host).  The accumulator is read in matrix-fragment layout: a lane needs eight shifts instead of 32
 //            (scale and shift fetched per column took 750-900 of a slab's 1 300 cycles) and stores with stmatrix.
 //   K side   S[256 tok x 2R] += slab . (W4^T q rows)^T, over all sources: rows of heads that another source serves are
 //            zero, so the sources simply add up.  Columns R r .. belong to CTA r (its own sequence's queries)
@@ -42,6 +43,13 @@
 // which leaves 64 KB for hidden slabs and 48 KB for weight slabs; 192 columns per chunk because 2 x 192 + 2 x 64 fill
 // tensor memory.
 //
+// Instruction fetch is the other bound: 24 warps run five programs, and with every wait's time limit inlined, U's blocks unrolled and
+// two forms of the epilogue the kernel was 88 KB of code, of whose instruction-cache requests 18 % missed (trivial stretches took 300
+// cycles).  Waiting is a function now, loops are kept as loops, the epilogue has one form: 61 KB.  With the accumulator given back
+// before the ring is waited for, one wait for all of a job's places, and four to twelve query slabs in flight instead of two or three
+// (the shifts come through L1), 12-layer steps: GPT-2 8 x 1024 tokens 649 -> 609 us, TinyLLaMA (22 layers) 4 x 32768 1800 -> 1711,
+// 32 x 2048 1264 -> 1215.
+//
 // Two warps issue products, one the hidden jobs, one S and U: with a single issuing thread the two took turns (6 800
 // cycles per chunk, 2 700 of them pipe time), and each waited for what only the other needed.  A warp of the hidden
 // epilogue takes one slab of a job (three slabs, four lane quarters: twelve warps).
@@ -52,7 +60,7 @@
 // has some of its zero-point left over, that times the weights' row sum: nothing is rounded that the fp32 form does not round.  12-layer step of the GPT-2 shape,
 // 8 x 1024 tokens: 973 us, 6404 us in fp32 on the CUDA cores.
 //
-// Warp roles: 0 loads of latents, query rows and shifts, 1 hidden products (leader CTA) and tensor memory, 2 weight loads,
+// Warp roles: 0 loads of latents and query rows, 1 hidden products (leader CTA) and tensor memory, 2 weight loads,
 // 3 S and U products (leader CTA), 4-15 hidden warps, 16-23 output warps.  All waits are bounded and record a code in the
 // status word.
 #include <algorithm>
@@ -98,22 +106,19 @@ struct Params {
     float *upart, *ml;
     int32_t max_pages_per_seq, page_tokens;
     int32_t hq, m_pad, wq_batch;
-    int32_t nz, nh, nw, nqs, nt, m_t;  // places for latent, hidden, weight and query slabs; shift buffers and their floats
-    int32_t t_resident;                // every source has a shift buffer of its own
+    int32_t nz, nh, nw, nqs;           // places for latent, hidden, weight and query slabs
     int32_t wide;                      // latents come from the widened rows of the launch's tiles
     int32_t two_terms_k, two_terms_v;  // low parts of the query rows / of the probabilities are used
 };
 
 constexpr int MODE_BOTH = 0, MODE_K = 1, MODE_V = 2;
 
-template <int SLEEP_NS = 0>
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int32_t *status, volatile int *abort_flag, int code) {
-    if (mbar_try(bar, parity)) return;
+// The waiting itself, out of line: some twenty waits with the time limit inlined made the tile kernel 80 KB of code, far more than
+// the instruction cache holds (see decode_latent_kernel).
+__device__ __noinline__ void mbar_wait_long(uint32_t bar, uint32_t parity, int32_t *status, volatile int *abort_flag, int code) {
     uint32_t n = 0;
     uint64_t t0 = 0;
-    while (true) {
-        if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
-        if (mbar_try(bar, parity)) return;
+    while (!mbar_try(bar, parity)) {
         if ((++n & 255u) == 0) {
             const uint64_t now = global_ns();
             if (t0 == 0) t0 = now;
@@ -124,6 +129,9 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int32_t
             }
         }
     }
+}
+__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int32_t *status, volatile int *abort_flag, int code) {
+    if (!mbar_try(bar, parity)) mbar_wait_long(bar, parity, status, abort_flag, code);
 }
 
 // the tiles of one CTA, in order
@@ -164,30 +172,34 @@ struct TileWalk {
     }
 };
 
+__device__ __noinline__ int pool_row(const int32_t *table, int page_tokens, int tok) {
+    return table[tok / page_tokens] * page_tokens + tok % page_tokens;
+}
 __device__ __forceinline__ float redux_max(float v) {
     float r;
     asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
 }
-// N values per lane (N = 6, 8 or 16): afterwards lane L holds the maximum over the warp of value L (L < N); halves the values
-// while it halves the lanes' distance, so about N shuffles instead of 5 N
-template <int N>
-__device__ __forceinline__ float max_over_lanes(const float *v, int lane) {
+// N values per lane (N = 6, 8 or 16): afterwards lane L holds the maximum (or the sum) over the warp of value L (L < N); halves
+// the values while it halves the lanes' distance, so about N shuffles instead of 5 N
+template <int N, bool SUM>
+__device__ __forceinline__ float over_lanes(const float *v, int lane) {
     constexpr int P = N <= 8 ? 8 : 16;
     float x[P];
+    auto fold = [](float a, float b) { return SUM ? a + b : fmaxf(a, b); };
 #pragma unroll
-    for (int i = 0; i < P; ++i) x[i] = i < N ? v[i] : -INFINITY;
+    for (int i = 0; i < P; ++i) x[i] = i < N ? v[i] : SUM ? 0.f : -INFINITY;
 #pragma unroll
     for (int w = P / 2; w > 0; w >>= 1) {
         const bool up = (lane & w) != 0;
 #pragma unroll
         for (int i = 0; i < w; ++i) {
             const float keep = up ? x[i + w] : x[i], give = up ? x[i] : x[i + w];
-            x[i] = fmaxf(keep, __shfl_xor_sync(0xffffffffu, give, w));
+            x[i] = fold(keep, __shfl_xor_sync(0xffffffffu, give, w));
         }
     }
 #pragma unroll
-    for (int w = P; w < 32; w <<= 1) x[0] = fmaxf(x[0], __shfl_xor_sync(0xffffffffu, x[0], w));
+    for (int w = P; w < 32; w <<= 1) x[0] = fold(x[0], __shfl_xor_sync(0xffffffffu, x[0], w));
     return x[0];
 }
 __device__ __forceinline__ float ex2(float x) {
@@ -195,18 +207,17 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-// `bytes` (a multiple of 16, both addresses 16-byte aligned) into this CTA's shared memory, counted on a barrier of it
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
-                 "r"(bytes), "r"(bar)
-                 : "memory");
-}
 __device__ __forceinline__ void stmatrix_x4(uint32_t addr, const uint32_t *w) {
     asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
                  : "memory");
 }
 __device__ __forceinline__ void st_smem_u16(uint32_t addr, uint16_t v) {
     asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(v) : "memory");
+}
+
+// *p = v if i < limit, without a branch
+__device__ __forceinline__ void st_global_below(float *p, float v, int i, int limit) {
+    asm volatile("{\n .reg .pred p;\n setp.lt.s32 p, %2, %3;\n @p st.global.f32 [%0], %1;\n}" ::"l"(p), "f"(v), "r"(i), "r"(limit) : "memory");
 }
 
 // what the warps share besides operands and barriers (everything is dynamic shared memory, so that the operand places
@@ -231,12 +242,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     const bool leader = rank == 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t s_z = smem_u32(smem_raw), s_h = s_z + a.nz * SLAB, s_w = s_h + a.nh * SLAB, s_q = s_w + a.nw * WSTAGE;
-    const uint32_t s_p = s_q + a.nqs * QSLAB, s_t = s_p + 2 * PSLAB, s_bar = s_t + a.nt * a.m_t * 4;
+    const uint32_t s_p = s_q + a.nqs * QSLAB, s_bar = s_p + 2 * PSLAB;
     const uint32_t w_full = s_bar, w_empty = w_full + 8 * a.nw;
     const uint32_t z_full = w_empty + 8 * a.nw, z_empty = z_full + 8 * a.nz;
     const uint32_t q_full = z_empty + 8 * a.nz, q_empty = q_full + 8 * a.nqs;
-    const uint32_t tb_full = q_empty + 8 * a.nqs, tb_empty = tb_full + 8 * a.nt;
-    const uint32_t h_ready = tb_empty + 8 * a.nt, h_free = h_ready + 8 * READY_BARS;
+    const uint32_t h_ready = q_empty + 8 * a.nqs, h_free = h_ready + 8 * READY_BARS;
     const uint32_t t_full = h_free + 8 * a.nh, t_empty = t_full + 16, o_full = t_empty + 16, o_empty = o_full + 16;
     const uint32_t p_ready = o_empty + 16;
     Scratch<NQ> &sh = *reinterpret_cast<Scratch<NQ> *>(smem_raw + (p_ready + 8 - s_z));
@@ -244,33 +254,42 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     // pair of runs, and which part of a side's hidden columns (one part unless the grid is small)
     const int pair = (int)(blockIdx.x >> 1) / a.n_parts, part = (int)(blockIdx.x >> 1) % a.n_parts;
     const int side_lo = a.mode == MODE_V ? 1 : 0, side_hi = a.mode == MODE_K ? 1 : 2;
-    auto list_of = [&](int side) -> const LatList & { return a.list[a.mode == MODE_BOTH ? side : part]; };
+    // (opaque to the compiler, as `lag` below: it would make two copies of every loop, one per mode)
+    int list0 = a.mode == MODE_BOTH ? 0 : part, list_step = a.mode == MODE_BOTH ? 1 : 0;
+    asm volatile("" : "+r"(list0), "+r"(list_step));
+    auto list_of = [&](int side) -> const LatList & { return a.list[list0 + side * list_step]; };
     // tiles of the cluster's longer run (the leader's); the other CTA idles through the last ones it does not have
     const int my_run = 2 * pair + (int)rank;
     const int n_it = max(0, min(a.sq.per, a.sq.n_tiles - 2 * pair * a.sq.per));
     const int my_first = my_run * a.sq.per;
+    // MODE_BOTH: in step `it` the K side of tile `it`, then the V side of the tile before
+    const int lag = list_step, n_steps = n_it > 0 ? n_it + lag : 0;
+    auto tile_of = [&](int it, int side) { return it - (side == 1 ? lag : 0); };
+    auto on = [&](int it, int side) { return tile_of(it, side) >= 0 && tile_of(it, side) < n_it; };
     launch_dependents();
 
     if (threadIdx.x == 0) {
         sh.abort_flag = 0;
+#pragma unroll 1
         for (int i = 0; i < a.nw; ++i) {
             mbar_init(w_full + 8 * i, 1);
             mbar_init(w_empty + 8 * i, 1);
         }
+#pragma unroll 1
         for (int i = 0; i < a.nz; ++i) {
             mbar_init(z_full + 8 * i, 1);
             mbar_init(z_empty + 8 * i, 1);
         }
+#pragma unroll 1
         for (int i = 0; i < a.nqs; ++i) {
             mbar_init(q_full + 8 * i, 1);
             mbar_init(q_empty + 8 * i, 1);
         }
-        for (int i = 0; i < a.nt; ++i) {
-            mbar_init(tb_full + 8 * i, 1);
-            mbar_init(tb_empty + 8 * i, N_HID);
-        }
+#pragma unroll 1
         for (int i = 0; i < a.nh; ++i) mbar_init(h_free + 8 * i, 1);
+#pragma unroll 1
         for (int i = 0; i < READY_BARS; ++i) mbar_init(h_ready + 8 * i, 2 * N_HID);
+#pragma unroll 1
         for (int i = 0; i < 2; ++i) {
             mbar_init(t_full + 8 * i, 1);
             mbar_init(t_empty + 8 * i, 2 * N_HID);
@@ -293,88 +312,83 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     const uint32_t tmem = sh.tmem_slot;
 
     if (warp == 0) {
-        // ============================== latents, query rows, shifts ==============================
-        // Three independent streams of loads, each into its own ring; one thread looks at the rings in turn and fills the
+        // ============================== latents, query rows ==============================
+        // Two independent streams of loads, each into its own ring; one thread looks at the rings in turn and fills the
         // one that has a place.
         if (elect_one()) {
             auto rows_of = [&](const TileWalk &t, int *r) {  // pool rows of the tile's two 64-token halves
                 r[0] = r[1] = 0;
                 const int v = t.valid(a.sq);
+                if (v == 0) return;
+                const int tok = t.chunk * TILE;
                 if (Q8) {  // widened rows lie in the order of the launch's tiles
-                    r[0] = v == 0 ? 0 : (t.first(a.sq, t.si) + t.chunk) * TILE;
+                    r[0] = (t.first(a.sq, t.si) + t.chunk) * TILE;
                     r[1] = r[0] + (v > 64 ? 64 : 0);
+                    return;
                 }
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    if (Q8 || v == 0) break;
-                    int tok = t.chunk * TILE + 64 * h;
-                    if (64 * h >= v) tok = t.chunk * TILE;  // no valid token there: re-read the first half
-                    const int page = a.block_table[(int64_t)a.sq.id[t.si] * a.max_pages_per_seq + tok / a.page_tokens];
-                    r[h] = page * a.page_tokens + tok % a.page_tokens;
-                }
+                const int32_t *table = a.block_table + (int64_t)a.sq.id[t.si] * a.max_pages_per_seq;
+                r[0] = pool_row(table, a.page_tokens, tok);
+                r[1] = v > 64 ? pool_row(table, a.page_tokens, tok + 64) : r[0];  // no valid token there: re-read the first half
             };
             struct Pos {
                 int it, side, s, k;
             };
-            Pos z{0, side_lo, 0, 0}, q{a.mode == MODE_V ? n_it : 0, 0, 0, 0}, t{0, side_lo, 0, 0};
+            Pos z{0, side_lo, 0, 0}, q{a.mode == MODE_V ? n_it : 0, 0, 0, 0};
             bool waited = false;  // for the launch before, which writes the query rows
-            uint32_t zslot = 0, zphase = 0, qslot = 0, qphase = 0, tslot = 0, tphase = 0;
+            uint32_t zslot = 0, zphase = 0, qslot = 0, qphase = 0;
             TileWalk zw, qw;
             zw.start(a.sq, my_first);
             qw = zw;
-            int row[2], nrow[2];
+            int prow[2] = {0, 0}, row[2], nrow[2] = {0, 0};  // of the tile before, of tile z.it, of the next
+            bool live = zw.left > 0, nlive = false;          // row, nrow are of a tile of this CTA
             rows_of(zw, row);
             const bool low_k = NQ <= 16 || a.two_terms_k;
-            const int t_its = a.t_resident ? min(1, n_it) : n_it;
             uint32_t idle = 0;
             uint64_t t0 = 0;
-            while (z.it < n_it || q.it < n_it || t.it < t_its) {
+            while (z.it < n_steps || q.it < n_it) {
                 bool moved = false;
-                if (z.it < n_it && mbar_test(z_empty + 8 * zslot, zphase ^ 1u)) {
+                if (z.it < n_steps && mbar_test(z_empty + 8 * zslot, zphase ^ 1u)) {
                     moved = true;
                     if (leader) mbar_expect_tx(z_full + 8 * zslot, 2 * SLAB);
                     const LatSrc &zp_ = list_of(z.side).src[z.s];
                     const CUtensorMap *map = &a.pool[z.side][zp_.map];
                     const uint32_t fb = map_to_cta(z_full + 8 * zslot, 0), dst = s_z + zslot * SLAB;
-                    tma_load_2d_pair(dst, map, z.k * 64, row[0], fb);
-                    tma_load_2d_pair(dst + SLAB / 2, map, z.k * 64, row[1], fb);
+                    const bool behind = tile_of(z.it, z.side) < z.it;  // the tile before
+                    tma_load_2d_pair(dst, map, z.k * 64, behind ? prow[0] : row[0], fb);
+                    tma_load_2d_pair(dst + SLAB / 2, map, z.k * 64, behind ? prow[1] : row[1], fb);
                     if (++zslot == (uint32_t)a.nz) { zslot = 0; zphase ^= 1u; }
                     const int ks1 = (zp_.d + 63) >> 6;
                     if (++z.k == ks1) {
-                        // the same rows of the next tile: from HBM into L2 while this one is worked on
+                        // the same rows of the tile after: from HBM into L2 while this one is worked on
                         if (z.side == side_lo && z.s == 0) {
                             zw.next(a.sq);
                             rows_of(zw, nrow);
+                            nlive = zw.left > 0;
                         }
-                        if (zw.left > 0)
+                        if (behind ? live : nlive) {
+                            const int r0 = behind ? row[0] : nrow[0], r1 = behind ? row[1] : nrow[1];
+#pragma unroll 1
                             for (int ks = 0; ks < ks1; ++ks) {
-                                tma_prefetch_2d(map, ks * 64, nrow[0]);
-                                if (nrow[1] != nrow[0]) tma_prefetch_2d(map, ks * 64, nrow[1]);
+                                tma_prefetch_2d(map, ks * 64, r0);
+                                if (r1 != r0) tma_prefetch_2d(map, ks * 64, r1);
                             }
+                        }
                         z.k = 0;
                         if (++z.s == list_of(z.side).n) {
                             z.s = 0;
-                            if (++z.side == side_hi) {
-                                z.side = side_lo;
-                                ++z.it;
-                                row[0] = nrow[0];
-                                row[1] = nrow[1];
-                            }
-                        }
-                    }
-                }
-                if (t.it < t_its && mbar_test(tb_empty + 8 * tslot, tphase ^ 1u)) {
-                    moved = true;
-                    const LatSrc &sp = list_of(t.side).src[t.s];
-                    const uint32_t bytes = (uint32_t)((sp.m + 31) & ~31) * 4u;
-                    mbar_expect_tx(tb_full + 8 * tslot, bytes);
-                    bulk_load(s_t + tslot * a.m_t * 4, sp.shift, bytes, tb_full + 8 * tslot);
-                    if (++tslot == (uint32_t)a.nt) { tslot = 0; tphase ^= 1u; }
-                    if (++t.s == list_of(t.side).n) {
-                        t.s = 0;
-                        if (++t.side == side_hi) {
-                            t.side = side_lo;
-                            ++t.it;
+                            do {
+                                if (++z.side == side_hi) {
+                                    z.side = side_lo;
+                                    ++z.it;
+#pragma unroll
+                                    for (int h = 0; h < 2; ++h) {
+                                        prow[h] = row[h];
+                                        row[h] = nrow[h];
+                                    }
+                                    live = nlive;
+                                    nlive = false;
+                                }
+                            } while (z.it < n_steps && !on(z.it, z.side));
                         }
                     }
                 }
@@ -422,16 +436,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         // ============================== weight loads ==============================
         if (elect_one()) {
             uint32_t slot = 0, phase = 0;
-            for (int it = 0; it < n_it; ++it)
+#pragma unroll 1
+            for (int it = 0; it < n_steps; ++it)
+#pragma unroll 1
                 for (int side = side_lo; side < side_hi; ++side)
-                    for (int s = 0; s < list_of(side).n; ++s) {
+#pragma unroll 1
+                    for (int s = 0; s < (on(it, side) ? list_of(side).n : 0); ++s) {
                         const LatSrc &sp = list_of(side).src[s];
                         const int ks1 = (sp.d + 63) >> 6, m = sp.m;
                         const CUtensorMap *map = &a.w1[side][sp.map];
+#pragma unroll 1
                         for (int c0 = 0; c0 < m; c0 += CN) {
                             const int y = sp.c0 + c0 + (int)rank * (min(CN, m - c0) >> 1);
+#pragma unroll 1
                             for (int ks = 0; ks < ks1; ++ks) {
-                                mbar_wait<32>(w_empty + 8 * slot, phase ^ 1u, a.status, &abort_flag, 0x602);
+                                mbar_wait(w_empty + 8 * slot, phase ^ 1u, a.status, &abort_flag, 0x602);
                                 if (leader) mbar_expect_tx(w_full + 8 * slot, 2 * WSTAGE);
                                 tma_load_2d_pair(s_w + slot * WSTAGE, map, ks * 64, y, map_to_cta(w_full + 8 * slot, 0));
                                 if (++slot == (uint32_t)a.nw) { slot = 0; phase ^= 1u; }
@@ -444,12 +463,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         if (leader && elect_one()) {
             uint32_t wslot = 0, wphase = 0, zslot = 0, zphase = 0, h = 0;
             const uint64_t z_desc = make_desc(s_z), w_desc = make_desc(s_w);
-            for (int it = 0; it < n_it; ++it)
+#pragma unroll 1
+            for (int it = 0; it < n_steps; ++it)
+#pragma unroll 1
                 for (int side = side_lo; side < side_hi; ++side)
-                    for (int s = 0; s < list_of(side).n; ++s) {
+#pragma unroll 1
+                    for (int s = 0; s < (on(it, side) ? list_of(side).n : 0); ++s) {
                         const int d = list_of(side).src[s].d, m = list_of(side).src[s].m;
                         const int ks1 = (d + 63) >> 6, nk_last = ((d - 1) & 63) / 16 + 1;
                         uint32_t zs = 0, zp = 0;
+#pragma unroll 1
                         for (int c0 = 0; c0 < m; c0 += CN, ++h) {
                             const bool first = c0 == 0, last = c0 + CN >= m;
                             const uint32_t buf = h & 1u, acc = tmem + CN * buf, idesc = make_idesc(256, min(CN, m - c0));
@@ -471,6 +494,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                                     umma_pair<1>(acc, da + 4u, db + 4u, idesc);
                                     umma_pair<1>(acc, da + 6u, db + 6u, idesc);
                                 } else {
+#pragma unroll 1
                                     for (int t = 1; t < nk_last; ++t) umma_pair<1>(acc, da + 2u * t, db + 2u * t, idesc);
                                 }
                                 umma_commit_pair(w_empty + 8 * wslot);
@@ -492,11 +516,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             constexpr uint32_t idesc_u = idesc | (1u << 15);  // row operand MN-major
             const uint64_t h_desc = make_desc(s_h), q_desc = make_desc(s_q), p_desc = make_desc(s_p);
             const bool two = NQ > 16 && a.two_terms_k;
-            for (int it = 0; it < n_it; ++it) {
-                if (side_lo == 0) {  // S
+#pragma unroll 1
+            for (int it = 0; it < n_steps; ++it) {
+                if (side_lo == 0 && on(it, 0)) {  // S
                     const uint32_t ob = o & 1u, acc = tmem + TM_OUT + 64u * ob;
                     mbar_wait(o_empty + 8 * ob, ((o >> 1) & 1u) ^ 1u, a.status, &abort_flag, 0x605);
                     bool begin = true;
+#pragma unroll 1
                     for (int s = 0; s < list_of(0).n; ++s) {
                         const int m = list_of(0).src[s].m, ksm = (m + 63) >> 6, nk_last = ((m - 1) & 63) / 16 + 1;
 #pragma unroll 1
@@ -535,7 +561,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                     ++o;
                 }
                 bool p_seen = false;
-                for (int s = 0; s < (side_hi == 2 ? list_of(1).n : 0); ++s) {  // U
+#pragma unroll 1
+                for (int s = 0; s < (side_hi == 2 && on(it, 1) ? list_of(1).n : 0); ++s) {  // U
                     const int ksm = (list_of(1).src[s].m + 63) >> 6;
                     hslot += hslot & 1u;  // slabs go in pairs: a source starts at an even place
                     if (hslot == (uint32_t)a.nh) hslot = 0;
@@ -551,7 +578,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                         if (++hslot == (uint32_t)a.nh) hslot = 0;
                         if (!(sl & 1) && sl + 1 < ksm) continue;
                         if (!p_seen) {
-                            mbar_wait(p_ready, (uint32_t)it & 1u, a.status, &abort_flag, 0x606);
+                            mbar_wait(p_ready, (uint32_t)tile_of(it, 1) & 1u, a.status, &abort_flag, 0x606);
                             p_seen = true;
                         }
                         const uint32_t ob = o & 1u, accu = tmem + TM_OUT + 64u * ob, h0 = hs & ~1u;
@@ -580,18 +607,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         // where this lane's row of the 8 x 8 blocks goes (row lane % 8 of 8, block lane / 8 of 4; 128-byte swizzle)
         const uint32_t st_row = (lane_base + (lane & 7)) * 128u;
         const uint32_t ready_leader = map_to_cta(h_ready, 0), empty_leader = map_to_cta(t_empty, 0);
-        uint32_t hslot = 0, hphase = 0, h = 0, tb = 0, tphase = 0;
+        uint32_t hslot = 0, hphase = 0, h = 0;
         TileWalk tw;
         tw.start(a.sq, my_first);
-        for (int it = 0; it < n_it; ++it, tw.next(a.sq)) {
-            const int valid = tw.valid(a.sq);
+        auto wide_row = [&]() { return !Q8 || tw.left == 0 ? 0 : (tw.first(a.sq, tw.si) + tw.chunk) * TILE; };
+        int k_valid = tw.valid(a.sq), k_row = wide_row(), v_valid = k_valid, v_row = k_row;  // of the K and of the V side's tile
+#pragma unroll 1
+        for (int it = 0; it < n_steps; ++it) {
+#pragma unroll 1
             for (int side = side_lo; side < side_hi; ++side) {
+                if (!on(it, side)) continue;
+                const int valid = side == 0 ? k_valid : v_valid;
                 const int n_src = list_of(side).n;
+#pragma unroll 1
                 for (int s = 0; s < n_src; ++s) {
                     const int m = list_of(side).src[s].m;
                     const float slope = list_of(side).src[s].slope;
                     const float2 slope2 = make_float2(slope, slope);
-                    const bool lr_max = slope <= 1.f;
                     // V side: rows past the tile's end may hold anything, and zero times a stray NaN is not zero
                     const bool clear = side == 1 && valid < TILE;
                     if (side == 1) {
@@ -601,7 +633,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                     float inv[4] = {1.f, 1.f, 1.f, 1.f}, left[4] = {0.f, 0.f, 0.f, 0.f};  // int8 rows: this lane's four tokens
                     bool any_left = false;
                     if (Q8) {
-                        const int r0 = valid == 0 ? 0 : (tw.first(a.sq, tw.si) + tw.chunk) * TILE;
+                        const int r0 = side == 0 ? k_row : v_row;
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
                             const int r = (int)lane_base + 8 * i + (lane >> 2);
@@ -614,78 +646,108 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                         }
                         any_left = __any_sync(0xffffffffu, any_left);
                     }
-                    const float *tbuf = reinterpret_cast<const float *>(smem_raw + (s_t - s_z)) + tb * a.m_t;
-                    if (it == 0 || !a.t_resident) mbar_wait(tb_full + 8 * tb, tphase, a.status, &abort_flag, 0x60f);
+                    const float *shift = list_of(side).src[s].shift;
+#pragma unroll 1
                     for (int c0 = 0; c0 < m; c0 += CN, ++h) {
                         const int nc = min(CN, m - c0);
                         const uint32_t buf = h & 1u, acc = tmem + CN * buf + (lane_base << 16);
+                        const int col0 = 64 * my_slab, halves = col0 >= nc ? 0 : col0 + 32 >= nc ? 1 : 2;
+                        const float4 *t4 = reinterpret_cast<const float4 *>(shift + c0 + col0) + 2 * (lane & 3);
+                        float4 ta = make_float4(0.f, 0.f, 0.f, 0.f), tb = ta;
+                        if (halves > 0) {
+                            ta = __ldg(t4);
+                            tb = __ldg(t4 + 1);
+                        }
                         mbar_wait(t_full + 8 * buf, (h >> 1) & 1u, a.status, &abort_flag, 0x609);
                         __syncwarp();
                         tc_fence_after();
-                        // The job's places in the ring.  A warp writes one of them but sees every one free: a phase that it
-                        // skipped would let a later wait on the same place pass one phase early.
-                        uint32_t slot = 0;
-                        bool mine = false;
-                        for (int sl = 0; 64 * sl < nc; ++sl) {
-                            if (sl == my_slab) {
-                                mine = true;
-                                slot = hslot;
-                            }
-                            mbar_wait(h_free + 8 * hslot, ((hphase >> hslot) & 1u) ^ 1u, a.status, &abort_flag, 0x60a);
-                            hphase ^= 1u << hslot;
-                            if (++hslot == (uint32_t)a.nh) hslot = 0;
-                        }
-                        __syncwarp();
-                        if (mine) {
+                        // The accumulator is read, and given back, before the job's places in the ring are free: the next
+                        // hidden products do not wait for the products that still read those places.
+                        uint32_t w[2][16];
 #pragma unroll
-                            for (int half = 0; half < 2; ++half) {
-                                const int col = 64 * my_slab + 32 * half;
-                                if (col < nc) {
-                                    const float4 *t4 = reinterpret_cast<const float4 *>(tbuf + c0 + col) + 2 * (lane & 3);
-                                    const float4 ta = t4[0], tb4 = t4[1];
-                                    const float2 t[4] = {make_float2(ta.x, ta.y), make_float2(ta.z, ta.w), make_float2(tb4.x, tb4.y),
-                                                         make_float2(tb4.z, tb4.w)};
-                                    uint32_t r[2][16];
-                                    tmem_ld_frag_x4(acc + (uint32_t)col, r[0]);
-                                    tmem_ld_frag_x4(acc + (16u << 16) + (uint32_t)col, r[1]);
-                                    tmem_ld_wait();
-                                    const uint32_t dst = s_h + slot * SLAB + st_row + (uint32_t)(((4 * half + (lane >> 3)) ^ (lane & 7)) << 4);
+                        for (int u = 0; u < 4; ++u) {  // 32 columns (u / 2) x 16 of the warp's 32 rows (u % 2)
+                            const int half = u >> 1, f = u & 1;
+                            if (half < halves) {
+                                uint32_t r[16];
+                                tmem_ld_frag_x4(acc + (uint32_t)f * (16u << 16) + (uint32_t)(col0 + 32 * half), r);
+                                if (u == 2) {
+                                    ta = __ldg(t4 + 8);
+                                    tb = __ldg(t4 + 9);
+                                }
+                                const float2 t[4] = {make_float2(ta.x, ta.y), make_float2(ta.z, ta.w), make_float2(tb.x, tb.y),
+                                                     make_float2(tb.z, tb.w)};
+                                tmem_ld_wait();
+                                if (f == 1 && half + 1 == halves) {
+                                    tc_fence_before();
+                                    __syncwarp();
+                                    if (elect_one()) mbar_arrive_remote(empty_leader + 8 * buf);
+                                }
+                                if (Q8 && any_left) {
 #pragma unroll
-                                    for (int i = 0; i < 4; ++i) {  // rows 8 i .. of the warp's 32
-                                        uint32_t w[4];
-#pragma unroll
-                                        for (int j = 0; j < 4; ++j) {
-                                            float2 h2 = make_float2(__uint_as_float(r[i >> 1][4 * j + 2 * (i & 1)]),
-                                                                    __uint_as_float(r[i >> 1][4 * j + 2 * (i & 1) + 1]));
-                                            if (Q8 && any_left) {
-                                                const float2 rs = __ldg(reinterpret_cast<const float2 *>(list_of(side).src[s].rowsum + c0 + col) +
-                                                                        4 * (lane & 3) + j);
-                                                h2 = __ffma2_rn(make_float2(-left[i], -left[i]), rs, h2);
-                                            }
-                                            const float2 x = Q8 ? __ffma2_rn(h2, make_float2(inv[i], inv[i]), t[j]) : __fadd2_rn(h2, t[j]);
-                                            const float2 y = __fmul2_rn(x, slope2);
-                                            // LeakyReLU: the larger of x and slope*x for slope <= 1, the smaller for slope > 1
-                                            w[j] = lr_max ? pack_bf16(fmaxf(x.x, y.x), fmaxf(x.y, y.y))
-                                                          : pack_bf16(fminf(x.x, y.x), fminf(x.y, y.y));
-                                            if (clear && (int)lane_base + 8 * i + (lane >> 2) >= valid) w[j] = 0u;
-                                        }
-                                        stmatrix_x4(dst + 1024u * i, w);
+                                    for (int e = 0; e < 8; ++e) {
+                                        const int i = e >> 2, j = e & 3;
+                                        const float2 rs = __ldg(reinterpret_cast<const float2 *>(list_of(side).src[s].rowsum + c0 + col0 + 32 * half) +
+                                                                4 * (lane & 3) + j);
+                                        r[4 * j + 2 * i] = __float_as_uint(fmaf(-left[2 * f + i], rs.x, __uint_as_float(r[4 * j + 2 * i])));
+                                        r[4 * j + 2 * i + 1] = __float_as_uint(fmaf(-left[2 * f + i], rs.y, __uint_as_float(r[4 * j + 2 * i + 1])));
                                     }
+                                }
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) {  // rows 8 (e / 4) .. of the 16
+                                    const int i = e >> 2, j = e & 3;
+                                    const float2 h2 = make_float2(__uint_as_float(r[4 * j + 2 * i]), __uint_as_float(r[4 * j + 2 * i + 1]));
+                                    const float iv = inv[2 * f + i];
+                                    const float2 x = Q8 ? __ffma2_rn(h2, make_float2(iv, iv), t[j]) : __fadd2_rn(h2, t[j]);
+                                    const float2 y = __fmul2_rn(x, slope2);
+                                    w[half][8 * f + e] = pack_bf16(fmaxf(x.x, y.x), fmaxf(x.y, y.y));  // slope <= 1
                                 }
                             }
                         }
-                        tc_fence_before();
+                        if (clear) {
+#pragma unroll
+                            for (int e = 0; e < 32; ++e)
+                                if ((int)lane_base + 8 * ((e & 15) >> 2) + (lane >> 2) >= valid) w[e >> 4][e & 15] = 0u;
+                        }
+                        if (halves == 0) {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (elect_one()) mbar_arrive_remote(empty_leader + 8 * buf);
+                        }
+                        // The job's places in the ring.  A warp writes one of them but sees every one free: a phase that it
+                        // skipped would let a later wait on the same place pass one phase early.
+                        // One lane per place.
+                        const int n_sl = (nc + 63) >> 6;
+                        const uint32_t nh = (uint32_t)a.nh, place = hslot + lane < nh ? hslot + lane : hslot + lane - nh;
+                        if (lane < n_sl) mbar_wait(h_free + 8 * place, ((hphase >> place) & 1u) ^ 1u, a.status, &abort_flag, 0x60a);
+                        const uint32_t slot = hslot + my_slab < nh ? hslot + my_slab : hslot + my_slab - nh;
+                        const uint32_t passed = ((1u << n_sl) - 1u) << hslot;
+                        hphase ^= (passed | passed >> nh) & ((1u << nh) - 1u);
+                        hslot = hslot + n_sl < nh ? hslot + n_sl : hslot + n_sl - nh;
+                        __syncwarp();
+                        const uint32_t dst = s_h + slot * SLAB + st_row;
+#pragma unroll
+                        for (int half = 0; half < 2; ++half)
+                            if (half < halves) {
+#pragma unroll
+                                for (int i = 0; i < 4; ++i)
+                                    stmatrix_x4(dst + (uint32_t)(((4 * half + (lane >> 3)) ^ (lane & 7)) << 4) + 1024u * i, w[half] + 4 * i);
+                            }
                         fence_async_smem();
                         __syncwarp();
-                        if (elect_one()) {
-                            mbar_arrive_remote(empty_leader + 8 * buf);
-                            mbar_arrive_remote(ready_leader + 8 * (h & 7u));
-                        }
+                        if (elect_one()) mbar_arrive_remote(ready_leader + 8 * (h & 7u));
                     }
-                    __syncwarp();
-                    if (!a.t_resident && elect_one()) mbar_arrive_local(tb_empty + 8 * tb);
-                    if (++tb == (uint32_t)a.nt || (a.t_resident && side + 1 == side_hi && s + 1 == n_src)) { tb = 0; tphase ^= 1u; }
                 }
+            }
+            if (lag) {
+                v_valid = k_valid;
+                v_row = k_row;
+            }
+            tw.next(a.sq);
+            k_valid = tw.valid(a.sq);
+            k_row = wide_row();
+            if (!lag) {
+                v_valid = k_valid;
+                v_row = k_row;
             }
         }
     } else {
@@ -700,13 +762,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         const uint32_t col = TM_OUT + R * rank + NT * half;
         const int q0 = NT * half;
         const bool low_v = a.two_terms_v != 0;
-        float acc[NB][NT], l[NT];
+        float acc[NB][NT], l = 0.f;  // l: lane q, this warp's part of head q0 + q's sum
 #pragma unroll
-        for (int q = 0; q < NT; ++q) {
-            l[q] = 0.f;
+        for (int q = 0; q < NT; ++q)
 #pragma unroll
             for (int b = 0; b < NB; ++b) acc[b][q] = 0.f;
-        }
         uint32_t o = 0;
         auto half_sync = [&]() {  // the four warps of this half
             if (half == 0)
@@ -731,123 +791,139 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
 #pragma unroll
             for (int q = 0; q < NT; ++q) v[q] = NQ <= 16 ? r[q] + r[8 + q] : r[q];  // the low terms have columns of their own
         };
+        // probabilities of the tile whose scores are s
+        auto probabilities = [&](float *s, int valid, int par) {
+#pragma unroll
+            for (int q = 0; q < NT; ++q)
+                if (row >= valid) s[q] = -INFINITY;
+            const float keep = over_lanes<NT, false>(s, lane);
+            if (lane < NT) sh.red[par][q0 + lane][quarter] = keep;
+            half_sync();
+            // reference maxima: one head per lane, then broadcast by shuffles of the few values that follow from them
+            float m_new = 0.f, f = 1.f;
+            if (lane < NT) {
+                const float *r = sh.red[par][q0 + lane];
+                const float m_old = sh.mrun[par][q0 + lane];
+                m_new = fmaxf(m_old, fmaxf(fmaxf(r[0], r[1]), fmaxf(r[2], r[3])));
+                if (m_new != m_old) f = ex2(m_old - m_new);
+                if (quarter == 0) sh.mrun[par ^ 1][q0 + lane] = m_new;
+            }
+            const uint32_t t6 = row & 63;
+            const uint32_t pbase = s_p + (uint32_t)(row >> 6) * PSLAB + (t6 & 7u) * 2u;
+#pragma unroll
+            for (int q = 0; q < NT; ++q) {
+                const float mq = __shfl_sync(0xffffffffu, m_new, q);
+                const float p = valid > 0 ? ex2(s[q] - mq) : 0.f;
+                s[q] = p;
+                // operand row q0 + q, token t6 of atom row >> 6 (K-major, 128-byte swizzle)
+                const uint32_t qr = q0 + q;
+                const __nv_bfloat16 hi = __float2bfloat16_rn(p);
+                st_smem_u16(pbase + qr * 128u + (((t6 >> 3) ^ (qr & 7u)) << 4), __bfloat16_as_ushort(hi));
+                if (NQ <= 16) {
+                    const uint32_t ql = qr + NQ;
+                    const __nv_bfloat16 lo = __float2bfloat16_rn(low_v ? p - __bfloat162float(hi) : 0.f);
+                    st_smem_u16(pbase + ql * 128u + (((t6 >> 3) ^ (ql & 7u)) << 4), __bfloat16_as_ushort(lo));
+                }
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (elect_one()) mbar_arrive_remote(pready_leader);
+            // the running sums, while the products run
+            l = l * f + over_lanes<NT, true>(s, lane);
+            if (__any_sync(0xffffffffu, f != 1.f)) {
+#pragma unroll
+                for (int q = 0; q < NT; ++q) {
+                    const float fq = __shfl_sync(0xffffffffu, f, q);
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) acc[b][q] *= fq;
+                }
+            }
+        };
         TileWalk tw;
         tw.start(a.sq, my_first);
-        for (int it = 0; it < n_it; ++it, tw.next(a.sq)) {
-            const int valid = tw.valid(a.sq), par = it & 1;
+        int u_si = 0;          // the tile whose U comes next: its sequence, and whether it ends the run
+        bool u_ends = false;
+        // in step `it` the scores of tile `it`, U of the tile before, then the probabilities of tile `it`
+#pragma unroll 1
+        for (int it = 0; it <= n_it; ++it) {
             float s[NT];
-            if (a.mode != MODE_V) {
+            if (it < n_it && a.mode != MODE_V) {
                 fetch(s);
-            } else {
+            } else if (it < n_it) {
                 if (it == 0) grid_dependency_wait();  // the launch before holds the scores
 #pragma unroll
                 for (int q = 0; q < NT; ++q) s[q] = 0.f;
-                for (int p = 0; p < a.k_parts; ++p) {
-                    const float *sp = a.score + ((int64_t)((pair * a.k_parts + p) * 2 + (int)rank) * NQ + q0) * TILE + row;
+                const float *sp = a.score + ((int64_t)(pair * a.k_parts * 2 + (int)rank) * NQ + q0) * TILE + row;
+#pragma unroll 4
+                for (int p = 0; p < a.k_parts; ++p, sp += 2 * NQ * TILE) {
 #pragma unroll
                     for (int q = 0; q < NT; ++q) s[q] += sp[q * TILE];
                 }
             }
             if (a.mode == MODE_K) {  // one cluster's part of the sums over the hidden columns
+                if (it == n_it) break;
                 float *sp = a.score + ((int64_t)blockIdx.x * NQ + q0) * TILE + row;
 #pragma unroll
                 for (int q = 0; q < NT; ++q) sp[q * TILE] = s[q];
                 continue;
             }
-            {
-#pragma unroll
-                for (int q = 0; q < NT; ++q)
-                    if (row >= valid) s[q] = -INFINITY;
-                const float keep = max_over_lanes<NT>(s, lane);
-                if (lane < NT) sh.red[par][q0 + lane][quarter] = keep;
-                half_sync();
-                // reference maxima: one head per lane, then broadcast by shuffles of the few values that follow from them
-                float m_new = 0.f, f = 1.f;
-                if (lane < NT) {
-                    const float *r = sh.red[par][q0 + lane];
-                    const float m_old = sh.mrun[par][q0 + lane];
-                    m_new = fmaxf(m_old, fmaxf(fmaxf(r[0], r[1]), fmaxf(r[2], r[3])));
-                    if (m_new != m_old) f = ex2(m_old - m_new);
-                    if (quarter == 0) sh.mrun[par ^ 1][q0 + lane] = m_new;
-                }
-                if (__any_sync(0xffffffffu, f != 1.f)) {
-#pragma unroll
-                    for (int q = 0; q < NT; ++q) {
-                        const float fq = __shfl_sync(0xffffffffu, f, q);
-                        l[q] *= fq;
-#pragma unroll
-                        for (int b = 0; b < NB; ++b) acc[b][q] *= fq;
-                    }
-                }
-                const uint32_t t6 = row & 63;
-                const uint32_t pbase = s_p + (uint32_t)(row >> 6) * PSLAB + (t6 & 7u) * 2u;
-#pragma unroll
-                for (int q = 0; q < NT; ++q) {
-                    const float mq = __shfl_sync(0xffffffffu, m_new, q);
-                    const float p = valid > 0 ? ex2(s[q] - mq) : 0.f;
-                    l[q] += p;
-                    // operand row q0 + q, token t6 of atom row >> 6 (K-major, 128-byte swizzle)
-                    const uint32_t qr = q0 + q;
-                    const __nv_bfloat16 hi = __float2bfloat16_rn(p);
-                    st_smem_u16(pbase + qr * 128u + (((t6 >> 3) ^ (qr & 7u)) << 4), __bfloat16_as_ushort(hi));
-                    if (NQ <= 16) {
-                        const uint32_t ql = qr + NQ;
-                        const __nv_bfloat16 lo = __float2bfloat16_rn(low_v ? p - __bfloat162float(hi) : 0.f);
-                        st_smem_u16(pbase + ql * 128u + (((t6 >> 3) ^ (ql & 7u)) << 4), __bfloat16_as_ushort(lo));
-                    }
-                }
-                fence_async_smem();
-                __syncwarp();
-                if (elect_one()) mbar_arrive_remote(pready_leader);
-            }
-            for (int si = 0; si < list_of(1).n; ++si) {
+#pragma unroll 1
+            for (int si = 0; si < (it > 0 ? list_of(1).n : 0); ++si) {
                 const int n_blk = (((list_of(1).src[si].m + 63) >> 6) + 1) >> 1;
                 const uint32_t mask = list_of(1).src[si].mask >> q0;
+#pragma unroll 1
+                for (int blk = 0; blk < n_blk; ++blk) {
+                    float u[NT];
+                    fetch(u);
 #pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    if (b < n_blk) {
-                        float u[NT];
-                        fetch(u);
+                    for (int q = 0; q < NT; ++q)
+                        if (!((mask >> q) & 1u)) u[q] = 0.f;
 #pragma unroll
-                        for (int q = 0; q < NT; ++q)
-                            if ((mask >> q) & 1u) acc[b][q] += u[q];
-                    }
+                    for (int b = 0; b < NB; ++b)
+                        if (b == blk) {
+#pragma unroll
+                            for (int q = 0; q < NT; ++q) acc[b][q] += u[q];
+                        }
                 }
             }
-            if (tw.ends_run()) {
-                const int64_t run = (int64_t)my_run + tw.si;  // run and sequence only ever grow along the runs: unique
+            if (u_ends) {
+                const int64_t run = (int64_t)my_run + u_si;  // run and sequence only ever grow along the runs: unique
+#pragma unroll 1
                 for (int si = 0; si < list_of(1).n; ++si) {
-                    const int m = list_of(1).src[si].m;
+                    const int m_left = list_of(1).src[si].m - row;
                     const uint32_t mask = list_of(1).src[si].mask >> q0;
                     float *u = a.upart + (run * a.hq + q0) * a.m_pad + list_of(1).src[si].c0 + row;
 #pragma unroll
-                    for (int b = 0; b < NB; ++b)
+                    for (int q = 0; q < NT; ++q, u += a.m_pad) {
+                        const int limit = (mask >> q) & 1u ? m_left : 0;
 #pragma unroll
-                        for (int q = 0; q < NT; ++q)
-                            if (((mask >> q) & 1u) && 128 * b + row < m) u[(int64_t)q * a.m_pad + 128 * b] = acc[b][q];
+                        for (int b = 0; b < NB; ++b) st_global_below(u + 128 * b, acc[b][q], 128 * b, limit);
+                    }
                 }
-                float keep = 0.f;
 #pragma unroll
-                for (int q = 0; q < NT; ++q) {
-                    float v = l[q];
-#pragma unroll
-                    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-                    if (lane == q) keep = v;
-                    l[q] = 0.f;
+                for (int q = 0; q < NT; ++q)
 #pragma unroll
                     for (int b = 0; b < NB; ++b) acc[b][q] = 0.f;
-                }
-                if (lane < NT) sh.lred[q0 + lane][quarter] = keep;
+                if (lane < NT) sh.lred[q0 + lane][quarter] = l;
+                l = 0.f;
                 half_sync();
                 if (quarter == 0 && lane < NT) {
+                    float *m_run = &sh.mrun[it & 1][q0 + lane];
                     if (q0 + lane < a.hq && part == 0) {
                         const float *r = sh.lred[q0 + lane];
                         float *ml = a.ml + (run * a.hq + q0 + lane) * 2;
-                        ml[0] = sh.mrun[par ^ 1][q0 + lane];
+                        ml[0] = *m_run;
                         ml[1] = (r[0] + r[1]) + (r[2] + r[3]);
                     }
-                    sh.mrun[par ^ 1][q0 + lane] = -INFINITY;
+                    *m_run = -INFINITY;
                 }
+                u_ends = false;
+            }
+            if (it < n_it) {
+                probabilities(s, tw.valid(a.sq), it & 1);
+                u_si = tw.si;
+                u_ends = tw.ends_run();
+                tw.next(a.sq);
             }
         }
     }
@@ -1191,10 +1267,10 @@ const Kernel kernels[2][6] = {{decode_latent_kernel<12, 2, false>, decode_latent
 constexpr int KERNEL_NQ[] = {12, 12, 16, 16, 32, 32}, KERNEL_NB[] = {2, 5, 5, 8, 2, 3};
 constexpr int N_KERNELS = 6;
 
-int smem_bytes(int nq, int nz, int nh, int nw, int nqs, int nt, int m_t) {
+int smem_bytes(int nq, int nz, int nh, int nw, int nqs) {
     const int scratch = nq == 12 ? sizeof(Scratch<12>) : nq == 16 ? sizeof(Scratch<16>) : sizeof(Scratch<32>);
-    return (nz + nh) * SLAB + nw * WSTAGE + nqs * wq_slab(nq) + 2 * op_rows(nq) * 128 + nt * m_t * 4 +
-           8 * (2 * (nz + nw + nqs + nt) + nh + READY_BARS + 9) + scratch;
+    return (nz + nh) * SLAB + nw * WSTAGE + nqs * wq_slab(nq) + 2 * op_rows(nq) * 128 +
+           8 * (2 * (nz + nw + nqs) + nh + READY_BARS + 9) + scratch;
 }
 constexpr int SMEM_MAX = 227 * 1024;
 
@@ -1301,7 +1377,7 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
                 d.map = s;
                 d.d = sp.d;
                 d.m = sp.m;
-                d.slope = sp.slope;
+                d.slope = sp.slope > 1.f ? 1.f / sp.slope : sp.slope;  // see put_signed_fc1
                 d.mask = 0;
                 hp.src[w][s] = {sp.w2k, sp.w2t, sp.b2, sp.sabs, sp.m, sp.in_dim};
                 for (int i = 0; i < sp.n_need; ++i) {
@@ -1334,25 +1410,20 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
         // Staging places.  A side's latents stay for all its chunks (nz >= their slabs).  One-chunk layers get places for the
         // other side's latents and six hidden slabs, because their jobs are shorter than the way from S to P; the others four
         // hidden slabs: a chunk's three and the one its predecessor may leave unpaired.
-        const int m_t = (lm + 31) & ~31, n_all = ly.list[0].n + ly.list[1].n;
-        int nh = chunks == 1 ? 6 : 4, nz = chunks == 1 ? std::max(4, 2 * ks) : ks, nw = 4, nqs = chunks == 1 ? 3 : 2;
-        int nt = chunks == 1 ? std::min(n_all, 4) : 1;
-        auto fits = [&]() { return smem_bytes(st.nq, nz, nh, nw, nqs, nt, m_t) <= SMEM_MAX; };
+        int nh = chunks == 1 ? 6 : 4, nz = chunks == 1 ? std::max(4, 2 * ks) : ks, nw = 4, nqs = 4;
+        auto fits = [&]() { return smem_bytes(st.nq, nz, nh, nw, nqs) <= SMEM_MAX; };
         while (nw > 3 && !fits()) --nw;
         while (nqs > 2 && !fits()) --nqs;
         while (nz > ks && !fits()) --nz;
         while (nw > 2 && !fits()) --nw;
         if (!fits()) continue;
-        while (nt < n_all && (++nt, fits())) {}
-        if (!fits()) --nt;
+        while (nqs < 12 && (++nqs, fits())) {}
+        if (!fits()) --nqs;
         lc.nz = (uint8_t)nz;
         lc.nh = (uint8_t)nh;
         lc.nw = (uint8_t)nw;
         lc.nqs = (uint8_t)nqs;
-        lc.nt = (uint8_t)nt;
-        lc.m_t = m_t;
-        lc.t_resident = nt >= n_all;
-        lc.smem = std::max(smem_bytes(st.nq, nz, nh, nw, nqs, nt, m_t), 120 * 1024);  // one CTA per SM: each takes all of tensor memory
+        lc.smem = std::max(smem_bytes(st.nq, nz, nh, nw, nqs), 120 * 1024);  // one CTA per SM: each takes all of tensor memory
         lc.variant = (uint8_t)v;
         lc.max_m = lm;
         lc.max_mk = lmk;
@@ -1476,9 +1547,6 @@ static cudaError_t launch_group(LatState &st, const DecodeArgs &a, const SeqList
     p.nh = lc.nh;
     p.nw = lc.nw;
     p.nqs = lc.nqs;
-    p.nt = lc.nt;
-    p.m_t = lc.m_t;
-    p.t_resident = lc.t_resident;
     p.two_terms_k = two_k;
     p.two_terms_v = two_v;
     const int pairs = (((p.sq.n_tiles + p.sq.per - 1) / p.sq.per) + 1) / 2, slots = st.n_sms / 2;

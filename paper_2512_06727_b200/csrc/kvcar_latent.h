@@ -68,9 +68,7 @@ struct LatCodes {
 struct LatLayerCfg {
     uint8_t ok = 0;
     uint8_t variant = 0;                              // kernel instantiation
-    uint8_t nz = 0, nh = 0, nw = 0, nqs = 0, nt = 0;  // staging places: latent, hidden, weight, query slabs; shift buffers
-    uint8_t t_resident = 0;                           // every source has a shift buffer of its own
-    int32_t m_t = 0;
+    uint8_t nz = 0, nh = 0, nw = 0, nqs = 0;          // staging places: latent, hidden, weight, query slabs
     int32_t smem = 0;
     int32_t max_mk = 0, max_m = 0;  // widest hidden layer of the K sources, of all
 };

@@ -166,6 +166,28 @@ def test_uncompressed_twin_with_query_groups(heads):
         _check_step(p.decode_step(seqs, step), "bf16", f"raw group {hq // hkv} step {step}")
 
 
+@pytest.mark.parametrize("cfg,slope,int8", [("c2", 0.01, False), ("c2", 1.5, False), ("c2", 1.5, True), ("c3", 1.5, False)])
+def test_runs_of_several_tiles(cfg, slope, int8):
+    """More tiles than blocks, so that each walks several (the K side one tile ahead) across sequence ends and partial tiles; slopes of
+    both sides of 1, of which the upper one is turned round when the weights are laid out.  Three sequences against the oracle."""
+    w = synth.scaled(synth.CONFIGS[cfg], n_layers=2, batch=48, reuse_frac=0.3)
+    seqs = list(range(48))
+    lens = [128 * (5 * s % 8) + (1, 127, 128, 60)[s % 4] for s in seqs]
+    assert sum((n + 127) // 128 for n in lens) > 148
+    p = Pair(w, max_seqs=48, max_pages=48 * 17, max_pages_per_seq=17, ae_kwargs={"leaky_slope": slope}, latent_quant=int8)
+    p.oracle_seqs = {0, 23, 47}
+    p.open(seqs)
+    for s_, n in zip(seqs, lens):
+        p.prefill([s_], n)
+    assert all(p.s.ctx.layer_kernel(l) == B.KERNEL_TENSOR for l in range(w.n_layers))
+    for step in range(2):
+        for l, (got, ref, rows) in p.decode_step(seqs, step, fused=True).items():
+            # the bound of slope 0.01 grows with the hidden vector, half of whose features the slope multiplies: rms sqrt((1 + slope^2) / 2)
+            grow = max(1.0, (1 + slope * slope) ** 0.5)
+            what = f"{cfg} slope {slope} int8 {int8} step {step} layer {l}"
+            assert_close(got[rows] / grow, ref / grow, "bf16", what)
+
+
 @pytest.mark.parametrize("storage,page_tokens,batch", [("bf16", 64, 1), ("bf16", 16, 5), ("bf16", 64, 33), ("f32", 64, 5)])
 def test_uncompressed_single_call_steps(storage, page_tokens, batch):
     """Raw layers through the single call, whose tile launch also appends the rows: pages of less than a 32-token step (plain copies)
