@@ -41,11 +41,12 @@ struct Vec16<__nv_bfloat16> {
 
 // acc[f][r] += sum over this lane's share of w_f[0..n) * x[r][0..n); `pre` holds the lane's first vector of each row already
 template <typename T, int NF>
-__device__ __forceinline__ void lane_dots(const T *wrow, const uint4 *pre, const float *x, int n, int lane, float (*acc)[RB]) {
+__device__ __forceinline__ void lane_dots(const T *wrow, const uint4 *pre, const float *x, int n, int rows, int lane, float (*acc)[RB]) {
     constexpr int VL = Vec16<T>::N;
     uint4 cur[NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) cur[f] = pre[f];
+#pragma unroll 1
     for (int k0 = lane * VL; k0 < n; k0 += 32 * VL) {
         const int kn = k0 + 32 * VL;
         uint4 nxt[NF];
@@ -56,6 +57,7 @@ __device__ __forceinline__ void lane_dots(const T *wrow, const uint4 *pre, const
         for (int f = 0; f < NF; ++f) Vec16<T>::unpack(cur[f], w[f]);
 #pragma unroll
         for (int r = 0; r < RB; ++r) {
+            if (r % 4 == 0 && r >= rows) break;  // rows in fours, as xs is filled
             const float4 *xr = reinterpret_cast<const float4 *>(x + r * n + k0);
 #pragma unroll
             for (int i = 0; i < VL / 4; ++i) {
@@ -177,7 +179,7 @@ __device__ __forceinline__ void encode_fc_block(const EncodeArgs &a, const int32
     if (EARLY) launch_dependents();
     grid_dependency_wait();  // inputs, page table and (stage 2) the hidden scratch are final from here on
 
-    const int rows_here = min(RB, n_rows - r0);
+    const int rows_here = min(RB, n_rows - r0), rows4 = (rows_here + 3) & ~3;
     const int my_row = row_of_lane(lane);
     int64_t prow = -1;  // stage 2: cache row of the input row this lane will write
     if (STAGE == 2 && active && !(lane & 1) && my_row < rows_here) {
@@ -188,6 +190,7 @@ __device__ __forceinline__ void encode_fc_block(const EncodeArgs &a, const int32
     if (STAGE == 1) {
         const int wv = a.kv_width / VL;  // 16-byte vectors per input row (head_dim is a multiple of the vector)
         if (bx == 0) {  // exact current-token rows (all heads)
+#pragma unroll 1
             for (int idx = threadIdx.x; idx < rows_here * wv; idx += blockDim.x) {
                 const int rr = idx / wv, cv = idx % wv, r = r0 + rr;
                 reinterpret_cast<uint4 *>(reinterpret_cast<T *>(pl.cur) + (int64_t)seq_ids[r] * a.kv_width)[cv] =
@@ -196,6 +199,7 @@ __device__ __forceinline__ void encode_fc_block(const EncodeArgs &a, const int32
         }
         if (!compressed) {
             const int nv = in_dim / VL;
+#pragma unroll 1
             for (int idx = bx * blockDim.x + threadIdx.x; idx < rows_here * nv; idx += nbx * blockDim.x)
                 copy_raw_vec<T>(a, pl, src, seq_ids, r0 + idx / nv, (idx % nv) * VL);
             return;
@@ -203,6 +207,7 @@ __device__ __forceinline__ void encode_fc_block(const EncodeArgs &a, const int32
         if (bx * NW >= n_out) return;
         // stage the stored heads' slices of this block's rows as fp32, 16 bytes per load, four loads in flight
         const int nv = in_dim / VL, total = rows_here * nv;
+#pragma unroll 1
         for (int base = threadIdx.x; base < total; base += 4 * blockDim.x) {
             uint4 v[4];
             int dst[4];
@@ -226,11 +231,13 @@ __device__ __forceinline__ void encode_fc_block(const EncodeArgs &a, const int32
                         *reinterpret_cast<float4 *>(xs + dst[u] + i) = make_float4(w[i], w[i + 1], w[i + 2], w[i + 3]);
                 }
         }
-        for (int idx = rows_here * in_dim + threadIdx.x; idx < RB * in_dim; idx += blockDim.x) xs[idx] = 0.f;
+#pragma unroll 1
+        for (int idx = rows_here * in_dim + threadIdx.x; idx < rows4 * in_dim; idx += blockDim.x) xs[idx] = 0.f;
     } else {
         if (!compressed || bx * NW >= n_out) return;
         const float *h = hid + ((int64_t)which * max_batch + r0) * hid_pitch;
         const int nv = m / 4, total = rows_here * nv;
+#pragma unroll 1
         for (int base = threadIdx.x; base < total; base += 4 * blockDim.x) {
             float4 v[4];
 #pragma unroll
@@ -244,7 +251,8 @@ __device__ __forceinline__ void encode_fc_block(const EncodeArgs &a, const int32
                 if (idx < total) *reinterpret_cast<float4 *>(xs + (idx / nv) * m + (idx % nv) * 4) = v[u];
             }
         }
-        for (int idx = rows_here * m + threadIdx.x; idx < RB * m; idx += blockDim.x) xs[idx] = 0.f;
+#pragma unroll 1
+        for (int idx = rows_here * m + threadIdx.x; idx < rows4 * m; idx += blockDim.x) xs[idx] = 0.f;
     }
     __syncthreads();
     if (!active) return;
@@ -253,7 +261,7 @@ __device__ __forceinline__ void encode_fc_block(const EncodeArgs &a, const int32
     for (int f = 0; f < NF; ++f)
 #pragma unroll
         for (int r = 0; r < RB; ++r) acc[f][r] = 0.f;
-    lane_dots<T, NF>(wrow, pre, xs, n_in, lane, acc);
+    lane_dots<T, NF>(wrow, pre, xs, n_in, rows_here, lane, acc);
     float sum[NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) sum[f] = reduce_rows(acc[f], lane);

@@ -944,6 +944,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
 // log2(e): the tile kernel's exponentials are powers of two.  Bound by the latency of the weight loads at few sequences, so all
 // of them are in flight before the wait for the preceding kernels; everything else comes from the parameters.  Operand rows of
 // sources that do not serve the head are zeroed.
+// Every block runs its code once, so instruction fetch counts like the loads: with loops unrolled only where that keeps loads in flight,
+// addresses stepped instead of computed per load and the encoder's rows bounded, this kernel went from 63 to 39 KB of code and
+// latent_back_kernel from 41-47 to 33-37; 12 layers of GPT-2's shape, 1 x 200 tokens 355 -> 314 us, 8 x 1024 609 -> 580; 22 of
+// TinyLLaMA's, 32 x 2048 1213 -> 1174.
 constexpr int LQ_SB = 8, LQ_COLS = 256, LF_THREADS = 256;
 struct QueryArgs {
     const __nv_bfloat16 *q;
@@ -960,12 +964,13 @@ __device__ __forceinline__ void query_block(const LatHeads &hp, const QueryArgs 
     const int kvh = qh / a.group, s = hp.idx[0][kvh], slot = hp.slot[0][kvh];
     const LatHeads::Src &sp = hp.src[0][s];
     const int m2 = sp.m >> 1, j = cb * (LQ_COLS / 2) + (tid & 127);
-    const uint32_t *w = reinterpret_cast<const uint32_t *>(sp.w2k) + (int64_t)slot * 64 * m2 + j;
+    // threads past the last feature pair take the last one's weights and store nothing
+    const int jj = min(j, m2 - 1);
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(sp.w2k) + (int64_t)slot * 64 * m2 + jj;
     uint32_t u[64];
-    float2 sab = make_float2(0.f, 0.f);  // the hidden vector is short of these
 #pragma unroll
-    for (int c = 0; c < 64; ++c) u[c] = j < m2 ? __ldg(w + (int64_t)c * m2) : 0u;
-    if (j < m2) sab = __ldg(reinterpret_cast<const float2 *>(sp.sabs) + j);
+    for (int c = 0; c < 64; ++c, w += m2) u[c] = __ldg(w);
+    const float2 sab = __ldg(reinterpret_cast<const float2 *>(sp.sabs) + jj);  // the hidden vector is short of these
     grid_dependency_wait();
     launch_dependents();
     for (int i = tid; i < 64 * LQ_SB; i += LF_THREADS) {
@@ -988,19 +993,25 @@ __device__ __forceinline__ void query_block(const LatHeads &hp, const QueryArgs 
         y[3] = fmaf(w1, q4.w, y[3]);
     }
     const int rows = wq_rows(a.nq);  // operand rows per (source, sequence): high terms, then low terms
+    uint32_t hi[4], lo[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        if (i0 + i >= n_here) break;
         x[i] *= sab.x;
         y[i] *= sab.y;
-        const uint32_t hi = pack_bf16(x[i], y[i]);
-        const uint32_t lo = a.two_terms ? pack_bf16(x[i] - __uint_as_float(hi << 16), y[i] - __uint_as_float(hi & 0xffff0000u)) : 0u;
-        for (int ss = 0; ss < hp.n_src[0]; ++ss) {
-            if (j >= (hp.src[0][ss].m >> 1)) continue;
-            uint32_t *r = reinterpret_cast<uint32_t *>(a.wq + (((int64_t)ss * a.batch + si0 + i0 + i) * rows + qh) * a.m_pad) + j;
-            r[0] = ss == s ? hi : 0u;
-            r[(int64_t)a.nq * a.m_pad / 2] = ss == s ? lo : 0u;
-        }
+        hi[i] = pack_bf16(x[i], y[i]);
+        lo[i] = a.two_terms ? pack_bf16(x[i] - __uint_as_float(hi[i] << 16), y[i] - __uint_as_float(hi[i] & 0xffff0000u)) : 0u;
+    }
+    const int64_t seq_step = (int64_t)rows * (a.m_pad >> 1), low = (int64_t)a.nq * (a.m_pad >> 1);
+    uint32_t *r = reinterpret_cast<uint32_t *>(a.wq) + (int64_t)(si0 + i0) * seq_step + (int64_t)qh * (a.m_pad >> 1) + j;
+#pragma unroll 1
+    for (int ss = 0; ss < hp.n_src[0]; ++ss, r += a.batch * seq_step) {
+        if (j >= (hp.src[0][ss].m >> 1)) continue;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i0 + i < n_here) {
+                r[i * seq_step] = ss == s ? hi[i] : 0u;
+                r[i * seq_step + low] = ss == s ? lo[i] : 0u;
+            }
     }
     if (cb != 0) return;
     const int warp = tid >> 5, lane = tid & 31;
@@ -1080,8 +1091,10 @@ __device__ __forceinline__ void merge_block(const LatHeads &hp, const LatSeqs &s
         const int n_run = runs(si, k0);
         const float2 *p = reinterpret_cast<const float2 *>(a.ml) + (int64_t)(k0 + si) * a.hq + qh;
         float M = -INFINITY, S = 0.f;
+#pragma unroll 1
         for (int r = lane; r < n_run; r += 32) M = fmaxf(M, p[(int64_t)r * a.hq].x);
         M = redux_max(M);
+#pragma unroll 1
         for (int r = lane; r < n_run; r += 32) {
             const float2 v = p[(int64_t)r * a.hq];
             const float wr = ex2(v.x - M);
@@ -1103,7 +1116,7 @@ __device__ __forceinline__ void merge_block(const LatHeads &hp, const LatSeqs &s
         const int n_run = runs(si0 + i, k0);
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         const float *p = a.upart + ((int64_t)(k0 + si0 + i) * a.hq + qh) * m_pad + f;
-#pragma unroll 8
+#pragma unroll 4
         for (int r = r0; r < n_run; r += step) {
             const float4 v = *reinterpret_cast<const float4 *>(p + (int64_t)r * a.hq * m_pad);
             const float wr = wts[i][r];
@@ -1126,6 +1139,7 @@ __device__ __forceinline__ void merge_block(const LatHeads &hp, const LatSeqs &s
         part[tid] = acc;
         __syncthreads();
         if (tid < nf) {
+#pragma unroll 2
             for (int g = 1; g < n_grp; ++g) {
                 const float4 v = part[tid + g * nf];
                 acc.x += v.x;
@@ -1136,6 +1150,7 @@ __device__ __forceinline__ void merge_block(const LatHeads &hp, const LatSeqs &s
             put(0, 4 * tid, acc);
         }
     } else {
+#pragma unroll 1
         for (int t = tid; t < SB * nf; t += LM_THREADS) {
             const int i = t / nf, f = 4 * (t % nf);
             put(i, f, i < n_here ? add_runs(i, f, 0, 1) : make_float4(0.f, 0.f, 0.f, 0.f));
@@ -1162,7 +1177,7 @@ __device__ __forceinline__ void merge_block(const LatHeads &hp, const LatSeqs &s
                 if (j < m) add(pre[k], j);
             }
         }
-#pragma unroll 16
+#pragma unroll(SB == 1 ? 2 : 16)
         for (int j = warp + (SB == 1 ? LM_PRE * LM_WARPS : 0); j < m; j += LM_WARPS) add(__ldg(w + j * pitch), j);
 #pragma unroll
         for (int i = 0; i < SB; ++i) *reinterpret_cast<float2 *>(&osum[warp][i][2 * lane]) = make_float2(x[i], y[i]);
@@ -1172,7 +1187,7 @@ __device__ __forceinline__ void merge_block(const LatHeads &hp, const LatSeqs &s
     // one warp per sequence: add up, the head's bias, the exact current token
     const int si = si0 + warp;
     float o[2] = {0.f, 0.f};
-#pragma unroll
+#pragma unroll 4
     for (int k = 0; k < LM_WARPS; ++k) {
         o[0] += osum[k][warp][lane];
         o[1] += osum[k][warp][lane + 32];
