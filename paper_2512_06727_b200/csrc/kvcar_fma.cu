@@ -10,10 +10,14 @@
 //   fma_merge_kernel   tiles of a sequence -> W4_h U + b4_h sum, the exact current token, the output row
 // Bound: FMA.  Tiles of 64 x 64 (8 x 4 per thread: three 16-byte shared loads per 32 FMA) where they fill the machine, else of
 // 32 x 32 (a sequence of 128 tokens is 72 blocks per side instead of 18).
+// The first three are programmatic dependent launches, and both hidden kernels work out their activations before they wait for what the
+// launch before left.  One GPT-2-shaped fp32 layer, us, with plain launches and 256-thread merges -> now: 1 x 128 tokens 95 -> 88,
+// 1 x 17 86 -> 60, 8 x 500 246 -> 211, 32 x 900 890 -> 865.
 #include <algorithm>
 #include <cmath>
 
 #include "kvcar_fma.h"
+#include "kvcar_pdl.cuh"
 
 namespace kvcar {
 
@@ -72,7 +76,10 @@ __global__ void __launch_bounds__(HC * 2) fma_hidden_kernel(const __grid_constan
     __shared__ float scl[TT], zp[TT];   // int8 rows: scale and zero-point
     const int tid = threadIdx.x, si = blockIdx.z, t0 = blockIdx.x * TT;
     const int len = sq.len[si], hq = a.hq, group = a.group;
-    if (t0 >= len) return;
+    if (t0 >= len) {
+        grid_dependency_wait();
+        return;
+    }
     const int valid = min(TT, len - t0), seq = sq.id[si];
     // which source and chunk
     int s = 0, ch = blockIdx.y;
@@ -169,6 +176,10 @@ __global__ void __launch_bounds__(HC * 2) fma_hidden_kernel(const __grid_constan
         }
     }
     const int nc = min(HC, m - c0);
+    // The launch before left what is read from here on (W4^T q, scores); it waited itself before it let this one start, so all that
+    // is older - rows, tables - was there from the beginning, and the hidden layer ran beside it.
+    grid_dependency_wait();
+    launch_dependents();
     if (SIDE == 0) {
         const float *wq = a.wq + ((int64_t)s * a.batch + sq.first_listed + si) * hq * a.max_m + c0;
         for (int i = tid; i < hq * HC; i += NT) aux[i] = i % HC < nc ? wq[(int64_t)(i / HC) * a.max_m + i % HC] : 0.f;
@@ -198,6 +209,7 @@ __global__ void __launch_bounds__(HC * 2) fma_hidden_kernel(const __grid_constan
                 const int t = lane + 32 * u;
                 if (t < whole) {
                     float x = 0.f;
+#pragma unroll 9
                     for (int c = 0; c < n_part; ++c) x += a.score[(((int64_t)c * a.n_tiles + tile) * hq + h) * FM_TOK + t];
                     v[u] = x;
                 }
@@ -242,6 +254,8 @@ __global__ void __launch_bounds__(256) fma_query_kernel(const __grid_constant__ 
     const int qh = blockIdx.x, si0 = blockIdx.z * SB, n_here = min(SB, n_seqs - si0), tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int kvh = qh / group, s = L.idx[0][kvh], slot = L.slot[0][kvh];
     const FmaSrc &sp = L.src[0][s];
+    grid_dependency_wait();
+    launch_dependents();
     for (int i = tid; i < SB * hd; i += 256) {
         const int k = i / hd, c = i % hd;
         qs[k][c] = k < n_here ? ld1(q + ((int64_t)(si0 + k) * hq + qh) * hd + c) * scale : 0.f;
@@ -268,7 +282,8 @@ __global__ void __launch_bounds__(256) fma_query_kernel(const __grid_constant__ 
     }
 }
 
-// Merge of the tiles of one (query head, sequence), 256 threads.  FINAL: apply the last decoder layer and write the output row;
+// Merge of the tiles of one (query head, sequence).  A block's time is that of its chain of loads of W4 (576 rows of 64 channels at the
+// GPT-2 shape), so few blocks get 1024 threads, many 256.  FINAL: apply the last decoder layer and write the output row;
 // else leave one partial result for the sequence.  `parts`: pieces of U per partial result.
 struct MergeArgs {
     const float *upart, *ml;
@@ -278,11 +293,14 @@ struct MergeArgs {
     int32_t hq, group, hd, kv_width, max_m, parts, with_current, tok;  // tok: tokens of a partial result
     float scale;
 };
-template <typename T, bool FINAL>
-__global__ void __launch_bounds__(256) fma_merge_kernel(const __grid_constant__ FmaLayer L, const __grid_constant__ FmaSeqs sq,
+template <typename T, bool FINAL, int THREADS>
+__global__ void __launch_bounds__(THREADS) fma_merge_kernel(const __grid_constant__ FmaLayer L, const __grid_constant__ FmaSeqs sq,
                                                         const __grid_constant__ MergeArgs a) {
-    extern __shared__ float u[];  // [max_m], then [256] partial sums
-    __shared__ float red[8], bred[8];
+    extern __shared__ float u[];  // [max_m], then [THREADS] partial sums
+    constexpr int WARPS = THREADS / 32;
+    __shared__ float red[WARPS], bred[WARPS];
+    grid_dependency_wait();
+    launch_dependents();
     const int qh = blockIdx.x, si = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, hd = a.hd;
     const int listed = sq.first_listed + si;
     const int kvh = qh / a.group, slot = L.slot[1][kvh];
@@ -295,7 +313,7 @@ __global__ void __launch_bounds__(256) fma_merge_kernel(const __grid_constant__ 
         if (lane == 0) red[warp] = v;
         __syncthreads();
         v = red[0];
-        for (int i = 1; i < 8; ++i) v = fmaxf(v, red[i]);
+        for (int i = 1; i < WARPS; ++i) v = fmaxf(v, red[i]);
         return v;
     };
     auto block_sum = [&](float v, float *buf) {
@@ -304,17 +322,17 @@ __global__ void __launch_bounds__(256) fma_merge_kernel(const __grid_constant__ 
         if (lane == 0) buf[warp] = v;
         __syncthreads();
         v = buf[0];
-        for (int i = 1; i < 8; ++i) v += buf[i];
+        for (int i = 1; i < WARPS; ++i) v += buf[i];
         return v;
     };
     float M = -INFINITY, S = 0.f;
-    for (int t = tid; t < n; t += 256) M = fmaxf(M, a.ml[((t0 + t) * a.hq + qh) * 2]);
+    for (int t = tid; t < n; t += THREADS) M = fmaxf(M, a.ml[((t0 + t) * a.hq + qh) * 2]);
     M = block_max(M);
-    for (int t = tid; t < n; t += 256) S += ex2(a.ml[((t0 + t) * a.hq + qh) * 2] - M) * a.ml[((t0 + t) * a.hq + qh) * 2 + 1];
+    for (int t = tid; t < n; t += THREADS) S += ex2(a.ml[((t0 + t) * a.hq + qh) * 2] - M) * a.ml[((t0 + t) * a.hq + qh) * 2 + 1];
     __syncthreads();
     S = block_sum(S, bred);
     const int tpp = FM_TOK / a.parts;  // tokens of a piece
-    for (int j = tid; j < sp.m; j += 256) {
+    for (int j = tid; j < sp.m; j += THREADS) {
         float acc = 0.f;
         for (int t = 0; t < n; ++t) {
             const float w = ex2(a.ml[((t0 + t) * a.hq + qh) * 2] - M);
@@ -336,11 +354,11 @@ __global__ void __launch_bounds__(256) fma_merge_kernel(const __grid_constant__ 
     __syncthreads();
     // thread = (channel, share of the hidden range)
     float *sums = u + a.max_m;
-    const int np = 256 / hd, c = tid % hd, part = tid / hd;
+    const int np = THREADS / hd, c = tid % hd, part = tid / hd;
     float o = 0.f;
     if (part < np) {
         const T *w = reinterpret_cast<const T *>(sp.w2t) + slot * hd + c;
-#pragma unroll 8
+#pragma unroll 12
         for (int j = part; j < sp.m; j += np) o = fmaf(ld1(w + (int64_t)j * sp.in_dim), u[j], o);
     }
     sums[tid] = o;
@@ -386,11 +404,9 @@ cudaError_t launch_hidden(const FmaLayer &L, const FmaSeqs &sq, const HiddenArgs
     for (int w = 0; w < 2; ++w)
         for (int s = 0; s < L.n_src[w]; ++s) units[w] += (L.src[w][s].m + HC - 1) / HC;
     const int tiles = (max_len + TT - 1) / TT;
-    k<<<dim3(tiles, units[0], sq.n), HC * 2, smem, st>>>(L, sq, h);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(k, dim3(tiles, units[0], sq.n), HC * 2, smem, st, L, sq, h);
     if (e != cudaSuccess) return e;
-    v<<<dim3(tiles, units[1], sq.n), HC * 2, smem, st>>>(L, sq, h);
-    return cudaGetLastError();
+    return launch_pdl(v, dim3(tiles, units[1], sq.n), HC * 2, smem, st, L, sq, h);
 }
 
 template <typename T, bool Q8>
@@ -398,9 +414,9 @@ cudaError_t launch_tiles(FmaState &st, const kvcar_config &cfg, const DecodeArgs
                          const FmaLayer &L, cudaStream_t stream, int *n_launches) {
     int max_mk = 0;
     for (int s = 0; s < L.n_src[0]; ++s) max_mk = std::max(max_mk, L.src[0][s].m);
-    fma_query_kernel<T><<<dim3(a.hq, (max_mk + 63) / 64, (seqs.n + 7) / 8), 256, 0, stream>>>(
-        L, reinterpret_cast<const T *>(a.q), st.wq, seqs.n, a.hq, a.hq / a.hkv, a.hd, a.scale * LOG2E, st.batch, st.max_m);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(fma_query_kernel<T>, dim3(a.hq, (max_mk + 63) / 64, (seqs.n + 7) / 8), 256, 0, stream, L,
+                               reinterpret_cast<const T *>(a.q), st.wq, seqs.n, a.hq, a.hq / a.hkv, a.hd, a.scale * LOG2E, st.batch,
+                               (int)st.max_m);
     if (e != cudaSuccess) return e;
     *n_launches = 1;
     int n_all = 0;
@@ -459,8 +475,7 @@ cudaError_t launch_tiles(FmaState &st, const kvcar_config &cfg, const DecodeArgs
             m.max_m = st.max_m;
             m.parts = small ? 2 : 1;
             m.tok = FM_TOK;
-            fma_merge_kernel<T, false><<<dim3(a.hq, g.n), 256, 0, stream>>>(L, g, m);
-            e = cudaGetLastError();
+            e = launch_pdl(fma_merge_kernel<T, false, 256>, dim3(a.hq, g.n), 256, 0, stream, L, g, m);
             if (e != cudaSuccess) return e;
             ++*n_launches;
         }
@@ -496,8 +511,10 @@ cudaError_t launch_merge(FmaState &st, const kvcar_config &cfg, const DecodeArgs
     m.tok = FM_TOK;
     m.with_current = (a.flags & KVCAR_INCLUDE_CURRENT_EXACT) != 0;
     m.scale = a.scale * LOG2E;
-    fma_merge_kernel<T, true><<<dim3(a.hq, seqs.n), 256, (size_t)(st.max_m + 256) * sizeof(float), stream>>>(L, g, m);
-    return cudaGetLastError();
+    const bool few = a.hq * seqs.n <= 2 * st.n_sms && (st.max_m + 1024) * sizeof(float) <= 48 * 1024;
+    const int threads = few ? 1024 : 256;
+    return launch_pdl(few ? fma_merge_kernel<T, true, 1024> : fma_merge_kernel<T, true, 256>, dim3(a.hq, seqs.n), threads,
+                      (size_t)(st.max_m + threads) * sizeof(float), stream, L, g, m);
 }
 
 }  // namespace

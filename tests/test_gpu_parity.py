@@ -188,6 +188,19 @@ def test_runs_of_several_tiles(cfg, slope, int8):
             assert_close(got[rows] / grow, ref / grow, "bf16", what)
 
 
+@pytest.mark.parametrize("batch", [24, 25])
+def test_fp32_merge_on_both_block_sizes(batch):
+    """12 heads x 24 sequences merge in blocks of 1024 threads, 12 x 25 (more than two per SM) in blocks of 256."""
+    w = synth.scaled(synth.CONFIGS["c2"], n_layers=1, batch=batch, storage="f32", reuse_frac=0.0)
+    seqs = list(range(batch))
+    p = Pair(w, max_seqs=batch, max_pages=2 * batch, max_pages_per_seq=2)
+    p.oracle_seqs = {0, 7, batch - 1}
+    p.open(seqs)
+    for s_ in seqs:
+        p.prefill([s_], (1, 31, 64, 100)[s_ % 4])
+    _check_step(p.decode_step(seqs, 0, fused=True), "f32", f"batch {batch}")
+
+
 @pytest.mark.parametrize("storage,page_tokens,batch", [("bf16", 64, 1), ("bf16", 16, 5), ("bf16", 64, 33), ("f32", 64, 5)])
 def test_uncompressed_single_call_steps(storage, page_tokens, batch):
     """Raw layers through the single call, whose tile launch also appends the rows: pages of less than a 32-token step (plain copies)
