@@ -255,21 +255,41 @@ void compute_layout(kvcar_ctx *c) {
     c->ws_bytes = s;
 }
 
+// round to nearest even, as __float2bfloat16_rn, in a form that compilers vectorise
+inline uint16_t bf16_bits(float f) {
+    uint32_t u;
+    memcpy(&u, &f, 4);
+    const uint32_t r = (u + 0x7fffu + ((u >> 16) & 1u)) >> 16;
+    return (uint16_t)((u & 0x7fffffffu) > 0x7f800000u ? 0x7fffu : r);
+}
+
 void put_elems(char *dst, const float *src, size_t n, int dtype) {
     if (dtype == KVCAR_F32) {
         memcpy(dst, src, n * 4);
     } else {
-        __nv_bfloat16 *d = reinterpret_cast<__nv_bfloat16 *>(dst);
-        for (size_t i = 0; i < n; ++i) d[i] = __float2bfloat16_rn(src[i]);
+        uint16_t *d = reinterpret_cast<uint16_t *>(dst);
+        for (size_t i = 0; i < n; ++i) d[i] = bf16_bits(src[i]);
     }
 }
 
-// transposed copy: src [rows][cols] -> dst [cols][rows]
-void put_transposed(char *dst, const float *src, int rows, int cols, int dtype) {
-    std::vector<float> t((size_t)rows * cols);
-    for (int r = 0; r < rows; ++r)
-        for (int cc = 0; cc < cols; ++cc) t[(size_t)cc * rows + r] = src[(size_t)r * cols + cc];
-    put_elems(dst, t.data(), t.size(), dtype);
+// transposed copy: src [rows][cols] -> dst [cols][rows], square blocks at a time so that both sides stay in cache
+template <typename E>
+void transpose(E *dst, const E *src, int rows, int cols) {
+    constexpr int B = 32;
+    for (int r0 = 0; r0 < rows; r0 += B)
+        for (int c0 = 0; c0 < cols; c0 += B) {
+            const int r1 = std::min(rows, r0 + B), c1 = std::min(cols, c0 + B);
+            for (int c = c0; c < c1; ++c)
+                for (int r = r0; r < r1; ++r) dst[(size_t)c * rows + r] = src[(size_t)r * cols + c];
+        }
+}
+
+// `rows` x `cols` elements that put_elems has written
+void put_transposed(char *dst, const char *elems, int rows, int cols, int dtype) {
+    if (dtype == KVCAR_F32)
+        transpose(reinterpret_cast<uint32_t *>(dst), reinterpret_cast<const uint32_t *>(elems), rows, cols);
+    else
+        transpose(reinterpret_cast<uint16_t *>(dst), reinterpret_cast<const uint16_t *>(elems), rows, cols);
 }
 
 // bias + BatchNorm(inference) as one scale/shift per feature
@@ -287,22 +307,27 @@ void fuse_bn(const std::vector<float> &b1, const std::vector<float> &bn, int m, 
 // that is left to the epilogue, |s| goes to the neighbours of the hidden vector (W4^T q and the weighted sum, both fp32).  A
 // scale too small to divide by leaves the constant LeakyReLU(t).  A slope above 1 is turned into one below: LeakyReLU(x) is then
 // -slope max(-x, -x / slope), so rows and shift change their sign and -slope goes with |s|; the kernel knows the larger-of form only.
-void put_signed_fc1(char *dst, float *sabs, size_t stride, const float *w, const float *s, const float *t, float slope, int m, int d) {
+// `w`: the layer in bf16.
+void put_signed_fc1(char *dst, float *sabs, size_t stride, const char *w, const float *s, const float *t, float slope, int m, int d) {
     const float flip = slope > 1.f ? -1.f : 1.f, gain = slope > 1.f ? -slope : 1.f;
-    __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(dst);
     float *shift = sabs + stride, *rowsum = shift + stride;
     for (int j = 0; j < m; ++j) {
         const bool tiny = std::fabs(s[j]) < 1e-20f;
-        const float sign = tiny ? 0.f : s[j] < 0.f ? -flip : flip;
+        const uint16_t sign = (s[j] < 0.f) != (flip < 0.f) ? 0x8000 : 0, keep = tiny ? 0 : 0xffff;
         const float size = tiny ? 1.f : std::fabs(s[j]);
         sabs[j] = gain * size;
         shift[shift_place(j)] = flip * t[j] / size;
-        double sum = 0.0;
+        const uint16_t *in = reinterpret_cast<const uint16_t *>(w) + (size_t)j * d;
+        uint16_t *o = reinterpret_cast<uint16_t *>(dst) + (size_t)j * d;
+        double sum[8] = {};
         for (int k = 0; k < d; ++k) {
-            o[(size_t)j * d + k] = __float2bfloat16_rn(sign * w[(size_t)j * d + k]);
-            sum += (double)__bfloat162float(o[(size_t)j * d + k]);
+            o[k] = (uint16_t)((in[k] ^ sign) & keep);
+            const uint32_t u = (uint32_t)o[k] << 16;
+            float x;
+            memcpy(&x, &u, 4);
+            sum[k & 7] += (double)x;
         }
-        rowsum[shift_place(j)] = (float)sum;
+        rowsum[shift_place(j)] = (float)(((sum[0] + sum[1]) + (sum[2] + sum[3])) + ((sum[4] + sum[5]) + (sum[6] + sum[7])));
     }
 }
 
@@ -547,33 +572,39 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
         p.enc_b2 = p.dec_t + M * 4;
         p.dec_b2 = p.enc_b2 + D * 4;
         w = align_up(w + (4 * M + D + I) * 4, 256);
-        put_transposed(&img[p.enc_w1t], a.enc_w1.data(), (int)M, (int)I, g.storage);  // [M][I] -> [I][M]
-        put_transposed(&img[p.enc_w2t], a.enc_w2.data(), (int)D, (int)M, g.storage);  // [D][M] -> [M][D]
-        put_transposed(&img[p.dec_w1t], a.dec_w1.data(), (int)M, (int)D, g.storage);  // [M][D] -> [D][M]
-        put_transposed(&img[p.dec_w2t], a.dec_w2.data(), (int)I, (int)M, g.storage);  // [I][M] -> [M][I]
         fuse_bn(a.enc_b1, a.enc_bn, (int)M, a.eps, (float *)&img[p.enc_s], (float *)&img[p.enc_t]);
         fuse_bn(a.dec_b1, a.dec_bn, (int)M, a.eps, (float *)&img[p.dec_s], (float *)&img[p.dec_t]);
         memcpy(&img[p.enc_b2], a.enc_b2.data(), D * 4);
         memcpy(&img[p.dec_b2], a.dec_b2.data(), I * 4);
+        // each matrix once from fp32, then its other layouts from that
+        p.enc_w1r = w;
+        p.enc_w2r = p.enc_w1r + M * I * E;
+        w = align_up(w + (M * I + D * M) * E, 256);
+        put_elems(&img[p.enc_w1r], a.enc_w1.data(), M * I, g.storage);
+        put_elems(&img[p.enc_w2r], a.enc_w2.data(), D * M, g.storage);
+        const char *fc1 = (const char *)a.dec_w1.data(), *fc2 = (const char *)a.dec_w2.data();
         if (g.storage == KVCAR_BF16) {
             p.w1k = w;
             p.w2k = p.w1k + M * D * 2;
             w = align_up(w + (M * D + I * M) * 2, 256);
             put_elems(&img[p.w1k], a.dec_w1.data(), M * D, KVCAR_BF16);
             put_elems(&img[p.w2k], a.dec_w2.data(), I * M, KVCAR_BF16);
+            fc1 = &img[p.w1k];
+            fc2 = &img[p.w2k];
+        }
+        put_transposed(&img[p.enc_w1t], &img[p.enc_w1r], (int)M, (int)I, g.storage);  // [M][I] -> [I][M]
+        put_transposed(&img[p.enc_w2t], &img[p.enc_w2r], (int)D, (int)M, g.storage);  // [D][M] -> [M][D]
+        put_transposed(&img[p.dec_w1t], fc1, (int)M, (int)D, g.storage);              // [M][D] -> [D][M]
+        put_transposed(&img[p.dec_w2t], fc2, (int)I, (int)M, g.storage);              // [I][M] -> [M][I]
+        if (g.storage == KVCAR_BF16) {
             p.w1n = w;
             w = align_up(w + M * D * 2, 256);
             p.sabs = w;  // then the shifts, then the row sums
             const size_t M32 = (M + 31) & ~(size_t)31;
             w = align_up(w + 3 * M32 * 4, 256);
-            put_signed_fc1(&img[p.w1n], (float *)&img[p.sabs], M32, a.dec_w1.data(),
-                           (const float *)&img[p.dec_s], (const float *)&img[p.dec_t], a.slope, (int)M, (int)D);
+            put_signed_fc1(&img[p.w1n], (float *)&img[p.sabs], M32, &img[p.w1k], (const float *)&img[p.dec_s],
+                           (const float *)&img[p.dec_t], a.slope, (int)M, (int)D);
         }
-        p.enc_w1r = w;
-        p.enc_w2r = p.enc_w1r + M * I * E;
-        w = align_up(w + (M * I + D * M) * E, 256);
-        put_elems(&img[p.enc_w1r], a.enc_w1.data(), M * I, g.storage);
-        put_elems(&img[p.enc_w2r], a.enc_w2.data(), D * M, g.storage);
     }
 
     // per-layer decode plans
