@@ -55,9 +55,9 @@ typedef enum { KVCAR_K = 0, KVCAR_V = 1 } kvcar_which;
 
 /* kernel families (kvcar_set_kernel) */
 typedef enum {
-    KVCAR_KERNEL_AUTO = 0,    /* tensor-core kernel where the shape allows, else generic */
-    KVCAR_KERNEL_GENERIC = 1, /* fp32-FMA kernels (any supported shape, both dtypes)     */
-    KVCAR_KERNEL_TENSOR = 2,  /* tcgen05/TMEM fused kernel (bf16 storage only)           */
+    KVCAR_KERNEL_AUTO = 0,    /* tensor-core kernels where the shape allows, else fp32 FMA */
+    KVCAR_KERNEL_GENERIC = 1, /* plain fp32 kernel (any supported shape, both dtypes)      */
+    KVCAR_KERNEL_TENSOR = 2,  /* tcgen05/TMEM kernels (bf16 storage, bf16 or int8 rows)    */
     KVCAR_KERNEL_RAW = 3      /* reported only: streaming kernel AUTO picks for a layer
                                  whose K and V are all stored raw (no autoencoder)       */
 } kvcar_kernel;
@@ -214,16 +214,13 @@ kvcar_status kvcar_advance(kvcar_ctx *ctx, const int32_t *seqs, int32_t n_seqs, 
  * "Network Architecture": FC, BatchNorm, LeakyReLU, FC, nothing after it), so
  * a head's score q.k' with k' = W4_h a + b4_h equals a.(W4_h^T q) + q.b4_h,
  * where a is the token's activated hidden vector: the restored K rows are then
- * never formed.  The same result up to rounding (W4_h^T q is rounded to the
- * storage type once per sequence and head); honoured by the tensor-core kernel
- * for K when the launch fills the machine, ignored (plain form computed) by
- * every other kernel.  KVCAR_ABSORBED_V (only together with KVCAR_ABSORBED): the
- * same for V, sum_t p_t v'_t = W4_h (sum_t p_t a_t) + b4_h sum_t p_t: a tile
- * hands on sum_t p_t a_t (m values per query head) and the last layer is applied
- * once per sequence and head when the tiles are merged; the probabilities enter
- * that product rounded to the storage type.  For at most 32 query heads and
- * hidden layers whose feature chunks fit one accumulator buffer (576 columns with
- * up to 16 query heads, 512 with up to 32); ignored elsewhere.
+ * never formed, and sum_t p_t v'_t = W4_h (sum_t p_t a_t) + b4_h sum_t p_t.  The
+ * tensor-core and fp32 kernels use this form in any case, with W4_h^T q and the
+ * probabilities in fp32 or as two bf16 terms; the flag lets them take one bf16
+ * term of W4_h^T q (rounded to the storage type once per sequence and head),
+ * KVCAR_ABSORBED_V (only together with KVCAR_ABSORBED) one bf16 term of the
+ * probabilities.  With 17 to 32 query heads the probabilities have one term
+ * anyway.  Kernels that restore the heads ignore the flags.
  */
 kvcar_status kvcar_decode_attention(kvcar_ctx *ctx, int32_t layer, const int32_t *seqs, int32_t n_seqs,
                                     const void *q, void *out, uint32_t flags, void *stream);
@@ -234,11 +231,12 @@ kvcar_status kvcar_decode_attention(kvcar_ctx *ctx, int32_t layer, const int32_t
  * results, all DEVICE buffers.  Because the cached rows that the decoder reads
  * do not depend on the row the encoder appends (Sec. "Network Architecture":
  * the restored (l-1) x D matrices are concatenated with the current token's
- * exact vectors, which enter only when the tiles are merged), the library runs
- * the tile kernel on a stream of its own, forked from `stream` at the call and
- * joined back before the merge, beside the encoder's launches.  On return all
- * work is enqueued and ordered after what `stream` held at the call and before
- * what is enqueued on it afterwards.
+ * exact vectors, which enter only when the tiles are merged), the encoder's work
+ * shares launches with the attention's (or, for shapes that only the restoring
+ * and fp32 kernels take, runs beside the tiles, those on a stream of the library's
+ * own that forks from `stream` at the call and joins it before the merge).  On
+ * return all work is enqueued and ordered after what `stream` held at the call
+ * and before what is enqueued on it afterwards.
  * Errors as for the two calls; on KVCAR_ERR_OOM_PAGES nothing is written.
  */
 kvcar_status kvcar_step_layer(kvcar_ctx *ctx, int32_t layer, const int32_t *seqs, int32_t n_seqs, const void *k,
@@ -254,7 +252,7 @@ kvcar_status kvcar_step_layer(kvcar_ctx *ctx, int32_t layer, const int32_t *seqs
  * that `stream` still holds (the call waits for the copy that used the slot eight
  * calls earlier), so k_host, v_host and q_host may be reused as soon as the
  * call returns; out_host should be page-locked: it is then written by the last
- * kernel of the step (or, if large, copied asynchronously).
+ * kernel of the step.
  */
 kvcar_status kvcar_step_layer_host(kvcar_ctx *ctx, int32_t layer, const int32_t *seqs, int32_t n_seqs,
                                    const void *k_host, const void *v_host, const void *q_host, void *out_host,
