@@ -252,7 +252,9 @@ kvcar_status kvcar_step_layer(kvcar_ctx *ctx, int32_t layer, const int32_t *seqs
  * that `stream` still holds (the call waits for the copy that used the slot eight
  * calls earlier), so k_host, v_host and q_host may be reused as soon as the
  * call returns; out_host should be page-locked: it is then written by the last
- * kernel of the step.
+ * kernel of the step.  Under stream capture the three copies are part of the
+ * graph, which reads k_host, v_host and q_host (page-locked) at every replay;
+ * replays and direct calls of a context may be mixed on one stream.
  */
 kvcar_status kvcar_step_layer_host(kvcar_ctx *ctx, int32_t layer, const int32_t *seqs, int32_t n_seqs,
                                    const void *k_host, const void *v_host, const void *q_host, void *out_host,

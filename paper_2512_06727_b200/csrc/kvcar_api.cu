@@ -225,8 +225,8 @@ void compute_layout(kvcar_ctx *c) {
     c->part_off = s;
     const int nb = std::min(g.max_seqs, KVCAR_MAX_BATCH);
     s = align_up(s + (size_t)nb * c->max_chunks * g.n_q_heads * (g.head_dim + 2) * sizeof(float), 256);
-    c->stage_off = s;  // host-buffer entry point: H_SLOTS slots of k, v and q, then one out
-    s = align_up(s + (kvcar_ctx::H_SLOTS * (2 * align_up((size_t)nb * W * c->elem, 256) + align_up((size_t)nb * g.n_q_heads * g.head_dim * c->elem, 256)) +
+    c->stage_off = s;  // host-buffer entry point: H_SLOTS slots of k, v and q, one for calls under capture, then one out
+    s = align_up(s + ((kvcar_ctx::H_SLOTS + 1) * (2 * align_up((size_t)nb * W * c->elem, 256) + align_up((size_t)nb * g.n_q_heads * g.head_dim * c->elem, 256)) +
                       (size_t)nb * g.n_q_heads * g.head_dim * c->elem), 256);
     c->enchid_off = s;  // hidden activations between the decode-time encoder's launches; int8 rows: then the fp32 latents
     s = align_up(s + (size_t)2 * nb * (c->max_m + (g.latent_quant ? c->max_d : 0)) * sizeof(float), 256);
@@ -750,10 +750,9 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
         if (static_scratch_for_current_device(&p) != cudaSuccess) cudaGetLastError();
         c->static_scratch = p;
     }
+    c->hslot_bytes = 2 * align_up((size_t)std::min(g.max_seqs, KVCAR_MAX_BATCH) * hkv * hd * c->elem, 256) +
+                     align_up((size_t)std::min(g.max_seqs, KVCAR_MAX_BATCH) * g.n_q_heads * hd * c->elem, 256);
     if (!c->hstage) {  // set-up time: the host-buffer entry point's staging slots (without them it copies k, v, q singly)
-        const size_t nbatch = (size_t)std::min(g.max_seqs, KVCAR_MAX_BATCH);
-        const size_t kvb = align_up(nbatch * hkv * hd * c->elem, 256), qb = align_up(nbatch * g.n_q_heads * hd * c->elem, 256);
-        c->hslot_bytes = 2 * kvb + qb;
         bool ok = cudaHostAlloc((void **)&c->hstage, c->hslot_bytes * kvcar_ctx::H_SLOTS, cudaHostAllocDefault) == cudaSuccess;
         ok = ok && cudaStreamCreateWithFlags(&c->copy, cudaStreamNonBlocking) == cudaSuccess;
         for (int i = 0; ok && i < kvcar_ctx::H_SLOTS; ++i)
@@ -1172,13 +1171,15 @@ kvcar_status kvcar_step_layer_host(kvcar_ctx *c, int32_t layer, const int32_t *s
     cudaStream_t st = (cudaStream_t)stream;
     const size_t kv_bytes = (size_t)n_seqs * g.n_kv_heads * g.head_dim * c->elem;
     const size_t q_bytes = (size_t)n_seqs * g.n_q_heads * g.head_dim * c->elem;
-    const unsigned slot = c->hslot++ % kvcar_ctx::H_SLOTS;
-    char *dk = c->ws + c->stage_off + (size_t)slot * c->hslot_bytes, *dv = dk + kvb, *dq = dv + kvb;
-    char *dout = c->ws + c->stage_off + (size_t)kvcar_ctx::H_SLOTS * c->hslot_bytes;
     cudaError_t e = cudaSuccess;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
     const bool ahead = c->hstage && cap == cudaStreamCaptureStatusNone;
+    // A captured call leaves no event behind for the replays that will read its device slot, so it takes a slot that no copy
+    // running ahead of the caller's stream ever writes.
+    const unsigned slot = ahead ? c->hslot++ % kvcar_ctx::H_SLOTS : kvcar_ctx::H_SLOTS;
+    char *dk = c->ws + c->stage_off + (size_t)slot * c->hslot_bytes, *dv = dk + kvb, *dq = dv + kvb;
+    char *dout = c->ws + c->stage_off + (size_t)(kvcar_ctx::H_SLOTS + 1) * c->hslot_bytes;
     if (ahead) {
         // One copy: k, v, q gathered in a pinned slot with the device slot's layout.  It depends on nothing in the caller's stream
         // but the step that read the device slot eight calls ago, so it runs ahead of the steps before this one

@@ -410,6 +410,48 @@ def test_host_buffer_steps_equal_device_steps(pinned_out):
     assert torch.equal(out, ref.cpu())
 
 
+def test_host_buffer_steps_mix_with_graph_replays():
+    """A captured host-buffer step of layer 0, replayed behind queued work, and direct host-buffer steps of layer 1 behind it
+    (more than the library has staging slots, whose copies run ahead of the stream): neither reads the other's inputs."""
+    w = synth.scaled(synth.CONFIGS["c3"], n_layers=2, batch=2, reuse_frac=0.0)
+    seqs, calls = [0, 1], 9
+    p = Pair(w, max_seqs=2, max_pages=8, max_pages_per_seq=4, with_oracle=False)
+    p.open(seqs)
+    p.prefill(seqs, 50)
+    p.decode_step(seqs, 0)
+    p.s.ctx.reserve(seqs, 1)
+    dt = p.s.dtype
+    shape = [(2, w.n_kv_heads, w.head_dim)] * 2 + [(2, w.n_q_heads, w.head_dim)]
+    gen = torch.Generator().manual_seed(6)
+    sets = [[torch.randn(s, generator=gen).to(dt).pin_memory() for s in shape] for _ in range(1 + calls)]
+    outs = [torch.zeros(shape[2], dtype=dt).pin_memory() for _ in sets]
+
+    def call(layer, i):
+        p.s.ctx.step_layer_host(layer, seqs, *(t.data_ptr() for t in sets[i]), outs[i].data_ptr(), B.INCLUDE_CURRENT_EXACT, p.s.stream())
+
+    def device(layer, i):
+        d, out = [t.cuda() for t in sets[i]], torch.empty(shape[2], dtype=dt, device="cuda")
+        p.s.ctx.step_layer(layer, seqs, *(t.data_ptr() for t in d), out.data_ptr(), B.INCLUDE_CURRENT_EXACT, p.s.stream())
+        return out.cpu()
+    ref = [device(0, 0)] + [device(1, i) for i in range(1, 1 + calls)]
+    call(0, 0)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(0, 0)
+    x = torch.randn(4096, 4096, device="cuda")
+    for _ in range(3):
+        for o in outs:
+            o.zero_()
+        for _ in range(10):
+            x = (x @ x).clamp_(-1, 1)
+        graph.replay()
+        for i in range(1, 1 + calls):
+            call(1, i)
+        p.s.ctx.sync_status(p.s.stream())
+        assert all(torch.equal(a, b) for a, b in zip(outs, ref))
+
+
 def test_errors_leave_state_untouched():
     w = synth.scaled(synth.CONFIGS["c3"], n_layers=1, batch=1, reuse_frac=0.0)
     p = Pair(w, max_seqs=2, max_pages=2, max_pages_per_seq=2, with_oracle=False)
