@@ -175,6 +175,8 @@ kvcar_status kvcar_reserve(kvcar_ctx *ctx, const int32_t *seqs, int32_t n_seqs, 
  * token's exact rows are also kept as the layer's "current token".  seq_len is
  * NOT changed: call kvcar_advance once per step after all layers.
  * seqs: HOST int32 [n_seqs], distinct open sequences, n_seqs <= KVCAR_MAX_BATCH.
+ * A list longer than max_seqs (so with a repeated id) is KVCAR_ERR_INVALID_ARG
+ * here for n_tokens = 1 and in the attention and step calls; nothing is written.
  */
 kvcar_status kvcar_encode_append(kvcar_ctx *ctx, int32_t layer, const int32_t *seqs, int32_t n_seqs,
                                  int32_t n_tokens, const void *k, const void *v, void *stream);

@@ -339,6 +339,12 @@ bool check_seqs(kvcar_ctx *c, const int32_t *seqs, int n) {
     return true;
 }
 
+// Workspace and staging areas hold one row per sequence id: a longer list names a sequence twice and would run past them.
+kvcar_status check_rows(kvcar_ctx *c, int n) {
+    if (n <= c->cfg.max_seqs) return KVCAR_OK;
+    return fail(c, KVCAR_ERR_INVALID_ARG, "the list names a sequence twice (it is longer than max_seqs)");
+}
+
 kvcar_status reserve_pages(kvcar_ctx *c, const int32_t *seqs, int n, int n_tokens) {
     const int P = c->cfg.page_tokens;
     size_t need_total = 0;
@@ -823,7 +829,9 @@ kvcar_status kvcar_encode_append(kvcar_ctx *c, int32_t layer, const int32_t *seq
         return fail(c, KVCAR_ERR_INVALID_ARG, "bad layer, pointer or token count");
     if (!check_seqs(c, seqs, n_seqs)) return fail(c, KVCAR_ERR_INVALID_ARG, "bad sequence list");
     if (((uintptr_t)k | (uintptr_t)v) & 15) return fail(c, KVCAR_ERR_INVALID_ARG, "k/v must be 16-byte aligned");
-    kvcar_status s = reserve_pages(c, seqs, n_seqs, n_tokens);
+    kvcar_status s = n_tokens == 1 ? check_rows(c, n_seqs) : KVCAR_OK;
+    if (s != KVCAR_OK) return s;
+    s = reserve_pages(c, seqs, n_seqs, n_tokens);
     if (s != KVCAR_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     s = flush_tables(c, st);
@@ -1082,7 +1090,7 @@ static kvcar_status check_decode_args(kvcar_ctx *c, int32_t layer, const int32_t
     if (!check_seqs(c, seqs, n_seqs)) return fail(c, KVCAR_ERR_INVALID_ARG, "bad sequence list");
     if (((uintptr_t)q | (uintptr_t)out) & 15) return fail(c, KVCAR_ERR_INVALID_ARG, "q/out must be 16-byte aligned");
     if (flags & ~(KVCAR_INCLUDE_CURRENT_EXACT | KVCAR_ABSORBED | KVCAR_ABSORBED_V)) return fail(c, KVCAR_ERR_INVALID_ARG, "unknown flag");
-    return KVCAR_OK;
+    return check_rows(c, n_seqs);
 }
 
 kvcar_status kvcar_decode_attention(kvcar_ctx *c, int32_t layer, const int32_t *seqs, int32_t n_seqs, const void *q,
@@ -1165,6 +1173,7 @@ kvcar_status kvcar_step_layer_host(kvcar_ctx *c, int32_t layer, const int32_t *s
     if (!c->bound) return fail(c, KVCAR_ERR_STATE, "bind memory first");
     if (!k_host || !v_host || !q_host || !out_host) return fail(c, KVCAR_ERR_INVALID_ARG, "null host buffer");
     if (!check_seqs(c, seqs, n_seqs)) return fail(c, KVCAR_ERR_INVALID_ARG, "bad sequence list");
+    if (kvcar_status s = check_rows(c, n_seqs); s != KVCAR_OK) return s;
     const kvcar_config &g = c->cfg;
     const size_t kvb = align_up((size_t)n_seqs * g.n_kv_heads * g.head_dim * c->elem, 256);
     const size_t qb = align_up((size_t)n_seqs * g.n_q_heads * g.head_dim * c->elem, 256);

@@ -583,7 +583,6 @@ void fma_setup(FmaState &st, const kvcar_config &cfg, const std::vector<LayerPla
 
 cudaError_t fma_launch_tiles(FmaState &st, const kvcar_config &cfg, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens,
                              int layer, cudaStream_t stream, int *n_launches) {
-    if (seqs.n > st.batch) return cudaErrorInvalidValue;  // the list names a sequence twice
     const FmaLayer &L = st.layer[layer];
     if (cfg.storage == KVCAR_F32) return launch_tiles<float, false>(st, cfg, a, seqs, lens, L, stream, n_launches);
     return L.quant ? launch_tiles<__nv_bfloat16, true>(st, cfg, a, seqs, lens, L, stream, n_launches)

@@ -1620,7 +1620,6 @@ static cudaError_t launch_group(LatState &st, const DecodeArgs &a, const SeqList
 
 cudaError_t lat_launch(LatState &st, const DecodeArgs &a, const SeqList &seqs, const int32_t *lens, int layer, const LatEncode *enc,
                        cudaStream_t stream, int *n_launches) {
-    if (seqs.n > st.batch) return cudaErrorInvalidValue;  // the list names a sequence twice
     *n_launches = 0;
     if (!st.quant) return launch_group(st, a, seqs, seqs, lens, layer, enc, stream, n_launches);
     // int8 rows: as many sequences at a time as the widened rows have room for; the encoder goes with the first

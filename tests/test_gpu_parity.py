@@ -468,6 +468,30 @@ def test_errors_leave_state_untouched():
     assert e.value.status == 1
 
 
+@pytest.mark.parametrize("kernel", KERNELS, ids=lambda k: KNAME[k])
+def test_a_list_longer_than_max_seqs_is_refused_before_anything_is_copied(kernel):
+    """Staging slots and workspace rows are one per sequence id; a longer list (which names a sequence twice) is an argument error
+    of every call that fills them, and the next step of the context is right."""
+    w = synth.scaled(synth.CONFIGS["c3"], n_layers=1, batch=1, reuse_frac=0.0)
+    p = Pair(w, max_seqs=1, max_pages=2, max_pages_per_seq=2, kernel=kernel)
+    p.open([0])
+    p.prefill([0], 40)
+    n = 9
+    host = torch.zeros(n, w.n_q_heads * w.head_dim, dtype=p.s.dtype).pin_memory()
+    dev = host.cuda()
+    h, d, st, ctx = host.data_ptr(), dev.data_ptr(), p.s.stream(), p.s.ctx
+    before = ctx.launch_count()
+    for call in (lambda: ctx.step_layer_host(0, [0] * n, h, h, h, h, B.INCLUDE_CURRENT_EXACT, st),
+                 lambda: ctx.step_layer(0, [0] * n, d, d, d, d, B.INCLUDE_CURRENT_EXACT, st),
+                 lambda: ctx.decode_attention(0, [0] * n, d, d, 0, st),
+                 lambda: ctx.encode_append(0, [0] * n, 1, d, d, st)):
+        with pytest.raises(B.KvcarError) as e:
+            call()
+        assert e.value.status == 1
+    assert ctx.launch_count() == before
+    _check_step(p.decode_step([0], 0, fused=True), "bf16", "after refused calls")
+
+
 def test_device_side_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     """A bounded device-side wait that nothing completes: the kernel gives up after its limit (1 ms here), records a
     code in the status word and returns; kvcar_sync_status reports KVCAR_ERR_DEVICE_TIMEOUT exactly once, and the
