@@ -109,6 +109,7 @@ kvcar_status fail(kvcar_ctx *c, kvcar_status s, const std::string &msg) {
     return s;
 }
 kvcar_status cuda_fail(kvcar_ctx *c, cudaError_t e, const char *what) {
+    cudaGetLastError();  // reported here: the next launch's check must not meet it again
     return fail(c, KVCAR_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
@@ -416,6 +417,33 @@ bool layer_is_raw(const kvcar_ctx *c, int layer) {
 bool use_tensor_kernel(const kvcar_ctx *c) {
     if (c->kernel == KVCAR_KERNEL_GENERIC) return false;
     return c->tc.available || c->lat.available;
+}
+
+// Device address of `bytes` bytes of page-locked host memory at p; null where any of them lies outside the one page-locked range.
+char *mapped_host(void *p, size_t bytes) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (at.type != cudaMemoryTypeHost || !at.devicePointer) return nullptr;
+    typedef CUresult (*Fn)(void *, CUpointer_attribute, CUdeviceptr);
+    static const Fn attribute = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttribute", &fn, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<Fn>(fn);
+    }();
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    const CUdeviceptr a = (CUdeviceptr)(uintptr_t)p;
+    if (!attribute || attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, a) != CUDA_SUCCESS ||
+        attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, a) != CUDA_SUCCESS)
+        return nullptr;
+    return a >= start && a - start + bytes <= size ? (char *)at.devicePointer : nullptr;
 }
 
 // device address of the library's built-in scratch array on the current device (defined with the array, below)
@@ -1217,14 +1245,8 @@ kvcar_status kvcar_step_layer_host(kvcar_ctx *c, int32_t layer, const int32_t *s
     // A page-locked output is written by the step's last kernel itself: each value once, and a copy behind the kernel costs the stream
     // more than the writes do at every size (12 layers of GPT-2's shape, 128 tokens: batch 8, 12 KB, 538 us with the copy and 471
     // without; batch 256, 384 KB, 2425 and 2269).
-    char *out = dout;
-    cudaPointerAttributes at;
-    if (((uintptr_t)out_host & 15) == 0) {
-        if (cudaPointerGetAttributes(&at, out_host) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer)
-            out = (char *)at.devicePointer;
-        else
-            cudaGetLastError();
-    }
+    char *out = ((uintptr_t)out_host & 15) == 0 ? mapped_host(out_host, q_bytes) : nullptr;
+    if (!out) out = dout;
     kvcar_status s = kvcar_step_layer(c, layer, seqs, n_seqs, dk, dv, dq, out, flags, stream);
     if (ahead) c->ev_d_used[slot] = cudaEventRecord(c->ev_d[slot], st) == cudaSuccess;
     if (s != KVCAR_OK || out != dout) return s;

@@ -410,6 +410,40 @@ def test_host_buffer_steps_equal_device_steps(pinned_out):
     assert torch.equal(out, ref.cpu())
 
 
+def test_output_buffer_that_is_page_locked_in_part_is_not_written_by_a_kernel():
+    """The first page of an output buffer is registered, the rest is not: the output arrives by a copy (or the copy refuses such a
+    range), never from a kernel, and the context goes on.  The same buffer registered whole is written in place."""
+    import mmap
+    w = synth.scaled(synth.CONFIGS["c3"], n_layers=1, batch=2, reuse_frac=0.0)
+    seqs = [0, 1]
+    p = Pair(w, max_seqs=2, max_pages=4, max_pages_per_seq=2, with_oracle=False)
+    p.open(seqs)
+    p.prefill(seqs, 50)
+    dt, st, page = p.s.dtype, p.s.stream(), mmap.PAGESIZE
+    gen = torch.Generator().manual_seed(7)
+    ins = [torch.randn(s, generator=gen).to(dt).pin_memory()
+           for s in [(2, w.n_kv_heads, w.head_dim)] * 2 + [(2, w.n_q_heads, w.head_dim)]]
+    d, ref = [t.cuda() for t in ins], torch.empty_like(ins[2], device="cuda")
+    p.s.ctx.step_layer(0, seqs, *(t.data_ptr() for t in d), ref.data_ptr(), B.INCLUDE_CURRENT_EXACT, st)
+    mem = mmap.mmap(-1, 4 * page)
+    buf = torch.frombuffer(mem, dtype=dt)
+    start = (page - 256) // 2                       # 256 bytes of the output lie in the first page
+    out = buf[start:start + ins[2].numel()].view(ins[2].shape)
+    rt = torch.cuda.cudart()
+    for registered in (page, 4 * page):
+        assert int(rt.cudaHostRegister(buf.data_ptr(), registered, 0)) == 0
+        try:
+            p.s.ctx.step_layer_host(0, seqs, *(t.data_ptr() for t in ins), out.data_ptr(), B.INCLUDE_CURRENT_EXACT, st)
+            p.s.ctx.sync_status(st)
+            assert torch.equal(out, ref.cpu())
+        except B.KvcarError as e:
+            assert registered == page and e.status == 6
+        finally:
+            torch.cuda.synchronize()
+            rt.cudaHostUnregister(buf.data_ptr())
+        buf.zero_()
+
+
 def test_host_buffer_steps_mix_with_graph_replays():
     """A captured host-buffer step of layer 0, replayed behind queued work, and direct host-buffer steps of layer 1 behind it
     (more than the library has staging slots, whose copies run ahead of the stream): neither reads the other's inputs."""
