@@ -315,6 +315,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
                 if (!SPLIT) {
                     store_block(b64, 0);
                 } else {
+                    float2 rest = make_float2(0.f, 0.f);  // sum of what the first term leaves out: not finite if a value is not
 #pragma unroll
                     for (int plane = 0; plane < PREFILL_TC_PLANES; ++plane) {
 #pragma unroll
@@ -327,10 +328,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
                                 w[e] = pack_bf16(x0, x1);
                                 x0 -= __uint_as_float(w[e] << 16);  // what this term leaves out goes to the next plane
                                 x1 -= __uint_as_float(w[e] & 0xffff0000u);
+                                if (plane == 0) rest = __fadd2_rn(rest, make_float2(x0, x1));
                             }
                             stage_chunk(ch, w);
                         }
                         store_block(b64, (int64_t)plane * a.hid_rows * a.hid_pitch);
+                        // an infinity is whole in its first term (inf - inf would turn it into NaN in the next)
+                        if (plane == 0 && __any_sync(0xffffffffu, !(fabsf(rest.x + rest.y) <= 3.4e38f))) {
+#pragma unroll
+                            for (int i = 0; i < (SPLIT ? 64 : 32); ++i)
+                                if (!(fabsf(v[i]) <= 3.4e38f)) v[i] = 0.f;
+                        }
                     }
                 }
             }

@@ -71,3 +71,35 @@ def test_bulk_append_keeps_the_hidden_activations_in_fp32(batch, tokens):
     p.open(seqs)
     p.prefill(seqs, tokens)
     p.check_latents(seqs)
+
+
+@pytest.mark.parametrize("beta", [3.3e38, float("inf")], ids=["large", "infinite"])
+def test_bulk_append_with_hidden_values_at_the_end_of_the_range(beta, monkeypatch):
+    """One hidden value of every row is 3.3e38 or infinite.  The rows of the bulk call agree with those of one call per token, whose
+    hidden values stay in fp32: within one bf16 step, infinities in the same places."""
+    real = synth.make_stack_autoencoders
+
+    def ends(*a, **kw):
+        aes = real(*a, **kw)
+        for ae in aes.values():
+            ae["enc_bn"][1, 7] = beta
+            ae["enc_w2"][:, 7] = 2.0 ** -127        # every latent has a share of it, 2 where it is finite
+        return aes
+    monkeypatch.setattr(synth, "make_stack_autoencoders", ends)
+    w = synth.scaled(synth.CONFIGS["c3"], n_layers=1, batch=2, reuse_frac=0.0)
+    p = Pair(w, max_seqs=2, max_pages=2, max_pages_per_seq=1, with_oracle=False)
+    p.open([0, 1])
+    rows = np.stack([synth.make_kv(w, 0, which, 0, 0, 5) for which in (0, 1)])
+    p.append(0, [0], rows[0][None], rows[1][None])
+    p.advance([0], 5)
+    for t in range(5):
+        p.append(0, [1], rows[0][None, t:t + 1], rows[1][None, t:t + 1])
+        p.advance([1], 1)
+    for which in (0, 1):
+        c = p.s.pool_rows(0, which).float().cpu().numpy()
+        a, b = c[p.s.ctx.debug_locate(0, 0)[1]:][:5], c[p.s.ctx.debug_locate(1, 0)[1]:][:5]
+        assert not np.isnan(b).any()
+        np.testing.assert_array_equal(np.isinf(a), np.isinf(b))
+        assert np.isinf(b).all() == np.isinf(beta)
+        if np.isfinite(beta):
+            assert np.all(np.abs(a - b) <= 2.0 ** -7 * np.abs(b) + 1e-6)
