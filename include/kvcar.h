@@ -221,8 +221,11 @@ kvcar_status kvcar_advance(kvcar_ctx *ctx, const int32_t *seqs, int32_t n_seqs, 
  * probabilities in fp32 or as two bf16 terms; the flag lets them take one bf16
  * term of W4_h^T q (rounded to the storage type once per sequence and head),
  * KVCAR_ABSORBED_V (only together with KVCAR_ABSORBED) one bf16 term of the
- * probabilities.  With 17 to 32 query heads the probabilities have one term
- * anyway.  Kernels that restore the heads ignore the flags.
+ * probabilities.  bf16 rows with 17 to 32 query heads in groups of more than
+ * two take one term of the probabilities anyway.  The hidden vectors a are one
+ * bf16 term over bf16 rows and two over int8 rows (latent_quant), so that int8
+ * rows lose nothing against fp32 arithmetic but the rounding of the output.
+ * Kernels that restore the heads ignore the flags.
  */
 kvcar_status kvcar_decode_attention(kvcar_ctx *ctx, int32_t layer, const int32_t *seqs, int32_t n_seqs,
                                     const void *q, void *out, uint32_t flags, void *stream);

@@ -57,11 +57,14 @@
 // int8 latent rows (Eq. 4: x = (code - zero-point) / scale).  latent_widen_kernel, ahead of the front, writes code - z0 as bf16 rows
 // into the workspace, z0 the zero-point kept to [-128, 128]: whole numbers of at most 256, exact in bf16 (a row whose range holds
 // zero, as latents have it, has z0 = zero-point).  The hidden warps of the Q8 builds then apply 1 / scale per token, and where a row
-// has some of its zero-point left over, that times the weights' row sum: nothing is rounded that the fp32 form does not round.  12-layer step of the GPT-2 shape,
-// 8 x 1024 tokens: 763 us, 6404 us in fp32 on the CUDA cores.
+// has some of its zero-point left over, that times the weights' row sum.  The fp32 kernels that these builds stand in for keep hidden
+// vectors and probabilities in fp32, so here both are two bf16 terms (2^-17 of the value is left out; one term of the hidden vectors
+// made the outputs' error 1.8 times that of fp32 at queries of 8 times the usual size, two terms leave it where it was).  A job is 128
+// columns then: a pair of slabs of high terms, a pair of low ones, which S and U take into the same accumulators one after the other.
+// 12-layer step of the GPT-2 shape, 8 x 1024 tokens: 1024 us (763 with one term), 6404 us in fp32 on the CUDA cores.
 //
 // Warp roles: 0 loads of latents and query rows, 1 hidden products (leader CTA) and tensor memory, 2 weight loads,
-// 3 S and U products (leader CTA), 4-15 hidden warps, 16-23 output warps.  All waits are bounded and record a code in the
+// 3 S and U products (leader CTA), then the hidden warps (twelve; eight where a job is 128 columns) and eight output warps.  All waits are bounded and record a code in the
 // status word.
 #include <algorithm>
 #include <cmath>
@@ -79,17 +82,17 @@ namespace {
 
 constexpr int TILE = 128;                 // tokens per CTA tile
 constexpr int SLAB = 16384;               // 128 rows x 64 bf16, 128-byte swizzle
-constexpr int CN = 192;                   // hidden columns per job
-constexpr int CSLABS = CN / 64;
-constexpr int WSTAGE = CN / 2 * 128;      // this CTA's half of a weight slab
-constexpr int TM_OUT = 2 * CN;            // tensor-memory columns: hidden 0, 192; outputs 384, 448
-constexpr int HID_WARP = 4, N_HID = 4 * CSLABS, OUT_WARP = HID_WARP + N_HID, N_OUT = 8, N_WARPS = OUT_WARP + N_OUT;
-constexpr int NTHREADS = 32 * N_WARPS;
-constexpr int READY_BARS = 8;             // hidden jobs between their epilogue and their product: at most as many as slabs
+constexpr int HID_WARP = 4, N_OUT = 8;    // first hidden warp, output warps
+constexpr int READY_BARS = 8;             // jobs' terms between their epilogue and their product: at most as many as slabs
+
+// What follows from the hidden columns of a job: 192 where the hidden vector is one bf16 term, 128 where it is two (two slabs
+// of each term: U's products take their 128 features from a pair of slabs, so a job is one such pair per term).
+__host__ __device__ constexpr int wstage(int cn) { return cn / 2 * 128; }  // this CTA's half of a weight slab
+__host__ __device__ constexpr int n_threads(int cn) { return 32 * (HID_WARP + 4 * (cn / 64) + N_OUT); }
 
 // Query heads padded to NQ.  Up to 16: high and low terms of an operand are rows of one operand.  32: the terms of W4^T q
-// are two operands, and the probabilities have one term (groups of more than two heads, whose restoring form rounds
-// restored K, restored V and the probabilities to bf16: the same class).
+// are two operands, and so are those of the probabilities in the P2 builds.  The others take one term of the probabilities: bf16 rows
+// of groups of more than two heads, whose restoring form rounds restored K, restored V and the probabilities to bf16, the same class.
 __host__ __device__ constexpr int op_rows(int nq) { return nq <= 16 ? 2 * nq : nq; }  // operand rows of a CTA in S and U
 __host__ __device__ constexpr int wq_rows(int nq) { return 2 * nq; }                  // rows of W4^T q per sequence and source
 __host__ __device__ constexpr int wq_slab(int nq) { return wq_rows(nq) * 128; }       // one 64-column slab of them
@@ -231,18 +234,24 @@ struct __align__(8) Scratch {
     float lred[NQ][4];    // sums of the four lane quarters at the end of a run
 };
 
-// NQ: query heads padded.  NB: U blocks of 128 hidden features at most; fixes the registers of the running sums.
-template <int NQ, int NB, bool Q8>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
+// NQ: query heads padded.  NB: U blocks of 128 hidden features at most; fixes the registers of the running sums.  CN: hidden columns
+// of a job.  Q8: int8 rows, whose hidden vectors are two bf16 terms.  P2: two operands for the probabilities (NQ = 32).
+template <int NQ, int NB, int CN, bool Q8, bool P2>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
     decode_latent_kernel(const __grid_constant__ Params a) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    constexpr int R = op_rows(NQ), PSLAB = R * 128, QSLAB = wq_slab(NQ);
+    constexpr int R = op_rows(NQ), PSLAB = R * 128, QSLAB = wq_slab(NQ), WSTAGE = wstage(CN), CSLABS = CN / 64;
+    constexpr int TERMS = Q8 ? 2 : 1, P_SLABS = P2 ? 4 : 2;
+    constexpr int TM_OUT = 2 * CN;  // tensor-memory columns: hidden 0, CN; outputs 2 CN, 2 CN + 64
+    constexpr int N_HID = 4 * CSLABS, OUT_WARP = HID_WARP + N_HID;
+    static_assert(TERMS == 1 || CSLABS == 2, "a term of a job is a pair of slabs");
+    static_assert(!P2 || NQ > 16, "up to 16 heads both terms of the probabilities are rows of one operand");
 
     const uint32_t rank = blockIdx.x & 1u;
     const bool leader = rank == 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t s_z = smem_u32(smem_raw), s_h = s_z + a.nz * SLAB, s_w = s_h + a.nh * SLAB, s_q = s_w + a.nw * WSTAGE;
-    const uint32_t s_p = s_q + a.nqs * QSLAB, s_bar = s_p + 2 * PSLAB;
+    const uint32_t s_p = s_q + a.nqs * QSLAB, s_bar = s_p + P_SLABS * PSLAB;
     const uint32_t w_full = s_bar, w_empty = w_full + 8 * a.nw;
     const uint32_t z_full = w_empty + 8 * a.nw, z_empty = z_full + 8 * a.nz;
     const uint32_t q_full = z_empty + 8 * a.nz, q_empty = q_full + 8 * a.nqs;
@@ -525,6 +534,47 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
 #pragma unroll 1
                     for (int s = 0; s < list_of(0).n; ++s) {
                         const int m = list_of(0).src[s].m, ksm = (m + 63) >> 6, nk_last = ((m - 1) & 63) / 16 + 1;
+                        if constexpr (TERMS == 2) {
+#pragma unroll 1
+                            for (int sl0 = 0; sl0 < ksm; sl0 += CSLABS) {
+                                const int n_sl = min(CSLABS, ksm - sl0);
+                                uint32_t qs = qslot, qp = qphase;
+#pragma unroll 1
+                                for (int term = 0; term < TERMS; ++term) {  // both terms meet the same query slabs
+                                    hslot += hslot & 1u;
+                                    if (hslot == (uint32_t)a.nh) hslot = 0;
+                                    mbar_wait(h_ready + 8 * (h & 7u), (h >> 3) & 1u, a.status, &abort_flag, 0x604);
+                                    tc_fence_after();
+                                    ++h;
+                                    qs = qslot;
+                                    qp = qphase;
+#pragma unroll 1
+                                    for (int i = 0; i < n_sl; ++i) {
+                                        mbar_wait(q_full + 8 * qs, qp, a.status, &abort_flag, 0x60e);
+                                        const uint64_t da = h_desc + hslot * (SLAB >> 4), db = q_desc + qs * (QSLAB >> 4);
+                                        const int nk = sl0 + i + 1 < ksm ? 4 : nk_last;
+                                        if (begin)
+                                            umma_pair<0>(acc, da, db, idesc);
+                                        else
+                                            umma_pair<1>(acc, da, db, idesc);
+                                        begin = false;
+#pragma unroll 1
+                                        for (int t = 1; t < nk; ++t) umma_pair<1>(acc, da + 2u * t, db + 2u * t, idesc);
+                                        if (two && term == 0) {
+#pragma unroll 1
+                                            for (int t = 0; t < nk; ++t) umma_pair<1>(acc, da + 2u * t, db + (QSLAB / 2 >> 4) + 2u * t, idesc);
+                                        }
+                                        umma_commit_pair(h_free + 8 * hslot);
+                                        if (term + 1 == TERMS) umma_commit_pair(q_empty + 8 * qs);
+                                        if (++hslot == (uint32_t)a.nh) hslot = 0;
+                                        if (++qs == (uint32_t)a.nqs) { qs = 0; qp ^= 1u; }
+                                    }
+                                }
+                                qslot = qs;
+                                qphase = qp;
+                            }
+                            continue;
+                        }
 #pragma unroll 1
                         for (int sl = 0, in_job = 0; sl < ksm; ++sl) {
                             if (in_job == 0) {  // the job's slabs, written by both CTAs
@@ -564,6 +614,48 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
 #pragma unroll 1
                 for (int s = 0; s < (side_hi == 2 && on(it, 1) ? list_of(1).n : 0); ++s) {  // U
                     const int ksm = (list_of(1).src[s].m + 63) >> 6;
+                    if constexpr (TERMS == 2) {
+#pragma unroll 1
+                        for (int sl0 = 0; sl0 < ksm; sl0 += CSLABS) {
+                            const uint32_t ob = o & 1u, accu = tmem + TM_OUT + 64u * ob;
+#pragma unroll 1
+                            for (int term = 0; term < TERMS; ++term) {
+                                hslot += hslot & 1u;
+                                if (hslot == (uint32_t)a.nh) hslot = 0;
+                                mbar_wait(h_ready + 8 * (h & 7u), (h >> 3) & 1u, a.status, &abort_flag, 0x604);
+                                ++h;
+                                if (!p_seen) {
+                                    mbar_wait(p_ready, (uint32_t)tile_of(it, 1) & 1u, a.status, &abort_flag, 0x606);
+                                    p_seen = true;
+                                }
+                                if (term == 0) mbar_wait(o_empty + 8 * ob, ((o >> 1) & 1u) ^ 1u, a.status, &abort_flag, 0x605);
+                                tc_fence_after();
+                                uint64_t da = h_desc + hslot * (SLAB >> 4);  // as below
+                                da = (da & ~((uint64_t)0x3FFF << 16)) | ((uint64_t)(SLAB >> 4) << 16);
+                                if (term == 0)
+                                    umma_pair<0>(accu, da, p_desc, idesc_u);
+                                else
+                                    umma_pair<1>(accu, da, p_desc, idesc_u);
+#pragma unroll
+                                for (int t = 1; t < TILE / 16; ++t)
+                                    umma_pair<1>(accu, da + (uint64_t)(t * (16 * 128 >> 4)),
+                                                 p_desc + (uint64_t)((t >> 2) * (PSLAB >> 4) + (t & 3) * 2), idesc_u);
+                                if (P2 && term == 0 && a.two_terms_v) {
+#pragma unroll
+                                    for (int t = 0; t < TILE / 16; ++t)
+                                        umma_pair<1>(accu, da + (uint64_t)(t * (16 * 128 >> 4)),
+                                                     p_desc + (uint64_t)((2 + (t >> 2)) * (PSLAB >> 4) + (t & 3) * 2), idesc_u);
+                                }
+                                umma_commit_pair(h_free + 8 * hslot);
+                                if (sl0 + 1 < ksm) umma_commit_pair(h_free + 8 * (hslot + 1));
+                                hslot += min(CSLABS, ksm - sl0);
+                                if (hslot == (uint32_t)a.nh) hslot = 0;
+                            }
+                            umma_commit_pair(o_full + 8 * ob);
+                            ++o;
+                        }
+                        continue;
+                    }
                     hslot += hslot & 1u;  // slabs go in pairs: a source starts at an even place
                     if (hslot == (uint32_t)a.nh) hslot = 0;
 #pragma unroll 1
@@ -607,7 +699,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         // where this lane's row of the 8 x 8 blocks goes (row lane % 8 of 8, block lane / 8 of 4; 128-byte swizzle)
         const uint32_t st_row = (lane_base + (lane & 7)) * 128u;
         const uint32_t ready_leader = map_to_cta(h_ready, 0), empty_leader = map_to_cta(t_empty, 0);
-        uint32_t hslot = 0, hphase = 0, h = 0;
+        uint32_t hslot = 0, hphase = 0, h = 0, r_job = 0;  // h: accumulators read, r_job: terms written
         TileWalk tw;
         tw.start(a.sq, my_first);
         auto wide_row = [&]() { return !Q8 || tw.left == 0 ? 0 : (tw.first(a.sq, tw.si) + tw.chunk) * TILE; };
@@ -663,7 +755,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                         tc_fence_after();
                         // The accumulator is read, and given back, before the job's places in the ring are free: the next
                         // hidden products do not wait for the products that still read those places.
-                        uint32_t w[2][16];
+                        uint32_t w[TERMS][2][16];
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {  // 32 columns (u / 2) x 16 of the warp's 32 rows (u % 2)
                             const int half = u >> 1, f = u & 1;
@@ -699,14 +791,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                                     const float iv = inv[2 * f + i];
                                     const float2 x = Q8 ? __ffma2_rn(h2, make_float2(iv, iv), t[j]) : __fadd2_rn(h2, t[j]);
                                     const float2 y = __fmul2_rn(x, slope2);
-                                    w[half][8 * f + e] = pack_bf16(fmaxf(x.x, y.x), fmaxf(x.y, y.y));  // slope <= 1
+                                    const float2 v = make_float2(fmaxf(x.x, y.x), fmaxf(x.y, y.y));  // slope <= 1
+                                    const uint32_t hi = pack_bf16(v.x, v.y);
+                                    w[0][half][8 * f + e] = hi;
+                                    if (TERMS == 2)
+                                        w[TERMS - 1][half][8 * f + e] = pack_bf16(v.x - __uint_as_float(hi << 16), v.y - __uint_as_float(hi & 0xffff0000u));
                                 }
                             }
                         }
                         if (clear) {
 #pragma unroll
                             for (int e = 0; e < 32; ++e)
-                                if ((int)lane_base + 8 * ((e & 15) >> 2) + (lane >> 2) >= valid) w[e >> 4][e & 15] = 0u;
+                                if ((int)lane_base + 8 * ((e & 15) >> 2) + (lane >> 2) >= valid) {
+                                    w[0][e >> 4][e & 15] = 0u;
+                                    w[TERMS - 1][e >> 4][e & 15] = 0u;
+                                }
                         }
                         if (halves == 0) {
                             tc_fence_before();
@@ -717,24 +816,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                         // skipped would let a later wait on the same place pass one phase early.
                         // One lane per place.
                         const int n_sl = (nc + 63) >> 6;
-                        const uint32_t nh = (uint32_t)a.nh, place = hslot + lane < nh ? hslot + lane : hslot + lane - nh;
-                        if (lane < n_sl) mbar_wait(h_free + 8 * place, ((hphase >> place) & 1u) ^ 1u, a.status, &abort_flag, 0x60a);
-                        const uint32_t slot = hslot + my_slab < nh ? hslot + my_slab : hslot + my_slab - nh;
-                        const uint32_t passed = ((1u << n_sl) - 1u) << hslot;
-                        hphase ^= (passed | passed >> nh) & ((1u << nh) - 1u);
-                        hslot = hslot + n_sl < nh ? hslot + n_sl : hslot + n_sl - nh;
-                        __syncwarp();
-                        const uint32_t dst = s_h + slot * SLAB + st_row;
+                        const uint32_t nh = (uint32_t)a.nh;
 #pragma unroll
-                        for (int half = 0; half < 2; ++half)
-                            if (half < halves) {
-#pragma unroll
-                                for (int i = 0; i < 4; ++i)
-                                    stmatrix_x4(dst + (uint32_t)(((4 * half + (lane >> 3)) ^ (lane & 7)) << 4) + 1024u * i, w[half] + 4 * i);
+                        for (int term = 0; term < TERMS; ++term) {
+                            if (TERMS == 2) {
+                                hslot += hslot & 1u;
+                                if (hslot == nh) hslot = 0;
                             }
-                        fence_async_smem();
-                        __syncwarp();
-                        if (elect_one()) mbar_arrive_remote(ready_leader + 8 * (h & 7u));
+                            const uint32_t place = hslot + lane < nh ? hslot + lane : hslot + lane - nh;
+                            if (lane < n_sl) mbar_wait(h_free + 8 * place, ((hphase >> place) & 1u) ^ 1u, a.status, &abort_flag, 0x60a);
+                            const uint32_t slot = hslot + my_slab < nh ? hslot + my_slab : hslot + my_slab - nh;
+                            const uint32_t passed = ((1u << n_sl) - 1u) << hslot;
+                            hphase ^= (passed | passed >> nh) & ((1u << nh) - 1u);
+                            hslot = hslot + n_sl < nh ? hslot + n_sl : hslot + n_sl - nh;
+                            __syncwarp();
+                            const uint32_t dst = s_h + slot * SLAB + st_row;
+#pragma unroll
+                            for (int half = 0; half < 2; ++half)
+                                if (half < halves) {
+#pragma unroll
+                                    for (int i = 0; i < 4; ++i)
+                                        stmatrix_x4(dst + (uint32_t)(((4 * half + (lane >> 3)) ^ (lane & 7)) << 4) + 1024u * i, w[term][half] + 4 * i);
+                                }
+                            fence_async_smem();
+                            __syncwarp();
+                            if (elect_one()) mbar_arrive_remote(ready_leader + 8 * (r_job & 7u));
+                            ++r_job;
+                        }
                     }
                 }
             }
@@ -823,6 +931,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                     const uint32_t ql = qr + NQ;
                     const __nv_bfloat16 lo = __float2bfloat16_rn(low_v ? p - __bfloat162float(hi) : 0.f);
                     st_smem_u16(pbase + ql * 128u + (((t6 >> 3) ^ (ql & 7u)) << 4), __bfloat16_as_ushort(lo));
+                } else if (P2) {  // an operand of its own, behind the high terms
+                    const __nv_bfloat16 lo = __float2bfloat16_rn(p - __bfloat162float(hi));
+                    st_smem_u16(pbase + 2 * PSLAB + qr * 128u + (((t6 >> 3) ^ (qr & 7u)) << 4), __bfloat16_as_ushort(lo));
                 }
             }
             fence_async_smem();
@@ -1275,16 +1386,25 @@ __global__ void __launch_bounds__(256) latent_widen_kernel(const __grid_constant
 }
 
 using Kernel = void (*)(const Params);
-const Kernel kernels[2][6] = {{decode_latent_kernel<12, 2, false>, decode_latent_kernel<12, 5, false>, decode_latent_kernel<16, 5, false>,
-                               decode_latent_kernel<16, 8, false>, decode_latent_kernel<32, 2, false>, decode_latent_kernel<32, 3, false>},
-                              {decode_latent_kernel<12, 2, true>, decode_latent_kernel<12, 5, true>, decode_latent_kernel<16, 5, true>,
-                               decode_latent_kernel<16, 8, true>, decode_latent_kernel<32, 2, true>, decode_latent_kernel<32, 3, true>}};
-constexpr int KERNEL_NQ[] = {12, 12, 16, 16, 32, 32}, KERNEL_NB[] = {2, 5, 5, 8, 2, 3};
-constexpr int N_KERNELS = 6;
+// Builds, the narrowest first of each kind.
+struct Build {
+    int nq, nb, cn;
+    bool quant, p2;
+    Kernel kernel;
+};
+template <int NQ, int NB, int CN, bool Q8, bool P2>
+constexpr Build build() {
+    return {NQ, NB, CN, Q8, P2, decode_latent_kernel<NQ, NB, CN, Q8, P2>};
+}
+const Build builds[] = {build<12, 2, 192, false, false>(), build<12, 5, 192, false, false>(), build<16, 5, 192, false, false>(),
+                        build<16, 8, 192, false, false>(), build<32, 2, 192, false, false>(), build<32, 3, 192, false, false>(),
+                        build<12, 2, 128, true, false>(),  build<12, 5, 128, true, false>(),  build<16, 5, 128, true, false>(),
+                        build<16, 8, 128, true, false>(),  build<32, 2, 128, true, true>(),   build<32, 3, 128, true, true>()};
+constexpr int N_BUILDS = sizeof(builds) / sizeof(builds[0]);
 
-int smem_bytes(int nq, int nz, int nh, int nw, int nqs) {
-    const int scratch = nq == 12 ? sizeof(Scratch<12>) : nq == 16 ? sizeof(Scratch<16>) : sizeof(Scratch<32>);
-    return (nz + nh) * SLAB + nw * WSTAGE + nqs * wq_slab(nq) + 2 * op_rows(nq) * 128 +
+int smem_bytes(const Build &b, int nz, int nh, int nw, int nqs) {
+    const int scratch = b.nq == 12 ? sizeof(Scratch<12>) : b.nq == 16 ? sizeof(Scratch<16>) : sizeof(Scratch<32>);
+    return (nz + nh) * SLAB + nw * wstage(b.cn) + nqs * wq_slab(b.nq) + (b.p2 ? 4 : 2) * op_rows(b.nq) * 128 +
            8 * (2 * (nz + nw + nqs) + nh + READY_BARS + 9) + scratch;
 }
 constexpr int SMEM_MAX = 227 * 1024;
@@ -1375,6 +1495,7 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
         LatLayerCfg &lc = st.cfg[l];
         bool ok = true;
         int ks = 0, lm = 0, lmk = 0, chunks = 0;
+        const int cn = st.quant ? 128 : 192;
         for (int w = 0; w < 2 && ok; ++w) {
             const WhichPlan &wp = plans[l].w[w];
             ok = wp.n_src > 0 && wp.n_src <= LT_MAX_SRC;
@@ -1411,26 +1532,27 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
                 }
                 ok = (st.quant ? encode_bf16_map(fn, &ly.pool[w][s], reinterpret_cast<__nv_bfloat16 *>(st.wide) + region * max_d, wide_rows, sp.d, max_d)
                                : encode_bf16_map(fn, &ly.pool[w][s], sp.pool, pool_rows, sp.width, sp.width)) &&
-                     encode_bf16_map(fn, &ly.w1[w][s], sp.w1n, sp.m, sp.d, sp.d, CN / 2);
+                     encode_bf16_map(fn, &ly.w1[w][s], sp.w1n, sp.m, sp.d, sp.d, cn / 2);
                 ks = std::max(ks, (sp.d + 63) / 64);
                 lm = std::max(lm, sp.m);
                 if (w == 0) lmk = std::max(lmk, sp.m);
-                chunks = std::max(chunks, (sp.m + CN - 1) / CN);
+                chunks = std::max(chunks, (sp.m + cn - 1) / cn);
             }
         }
         if (!ok) continue;
         int v = 0;
-        while (v < N_KERNELS && (KERNEL_NQ[v] < st.nq || KERNEL_NB[v] * 128 < lm)) ++v;
-        if (v == N_KERNELS || KERNEL_NQ[v] != st.nq) continue;
+        while (v < N_BUILDS && (builds[v].nq != st.nq || builds[v].quant != st.quant || builds[v].nb * 128 < lm)) ++v;
+        if (v == N_BUILDS) continue;
         // Staging places.  A side's latents stay for all its chunks (nz >= their slabs).  One-chunk layers get places for the
         // other side's latents and six hidden slabs, because their jobs are shorter than the way from S to P; the others four
-        // hidden slabs: a chunk's three and the one its predecessor may leave unpaired.
+        // hidden slabs: a chunk's three and the one its predecessor may leave unpaired, or a chunk's two terms of two.
         int nh = chunks == 1 ? 6 : 4, nz = chunks == 1 ? std::max(4, 2 * ks) : ks, nw = 4, nqs = 4;
-        auto fits = [&]() { return smem_bytes(st.nq, nz, nh, nw, nqs) <= SMEM_MAX; };
+        auto fits = [&]() { return smem_bytes(builds[v], nz, nh, nw, nqs) <= SMEM_MAX; };
         while (nw > 3 && !fits()) --nw;
         while (nqs > 2 && !fits()) --nqs;
         while (nz > ks && !fits()) --nz;
         while (nw > 2 && !fits()) --nw;
+        if (!fits() && st.quant) nh = 2;  // one term of a job at a time
         if (!fits()) continue;
         while (nqs < 12 && (++nqs, fits())) {}
         if (!fits()) --nqs;
@@ -1438,11 +1560,11 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
         lc.nh = (uint8_t)nh;
         lc.nw = (uint8_t)nw;
         lc.nqs = (uint8_t)nqs;
-        lc.smem = std::max(smem_bytes(st.nq, nz, nh, nw, nqs), 120 * 1024);  // one CTA per SM: each takes all of tensor memory
+        lc.smem = std::max(smem_bytes(builds[v], nz, nh, nw, nqs), 120 * 1024);  // one CTA per SM: each takes all of tensor memory
         lc.variant = (uint8_t)v;
         lc.max_m = lm;
         lc.max_mk = lmk;
-        if (cudaFuncSetAttribute(kernels[st.quant][v], cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess) {
+        if (cudaFuncSetAttribute(builds[v].kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess) {
             cudaGetLastError();
             continue;
         }
@@ -1460,15 +1582,15 @@ bool lat_layer_supported(const LatState &st, int layer, uint32_t flags) {
 
 namespace {
 
-// A side's hidden columns in `n` parts of whole 192-column chunks, of about the same number of products each; a part holds one
+// A side's hidden columns in `n` parts of whole chunks of `cn` columns, of about the same number of products each; a part holds one
 // range of columns per source at most (the ranges of a source follow one another).  False where a part would be empty.
-bool split_side(const LatList &all, int n, LatList *out) {
+bool split_side(const LatList &all, int cn, int n, LatList *out) {
     int total = 0, done = 0;
     for (int s = 0; s < all.n; ++s) total += (all.src[s].d + 63) / 64 * ((all.src[s].m + 63) / 64);
     for (int p = 0; p < n; ++p) out[p].n = 0;
     for (int s = 0; s < all.n; ++s)
-        for (int c0 = 0; c0 < all.src[s].m; c0 += CN) {
-            const int w = std::min(CN, all.src[s].m - c0), cost = (all.src[s].d + 63) / 64 * ((w + 63) / 64);
+        for (int c0 = 0; c0 < all.src[s].m; c0 += cn) {
+            const int w = std::min(cn, all.src[s].m - c0), cost = (all.src[s].d + 63) / 64 * ((w + 63) / 64);
             LatList &l = out[std::min(n - 1, (int)((int64_t)(2 * done + cost) * n / (2 * total)))];  // by the chunk's middle
             done += cost;
             if (l.n > 0 && l.src[l.n - 1].map == all.src[s].map) {
@@ -1486,9 +1608,9 @@ bool split_side(const LatList &all, int n, LatList *out) {
         if (out[p].n == 0) return false;
     return true;
 }
-int count_chunks(const LatList &l) {
+int count_chunks(const LatList &l, int cn) {
     int n = 0;
-    for (int s = 0; s < l.n; ++s) n += (l.src[s].m + CN - 1) / CN;
+    for (int s = 0; s < l.n; ++s) n += (l.src[s].m + cn - 1) / cn;
     return n;
 }
 
@@ -1499,6 +1621,7 @@ static cudaError_t launch_group(LatState &st, const DecodeArgs &a, const SeqList
                                 const LatEncode *enc_in, cudaStream_t stream, int *n_launches) {
     const LatLayerCfg &lc = st.cfg[layer];
     const LatLayer &ly = st.layer[layer];
+    const Build &b = builds[lc.variant];
     Params p;
     fill_seqs(p.sq, seqs, lens, st.n_sms);
     const bool two_k = !(a.flags & KVCAR_ABSORBED), two_v = !((a.flags & KVCAR_ABSORBED) && (a.flags & KVCAR_ABSORBED_V));
@@ -1569,26 +1692,26 @@ static cudaError_t launch_group(LatState &st, const DecodeArgs &a, const SeqList
     // are spread over as many clusters as there is room for.  The V launch starts beside the K launch (all of whose blocks run by
     // then), does its hidden layer meanwhile and waits for the K launch only before it sums the parts of the scores.  12-layer step
     // of the GPT-2 shape at 1 / 8 x 1024 tokens: 371 / 649 us, 625 / 712 us with one cluster per pair.
-    int kp = std::min({(slots / pairs + 1) / 2, count_chunks(ly.list[0]), LT_MAX_PARTS});
-    int vp = std::min({slots / pairs - kp, count_chunks(ly.list[1]), LT_MAX_PARTS});
+    int kp = std::min({(slots / pairs + 1) / 2, count_chunks(ly.list[0], b.cn), LT_MAX_PARTS});
+    int vp = std::min({slots / pairs - kp, count_chunks(ly.list[1], b.cn), LT_MAX_PARTS});
     *n_launches += 3;
     if (p.sq.per == 1 && kp >= 1 && vp >= 1) {
         p.mode = MODE_K;
-        while (!split_side(ly.list[0], kp, p.list)) --kp;
+        while (!split_side(ly.list[0], b.cn, kp, p.list)) --kp;
         p.n_parts = p.k_parts = kp;
-        err = launch_pdl(kernels[st.quant][lc.variant], dim3(2 * pairs * kp), NTHREADS, lc.smem, stream, p);
+        err = launch_pdl(b.kernel, dim3(2 * pairs * kp), n_threads(b.cn), lc.smem, stream, p);
         if (err != cudaSuccess) return err;
         p.mode = MODE_V;
-        while (!split_side(ly.list[1], vp, p.list)) --vp;
+        while (!split_side(ly.list[1], b.cn, vp, p.list)) --vp;
         p.n_parts = vp;
-        err = launch_pdl(kernels[st.quant][lc.variant], dim3(2 * pairs * vp), NTHREADS, lc.smem, stream, p);
+        err = launch_pdl(b.kernel, dim3(2 * pairs * vp), n_threads(b.cn), lc.smem, stream, p);
         ++*n_launches;
     } else {
         p.mode = MODE_BOTH;
         p.n_parts = p.k_parts = 1;
         p.list[0] = ly.list[0];
         p.list[1] = ly.list[1];
-        err = launch_pdl(kernels[st.quant][lc.variant], dim3(2 * pairs), NTHREADS, lc.smem, stream, p);
+        err = launch_pdl(b.kernel, dim3(2 * pairs), n_threads(b.cn), lc.smem, stream, p);
     }
     if (err != cudaSuccess) return err;
     // ---- back
