@@ -10,7 +10,7 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libkvcar.so")
-TRACE_LIB = os.path.join(PKG, "libkvcar_trace.so")  # the same sources with -DKVCAR_TC_TRACE (time stamps in the tensor kernel)
+TRACE_LIB = os.path.join(PKG, "libkvcar_trace.so")  # the same sources with -DKVCAR_TRACE (time stamps in the latent-attention kernel)
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-cudart", "static", "--expt-relaxed-constexpr"]
 
@@ -31,7 +31,7 @@ def needs_build(lib: str = LIB) -> bool:
 
 
 def build(force: bool = False, verbose: bool = False, trace: bool = False) -> str:
-    """trace: build libkvcar_trace.so instead, whose tensor kernel records time stamps (python -m
+    """trace: build libkvcar_trace.so instead, whose latent-attention kernel records time stamps (python -m
     paper_2512_06727_b200.trace reads them); the regular library carries none of that code."""
     lib = TRACE_LIB if trace else LIB
     if not force and not needs_build(lib):
@@ -44,7 +44,7 @@ def build(force: bool = False, verbose: bool = False, trace: bool = False) -> st
     for src in _sources():
         obj = os.path.join(bdir, os.path.basename(src)[:-3] + ".o")
         objs.append(obj)
-        cmd = [nvcc, *NVCC_FLAGS, *(["-DKVCAR_TC_TRACE"] if trace else []), "-I", os.path.join(ROOT, "include"), "-I", CSRC,
+        cmd = [nvcc, *NVCC_FLAGS, *(["-DKVCAR_TRACE"] if trace else []), "-I", os.path.join(ROOT, "include"), "-I", CSRC,
                "-c", src, "-o", obj]
         if verbose:
             cmd.insert(1, "-Xptxas=-v")

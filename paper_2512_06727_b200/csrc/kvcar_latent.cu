@@ -235,6 +235,34 @@ struct __align__(8) Scratch {
     float lred[NQ][4];    // sums of the four lane quarters at the end of a run
 };
 
+// ---------------------------------------------------------------------------- optional time stamps
+// Compiled with -DKVCAR_TRACE, six threads of one cluster (in both CTAs: the two loading ones, the two issuing ones of the leader,
+// lane 0 of the first hidden and of the first output warp) record (clock64 << 8) | tag at the points marked TR;
+// kvcar_debug_trace_select picks the cluster, kvcar_debug_trace_dump fetches the records of the last launch.  Without the macro the
+// marks compile to nothing.  Tags: loads 2 = a latent or weight slab's load issued, 3 = a query slab's; issuers 0x10 | kind = the
+// accumulator is free, a job begins (kind 1 = hidden chunk, 3 = S, 4 = a block of U), 0x30 = a slab's operands are in place, 0x31 = its
+// products and releases are issued, 0x19 = job committed; hidden and output warps (kind << 4) | phase with kind 4 = hidden chunk,
+// 7 = S and its probabilities, 8 = a block of U and phase 0 = waits for the job, 1 = job seen complete, 2 = accumulator read and given
+// back, 3 = done with the job.
+enum { TR_ROWS, TR_WEIGHTS, TR_HIDDEN_ISSUE, TR_HIDDEN, TR_OUT_ISSUE, TR_OUT, TR_ROLES };
+#ifdef KVCAR_TRACE
+constexpr int TRACE_LEN = 4096;
+__device__ unsigned long long g_trace[2][TR_ROLES][TRACE_LEN];
+__device__ int g_trace_n[2][TR_ROLES];
+__device__ int g_trace_cluster = 0;
+#define TR(role, tag)                                                                                       \
+    do {                                                                                                    \
+        if (tr_on) {                                                                                        \
+            if (tr_cnt < TRACE_LEN) g_trace[rank][role][tr_cnt++] = ((unsigned long long)clock64() << 8) | (unsigned)(tag); \
+            g_trace_n[rank][role] = tr_cnt;                                                                 \
+        }                                                                                                   \
+    } while (0)
+#else
+#define TR(role, tag) \
+    do {              \
+    } while (0)
+#endif
+
 // NQ: query heads padded.  NB: U blocks of 128 hidden features at most; fixes the registers of the running sums.  CN: hidden columns
 // of a job.  Q8: int8 rows, whose hidden vectors are two bf16 terms.  P2: two operands for the probabilities (NQ = 32).
 template <int NQ, int NB, int CN, bool Q8, bool P2>
@@ -251,6 +279,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
     const uint32_t rank = blockIdx.x & 1u;
     const bool leader = rank == 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#ifdef KVCAR_TRACE
+    // one thread of warps 0 to 3 runs their loops
+    const bool tr_on = (int)(blockIdx.x >> 1) == g_trace_cluster && (warp < HID_WARP || ((warp == HID_WARP || warp == OUT_WARP) && lane == 0));
+    int tr_cnt = 0;
+#endif
     const uint32_t s_z = smem_u32(smem_raw), s_h = s_z + a.nz * SLAB, s_w = s_h + a.nh * SLAB, s_q = s_w + a.nw * WSTAGE;
     const uint32_t s_p = s_q + a.nqs * QSLAB, s_bar = s_p + P_SLABS * PSLAB;
     const uint32_t w_full = s_bar, w_empty = w_full + 8 * a.nw;
@@ -366,6 +399,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                     const bool behind = tile_of(z.it, z.side) < z.it;  // the tile before
                     tma_load_2d_pair(dst, map, z.k * 64, behind ? prow[0] : row[0], fb);
                     tma_load_2d_pair(dst + SLAB / 2, map, z.k * 64, behind ? prow[1] : row[1], fb);
+                    TR(TR_ROWS, 2);
                     if (++zslot == (uint32_t)a.nz) { zslot = 0; zphase ^= 1u; }
                     const int ks1 = (zp_.d + 63) >> 6;
                     if (++z.k == ks1) {
@@ -414,6 +448,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                     const uint32_t fb = map_to_cta(q_full + 8 * qslot, 0), dst = s_q + qslot * QSLAB;
                     tma_load_2d_pair(dst, &a.tm_wq, x, y, fb);
                     if (NQ > 16 && low_k) tma_load_2d_pair(dst + QSLAB / 2, &a.tm_wq, x, y + R, fb);
+                    TR(TR_ROWS, 3);
                     if (++qslot == (uint32_t)a.nqs) { qslot = 0; qphase ^= 1u; }
                     if (++q.k == (sp.m + 63) >> 6) {
                         q.k = 0;
@@ -463,6 +498,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                                 mbar_wait(w_empty + 8 * slot, phase ^ 1u, a.status, &abort_flag, 0x602);
                                 if (leader) mbar_expect_tx(w_full + 8 * slot, 2 * WSTAGE);
                                 tma_load_2d_pair(s_w + slot * WSTAGE, map, ks * 64, y, map_to_cta(w_full + 8 * slot, 0));
+                                TR(TR_WEIGHTS, 2);
                                 if (++slot == (uint32_t)a.nw) { slot = 0; phase ^= 1u; }
                             }
                         }
@@ -488,12 +524,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                             const uint32_t buf = h & 1u, acc = tmem + CN * buf, idesc = make_idesc(256, min(CN, m - c0));
                             mbar_wait(t_empty + 8 * buf, ((h >> 1) & 1u) ^ 1u, a.status, &abort_flag, 0x607);
                             tc_fence_after();
+                            TR(TR_HIDDEN_ISSUE, 0x11);
                             zs = zslot;  // the source's latent slabs: places zslot ..
                             zp = zphase;
 #pragma unroll 1
                             for (int ks = 0; ks < ks1; ++ks) {
                                 if (first) mbar_wait(z_full + 8 * zs, zp, a.status, &abort_flag, 0x608);
                                 mbar_wait(w_full + 8 * wslot, wphase, a.status, &abort_flag, 0x603);
+                                TR(TR_HIDDEN_ISSUE, 0x30);
                                 const uint64_t da = z_desc + zs * (SLAB >> 4), db = w_desc + wslot * (WSTAGE >> 4);
                                 if (ks == 0)
                                     umma_pair<0>(acc, da, db, idesc);
@@ -509,10 +547,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                                 }
                                 umma_commit_pair(w_empty + 8 * wslot);
                                 if (last) umma_commit_pair(z_empty + 8 * zs);
+                                TR(TR_HIDDEN_ISSUE, 0x31);
                                 if (++wslot == (uint32_t)a.nw) { wslot = 0; wphase ^= 1u; }
                                 if (++zs == (uint32_t)a.nz) { zs = 0; zp ^= 1u; }
                             }
                             umma_commit_pair(t_full + 8 * buf);
+                            TR(TR_HIDDEN_ISSUE, 0x19);
                         }
                         zslot = zs;
                         zphase = zp;
@@ -531,6 +571,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                 if (side_lo == 0 && on(it, 0)) {  // S
                     const uint32_t ob = o & 1u, acc = tmem + TM_OUT + 64u * ob;
                     mbar_wait(o_empty + 8 * ob, ((o >> 1) & 1u) ^ 1u, a.status, &abort_flag, 0x605);
+                    TR(TR_OUT_ISSUE, 0x13);
                     bool begin = true;
 #pragma unroll 1
                     for (int s = 0; s < list_of(0).n; ++s) {
@@ -552,6 +593,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
 #pragma unroll 1
                                     for (int i = 0; i < n_sl; ++i) {
                                         mbar_wait(q_full + 8 * qs, qp, a.status, &abort_flag, 0x60e);
+                                        TR(TR_OUT_ISSUE, 0x30);
                                         const uint64_t da = h_desc + hslot * (SLAB >> 4), db = q_desc + qs * (QSLAB >> 4);
                                         const int nk = sl0 + i + 1 < ksm ? 4 : nk_last;
                                         if (begin)
@@ -567,6 +609,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                                         }
                                         umma_commit_pair(h_free + 8 * hslot);
                                         if (term + 1 == TERMS) umma_commit_pair(q_empty + 8 * qs);
+                                        TR(TR_OUT_ISSUE, 0x31);
                                         if (++hslot == (uint32_t)a.nh) hslot = 0;
                                         if (++qs == (uint32_t)a.nqs) { qs = 0; qp ^= 1u; }
                                     }
@@ -585,6 +628,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                             }
                             if (++in_job == CSLABS) in_job = 0;
                             mbar_wait(q_full + 8 * qslot, qphase, a.status, &abort_flag, 0x60e);
+                            TR(TR_OUT_ISSUE, 0x30);
                             const uint64_t da = h_desc + hslot * (SLAB >> 4), db = q_desc + qslot * (QSLAB >> 4);
                             if (begin)
                                 umma_pair<0>(acc, da, db, idesc);
@@ -604,11 +648,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                             }
                             umma_commit_pair(h_free + 8 * hslot);
                             umma_commit_pair(q_empty + 8 * qslot);
+                            TR(TR_OUT_ISSUE, 0x31);
                             if (++hslot == (uint32_t)a.nh) hslot = 0;
                             if (++qslot == (uint32_t)a.nqs) { qslot = 0; qphase ^= 1u; }
                         }
                     }
                     umma_commit_pair(o_full + 8 * ob);
+                    TR(TR_OUT_ISSUE, 0x19);
                     ++o;
                 }
                 bool p_seen = false;
@@ -629,8 +675,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                                     mbar_wait(p_ready, (uint32_t)tile_of(it, 1) & 1u, a.status, &abort_flag, 0x606);
                                     p_seen = true;
                                 }
-                                if (term == 0) mbar_wait(o_empty + 8 * ob, ((o >> 1) & 1u) ^ 1u, a.status, &abort_flag, 0x605);
+                                if (term == 0) {
+                                    mbar_wait(o_empty + 8 * ob, ((o >> 1) & 1u) ^ 1u, a.status, &abort_flag, 0x605);
+                                    TR(TR_OUT_ISSUE, 0x14);
+                                }
                                 tc_fence_after();
+                                TR(TR_OUT_ISSUE, 0x30);
                                 uint64_t da = h_desc + hslot * (SLAB >> 4);  // as below
                                 da = (da & ~((uint64_t)0x3FFF << 16)) | ((uint64_t)(SLAB >> 4) << 16);
                                 if (term == 0)
@@ -649,10 +699,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                                 }
                                 umma_commit_pair(h_free + 8 * hslot);
                                 if (sl0 + 1 < ksm) umma_commit_pair(h_free + 8 * (hslot + 1));
+                                TR(TR_OUT_ISSUE, 0x31);
                                 hslot += min(CSLABS, ksm - sl0);
                                 if (hslot == (uint32_t)a.nh) hslot = 0;
                             }
                             umma_commit_pair(o_full + 8 * ob);
+                            TR(TR_OUT_ISSUE, 0x19);
                             ++o;
                         }
                         continue;
@@ -677,6 +729,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                         const uint32_t ob = o & 1u, accu = tmem + TM_OUT + 64u * ob, h0 = hs & ~1u;
                         mbar_wait(o_empty + 8 * ob, ((o >> 1) & 1u) ^ 1u, a.status, &abort_flag, 0x605);
                         tc_fence_after();
+                        TR(TR_OUT_ISSUE, 0x14);
+                        TR(TR_OUT_ISSUE, 0x30);
                         // rows = features: two 64-feature atoms a slab apart, 8-token groups 1 KB apart (MN-major)
                         uint64_t da = h_desc + h0 * (SLAB >> 4);
                         da = (da & ~((uint64_t)0x3FFF << 16)) | ((uint64_t)(SLAB >> 4) << 16);
@@ -688,6 +742,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                         umma_commit_pair(h_free + 8 * h0);
                         if (hs != h0) umma_commit_pair(h_free + 8 * hs);
                         umma_commit_pair(o_full + 8 * ob);
+                        TR(TR_OUT_ISSUE, 0x31);
+                        TR(TR_OUT_ISSUE, 0x19);
                         ++o;
                     }
                 }
@@ -751,9 +807,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                             ta = __ldg(t4);
                             tb = __ldg(t4 + 1);
                         }
+                        TR(TR_HIDDEN, 0x40);
                         mbar_wait(t_full + 8 * buf, (h >> 1) & 1u, a.status, &abort_flag, 0x609);
                         __syncwarp();
                         tc_fence_after();
+                        TR(TR_HIDDEN, 0x41);
                         // The accumulator is read, and given back, before the job's places in the ring are free: the next
                         // hidden products do not wait for the products that still read those places.
                         uint32_t w[TERMS][2][16];
@@ -813,6 +871,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                             __syncwarp();
                             if (elect_one()) mbar_arrive_remote(empty_leader + 8 * buf);
                         }
+                        TR(TR_HIDDEN, 0x42);
                         // The job's places in the ring.  A warp writes one of them but sees every one free: a phase that it
                         // skipped would let a later wait on the same place pass one phase early.
                         // One lane per place.
@@ -844,6 +903,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                             if (elect_one()) mbar_arrive_remote(ready_leader + 8 * (r_job & 7u));
                             ++r_job;
                         }
+                        TR(TR_HIDDEN, 0x43);
                     }
                 }
             }
@@ -884,11 +944,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                 asm volatile("bar.sync 2, 128;" ::: "memory");
         };
         // this warp's columns of the next output accumulator: one value per query head of its half
-        auto fetch = [&](float *v) {
+        auto fetch = [&](float *v, int kind) {
             const uint32_t ob = o & 1u, addr = tmem + lane_sel + col + 64u * ob;
+            TR(TR_OUT, kind << 4);
             mbar_wait(o_full + 8 * ob, (o >> 1) & 1u, a.status, &abort_flag, 0x60b);
             __syncwarp();
             tc_fence_after();
+            TR(TR_OUT, kind << 4 | 1);
             float r[16];
             tmem_ld8(addr, r);
             tmem_ld8(NQ <= 16 ? addr + NQ : addr + 8u, r + 8);
@@ -896,6 +958,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
             tc_fence_before();
             __syncwarp();
             if (elect_one()) mbar_arrive_remote(empty_leader + 8 * ob);
+            TR(TR_OUT, kind << 4 | 2);
             ++o;
 #pragma unroll
             for (int q = 0; q < NT; ++q) v[q] = NQ <= 16 ? r[q] + r[8 + q] : r[q];  // the low terms have columns of their own
@@ -960,7 +1023,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
         for (int it = 0; it <= n_it; ++it) {
             float s[NT];
             if (it < n_it && a.mode != MODE_V) {
-                fetch(s);
+                fetch(s, 7);
             } else if (it < n_it) {
                 if (it == 0) grid_dependency_wait();  // the launch before holds the scores
 #pragma unroll
@@ -986,7 +1049,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
 #pragma unroll 1
                 for (int blk = 0; blk < n_blk; ++blk) {
                     float u[NT];
-                    fetch(u);
+                    fetch(u, 8);
 #pragma unroll
                     for (int q = 0; q < NT; ++q)
                         if (!((mask >> q) & 1u)) u[q] = 0.f;
@@ -996,6 +1059,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
 #pragma unroll
                             for (int q = 0; q < NT; ++q) acc[b][q] += u[q];
                         }
+                    TR(TR_OUT, 0x83);
                 }
             }
             if (u_ends) {
@@ -1033,6 +1097,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
             }
             if (it < n_it) {
                 probabilities(s, tw.valid(a.sq), it & 1);
+                TR(TR_OUT, 0x73);
                 u_si = tw.si;
                 u_ends = tw.ends_run();
                 tw.next(a.sq);
@@ -1768,3 +1833,13 @@ cudaError_t lat_launch(LatState &st, const DecodeArgs &a, const SeqList &seqs, c
 }
 
 }  // namespace kvcar
+
+#ifdef KVCAR_TRACE
+// out: [2 CTAs][6 roles][4096] records; n: records per CTA and role
+extern "C" int kvcar_debug_trace_select(int cluster) { return (int)cudaMemcpyToSymbol(kvcar::g_trace_cluster, &cluster, sizeof(int)); }
+extern "C" int kvcar_debug_trace_dump(unsigned long long *out, int *n) {
+    cudaError_t e = cudaMemcpyFromSymbol(out, kvcar::g_trace, sizeof(kvcar::g_trace));
+    if (e == cudaSuccess) e = cudaMemcpyFromSymbol(n, kvcar::g_trace_n, sizeof(kvcar::g_trace_n));
+    return (int)e;
+}
+#endif

@@ -1,12 +1,14 @@
-"""Time stamps of one cluster of the tensor-core decode kernel (decode_pair_kernel).
+"""Time stamps of one cluster of the tensor-core decode kernel (decode_latent_kernel).
 
     python -m paper_2512_06727_b200.trace --workload c5 --batch 32 --layer 0 --cluster 0
 
-builds the library with -DKVCAR_TC_TRACE (libkvcar_trace.so, beside the regular one), fills a cache of the
+builds the library with -DKVCAR_TRACE (libkvcar_trace.so, beside the regular one), fills a cache of the
 workload's shape with seeded random rows, runs kvcar_decode_attention on one layer three times and prints, from the
-stamps of the last launch, what the chosen cluster's MMA issuer and first epilogue warp did: per accumulator job its
-duration, the K slabs it walked, the time between a slab's release and the next slab's operands being seen ("wait")
-and the time spent issuing ("issue"), and per job the epilogue's wait and work.  Clock: clock64 of the leader CTA's SM.
+stamps of the last launch, what the chosen cluster's two issuing threads (hidden layers; scores and weighted sums) and
+its first hidden and first output warp did: per accumulator job its duration, the slabs it walked, the time between a
+slab's release and the next slab's operands being seen ("wait") and the time spent issuing ("issue"), and per job the
+consuming warp's wait and work.  Clock: clock64 of the leader CTA's SM.  (Small grids take two launches, K then V: the
+stamps are the later one's where both have the chosen cluster.)
 The stamps cost about 36 cycles each; the totals agree with an unstamped launch within a few per cent, but stamps
 placed between individual asynchronous instructions lengthen what they measure (each then waits for its predecessor).
 """
@@ -19,6 +21,8 @@ import os
 import sys
 
 import numpy as np
+
+ROLES = 6  # loads of rows, loads of weights, hidden issuer, first hidden warp, S and U issuer, first output warp
 
 
 def main(argv=None) -> int:
@@ -79,60 +83,29 @@ def main(argv=None) -> int:
     sess.ctx.sync_status(sess.stream())
     print(f"workload {w.name} batch {w.batch} layer {args.layer}: kvcar_decode_attention {1e3 * e0.elapsed_time(e1):.1f} us"
           f" (tile kernel + combine, stamps on)")
-    buf = (C.c_ulonglong * (2 * 4 * 4096))()
-    n = (C.c_int * 8)()
+    buf = (C.c_ulonglong * (2 * ROLES * 4096))()
+    n = (C.c_int * (2 * ROLES))()
     assert lib.kvcar_debug_trace_dump(buf, n) == 0
-    arr = np.frombuffer(buf, dtype=np.uint64).reshape(2, 4, 4096)
-    ev = {f"{c}.{r}": [(int(x >> 8), int(x & 0xFF)) for x in arr[c, r, :n[c * 4 + r]]] for c in range(2) for r in range(4)}
+    arr = np.frombuffer(buf, dtype=np.uint64).reshape(2, ROLES, 4096)
+    ev = {f"{c}.{r}": [(int(x >> 8), int(x & 0xFF)) for x in arr[c, r, :n[c * ROLES + r]]] for c in range(2) for r in range(ROLES)}
     if args.json:
         json.dump(ev, open(args.json, "w"))
     report(ev, args.jobs)
     return 0
 
 
-def ring_legs(ev):
-    """The staging ring's round trip in the head-group phase, from the producers' and the issuer's stamps of the
-    leader CTA: both producers stamp every slab once they are past its place (the one that loads it after the load
-    is issued), the issuer stamps operands seen (0x30) and products + release issued (0x31).  Slab i of a head-group
-    job re-uses the place of slab i - 3 (a ring of three places, as at the GPT-2 shape)."""
-    iss = ev["0.2"]
-    prod = [[t for t, g in ev[f"0.{r}"] if g in (2, 3)] for r in (0, 1)]
-    seen, rel, kind = [], [], []
-    k = None
-    for t, tag in iss:
-        if tag in (0x11, 0x12, 0x13, 0x14):
-            k = tag & 7
-        elif tag == 0x30:
-            seen.append(t)
-            kind.append(k)
-        elif tag == 0x31:
-            rel.append(t)
-    n = min(len(seen), len(rel), len(prod[0]), len(prod[1]))
-    if n < 8:
-        return
-    load, free, gap = [], [], []
-    for i in range(n):
-        if kind[i] != 2:
-            continue
-        issued = max(prod[0][i], prod[1][i])
-        load.append(seen[i] - issued)
-        if i + 3 < n and kind[i + 3] == 2:
-            free.append(min(prod[0][i + 3], prod[1][i + 3]) - rel[i])
-        if i > 0 and kind[i - 1] == 2:
-            gap.append(seen[i] - rel[i - 1])
-    if not load or not free:
-        return
-    med = lambda v: sorted(v)[len(v) // 2]
-    print(f"  head-group ring: load issued -> operands seen by the issuer: median {med(load)} cycles; products + release issued"
-          f" (slab i) -> place seen free for slab i+3: median {med(free)}; release issued -> next operands seen: median"
-          f" {med(gap)}; issue of a slab (0x30 -> 0x31): median {med([r - s for r, s, k in zip(rel, seen, kind) if k == 2])}")
-
-
 def report(ev, n_list):
-    iss, ep = ev["0.2"], ev["0.3"]
-    if not iss or not ep:
+    if not ev["0.2"] or not ev["0.3"]:
         print("no stamps: the chosen cluster does not exist in this launch, or the layer ran on another kernel")
         return
+    report_pair(ev["0.2"], ev["0.3"], n_list)
+    if ev.get("0.4") and ev.get("0.5"):
+        print("scores and weighted sums:")
+        report_pair(ev["0.4"], ev["0.5"], n_list)
+
+
+def report_pair(iss, ep, n_list):
+    """One issuing thread's records and those of the warp that reads its accumulators."""
     t_zero = min(iss[0][0], ep[0][0])
     jobs, cur, last = [], None, None
     for t, tag in iss:
@@ -148,16 +121,16 @@ def report(ev, n_list):
             cur["prev"] = t
         elif tag == 0x19:
             cur["t1"] = t
-    ejobs, c = [], None
+    ejobs, open_ = [], {}
     for t, tag in ep:
         ph, kind = tag & 0xF, tag >> 4
-        if ph == 0:
-            c = dict(kind=kind, w0=t)
-            ejobs.append(c)
+        if ph == 0:  # (a tile's probabilities are finished behind the weighted sums of the tile before: a job of each kind is open)
+            open_[kind] = dict(kind=kind, w0=t)
+            ejobs.append(open_[kind])
         elif ph == 1:
-            c["seen"] = t
+            open_[kind]["seen"] = t
         elif ph == 3:
-            c["done"] = t
+            open_[kind]["done"] = t
     names = {1: "hidden chunk", 2: "head group", 3: "K scores", 4: "V sums"}
     print("job  kind          start     cycles slabs   wait  issue | epilogue: job seen complete  work")
     for i, (j, e) in enumerate(zip(jobs, ejobs)):
@@ -174,8 +147,7 @@ def report(ev, n_list):
         if sel:
             print(f"  {names[kind]} jobs: {len(sel)}, mean {sum(j['t1'] - j['t0'] for j in sel) / len(sel):.0f} cycles,"
                   f" {sum(j['t1'] - j['t0'] for j in sel) / max(1, sum(j['slabs'] for j in sel)):.0f} per slab")
-    ring_legs(ev)
-    for kind, nm in ((4, "hidden chunk"), (5, "K head group"), (6, "V head group")):
+    for kind, nm in ((4, "hidden chunk"), (5, "K head group"), (6, "V head group"), (7, "K scores"), (8, "V sums")):
         sel = [e for e in ejobs if e["kind"] == kind and "done" in e and "seen" in e]
         if sel:
             print(f"  epilogue, {nm}: {len(sel)} jobs, mean wait {sum(e['seen'] - e['w0'] for e in sel) / len(sel):.0f},"

@@ -278,6 +278,14 @@ def test_trace_report_reads_synthetic_stamps(capsys):
     assert "epilogue, hidden chunk: 1 jobs, mean wait 900, mean work 1000 cycles" in out
     trace.report({"0.2": [], "0.3": []}, 5)
     assert "no stamps" in capsys.readouterr().out
+    # the second issuing thread (scores, weighted sums): probabilities of a tile end behind the sums of the tile before
+    iss2 = [(100, 0x13), (120, 0x30), (170, 0x31), (180, 0x19), (300, 0x14), (300, 0x30), (340, 0x31), (340, 0x19)]
+    ep2 = [(90, 0x70), (200, 0x71), (210, 0x72), (220, 0x80), (400, 0x81), (410, 0x82), (430, 0x83), (700, 0x73)]
+    trace.report({"0.2": iss, "0.3": ep, "0.4": iss2, "0.5": ep2}, 5)
+    out = capsys.readouterr().out
+    assert "K scores jobs: 1, mean 80 cycles" in out and "V sums jobs: 1, mean 40 cycles" in out
+    assert "epilogue, K scores: 1 jobs, mean wait 110, mean work 500 cycles" in out
+    assert "epilogue, V sums: 1 jobs, mean wait 180, mean work 30 cycles" in out
 
 
 
