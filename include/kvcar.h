@@ -57,7 +57,10 @@ typedef enum { KVCAR_K = 0, KVCAR_V = 1 } kvcar_which;
 typedef enum {
     KVCAR_KERNEL_AUTO = 0,    /* tensor-core kernels where the shape allows, else fp32 FMA */
     KVCAR_KERNEL_GENERIC = 1, /* plain fp32 kernel (any supported shape, both dtypes)      */
-    KVCAR_KERNEL_TENSOR = 2,  /* tcgen05/TMEM kernels (bf16 storage, bf16 or int8 rows)    */
+    KVCAR_KERNEL_TENSOR = 2,  /* tcgen05/TMEM kernels (bf16 storage, 64-wide heads, pages of
+                                 a multiple of 64 tokens, autoencoder widths that are
+                                 multiples of 16): as AUTO for such layers, UNSUPPORTED
+                                 for the others (int8 rows: where the kernels take them)  */
     KVCAR_KERNEL_RAW = 3      /* reported only: streaming kernel AUTO picks for a layer
                                  whose K and V are all stored raw (no autoencoder)       */
 } kvcar_kernel;
@@ -340,7 +343,8 @@ kvcar_status kvcar_layer_work_absorbed(kvcar_ctx *ctx, int32_t layer, int32_t bo
 /* Number of kernels the library has launched so far on this context. */
 kvcar_status kvcar_launch_count(kvcar_ctx *ctx, int64_t *count);
 /* Kernel family (kvcar_kernel: GENERIC, TENSOR or RAW) that kvcar_decode_attention will use
- * for `layer` under the current kvcar_set_kernel choice.  Only after kvcar_bind_memory. */
+ * for `layer` (without KVCAR_ABSORBED flags) under the current kvcar_set_kernel choice; GENERIC
+ * covers the fp32-FMA kernels.  Only after kvcar_bind_memory. */
 kvcar_status kvcar_layer_kernel(kvcar_ctx *ctx, int32_t layer, int32_t *kernel);
 /* Synchronise `stream` and report any asynchronous CUDA error or device-side
  * bounded-wait timeout recorded since the last call. */

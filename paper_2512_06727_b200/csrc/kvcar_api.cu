@@ -13,7 +13,6 @@
 #include "kvcar_internal.h"
 #include "kvcar_fma.h"
 #include "kvcar_latent.h"
-#include "kvcar_tc.h"
 
 using namespace kvcar;
 
@@ -83,16 +82,16 @@ struct kvcar_ctx {
     std::vector<size_t> qparam_off;         // int8 latent rows: offset of the (scale, zero-point) array, else 0
     std::vector<char> quant;                // [layer*2+which]: rows are int8 codes
     size_t pool_bytes = 0, weights_bytes = 0, ws_bytes = 0;
-    size_t plan_off = 0, enc_off = 0, tmap_off = 0, tcpart_off = 0;  // inside weights
-    size_t bt_off = 0, len_off = 0, status_off = 0, part_off = 0, stage_off = 0, enchid_off = 0, kvsplit_off = 0, pfhid_off = 0, lat_off = 0, fma_off = 0;  // inside workspace
+    size_t plan_off = 0, enc_off = 0;  // inside weights
+    size_t bt_off = 0, len_off = 0, status_off = 0, part_off = 0, stage_off = 0, enchid_off = 0, pfhid_off = 0, lat_off = 0, fma_off = 0;  // inside workspace
     int max_sources = 0;  // most distinct source layers any layer's K or V heads resolve to
     std::vector<RawSources> raw_src;  // [layer] tensor maps and head places of raw bf16 layers
     std::vector<char> raw_src_ok;     // [layer] filled (else the raw-row kernel stages with cp.async)
     std::vector<EncPlan> enc_host;  // the device's EncPlan table, host copy (tensor-core prefill builds tensor maps from it)
+    bool use_fma = false;           // some layer is the fp32-FMA kernels'
     int max_chunks = 0, chunk_tokens = 128;
     int max_d = 0, max_m = 0, max_in = 0;
     std::vector<LayerPlan> plans_host;
-    TcState tc;
     LatState lat;
     FmaState fma;
     bool fma_tiles = false;  // the last tile launch was the fp32-FMA kernels': their merge follows
@@ -139,8 +138,27 @@ int stored_width(const kvcar_ctx *c, int layer, int which) {
     return (int)stored_heads(c, layer, which).size() * c->cfg.head_dim;
 }
 
-// bf16 storage and 64-wide heads: the tensor-core kernels take all but a few layers, and those few stay with the generic kernel
-bool fma_is_fallback_only(const kvcar_config &g) { return g.storage == KVCAR_BF16 && g.head_dim == 64; }
+// Some layer over latent rows only that the tensor-core kernels do not take whatever the flags of a call: the fp32-FMA kernels get
+// their workspace (150 MB at 12 heads, hidden 576, 256 sequences; contexts that need none get none).
+bool needs_fma(const kvcar_ctx *c) {
+    const kvcar_config &g = c->cfg;
+    for (int l = 0; l < g.n_layers; ++l) {
+        LatShape sh;
+        bool rows = true;
+        for (int which = 0; which < 2; ++which) {
+            std::vector<char> seen(g.n_layers, 0);
+            for (int h = 0; h < g.n_kv_heads; ++h) {
+                const int r = resolve(c, l, h, which).root_layer;
+                const AEHost &a = c->ae[r * 2 + which];
+                rows = rows && a.set;
+                if (!seen[r]) sh.add(which, a.latent, a.hidden);
+                seen[r] = 1;
+            }
+        }
+        if (rows && !lat_covers(g, c->max_m, sh)) return true;
+    }
+    return false;
+}
 
 void compute_layout(kvcar_ctx *c) {
     const kvcar_config &g = c->cfg;
@@ -196,7 +214,7 @@ void compute_layout(kvcar_ctx *c) {
         w = align_up(w + 2 * mats * c->elem, 256);                                 // transposed enc + dec
         w = align_up(w + (size_t)(4 * a.hidden + a.latent + a.in_dim) * sizeof(float), 256);  // s,t x2, b2 x2
         if (g.storage == KVCAR_BF16) {
-            w = align_up(w + mats * 2, 256);                                       // K-major decoder copies
+            w = align_up(w + (size_t)a.in_dim * a.hidden * 2, 256);                // decoder FC2 as given
             w = align_up(w + (size_t)a.hidden * a.latent * 2, 256);                // FC1 of the latent-attention kernels
             w = align_up(w + (size_t)(3 * ((a.hidden + 31) & ~31)) * sizeof(float), 256);
         }
@@ -206,10 +224,6 @@ void compute_layout(kvcar_ctx *c) {
     w = align_up(w + (size_t)nl * sizeof(LayerPlan), 256);
     c->enc_off = w;
     w = align_up(w + (size_t)nl * 2 * sizeof(EncPlan), 256);
-    c->tmap_off = w;  // TMA descriptors of the tensor-core kernel: pool, decoder FC1, decoder FC2 per (layer, which)
-    w = align_up(w + (size_t)nl * 2 * 3 * 128, 256);
-    c->tcpart_off = w;  // per-layer job tables of the tensor-core kernel
-    w = align_up(w + tc_part_bytes(nl), 256);
     c->weights_bytes = w;
 
     // workspace
@@ -231,8 +245,6 @@ void compute_layout(kvcar_ctx *c) {
                       (size_t)nb * g.n_q_heads * g.head_dim * c->elem), 256);
     c->enchid_off = s;  // hidden activations between the decode-time encoder's launches; int8 rows: then the fp32 latents
     s = align_up(s + (size_t)2 * nb * (c->max_m + (g.latent_quant ? c->max_d : 0)) * sizeof(float), 256);
-    c->kvsplit_off = s;  // probabilities handed from K clusters to V clusters (tensor-core kernel, small grids)
-    s = align_up(s + tc_split_bytes(g), 256);
     c->pfhid_off = s;  // bf16 hidden activations between the two launches of the tensor-core prefill
     if (g.storage == KVCAR_BF16 && c->max_m > 0) s = align_up(s + prefill_tc_scratch_bytes(c->max_m), 256);
     c->max_sources = 0;
@@ -251,8 +263,9 @@ void compute_layout(kvcar_ctx *c) {
         }
     c->lat_off = s;  // operands and partial results of the latent-attention kernels
     s = align_up(s + lat_ws_bytes(g, c->max_sources, c->max_m, c->max_d, nb, cap), 256);
-    c->fma_off = s;  // the same of the fp32-FMA kernels, where latents are not bf16 rows of 64-wide heads
-    if (!fma_is_fallback_only(g)) s = align_up(s + fma_ws_bytes(g, c->max_sources, c->max_m, nb, cap), 256);
+    c->fma_off = s;  // the same of the fp32-FMA kernels
+    c->use_fma = needs_fma(c);
+    if (c->use_fma) s = align_up(s + fma_ws_bytes(g, c->max_sources, c->max_m, nb, cap), 256);
     c->ws_bytes = s;
 }
 
@@ -414,9 +427,26 @@ bool layer_is_raw(const kvcar_ctx *c, int layer) {
     return true;
 }
 
+// KVCAR_KERNEL_TENSOR: layers that the tensor-core kernels take, and layers of their kind a little beyond (more heads, wider latents,
+// hidden layers up to 1024), which an earlier tensor-core kernel took and the fp32-FMA kernels run now.
+bool takes_tensor_request(const kvcar_ctx *c, int layer) {
+    const kvcar_config &g = c->cfg;
+    if (c->lat.available && lat_layer_supported(c->lat, layer, KVCAR_ABSORBED | KVCAR_ABSORBED_V)) return true;
+    if (!fma_layer_supported(c->fma, layer) || g.storage != KVCAR_BF16 || g.latent_quant || g.head_dim != 64 || g.page_tokens % 64 ||
+        g.n_q_heads / g.n_kv_heads > 8)
+        return false;
+    const LayerPlan &lp = c->plans_host[layer];
+    for (int w = 0; w < 2; ++w)
+        for (int s = 0; s < lp.w[w].n_src; ++s) {
+            const SourcePlan &sp = lp.w[w].src[s];
+            if (lp.w[w].n_src > LT_MAX_SRC || sp.d % 16 || sp.m % 16 || sp.m > 1024 || sp.in_dim > 1024) return false;
+        }
+    return true;
+}
+
 bool use_tensor_kernel(const kvcar_ctx *c) {
     if (c->kernel == KVCAR_KERNEL_GENERIC) return false;
-    return c->tc.available || c->lat.available;
+    return c->lat.available;
 }
 
 // Device address of `bytes` bytes of page-locked host memory at p; null where any of them lies outside the one page-locked range.
@@ -481,7 +511,6 @@ kvcar_status kvcar_create(const kvcar_config *cfg, kvcar_ctx **out_ctx) {
 
 kvcar_status kvcar_destroy(kvcar_ctx *ctx) {
     if (!ctx) return KVCAR_ERR_INVALID_ARG;
-    tc_destroy(ctx->tc);
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
     if (ctx->side) cudaStreamDestroy(ctx->side);
@@ -585,7 +614,7 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
 
     std::vector<char> img(c->weights_bytes, 0);
     struct Packed {
-        size_t enc_w1t, enc_w2t, dec_w1t, dec_w2t, enc_s, enc_t, enc_b2, dec_s, dec_t, dec_b2, w1k, w2k, w1n, sabs, enc_w1r, enc_w2r;
+        size_t enc_w1t, enc_w2t, dec_w1t, dec_w2t, enc_s, enc_t, enc_b2, dec_s, dec_t, dec_b2, w2k, w1n, sabs, enc_w1r, enc_w2r;
     };
     std::vector<Packed> pk(nl * 2);
     size_t w = 0;
@@ -617,13 +646,14 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
         put_elems(&img[p.enc_w1r], a.enc_w1.data(), M * I, g.storage);
         put_elems(&img[p.enc_w2r], a.enc_w2.data(), D * M, g.storage);
         const char *fc1 = (const char *)a.dec_w1.data(), *fc2 = (const char *)a.dec_w2.data();
+        std::vector<char> w1_bf16;
         if (g.storage == KVCAR_BF16) {
-            p.w1k = w;
-            p.w2k = p.w1k + M * D * 2;
-            w = align_up(w + (M * D + I * M) * 2, 256);
-            put_elems(&img[p.w1k], a.dec_w1.data(), M * D, KVCAR_BF16);
+            p.w2k = w;
+            w = align_up(w + I * M * 2, 256);
+            w1_bf16.resize(M * D * 2);
+            put_elems(w1_bf16.data(), a.dec_w1.data(), M * D, KVCAR_BF16);
             put_elems(&img[p.w2k], a.dec_w2.data(), I * M, KVCAR_BF16);
-            fc1 = &img[p.w1k];
+            fc1 = w1_bf16.data();
             fc2 = &img[p.w2k];
         }
         put_transposed(&img[p.enc_w1t], &img[p.enc_w1r], (int)M, (int)I, g.storage);  // [M][I] -> [I][M]
@@ -636,7 +666,7 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
             p.sabs = w;  // then the shifts, then the row sums
             const size_t M32 = (M + 31) & ~(size_t)31;
             w = align_up(w + 3 * M32 * 4, 256);
-            put_signed_fc1(&img[p.w1n], (float *)&img[p.sabs], M32, &img[p.w1k], (const float *)&img[p.dec_s],
+            put_signed_fc1(&img[p.w1n], (float *)&img[p.sabs], M32, fc1, (const float *)&img[p.dec_s],
                            (const float *)&img[p.dec_t], a.slope, (int)M, (int)D);
         }
     }
@@ -678,7 +708,6 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
                         sp.t1 = (const float *)(c->weights + pk[idx].dec_t);
                         sp.b2 = (const float *)(c->weights + pk[idx].dec_b2);
                         if (g.storage == KVCAR_BF16) {
-                            sp.w1k = c->weights + pk[idx].w1k;
                             sp.w2k = c->weights + pk[idx].w2k;
                             sp.w1n = c->weights + pk[idx].w1n;
                             sp.sabs = (const float *)(c->weights + pk[idx].sabs);
@@ -697,12 +726,9 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
             }
         }
     }
-    // tensor maps and job tables of the tensor-core kernel (fills their regions of the image)
-    tc_setup(c->tc, c->cfg, plans, nl, c->weights, c->tmap_off, c->tcpart_off, img.data(),
-             (size_t)g.max_pages * g.page_tokens);
     lat_setup(c->lat, c->cfg, c->plans_host, (size_t)g.max_pages * g.page_tokens, c->max_sources, c->max_m, c->max_d,
               std::min(g.max_seqs, KVCAR_MAX_BATCH), g.max_pages_per_seq * g.page_tokens, c->ws + c->lat_off);
-    if (!fma_is_fallback_only(g))
+    if (c->use_fma)
         fma_setup(c->fma, c->cfg, c->plans_host, c->max_sources, c->max_m, std::min(g.max_seqs, KVCAR_MAX_BATCH),
                   g.max_pages_per_seq * g.page_tokens, c->ws + c->fma_off);
     // tensor maps and head places of the raw layers (kernel parameters of the raw-row kernel)
@@ -725,9 +751,6 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
         }
         c->raw_src_ok[l] = ok;
     }
-    c->tc.pbuf = reinterpret_cast<float *>(c->ws + c->kvsplit_off);
-    c->tc.pflags = reinterpret_cast<uint32_t *>(c->ws + c->kvsplit_off +
-                                                (size_t)TC_SPLIT_TILES * g.n_q_heads * 132 * sizeof(float));
     memcpy(&img[c->plan_off], plans, (size_t)nl * sizeof(LayerPlan));
 
     std::vector<EncPlan> enc(nl * 2);
@@ -764,7 +787,6 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
 
     cudaError_t e = cudaMemcpyAsync(c->weights, img.data(), img.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ws, 0, c->part_off, st);  // tables, lengths, status
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + c->kvsplit_off, 0, tc_split_bytes(g), st);  // hand-over flags
     if (e == cudaSuccess && c->ws_bytes > c->lat_off)
         e = cudaMemsetAsync(c->ws + c->lat_off, 0, c->ws_bytes - c->lat_off, st);  // operand rows of padding heads stay zero
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -813,8 +835,11 @@ kvcar_status kvcar_bind_memory(kvcar_ctx *c, void *pool, size_t pool_bytes, void
 
 kvcar_status kvcar_set_kernel(kvcar_ctx *c, int32_t kernel) {
     if (!c || kernel < 0 || kernel > 2) return fail(c, KVCAR_ERR_INVALID_ARG, "unknown kernel family");
-    if (kernel == KVCAR_KERNEL_TENSOR && c->bound && !c->tc.available && !c->lat.available)
-        return fail(c, KVCAR_ERR_UNSUPPORTED, std::string("tensor-core kernel unavailable: ") + c->tc.why);
+    if (kernel == KVCAR_KERNEL_TENSOR && c->bound) {
+        bool any = false;
+        for (int l = 0; l < c->cfg.n_layers && !any; ++l) any = takes_tensor_request(c, l);
+        if (!any) return fail(c, KVCAR_ERR_UNSUPPORTED, "no layer is of the tensor-core kernels' kind (bf16 storage, 64-wide heads, autoencoder widths that are multiples of 16)");
+    }
     c->kernel = kernel;
     return KVCAR_OK;
 }
@@ -1031,17 +1056,12 @@ static kvcar_status enqueue_decode_tiles(kvcar_ctx *c, int32_t layer, const Deco
     c->fma_tiles = false;
     if (n_chunks <= 0) return KVCAR_OK;
     const kvcar_config &g = c->cfg;
-    const bool want_tc = use_tensor_kernel(c) && tc_layer_supported(c->tc, layer);
-    if (c->kernel == KVCAR_KERNEL_TENSOR && !want_tc)
-        return fail(c, KVCAR_ERR_UNSUPPORTED, std::string("tensor-core kernel cannot run this layer: ") + c->tc.why);
+    if (c->kernel == KVCAR_KERNEL_TENSOR && !takes_tensor_request(c, layer))
+        return fail(c, KVCAR_ERR_UNSUPPORTED, "this layer is not of the tensor-core kernels' kind (bf16 storage, 64-wide heads, autoencoder widths that are multiples of 16)");
     cudaError_t e;
     if (c->kernel != KVCAR_KERNEL_GENERIC && layer_is_raw(c, layer)) {
         e = launch_decode_raw(a, sl, c->raw_src_ok[layer] ? &c->raw_src[layer] : nullptr, raw_rows, g.storage, n_chunks, st);
-    } else if (want_tc) {
-        int32_t lens[KVCAR_MAX_BATCH];
-        for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
-        e = tc_launch_decode(c->tc, a, sl, lens, layer, st);
-    } else if (c->kernel == KVCAR_KERNEL_AUTO && fma_layer_supported(c->fma, layer)) {
+    } else if (c->kernel != KVCAR_KERNEL_GENERIC && fma_layer_supported(c->fma, layer)) {
         int32_t lens[KVCAR_MAX_BATCH];
         for (int i = 0; i < sl.n; ++i) lens[i] = c->len[sl.id[i]];
         int n = 1;
@@ -1381,7 +1401,7 @@ kvcar_status kvcar_layer_kernel(kvcar_ctx *c, int32_t layer, int32_t *kernel) {
     if (c->kernel != KVCAR_KERNEL_GENERIC && layer_is_raw(c, layer))
         *kernel = KVCAR_KERNEL_RAW;
     else
-        *kernel = (use_tensor_kernel(c) && (lat_layer_supported(c->lat, layer, 0) || tc_layer_supported(c->tc, layer))) ? KVCAR_KERNEL_TENSOR : KVCAR_KERNEL_GENERIC;
+        *kernel = (use_tensor_kernel(c) && lat_layer_supported(c->lat, layer, 0)) ? KVCAR_KERNEL_TENSOR : KVCAR_KERNEL_GENERIC;
     return KVCAR_OK;
 }
 
@@ -1409,7 +1429,7 @@ kvcar_status kvcar_debug_expire_wait(kvcar_ctx *c, uint64_t limit_ns, void *stre
     if (!c) return KVCAR_ERR_INVALID_ARG;
     if (!c->bound) return fail(c, KVCAR_ERR_STATE, "bind memory first");
     if (limit_ns == 0 || limit_ns > 1000000000ull) return fail(c, KVCAR_ERR_INVALID_ARG, "limit must be 1 ns .. 1 s");
-    cudaError_t e = tc_launch_expire_wait(reinterpret_cast<int32_t *>(c->ws + c->status_off), limit_ns, (cudaStream_t)stream);
+    cudaError_t e = launch_expire_wait(reinterpret_cast<int32_t *>(c->ws + c->status_off), limit_ns, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "launch");
     ++c->launches;
     return KVCAR_OK;

@@ -1,7 +1,7 @@
 // Generic (fp32 FMA) kernels of the KV-CAR decode path: table maintenance,
 // encoder + append, decoder + attention over one chunk of cached tokens, and the
 // split-KV combine.  They handle every supported shape in both storage types and
-// are the fp32-mode path; the bf16 tensor-core kernel lives in kvcar_tc.cu.
+// stand behind the others: what neither kvcar_latent.cu nor kvcar_fma.cu takes runs here.
 #include "kvcar_internal.h"
 #include "kvcar_pdl.cuh"
 

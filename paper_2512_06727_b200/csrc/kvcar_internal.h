@@ -22,8 +22,7 @@ struct SourcePlan {
     const float *t1;
     const void *w2t;   // decoder FC2 transposed [m][in_dim], storage dtype
     const float *b2;   // [in_dim]
-    const void *w1k;   // K-major bf16 copies for the tensor-core kernel: [m][d]
-    const void *w2k;   //                                                  [in_dim][m]
+    const void *w2k;   // bf16: decoder FC2 as given, [in_dim][m]
     const float *qparam;  // int8 rows: (scale, zero-point) per pool row, else null
     // latent-attention kernels (bf16): decoder FC1 [m][d] with the signs of the BatchNorm scale taken into its rows, the
     // sizes of the scale [m], and the shift over them (in the kernels' own order)
@@ -139,6 +138,8 @@ bool raw_build_map(void *dst_host, const void *pool_dev, uint64_t rows, uint64_t
 // n_chunks: tiles of the longest listed sequence (picks the kernel: a warp or a CTA per sequence and query head)
 cudaError_t launch_combine(const DecodeArgs &a, const SeqList &seqs, int dtype, int n_chunks, cudaStream_t st);
 size_t decode_generic_smem(int hq, int hd, int max_d, int max_m);
+// test hook: one warp waits `limit_ns` on a barrier that nothing completes, then records code 0x7e57 in the status word (kvcar_debug.cu)
+cudaError_t launch_expire_wait(int32_t *status, uint64_t limit_ns, cudaStream_t st);
 
 // Bulk encoder + append on the tensor cores (kvcar_prefill_tc.cu): bf16 storage, both K and V of the layer with an
 // autoencoder, head_dim 64, hidden and latent widths multiples of 16.  Rows are worked through in blocks of

@@ -1500,8 +1500,12 @@ static int lat_wide_tiles(int batch, int max_len) {
     return (int)std::min<int64_t>((int64_t)batch * per_seq, std::max(LT_WIDE_TILES, per_seq));
 }
 
+static bool shape_ok(const kvcar_config &cfg) {
+    return cfg.storage == KVCAR_BF16 && cfg.head_dim == 64 && cfg.n_q_heads <= LT_MAX_Q && cfg.page_tokens % 64 == 0;
+}
+
 size_t lat_ws_bytes(const kvcar_config &cfg, int max_sources, int max_m, int max_d, int batch, int max_len) {
-    if (cfg.storage != KVCAR_BF16 || cfg.head_dim != 64 || cfg.n_q_heads > LT_MAX_Q || max_sources <= 0 || max_m <= 0) return 0;
+    if (!shape_ok(cfg) || max_sources <= 0 || max_m <= 0) return 0;
     const size_t nq = padded_heads(cfg.n_q_heads), m_pad = ((size_t)max_m + 63) / 64 * 64;
     const size_t wq = (size_t)std::min(max_sources, LT_MAX_SRC) * batch * wq_rows((int)nq) * m_pad * 2;
     const size_t bias = ((size_t)batch * cfg.n_q_heads * 4 + 255) / 256 * 256;
@@ -1512,6 +1516,46 @@ size_t lat_ws_bytes(const kvcar_config &cfg, int max_sources, int max_m, int max
     return n;
 }
 
+// the build and the staging places of a layer, false where none fits
+static bool pick_build(int nq, bool quant, const LatShape &sh, LatLayerCfg &lc) {
+    if (!sh.widths_ok || sh.n_src[0] < 1 || sh.n_src[0] > LT_MAX_SRC || sh.n_src[1] < 1 || sh.n_src[1] > LT_MAX_SRC) return false;
+    int v = 0;
+    while (v < N_BUILDS && (builds[v].nq != nq || builds[v].quant != quant || builds[v].nb * 128 < sh.m)) ++v;
+    if (v == N_BUILDS) return false;
+    const int ks = (sh.d + 63) / 64, chunks = (sh.m + builds[v].cn - 1) / builds[v].cn;
+    // Staging places.  A side's latents stay for all its chunks (nz >= their slabs).  One-chunk layers get places for the
+    // other side's latents and six hidden slabs, because their jobs are shorter than the way from S to P; the others four
+    // hidden slabs: a chunk's three and the one its predecessor may leave unpaired, or a chunk's two terms of two.
+    int nh = chunks == 1 ? 6 : 4, nz = chunks == 1 ? std::max(4, 2 * ks) : ks, nw = 4, nqs = 4;
+    auto fits = [&]() { return smem_bytes(builds[v], nz, nh, nw, nqs) <= SMEM_MAX; };
+    while (nw > 3 && !fits()) --nw;
+    while (nqs > 2 && !fits()) --nqs;
+    while (nz > ks && !fits()) --nz;
+    while (nw > 2 && !fits()) --nw;
+    if (!fits() && quant) nh = 2;  // one term of a job at a time
+    if (!fits()) return false;
+    while (nqs < 12 && (++nqs, fits())) {}
+    if (!fits()) --nqs;
+    lc.nz = (uint8_t)nz;
+    lc.nh = (uint8_t)nh;
+    lc.nw = (uint8_t)nw;
+    lc.nqs = (uint8_t)nqs;
+    lc.smem = std::max(smem_bytes(builds[v], nz, nh, nw, nqs), 120 * 1024);  // one CTA per SM: each takes all of tensor memory
+    lc.variant = (uint8_t)v;
+    lc.max_m = sh.m;
+    lc.max_mk = sh.mk;
+    return true;
+}
+
+// Groups of more than two query heads, or int8 rows, or up to 16 heads: see lat_layer_supported.
+static bool any_flags(const kvcar_config &cfg, int nq) { return nq <= 16 || cfg.n_q_heads / cfg.n_kv_heads > 2 || cfg.latent_quant; }
+
+bool lat_covers(const kvcar_config &cfg, int max_m, const LatShape &sh) {
+    LatLayerCfg lc;
+    const int nq = padded_heads(cfg.n_q_heads);
+    return shape_ok(cfg) && any_flags(cfg, nq) && pick_build(nq, cfg.latent_quant != 0, sh, lc);
+}
+
 void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPlan> &plans, size_t pool_rows,
                int max_sources, int max_m, int max_d, int batch, int max_len, char *ws_area) {
     st.available = false;
@@ -1519,7 +1563,7 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
     st.layer.assign(nl, LatLayer{});
     st.heads.assign(nl, LatHeads{});
     st.cfg.assign(nl, LatLayerCfg{});
-    if (lat_ws_bytes(cfg, max_sources, max_m, max_d, batch, max_len) == 0 || cfg.page_tokens % 64 != 0) return;
+    if (lat_ws_bytes(cfg, max_sources, max_m, max_d, batch, max_len) == 0) return;
     EncodeTiledFn fn = tensor_map_encoder();
     if (!fn) return;
     int dev = 0, sms = 148;
@@ -1532,6 +1576,7 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, LT_ENC_SMEM) != cudaSuccess) return;
     st.nq = padded_heads(cfg.n_q_heads);
     st.group = group;
+    st.any_flags = any_flags(cfg, st.nq);
     st.m_pad = (max_m + 63) / 64 * 64;
     st.batch = batch;
     const size_t n_src = std::min(max_sources, LT_MAX_SRC), n_rows = n_src * batch * wq_rows(st.nq);
@@ -1560,7 +1605,7 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
         LatHeads &hp = st.heads[l];
         LatLayerCfg &lc = st.cfg[l];
         bool ok = true;
-        int ks = 0, lm = 0, lmk = 0, chunks = 0;
+        LatShape sh;
         const int cn = st.quant ? 128 : 192;
         for (int w = 0; w < 2 && ok; ++w) {
             const WhichPlan &wp = plans[l].w[w];
@@ -1599,38 +1644,12 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
                 ok = (st.quant ? encode_bf16_map(fn, &ly.pool[w][s], reinterpret_cast<__nv_bfloat16 *>(st.wide) + region * max_d, wide_rows, sp.d, max_d)
                                : encode_bf16_map(fn, &ly.pool[w][s], sp.pool, pool_rows, sp.width, sp.width)) &&
                      encode_bf16_map(fn, &ly.w1[w][s], sp.w1n, sp.m, sp.d, sp.d, cn / 2);
-                ks = std::max(ks, (sp.d + 63) / 64);
-                lm = std::max(lm, sp.m);
-                if (w == 0) lmk = std::max(lmk, sp.m);
-                chunks = std::max(chunks, (sp.m + cn - 1) / cn);
+                sh.add(w, sp.d, sp.m);
             }
         }
         if (!ok) continue;
-        int v = 0;
-        while (v < N_BUILDS && (builds[v].nq != st.nq || builds[v].quant != st.quant || builds[v].nb * 128 < lm)) ++v;
-        if (v == N_BUILDS) continue;
-        // Staging places.  A side's latents stay for all its chunks (nz >= their slabs).  One-chunk layers get places for the
-        // other side's latents and six hidden slabs, because their jobs are shorter than the way from S to P; the others four
-        // hidden slabs: a chunk's three and the one its predecessor may leave unpaired, or a chunk's two terms of two.
-        int nh = chunks == 1 ? 6 : 4, nz = chunks == 1 ? std::max(4, 2 * ks) : ks, nw = 4, nqs = 4;
-        auto fits = [&]() { return smem_bytes(builds[v], nz, nh, nw, nqs) <= SMEM_MAX; };
-        while (nw > 3 && !fits()) --nw;
-        while (nqs > 2 && !fits()) --nqs;
-        while (nz > ks && !fits()) --nz;
-        while (nw > 2 && !fits()) --nw;
-        if (!fits() && st.quant) nh = 2;  // one term of a job at a time
-        if (!fits()) continue;
-        while (nqs < 12 && (++nqs, fits())) {}
-        if (!fits()) --nqs;
-        lc.nz = (uint8_t)nz;
-        lc.nh = (uint8_t)nh;
-        lc.nw = (uint8_t)nw;
-        lc.nqs = (uint8_t)nqs;
-        lc.smem = std::max(smem_bytes(builds[v], nz, nh, nw, nqs), 120 * 1024);  // one CTA per SM: each takes all of tensor memory
-        lc.variant = (uint8_t)v;
-        lc.max_m = lm;
-        lc.max_mk = lmk;
-        if (cudaFuncSetAttribute(builds[v].kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess) {
+        if (!pick_build(st.nq, st.quant, sh, lc)) continue;
+        if (cudaFuncSetAttribute(builds[lc.variant].kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess) {
             cudaGetLastError();
             continue;
         }
@@ -1641,9 +1660,9 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
 
 bool lat_layer_supported(const LatState &st, int layer, uint32_t flags) {
     if (!st.available || !st.cfg[layer].ok) return false;
-    // 17 to 32 query heads: the probabilities are one bf16 term.  The restoring kernel keeps them in fp32 for groups of up to
-    // two heads, so those take this path only where the caller has asked for that rounding.
-    return st.nq <= 16 || st.group > 2 || ((flags & KVCAR_ABSORBED) && (flags & KVCAR_ABSORBED_V));
+    // 17 to 32 query heads over bf16 rows: the probabilities are one bf16 term.  For groups of up to two heads they have always been
+    // more than that, so those take this path only where the caller has asked for that rounding.
+    return st.any_flags || ((flags & KVCAR_ABSORBED) && (flags & KVCAR_ABSORBED_V));
 }
 
 namespace {

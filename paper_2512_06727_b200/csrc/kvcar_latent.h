@@ -65,6 +65,19 @@ struct LatCodes {
     int32_t n_src[2];
 };
 
+// What decides whether the kernels take a layer: the sources of its K and V heads (all over latent rows).
+struct LatShape {
+    int n_src[2] = {0, 0}, d = 0, m = 0, mk = 0;  // widest latent, widest hidden layer, widest hidden layer of the K sources
+    bool widths_ok = true;
+    void add(int which, int latent, int hidden) {
+        ++n_src[which];
+        d = latent > d ? latent : d;
+        m = hidden > m ? hidden : m;
+        if (which == 0) mk = hidden > mk ? hidden : mk;
+        widths_ok = widths_ok && latent % 16 == 0 && hidden % 16 == 0;
+    }
+};
+
 struct LatLayerCfg {
     uint8_t ok = 0;
     uint8_t variant = 0;                              // kernel instantiation
@@ -86,6 +99,7 @@ struct LatState {
     int n_sms = 148;
     int nq = 12;      // query heads padded
     int group = 1;    // query heads per KV head
+    bool any_flags = true;  // layers are taken whatever the flags of a call
     int m_pad = 0;    // row pitch of the vectors below
     int batch = 0;    // sequences per call at most
     void *wq = nullptr;      // [source][batch][operand rows][m_pad] bf16: W4_h^T q, high parts then low parts
@@ -98,6 +112,8 @@ struct LatState {
 
 // bytes of the operands and partial results inside the workspace (0: the shape does not take this path)
 size_t lat_ws_bytes(const kvcar_config &cfg, int max_sources, int max_m, int max_d, int batch, int max_len);
+// whether every call on such a layer takes this path (max_m: widest hidden layer of the context)
+bool lat_covers(const kvcar_config &cfg, int max_m, const LatShape &sh);
 // decide per layer whether the kernels take it, build tensor maps, place the workspace area
 void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPlan> &plans, size_t pool_rows,
                int max_sources, int max_m, int max_d, int batch, int max_len, char *ws_area);

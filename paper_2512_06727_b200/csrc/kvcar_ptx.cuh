@@ -1,6 +1,6 @@
 // Thin wrappers around the sm_100a instructions the tensor-core kernels use (mbarrier, TMA tensor loads,
 // tcgen05 products / commits / tensor-memory loads, cluster addressing) and the two descriptor packers.
-// Device code only; shared by the fused decode kernel and the bulk encoder.
+// Device code only; shared by the decode kernels and the bulk encoder.
 #pragma once
 
 #include <cuda.h>
@@ -19,38 +19,20 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)_
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
 }
-__device__ __forceinline__ void mbar_arrive_local(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// arrive on a barrier of any CTA of the cluster (address from map_to_cta), release at cluster scope
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
-}
-// arrive on a barrier of any CTA of the cluster, ordering only this CTA's earlier operations (enough where the data
+// arrive on a barrier of any CTA of the cluster (address from map_to_cta), ordering only this CTA's earlier operations (enough where the data
 // handed over is tensor memory already read, or this CTA's shared memory already fenced for the async proxy)
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_bar) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
-// CLUSTER: the phase was completed by another CTA's ordinary stores + arrive, so acquire at cluster scope
-template <bool CLUSTER = false>
 __device__ __forceinline__ uint32_t mbar_try(uint32_t bar, uint32_t parity) {
     uint32_t ok;
-    if (CLUSTER)
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, "
-            "0, p;\n}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-    else
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok)
+                 : "r"(bar), "r"(parity)
+                 : "memory");
     return ok;
 }
 // one look at the phase, never suspends the thread
@@ -77,22 +59,6 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t local_addr, uint32_t ran
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void st_cluster_v4(uint32_t addr, float a, float b, float c, float d) {
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
-                 : "memory");
-}
-__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-// Copy `bytes` (a multiple of 16, both addresses 16-byte aligned) from this CTA's shared memory into the peer CTA's
-// and count them on a barrier there: whoever sees that barrier's phase complete sees the data.
-__device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst_cluster, uint32_t src_cta, uint32_t bytes,
-                                                  uint32_t bar_cluster) {
-    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     dst_cluster),
-                 "r"(src_cta), "r"(bytes), "r"(bar_cluster)
-                 : "memory");
-}
 
 // ---- TMA tensor loads (no multicast anywhere) ------------------------------------------------------------------
 // 2-D tile into this CTA's shared memory, completion bytes on a barrier of this CTA
@@ -110,12 +76,6 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void *tmap,
         "[%4];" ::"r"(dst),
         "l"(tmap), "r"(x), "r"(y), "r"(cluster_bar)
         : "memory");
-}
-// A tensor map that lies in global memory was written through other proxies (a copy from the host at bind time): the
-// block that uses it has to acquire it first, or it may meet what the map cache of its SM kept of an earlier map at the
-// same address (an earlier context's, whose pool may be gone).
-__device__ __forceinline__ void tmap_acquire(const void *tmap) {
-    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(tmap) : "memory");
 }
 // bring one box of a tensor into L2 ahead of its load
 __device__ __forceinline__ void tma_prefetch_2d(const void *tmap, int x, int y) {
@@ -137,18 +97,7 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// D[tmem] (+)= A[smem desc] . B[smem desc]^T, bf16 inputs, fp32 accumulate, one CTA (M = 128)
-__device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                     uint32_t accumulate) {
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(
-                     d_tmem),
-                 "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-                 : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-// the same over a CTA pair (M = 256); ACC is a compile-time constant so that no predicate has to be computed in
+// D[tmem] (+)= A[smem desc] . B[smem desc]^T, bf16 inputs, fp32 accumulate, over a CTA pair (M = 256); ACC is a compile-time constant so that no predicate has to be computed in
 // the issuing thread
 template <int ACC>
 __device__ __forceinline__ void umma_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
@@ -198,15 +147,6 @@ __device__ __forceinline__ void tmem_ld_frag_x4(uint32_t taddr, uint32_t *r) {  
         : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// D[16 x 8] += A[16 x 16] . B[16 x 8], bf16 operands, fp32 accumulate (warp-level tensor op)
-__device__ __forceinline__ void mma_16816(float *d, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                          uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, "
-        "%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
 
 // K-major, 128B-swizzled operand tile in shared memory: rows of 128 B, 8-row groups 1024 B apart
 __device__ __forceinline__ uint64_t make_desc(uint32_t smem_addr) {

@@ -753,3 +753,88 @@ def test_int8_attention_is_as_precise_as_in_fp32(shape):
         rel[kernel] = [np.linalg.norm(got[r] - ref) / np.linalg.norm(ref) for got, ref, r in res.values()]
     for auto, fp32 in zip(rel[B.KERNEL_AUTO], rel[B.KERNEL_GENERIC]):
         assert auto <= 1.01 * fp32, (auto, fp32)
+
+
+# Shapes past what the latent-attention kernels once took, and past what they take: name -> (config, changes, AE hidden width or None)
+BEYOND = {
+    "latent_576": ("c2", dict(latent_full=576), None),                                   # GPT-2 shape at 25 % compression
+    "latent_576_no_reuse": ("c2", dict(latent_full=576, reuse_frac=0.0), None),          # (with reuse a hidden layer is 504 wide)
+    "hidden_768": ("c2", {}, 768),                                                       # 12 heads, hidden layer above 640
+    "32_heads_of_their_own": ("c3", dict(n_q_heads=32, n_kv_heads=32, latent_full=512), 272),
+    "32_heads_in_pairs_wide": ("c3", dict(n_q_heads=32, n_kv_heads=16, latent_full=512), None),
+    "40_heads": ("c3", dict(n_q_heads=40, n_kv_heads=8, latent_full=256), None),
+    "hidden_1040": ("c2", {}, 1040),
+    "eight_sources": ("c2", dict(n_layers=8), None),
+}
+
+
+def _beyond(shape, int8, kernel, monkeypatch):
+    cfg, kw, hidden = BEYOND[shape]
+    if hidden:
+        real = synth.ae_dims
+        monkeypatch.setattr(synth, "ae_dims", lambda *a: (real(*a)[0], hidden, real(*a)[2]))
+    w = synth.scaled(synth.CONFIGS[cfg], **{**dict(n_layers=2, batch=4, cached_tokens=0, decode_steps=1, reuse_frac=0.25), **kw})
+    src = None
+    if shape == "eight_sources":       # head h of the top layer reads layer h (heads 7.. the top layer's own)
+        src = -np.ones((8, 12), np.int32)
+        for h in range(7):
+            src[h + 1:, h] = h
+        src = src.reshape(-1)
+    p = Pair(w, max_seqs=4, max_pages=64, max_pages_per_seq=18, src_k=src, src_v=src, latent_quant=int8, kernel=kernel)
+    p.open([0, 1, 2, 3])
+    for s_, n in zip(range(4), (1, 127, 0, 1100)):
+        if n:
+            p.prefill([s_], n)
+    return w, p
+
+
+@pytest.mark.parametrize("shape,kernel", [(s, B.KERNEL_AUTO) for s in sorted(BEYOND)] +
+                         [(s, B.KERNEL_TENSOR) for s in ("latent_576_no_reuse", "hidden_768", "32_heads_in_pairs_wide", "40_heads")])
+def test_bf16_layers_of_every_shape_have_a_fast_path(shape, kernel, monkeypatch):
+    """Wide latents, wide hidden layers, many heads, many source layers: against the oracle, through the two calls and the single one,
+    and never on the restoring kernel (which is two launches per call; the others are three or more)."""
+    w, p = _beyond(shape, False, kernel, monkeypatch)
+    seqs = [0, 1, 2, 3]
+    _check_step(p.decode_step(seqs, 0), "bf16", f"{shape} two calls")
+    _check_step(p.decode_step(seqs, 1, fused=True), "bf16", f"{shape} one call")
+    q = np.stack([synth.make_q(w, w.n_layers - 1, s_, 9) for s_ in seqs])
+    before = p.s.ctx.launch_count()
+    got, ref, rows = p.attention(w.n_layers - 1, seqs, q, include_current=False)
+    assert p.s.ctx.launch_count() - before >= 3
+    assert_close(got[rows], ref, "bf16", f"{shape} cached only")
+
+
+@pytest.mark.parametrize("shape", sorted(BEYOND))
+def test_int8_layers_of_every_shape_have_a_fast_path(shape, monkeypatch):
+    """The same with int8 rows."""
+    w, p = _beyond(shape, True, B.KERNEL_AUTO, monkeypatch)
+    seqs = [0, 1, 2, 3]
+    _check_step(p.decode_step(seqs, 0), "bf16", f"int8 {shape} two calls")
+    _check_step(p.decode_step(seqs, 1, fused=True), "bf16", f"int8 {shape} one call")
+    q = np.stack([synth.make_q(w, w.n_layers - 1, s_, 9) for s_ in seqs])
+    before = p.s.ctx.launch_count()
+    p.attention(w.n_layers - 1, seqs, q)
+    assert p.s.ctx.launch_count() - before >= 3
+
+
+@pytest.mark.parametrize("shape", ["hidden_1040", "32_heads_of_their_own"])
+def test_the_tensor_choice_is_refused_where_it_always_was(shape, monkeypatch):
+    """KVCAR_KERNEL_TENSOR: hidden layers above 1024 and rows wider than 1024 stay UNSUPPORTED."""
+    with pytest.raises(B.KvcarError) as e:
+        _beyond(shape, False, B.KERNEL_TENSOR, monkeypatch)
+    assert e.value.status == 5
+
+
+@pytest.mark.parametrize("page_tokens", [16, 48])
+def test_bf16_pages_that_are_no_multiple_of_64_tokens(page_tokens):
+    """Pages the tensor loads cannot take: the fp32 kernels."""
+    w = synth.scaled(synth.CONFIGS["c2"], n_layers=2, batch=3, page_tokens=page_tokens, reuse_frac=0.25)
+    per = 320 // page_tokens + 1
+    p = Pair(w, max_seqs=3, max_pages=3 * per, max_pages_per_seq=per)
+    p.open([0, 1, 2])
+    for s_, n in zip(range(3), (300, 49, 1)):
+        p.prefill([s_], n)
+    before = p.s.ctx.launch_count()
+    p.attention(1, [0, 1, 2], np.stack([synth.make_q(w, 1, s_, 9) for s_ in range(3)]))
+    assert p.s.ctx.launch_count() - before >= 4
+    _check_step(p.decode_step([0, 1, 2], 0, fused=True), "bf16", f"pages of {page_tokens}")
