@@ -343,7 +343,7 @@ kvcar_status kvcar_layer_work_absorbed(kvcar_ctx *ctx, int32_t layer, int32_t bo
 /* Number of kernels the library has launched so far on this context. */
 kvcar_status kvcar_launch_count(kvcar_ctx *ctx, int64_t *count);
 /* Kernel family (kvcar_kernel: GENERIC, TENSOR or RAW) that kvcar_decode_attention will use
- * for `layer` (without KVCAR_ABSORBED flags) under the current kvcar_set_kernel choice; GENERIC
+ * for `layer` under the current kvcar_set_kernel choice; GENERIC
  * covers the fp32-FMA kernels.  Only after kvcar_bind_memory. */
 kvcar_status kvcar_layer_kernel(kvcar_ctx *ctx, int32_t layer, int32_t *kernel);
 /* Synchronise `stream` and report any asynchronous CUDA error or device-side

@@ -138,7 +138,7 @@ int stored_width(const kvcar_ctx *c, int layer, int which) {
     return (int)stored_heads(c, layer, which).size() * c->cfg.head_dim;
 }
 
-// Some layer over latent rows only that the tensor-core kernels do not take whatever the flags of a call: the fp32-FMA kernels get
+// Some layer over latent rows only that the tensor-core kernels do not take: the fp32-FMA kernels get
 // their workspace (150 MB at 12 heads, hidden 576, 256 sequences; contexts that need none get none).
 bool needs_fma(const kvcar_ctx *c) {
     const kvcar_config &g = c->cfg;
@@ -431,7 +431,7 @@ bool layer_is_raw(const kvcar_ctx *c, int layer) {
 // hidden layers up to 1024), which an earlier tensor-core kernel took and the fp32-FMA kernels run now.
 bool takes_tensor_request(const kvcar_ctx *c, int layer) {
     const kvcar_config &g = c->cfg;
-    if (c->lat.available && lat_layer_supported(c->lat, layer, KVCAR_ABSORBED | KVCAR_ABSORBED_V)) return true;
+    if (lat_layer_supported(c->lat, layer)) return true;
     if (!fma_layer_supported(c->fma, layer) || g.storage != KVCAR_BF16 || g.latent_quant || g.head_dim != 64 || g.page_tokens % 64 ||
         g.n_q_heads / g.n_kv_heads > 8)
         return false;
@@ -1093,8 +1093,8 @@ static kvcar_status enqueue_combine(kvcar_ctx *c, int32_t layer, const DecodeArg
 }
 
 // the latent-attention kernels take this call
-static bool use_latent(const kvcar_ctx *c, int32_t layer, int n_chunks, uint32_t flags) {
-    return n_chunks > 0 && use_tensor_kernel(c) && lat_layer_supported(c->lat, layer, flags);
+static bool use_latent(const kvcar_ctx *c, int32_t layer, int n_chunks) {
+    return n_chunks > 0 && use_tensor_kernel(c) && lat_layer_supported(c->lat, layer);
 }
 // all of such a call; with k and v the encoder of the same step's rows goes along in the same launches
 static kvcar_status enqueue_latent(kvcar_ctx *c, int32_t layer, const DecodeArgs &a, const SeqList &sl, const void *k, const void *v,
@@ -1153,7 +1153,7 @@ kvcar_status kvcar_decode_attention(kvcar_ctx *c, int32_t layer, const int32_t *
     DecodeArgs a;
     SeqList sl;
     const int n_chunks = prepare_decode(c, layer, seqs, n_seqs, q, out, flags, a, sl);
-    if (use_latent(c, layer, n_chunks, flags)) return enqueue_latent(c, layer, a, sl, nullptr, nullptr, st);
+    if (use_latent(c, layer, n_chunks)) return enqueue_latent(c, layer, a, sl, nullptr, nullptr, st);
     s = enqueue_decode_tiles(c, layer, a, sl, n_chunks, st);
     if (s != KVCAR_OK) return s;
     return enqueue_combine(c, layer, a, sl, n_chunks, st);
@@ -1175,7 +1175,7 @@ kvcar_status kvcar_step_layer(kvcar_ctx *c, int32_t layer, const int32_t *seqs, 
     DecodeArgs a;
     SeqList sl;
     const int n_chunks = prepare_decode(c, layer, seqs, n_seqs, q, out, flags, a, sl);
-    if (use_latent(c, layer, n_chunks, flags)) return enqueue_latent(c, layer, a, sl, k, v, st);
+    if (use_latent(c, layer, n_chunks)) return enqueue_latent(c, layer, a, sl, k, v, st);
     // a raw layer has no encoder: its new rows are copied in the tile kernel's launch
     if (n_chunks > 0 && c->kernel != KVCAR_KERNEL_GENERIC && layer_is_raw(c, layer) && !c->ae[layer * 2].set && !c->ae[layer * 2 + 1].set) {
         const EncodeArgs rows = encode_args(c, layer, 1, k, v);
@@ -1401,7 +1401,7 @@ kvcar_status kvcar_layer_kernel(kvcar_ctx *c, int32_t layer, int32_t *kernel) {
     if (c->kernel != KVCAR_KERNEL_GENERIC && layer_is_raw(c, layer))
         *kernel = KVCAR_KERNEL_RAW;
     else
-        *kernel = (use_tensor_kernel(c) && lat_layer_supported(c->lat, layer, 0)) ? KVCAR_KERNEL_TENSOR : KVCAR_KERNEL_GENERIC;
+        *kernel = (use_tensor_kernel(c) && lat_layer_supported(c->lat, layer)) ? KVCAR_KERNEL_TENSOR : KVCAR_KERNEL_GENERIC;
     return KVCAR_OK;
 }
 

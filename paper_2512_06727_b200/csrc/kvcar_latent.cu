@@ -86,13 +86,15 @@ constexpr int HID_WARP = 4, N_OUT = 8;    // first hidden warp, output warps
 constexpr int READY_BARS = 8;             // jobs' terms between their epilogue and their product: at most as many as slabs
 
 // What follows from the hidden columns of a job: 192 where the hidden vector is one bf16 term, 128 where it is two (two slabs
-// of each term: U's products take their 128 features from a pair of slabs, so a job is one such pair per term).
+// of each term: U's products take their 128 features from a pair of slabs, so a job is one such pair per term), and where latents of
+// more than seven slabs leave no room for more (two or four hidden slabs and two weight slabs of 8 KB: latents up to 640 wide).
 __host__ __device__ constexpr int wstage(int cn) { return cn / 2 * 128; }  // this CTA's half of a weight slab
 __host__ __device__ constexpr int n_threads(int cn) { return 32 * (HID_WARP + 4 * (cn / 64) + N_OUT); }
 
 // Query heads padded to NQ.  Up to 16: high and low terms of an operand are rows of one operand.  32: the terms of W4^T q
 // are two operands, and so are those of the probabilities in the P2 builds.  The others take one term of the probabilities: bf16 rows
-// of groups of more than two heads, whose restoring form rounds restored K, restored V and the probabilities to bf16, the same class.
+// of groups of more than two heads, whose restoring form rounds restored K, restored V and the probabilities to bf16, the same class
+// (of groups of up to two it keeps the probabilities in fp32).
 __host__ __device__ constexpr int op_rows(int nq) { return nq <= 16 ? 2 * nq : nq; }  // operand rows of a CTA in S and U
 __host__ __device__ constexpr int wq_rows(int nq) { return 2 * nq; }                  // rows of W4^T q per sequence and source
 __host__ __device__ constexpr int wq_slab(int nq) { return wq_rows(nq) * 128; }       // one 64-column slab of them
@@ -739,6 +741,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                         for (int t = 1; t < TILE / 16; ++t)
                             umma_pair<1>(accu, da + (uint64_t)(t * (16 * 128 >> 4)),
                                          p_desc + (uint64_t)((t >> 2) * (PSLAB >> 4) + (t & 3) * 2), idesc_u);
+                        if (P2 && a.two_terms_v) {
+#pragma unroll
+                            for (int t = 0; t < TILE / 16; ++t)
+                                umma_pair<1>(accu, da + (uint64_t)(t * (16 * 128 >> 4)),
+                                             p_desc + (uint64_t)((2 + (t >> 2)) * (PSLAB >> 4) + (t & 3) * 2), idesc_u);
+                        }
                         umma_commit_pair(h_free + 8 * h0);
                         if (hs != h0) umma_commit_pair(h_free + 8 * hs);
                         umma_commit_pair(o_full + 8 * ob);
@@ -1452,7 +1460,7 @@ __global__ void __launch_bounds__(256) latent_widen_kernel(const __grid_constant
 }
 
 using Kernel = void (*)(const Params);
-// Builds, the narrowest first of each kind.
+// Builds, the narrowest first of each kind, jobs of 192 columns before those of 128.
 struct Build {
     int nq, nb, cn;
     bool quant, p2;
@@ -1464,6 +1472,7 @@ constexpr Build build() {
 }
 const Build builds[] = {build<12, 2, 192, false, false>(), build<12, 5, 192, false, false>(), build<16, 5, 192, false, false>(),
                         build<16, 8, 192, false, false>(), build<32, 2, 192, false, false>(), build<32, 3, 192, false, false>(),
+                        build<32, 3, 192, false, true>(),  build<12, 5, 128, false, false>(), build<16, 8, 128, false, false>(),
                         build<12, 2, 128, true, false>(),  build<12, 5, 128, true, false>(),  build<16, 5, 128, true, false>(),
                         build<16, 8, 128, true, false>(),  build<32, 2, 128, true, true>(),   build<32, 3, 128, true, true>()};
 constexpr int N_BUILDS = sizeof(builds) / sizeof(builds[0]);
@@ -1475,7 +1484,8 @@ int smem_bytes(const Build &b, int nz, int nh, int nw, int nqs) {
 }
 constexpr int SMEM_MAX = 227 * 1024;
 
-int padded_heads(int hq) { return hq <= 12 ? 12 : hq <= 16 ? 16 : 32; }
+// one padding for all layers of a context, whose W4^T q rows share their place (12 heads: up to 640 hidden features in registers)
+int padded_heads(int hq, int max_m) { return hq <= 12 && max_m <= 640 ? 12 : hq <= 16 ? 16 : 32; }
 
 void fill_seqs(LatSeqs &q, const SeqList &seqs, const int32_t *lens, int n_sms) {
     uint32_t t = 0;
@@ -1506,7 +1516,7 @@ static bool shape_ok(const kvcar_config &cfg) {
 
 size_t lat_ws_bytes(const kvcar_config &cfg, int max_sources, int max_m, int max_d, int batch, int max_len) {
     if (!shape_ok(cfg) || max_sources <= 0 || max_m <= 0) return 0;
-    const size_t nq = padded_heads(cfg.n_q_heads), m_pad = ((size_t)max_m + 63) / 64 * 64;
+    const size_t nq = padded_heads(cfg.n_q_heads, max_m), m_pad = ((size_t)max_m + 63) / 64 * 64;
     const size_t wq = (size_t)std::min(max_sources, LT_MAX_SRC) * batch * wq_rows((int)nq) * m_pad * 2;
     const size_t bias = ((size_t)batch * cfg.n_q_heads * 4 + 255) / 256 * 256;
     const size_t runs = (size_t)LT_MAX_CTAS + batch;
@@ -1516,23 +1526,18 @@ size_t lat_ws_bytes(const kvcar_config &cfg, int max_sources, int max_m, int max
     return n;
 }
 
-// the build and the staging places of a layer, false where none fits
-static bool pick_build(int nq, bool quant, const LatShape &sh, LatLayerCfg &lc) {
-    if (!sh.widths_ok || sh.n_src[0] < 1 || sh.n_src[0] > LT_MAX_SRC || sh.n_src[1] < 1 || sh.n_src[1] > LT_MAX_SRC) return false;
-    int v = 0;
-    while (v < N_BUILDS && (builds[v].nq != nq || builds[v].quant != quant || builds[v].nb * 128 < sh.m)) ++v;
-    if (v == N_BUILDS) return false;
-    const int ks = (sh.d + 63) / 64, chunks = (sh.m + builds[v].cn - 1) / builds[v].cn;
-    // Staging places.  A side's latents stay for all its chunks (nz >= their slabs).  One-chunk layers get places for the
-    // other side's latents and six hidden slabs, because their jobs are shorter than the way from S to P; the others four
-    // hidden slabs: a chunk's three and the one its predecessor may leave unpaired, or a chunk's two terms of two.
+// Staging places of a layer under a build.  A side's latents stay for all its chunks (nz >= their slabs).  One-chunk layers get
+// places for the other side's latents and six hidden slabs, because their jobs are shorter than the way from S to P; the others four
+// hidden slabs: a chunk's three and the one its predecessor may leave unpaired, or two chunks' two, or a chunk's two terms of two.
+static bool pick_places(const Build &b, const LatShape &sh, LatLayerCfg &lc) {
+    const int ks = (sh.d + 63) / 64, chunks = (sh.m + b.cn - 1) / b.cn;
     int nh = chunks == 1 ? 6 : 4, nz = chunks == 1 ? std::max(4, 2 * ks) : ks, nw = 4, nqs = 4;
-    auto fits = [&]() { return smem_bytes(builds[v], nz, nh, nw, nqs) <= SMEM_MAX; };
+    auto fits = [&]() { return smem_bytes(b, nz, nh, nw, nqs) <= SMEM_MAX; };
     while (nw > 3 && !fits()) --nw;
     while (nqs > 2 && !fits()) --nqs;
     while (nz > ks && !fits()) --nz;
     while (nw > 2 && !fits()) --nw;
-    if (!fits() && quant) nh = 2;  // one term of a job at a time
+    if (!fits() && b.cn == 128) nh = 2;  // one chunk, or one term of it, at a time
     if (!fits()) return false;
     while (nqs < 12 && (++nqs, fits())) {}
     if (!fits()) --nqs;
@@ -1540,20 +1545,29 @@ static bool pick_build(int nq, bool quant, const LatShape &sh, LatLayerCfg &lc) 
     lc.nh = (uint8_t)nh;
     lc.nw = (uint8_t)nw;
     lc.nqs = (uint8_t)nqs;
-    lc.smem = std::max(smem_bytes(builds[v], nz, nh, nw, nqs), 120 * 1024);  // one CTA per SM: each takes all of tensor memory
-    lc.variant = (uint8_t)v;
-    lc.max_m = sh.m;
-    lc.max_mk = sh.mk;
+    lc.smem = std::max(smem_bytes(b, nz, nh, nw, nqs), 120 * 1024);  // one CTA per SM: each takes all of tensor memory
     return true;
 }
 
-// Groups of more than two query heads, or int8 rows, or up to 16 heads: see lat_layer_supported.
-static bool any_flags(const kvcar_config &cfg, int nq) { return nq <= 16 || cfg.n_q_heads / cfg.n_kv_heads > 2 || cfg.latent_quant; }
+// the build and the staging places of a layer, false where none fits
+static bool pick_build(const kvcar_config &cfg, int max_m, const LatShape &sh, LatLayerCfg &lc) {
+    if (!sh.widths_ok || sh.n_src[0] < 1 || sh.n_src[0] > LT_MAX_SRC || sh.n_src[1] < 1 || sh.n_src[1] > LT_MAX_SRC) return false;
+    const int nq = padded_heads(cfg.n_q_heads, max_m);
+    const bool quant = cfg.latent_quant != 0, p2 = nq > 16 && (quant || cfg.n_q_heads / cfg.n_kv_heads <= 2);
+    for (int v = 0; v < N_BUILDS; ++v) {
+        const Build &b = builds[v];
+        if (b.nq != nq || b.quant != quant || b.p2 != p2 || b.nb * 128 < sh.m || !pick_places(b, sh, lc)) continue;
+        lc.variant = (uint8_t)v;
+        lc.max_m = sh.m;
+        lc.max_mk = sh.mk;
+        return true;
+    }
+    return false;
+}
 
 bool lat_covers(const kvcar_config &cfg, int max_m, const LatShape &sh) {
     LatLayerCfg lc;
-    const int nq = padded_heads(cfg.n_q_heads);
-    return shape_ok(cfg) && any_flags(cfg, nq) && pick_build(nq, cfg.latent_quant != 0, sh, lc);
+    return shape_ok(cfg) && pick_build(cfg, max_m, sh, lc);
 }
 
 void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPlan> &plans, size_t pool_rows,
@@ -1574,9 +1588,8 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, LT_ENC_SMEM) != cudaSuccess) return;
     for (auto k : {latent_front_kernel<1>, latent_front_kernel<2>})
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, LT_ENC_SMEM) != cudaSuccess) return;
-    st.nq = padded_heads(cfg.n_q_heads);
+    st.nq = padded_heads(cfg.n_q_heads, max_m);
     st.group = group;
-    st.any_flags = any_flags(cfg, st.nq);
     st.m_pad = (max_m + 63) / 64 * 64;
     st.batch = batch;
     const size_t n_src = std::min(max_sources, LT_MAX_SRC), n_rows = n_src * batch * wq_rows(st.nq);
@@ -1606,15 +1619,18 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
         LatLayerCfg &lc = st.cfg[l];
         bool ok = true;
         LatShape sh;
-        const int cn = st.quant ? 128 : 192;
+        for (int w = 0; w < 2; ++w)
+            for (int s = 0; s < plans[l].w[w].n_src; ++s) {
+                const SourcePlan &sp = plans[l].w[w].src[s];
+                ok = ok && sp.compressed && (sp.qparam != nullptr) == st.quant && sp.width == sp.d;
+                sh.add(w, sp.d, sp.m);
+            }
+        if (!ok || !pick_build(cfg, max_m, sh, lc)) continue;
         for (int w = 0; w < 2 && ok; ++w) {
             const WhichPlan &wp = plans[l].w[w];
-            ok = wp.n_src > 0 && wp.n_src <= LT_MAX_SRC;
             ly.list[w].n = hp.n_src[w] = wp.n_src;
             for (int s = 0; s < wp.n_src && ok; ++s) {
                 const SourcePlan &sp = wp.src[s];
-                ok = sp.compressed && (sp.qparam != nullptr) == st.quant && sp.d % 16 == 0 && sp.m % 16 == 0 && sp.width == sp.d;
-                if (!ok) break;
                 LatSrc &d = ly.list[w].src[s];
                 d.shift = sp.shift;
                 d.rowsum = sp.rowsum;
@@ -1643,12 +1659,10 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
                 }
                 ok = (st.quant ? encode_bf16_map(fn, &ly.pool[w][s], reinterpret_cast<__nv_bfloat16 *>(st.wide) + region * max_d, wide_rows, sp.d, max_d)
                                : encode_bf16_map(fn, &ly.pool[w][s], sp.pool, pool_rows, sp.width, sp.width)) &&
-                     encode_bf16_map(fn, &ly.w1[w][s], sp.w1n, sp.m, sp.d, sp.d, cn / 2);
-                sh.add(w, sp.d, sp.m);
+                     encode_bf16_map(fn, &ly.w1[w][s], sp.w1n, sp.m, sp.d, sp.d, builds[lc.variant].cn / 2);
             }
         }
         if (!ok) continue;
-        if (!pick_build(st.nq, st.quant, sh, lc)) continue;
         if (cudaFuncSetAttribute(builds[lc.variant].kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess) {
             cudaGetLastError();
             continue;
@@ -1658,12 +1672,7 @@ void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPla
     }
 }
 
-bool lat_layer_supported(const LatState &st, int layer, uint32_t flags) {
-    if (!st.available || !st.cfg[layer].ok) return false;
-    // 17 to 32 query heads over bf16 rows: the probabilities are one bf16 term.  For groups of up to two heads they have always been
-    // more than that, so those take this path only where the caller has asked for that rounding.
-    return st.any_flags || ((flags & KVCAR_ABSORBED) && (flags & KVCAR_ABSORBED_V));
-}
+bool lat_layer_supported(const LatState &st, int layer) { return st.available && st.cfg[layer].ok; }
 
 namespace {
 
@@ -1709,7 +1718,7 @@ static cudaError_t launch_group(LatState &st, const DecodeArgs &a, const SeqList
     const Build &b = builds[lc.variant];
     Params p;
     fill_seqs(p.sq, seqs, lens, st.n_sms);
-    const bool two_k = !(a.flags & KVCAR_ABSORBED), two_v = !((a.flags & KVCAR_ABSORBED) && (a.flags & KVCAR_ABSORBED_V));
+    const bool two_k = !(a.flags & KVCAR_ABSORBED), two_v = !((a.flags & KVCAR_ABSORBED) && (a.flags & KVCAR_ABSORBED_V)) && (b.nq <= 16 || b.p2);
     LatEncode e{};
     if (enc_in) e = *enc_in;
     EncodeGrid g{0, 1, 1};

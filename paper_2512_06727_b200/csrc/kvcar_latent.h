@@ -99,7 +99,6 @@ struct LatState {
     int n_sms = 148;
     int nq = 12;      // query heads padded
     int group = 1;    // query heads per KV head
-    bool any_flags = true;  // layers are taken whatever the flags of a call
     int m_pad = 0;    // row pitch of the vectors below
     int batch = 0;    // sequences per call at most
     void *wq = nullptr;      // [source][batch][operand rows][m_pad] bf16: W4_h^T q, high parts then low parts
@@ -112,13 +111,12 @@ struct LatState {
 
 // bytes of the operands and partial results inside the workspace (0: the shape does not take this path)
 size_t lat_ws_bytes(const kvcar_config &cfg, int max_sources, int max_m, int max_d, int batch, int max_len);
-// whether every call on such a layer takes this path (max_m: widest hidden layer of the context)
+// whether the kernels take such a layer (max_m: widest hidden layer of the context)
 bool lat_covers(const kvcar_config &cfg, int max_m, const LatShape &sh);
 // decide per layer whether the kernels take it, build tensor maps, place the workspace area
 void lat_setup(LatState &st, const kvcar_config &cfg, const std::vector<LayerPlan> &plans, size_t pool_rows,
                int max_sources, int max_m, int max_d, int batch, int max_len, char *ws_area);
-// flags: those of the call (17 to 32 query heads in groups of at most two only with KVCAR_ABSORBED_V, see kvcar_latent.cu)
-bool lat_layer_supported(const LatState &st, int layer, uint32_t flags);
+bool lat_layer_supported(const LatState &st, int layer);
 // The encoder of the same step's new rows, carried by the first and the last launch (null: none).
 struct LatEncode {
     EncodeArgs a;

@@ -761,11 +761,18 @@ BEYOND = {
     "latent_576_no_reuse": ("c2", dict(latent_full=576, reuse_frac=0.0), None),          # (with reuse a hidden layer is 504 wide)
     "hidden_768": ("c2", {}, 768),                                                       # 12 heads, hidden layer above 640
     "32_heads_of_their_own": ("c3", dict(n_q_heads=32, n_kv_heads=32, latent_full=512), 272),
+    "32_heads_in_pairs": ("c3", dict(n_q_heads=32, n_kv_heads=16, latent_full=256), 384),
+    "16_heads": ("c2", dict(n_q_heads=16, n_kv_heads=16, latent_full=512), None),
     "32_heads_in_pairs_wide": ("c3", dict(n_q_heads=32, n_kv_heads=16, latent_full=512), None),
     "40_heads": ("c3", dict(n_q_heads=40, n_kv_heads=8, latent_full=256), None),
     "hidden_1040": ("c2", {}, 1040),
     "eight_sources": ("c2", dict(n_layers=8), None),
 }
+
+
+# those of them that the latent-attention kernels take: with jobs of 128 columns (latents above 448), 12 heads padded to 16 (hidden layers
+# above 640), probabilities in two operands (32 heads in small groups)
+BEYOND_TENSOR = {"latent_576_no_reuse", "hidden_768", "32_heads_in_pairs", "16_heads"}
 
 
 def _beyond(shape, int8, kernel, monkeypatch):
@@ -795,6 +802,8 @@ def test_bf16_layers_of_every_shape_have_a_fast_path(shape, kernel, monkeypatch)
     and never on the restoring kernel (which is two launches per call; the others are three or more)."""
     w, p = _beyond(shape, False, kernel, monkeypatch)
     seqs = [0, 1, 2, 3]
+    if shape in BEYOND_TENSOR:
+        assert all(p.s.ctx.layer_kernel(l) == B.KERNEL_TENSOR for l in range(w.n_layers))
     _check_step(p.decode_step(seqs, 0), "bf16", f"{shape} two calls")
     _check_step(p.decode_step(seqs, 1, fused=True), "bf16", f"{shape} one call")
     q = np.stack([synth.make_q(w, w.n_layers - 1, s_, 9) for s_ in seqs])
@@ -817,11 +826,15 @@ def test_int8_layers_of_every_shape_have_a_fast_path(shape, monkeypatch):
     assert p.s.ctx.launch_count() - before >= 3
 
 
-@pytest.mark.parametrize("shape", ["hidden_1040", "32_heads_of_their_own"])
-def test_the_tensor_choice_is_refused_where_it_always_was(shape, monkeypatch):
-    """KVCAR_KERNEL_TENSOR: hidden layers above 1024 and rows wider than 1024 stay UNSUPPORTED."""
+def test_the_tensor_choice_is_refused_where_it_always_was(monkeypatch):
+    """KVCAR_KERNEL_TENSOR: hidden layers above 1024 and more than six source layers stay UNSUPPORTED."""
     with pytest.raises(B.KvcarError) as e:
-        _beyond(shape, False, B.KERNEL_TENSOR, monkeypatch)
+        _beyond("hidden_1040", False, B.KERNEL_TENSOR, monkeypatch)
+    assert e.value.status == 5
+    monkeypatch.undo()
+    w, p = _beyond("eight_sources", False, B.KERNEL_TENSOR, monkeypatch)
+    with pytest.raises(B.KvcarError) as e:
+        p.attention(7, [0, 1], np.stack([synth.make_q(w, 7, s_, 9) for s_ in (0, 1)]))
     assert e.value.status == 5
 
 
@@ -838,3 +851,24 @@ def test_bf16_pages_that_are_no_multiple_of_64_tokens(page_tokens):
     p.attention(1, [0, 1, 2], np.stack([synth.make_q(w, 1, s_, 9) for s_ in range(3)]))
     assert p.s.ctx.launch_count() - before >= 4
     _check_step(p.decode_step([0, 1, 2], 0, fused=True), "bf16", f"pages of {page_tokens}")
+
+
+@pytest.mark.parametrize("shape,int8", [("latent_576_no_reuse", False), ("latent_576_no_reuse", True), ("hidden_768", False),
+                                        ("32_heads_in_pairs", False), ("16_heads", True)])
+def test_runs_of_several_tiles_beyond(shape, int8, monkeypatch):
+    """The builds of the wider shapes with more tiles than blocks: each walks several, across sequence ends and partial tiles."""
+    cfg, kw, hidden = BEYOND[shape]
+    if hidden:
+        real = synth.ae_dims
+        monkeypatch.setattr(synth, "ae_dims", lambda *a: (real(*a)[0], hidden, real(*a)[2]))
+    w = synth.scaled(synth.CONFIGS[cfg], **{**dict(n_layers=1, batch=48, reuse_frac=0.0), **kw, "n_layers": 1})
+    seqs = list(range(48))
+    lens = [128 * (5 * s % 8) + (1, 127, 128, 60)[s % 4] for s in seqs]
+    p = Pair(w, max_seqs=48, max_pages=48 * 17, max_pages_per_seq=17, latent_quant=int8)
+    p.oracle_seqs = {0, 23, 47}
+    p.open(seqs)
+    for s_, n in zip(seqs, lens):
+        p.prefill([s_], n)
+    assert p.s.ctx.layer_kernel(0) == B.KERNEL_TENSOR
+    for step in range(2):
+        _check_step(p.decode_step(seqs, step, fused=True), "bf16", f"{shape} int8 {int8} step {step}")
