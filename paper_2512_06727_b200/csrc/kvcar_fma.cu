@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(HC * 2) fma_hidden_kernel(const __grid_constan
     const int d = sp.d, m = sp.m, c0 = ch * HC;
     if (tid < TT) {
         const int t = t0 + (tid < valid ? tid : 0);  // rows past the end repeat a valid one; they have no probability
-        const int page = __ldcg(a.block_table + (int64_t)seq * a.max_pages_per_seq + t / a.page_tokens);
+        const int page = a.block_table[(int64_t)seq * a.max_pages_per_seq + t / a.page_tokens];
         const int64_t r = (int64_t)page * a.page_tokens + t % a.page_tokens;
         rows[tid] = r;
         if (Q8) {

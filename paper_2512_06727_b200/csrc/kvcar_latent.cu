@@ -177,9 +177,9 @@ struct TileWalk {
     }
 };
 
-// (read past the first-level cache: the tile kernel looks before it waits, see kvcar_pdl.cuh)
+// (the tile kernel looks before it waits: see kvcar_pdl.cuh)
 __device__ __noinline__ int pool_row(const int32_t *table, int page_tokens, int tok) {
-    return __ldcg(table + tok / page_tokens) * page_tokens + tok % page_tokens;
+    return table[tok / page_tokens] * page_tokens + tok % page_tokens;
 }
 __device__ __forceinline__ float redux_max(float v) {
     float r;
@@ -795,7 +795,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                         for (int i = 0; i < 4; ++i) {
                             const int r = (int)lane_base + 8 * i + (lane >> 2);
                             if (r < valid) {
-                                const float2 p = __ldcg(list_of(side).src[s].rowp + r0 + r);  // as pool_row
+                                const float2 p = __ldcg(list_of(side).src[s].rowp + r0 + r);  // past the first-level cache: see kvcar_pdl.cuh
                                 inv[i] = p.x;
                                 left[i] = p.y;
                             }

@@ -4,10 +4,12 @@
 // What a kernel may read before its own wait.  The wait is what makes its predecessor's writes visible; launch_dependents is no
 // release.  decode_latent_kernel and fma_hidden_kernel start on page table, cached rows and (int8) widened rows before they wait.
 // Their predecessors in the stream (latent_front_kernel, fma_query_kernel) let them start only after a wait of their own, so whatever
-// was enqueued before those is complete and written back to L2 by then, and that is where these reads go: tensor loads (which know no
-// other cache) and __ldcg for the table and the row parameters, whose addresses are written again from call to call.  Cached rows
-// that fma_hidden_kernel reads through the first-level cache lie below the sequences' lengths: a row gets there by kvcar_advance,
-// whose table update is an ordinary launch, behind everything before it and in front of everything after it.
+// was enqueued before those is complete and written back to L2 by then.  What is left is an older line in an SM's first-level cache.
+//   - Page table and cached rows below the sequences' lengths are written, or counted in (kvcar_advance), by the table update, an
+//     ordinary launch: behind everything before it and in front of everything after it, so no kernel after it meets older lines.
+//   - The widened int8 rows and their parameters are written again by every layer of a step with dependent launches all the way, so
+//     they are read where no first-level cache stands between: tensor loads, and __ldcg for the parameters.
+// (The table past that cache as well: 12-layer step of GPT-2's shape, 1 x 200 tokens, 337 -> 341 us, TinyLLaMA 4 x 32768 1653 -> 1669.)
 #pragma once
 #include <cuda_runtime.h>
 
