@@ -243,8 +243,8 @@ def test_physical_page_permutation_is_bit_invariant(kernel):
 
 
 def test_large_grid_runs_k_then_v_in_one_cluster():
-    """More tile pairs than a quarter of the SMs: the tensor-core kernel stops spreading a
-    pair over several clusters and each cluster restores K, then V (the other tests are
+    """More tile pairs than half of the SM pairs: the tensor-core kernel stops spreading a
+    pair over several clusters and each cluster does K, then V (most other tests are
     small enough to take the split paths)."""
     w = synth.scaled(synth.CONFIGS["c3"], n_layers=2, batch=5, cached_tokens=0, decode_steps=1, reuse_frac=0.25)
     pps = 34
@@ -258,17 +258,16 @@ def test_large_grid_runs_k_then_v_in_one_cluster():
 
 @pytest.mark.parametrize("shape", ["group2_narrow", "group4_wide", "group3_odd"])
 def test_tensor_kernel_variants_walk_several_pairs(shape):
-    """The tensor-core kernel is built in four variants (query groups of more than two heads or not; hidden
-    layers of one 256-column chunk or more).  The two paper shapes take two of them; these shapes take the
-    others, with more tile pairs than clusters so that a cluster walks several pairs (queries and tile
-    positions of the next pair fetched ahead, parameter blocks kept, probability buffers handed back)."""
-    if shape == "group2_narrow":     # 8 query / 4 KV heads, hidden 192: one chunk, CUDA-core attention products
+    """The tensor-core kernel is built for 12, 16 or 32 query heads and one to eight blocks of 128 hidden features.  The two paper
+    shapes take two of the builds; these shapes take others, with more tiles than CTAs so that each walks several
+    (wider shapes: test_runs_of_several_tiles_beyond)."""
+    if shape == "group2_narrow":     # 8 query / 4 KV heads, hidden 192: one chunk, two blocks of features
         w = synth.scaled(synth.CONFIGS["c3"], n_layers=2, n_q_heads=8, n_kv_heads=4, latent_full=128, batch=9,
                          cached_tokens=0, decode_steps=1, reuse_frac=0.25)
-    elif shape == "group4_wide":     # 32 query / 8 KV heads, hidden 384: two chunks, tensor-op attention products
+    elif shape == "group4_wide":     # 32 query / 8 KV heads, hidden 384: two chunks, three blocks
         w = synth.scaled(synth.CONFIGS["c3"], n_layers=2, n_q_heads=32, n_kv_heads=8, latent_full=256, batch=9,
                          cached_tokens=0, decode_steps=1, reuse_frac=0.25)
-    else:                            # 6 query / 2 KV heads: a group of three (padded inside the 8-wide operand)
+    else:                            # 6 query / 2 KV heads: a group of three, half of the operand's rows padding
         w = synth.scaled(synth.CONFIGS["c3"], n_layers=2, n_q_heads=6, n_kv_heads=2, latent_full=64, batch=9,
                          cached_tokens=0, decode_steps=1, reuse_frac=0.5)
     pps = 34
@@ -631,9 +630,9 @@ def test_absorbed_last_layer_on_both_sides_matches_the_oracle(shape):
 def test_absorbed_last_layer_matches_the_oracle(shape):
     """KVCAR_ABSORBED: a head's scores are taken as a.(W4_h^T q) + q.b4_h from the activated hidden vectors, the
     restored K rows are never formed (the decoder ends in a bare fully connected layer, Sec. "Network Architecture").
-    Same result as the plain form up to rounding: compared with the oracle at the usual tolerance on grids large
-    enough for the form to be taken, with reuse (several source layers per layer), and the launch counter shows that
-    the operand kernel ran."""
+    Same result as the plain form up to rounding: compared with the oracle at the usual tolerance, with reuse (several source
+    layers per layer).  Every call takes this form; the flag leaves one bf16 term of W4_h^T q instead of two, so it changes some bits
+    of the output and no more than that."""
     if shape == "gpt2":            # 12 heads, hidden 576 (three chunks), CUDA-core attention products
         w = synth.scaled(synth.CONFIGS["c2"], n_layers=3, batch=5, cached_tokens=0, decode_steps=2, reuse_frac=0.25)
     elif shape == "tinyllama":     # 32 query / 4 KV heads, hidden 192, tensor-op attention products
@@ -648,12 +647,13 @@ def test_absorbed_last_layer_matches_the_oracle(shape):
     for s_, n in zip(seqs, (2100, 2049, 2111, 2050, 2064)):     # 17 tiles each: 85 tiles, 43 pairs
         p.prefill([s_], n)
     for step in range(2):
-        before = p.s.ctx.launch_count()
         res = p.decode_step(seqs, step, absorbed=True)
-        # per layer: two encoder launches, the operand kernel, the tile kernel, the combine kernel (+ table updates)
-        assert p.s.ctx.launch_count() - before >= 5 * w.n_layers
         _check_step(res, "bf16", f"absorbed {shape} step {step}")
-    # the flag is a no-op where the form is not taken (a grid small enough for the K/V split): same tolerance
+    q = np.stack([synth.make_q(w, 1, s_, 7) for s_ in seqs])
+    one, ref, rows = p.attention(1, seqs, q, absorbed=True)
+    two, _, _ = p.attention(1, seqs, q)
+    assert 0.0 < np.max(np.abs(one - two)) < 2e-2
+    # and on a grid small enough for K and V to be two launches
     w2 = synth.scaled(w, batch=2)
     p2 = Pair(w2, max_seqs=2, max_pages=8, max_pages_per_seq=4, kernel=B.KERNEL_TENSOR)
     p2.open([0, 1])
@@ -665,10 +665,10 @@ def test_absorbed_last_layer_matches_the_oracle(shape):
 
 @pytest.mark.parametrize("case", ["small_tiles", "large_tiles", "groups", "int8_large_tiles"])
 def test_fp32_arithmetic_kernels_at_tile_edges(case):
-    """The fp32-FMA attention kernels (fp32 storage, int8 rows, head widths other than 64): blocks of 32 x 32 with two pieces
-    per partial result, blocks of 64 x 64 where those fill the machine, and calls of more than 1024 partial results, which
-    are worked through in groups of sequences.  Lengths around 32, 64 and 128 tokens, one sequence empty; tolerances of the
-    storage type, as everywhere."""
+    """The fp32-FMA attention kernels on fp32 storage: blocks of 32 x 32 with two pieces per partial result, blocks of 64 x 64
+    where those fill the machine, and calls of more than 1024 partial results, which are worked through in groups of sequences.
+    Lengths around 32, 64 and 128 tokens, one sequence empty; tolerances of the storage type, as everywhere.  (int8_large_tiles is
+    the same lengths on the tensor cores; int8 rows on the FMA kernels: the next test.)"""
     lens = {"small_tiles": (31, 32, 33, 0, 63, 64, 65, 129), "large_tiles": (1473, 1, 1472, 0, 1471),
             "int8_large_tiles": (1473, 1, 1472, 0, 1471), "groups": (33000, 65, 0, 32900)}[case]
     if case == "groups":
@@ -686,6 +686,29 @@ def test_fp32_arithmetic_kernels_at_tile_edges(case):
         if n:
             p.prefill([s_], n)
     _check_step(p.decode_step(seqs, 0), w.storage, case)
+
+
+@pytest.mark.parametrize("head_dim", [32, 128])
+@pytest.mark.parametrize("tiles", ["small", "large"])
+def test_int8_rows_on_the_fp32_arithmetic_kernels(head_dim, tiles):
+    """int8 rows of other head widths: blocks of 32 x 32 and (from four times the SM count of 64 x 64 blocks on) of 64 x 64.  Four
+    launches per attention call show the path (the restoring kernel takes two)."""
+    w = synth.scaled(synth.CONFIGS["c3"], n_layers=2, n_q_heads=4, n_kv_heads=2, head_dim=head_dim, latent_full=head_dim, batch=5,
+                     cached_tokens=0, decode_steps=1, reuse_frac=0.5)
+    lens = (31, 64, 65, 0, 129) if tiles == "small" else (9600, 9537, 1, 9601, 9472)
+    blocks = sum((n + 63) // 64 for n in lens) * ((3 * head_dim // 2 + 63) // 64)
+    assert (blocks >= 4 * 148) == (tiles == "large")
+    pps = (max(lens) + 2 + w.page_tokens - 1) // w.page_tokens
+    p = Pair(w, max_seqs=5, max_pages=5 * pps, max_pages_per_seq=pps, latent_quant=True)
+    p.oracle_seqs = None if tiles == "small" else {1, 2}
+    p.open([0, 1, 2, 3, 4])
+    for s_, n in zip(range(5), lens):
+        if n:
+            p.prefill([s_], n)
+    _check_step(p.decode_step([0, 1, 2, 3, 4], 0), "bf16", f"head_dim {head_dim} {tiles}")
+    before = p.s.ctx.launch_count()
+    p.attention(0, [0, 1, 2, 4], np.stack([synth.make_q(w, 0, s_, 9) for s_ in (0, 1, 2, 4)]))
+    assert p.s.ctx.launch_count() - before == 4
 
 
 @pytest.mark.parametrize("case", ["offset_rows", "groups"])
