@@ -46,19 +46,19 @@ def parse():
     ap.add_argument("--kernel", default="auto", choices=["auto", "generic", "tensor"])
     ap.add_argument("--uncompressed", action="store_true", help="raw K/V pages (the uncompressed twin)")
     ap.add_argument("--absorbed", action="store_true",
-                    help="pass KVCAR_ABSORBED: K scores from the hidden vectors (absorbed last decoder layer); the roofline "
-                         "then counts that form's own, smaller number of operations")
+                    help="pass KVCAR_ABSORBED: one bf16 term of W4^T q instead of two")
     ap.add_argument("--absorbed-v", action="store_true",
-                    help="with --absorbed: KVCAR_ABSORBED_V as well (the V side through the hidden vectors too)")
+                    help="with --absorbed: KVCAR_ABSORBED_V as well (one bf16 term of the probabilities)")
     ap.add_argument("--api", default="fused", choices=["fused", "split"],
-                    help="a layer's step through kvcar_step_layer (one call; the tile kernel runs beside the encoder) "
+                    help="a layer's step through kvcar_step_layer (one call; the encoder shares its launches) "
                          "or through kvcar_encode_append + kvcar_decode_attention")
     ap.add_argument("--head-l1", action="store_true",
                     help="instead of the decode step: time Alg. 2's head-distance reduction on K rows shaped like "
                          "the workload (layers x batch*cached_tokens x KV width) and print its own JSON line")
     ap.add_argument("--prefill", action="store_true",
                     help="instead of the decode step: time the bulk encoder + append of 1024 tokens per sequence, on the "
-                         "tensor cores (kvcar_encode_append_tensor) and on the CUDA cores, and print its own JSON line")
+                         "tensor cores with hidden activations in bf16 (kvcar_encode_append_tensor) and in fp32 "
+                         "(kvcar_encode_append), and print its own JSON line")
     ap.add_argument("--capacity", action="store_true",
                     help="instead of the decode step: longest sequence that fits per batch size at 0/25/50/75 %% compression from the\n"
                          "library's own bytes-per-token accounting, plus one batch actually held in memory compressed vs raw")
@@ -499,7 +499,7 @@ def run_prefill(args):
     K_, W_ = args.steps, max(args.warmup, 3)
     peaks = measured_peaks()
     out = {}
-    for name in ("tensor", "cuda_cores"):
+    for name in ("tensor", "fp32_hidden"):
         sess, src, aes = build_session(synth.scaled(w, cached_tokens=0), args, torch, chunk * (K_ + W_) + 8)
         seqs = list(range(w.batch))
         for q in seqs:
@@ -534,16 +534,16 @@ def run_prefill(args):
                       "roofline": {"bound": "tensor", "achieved": tf, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
                                    "frac": tf / peaks["bf16_tflops"], "traffic": None, "peak_source": peaks["source"] + " (burst)",
                                    "algorithmic_flops_per_step": flops},
-                      "cuda_core_encoder_ms_per_step": out["cuda_cores"]}))
+                      "fp32_hidden_encoder_ms_per_step": out["fp32_hidden"]}))
 
 
 NOMINAL_BF16_TFLOPS = 2250.0     # dense bf16 per B200 (vendor figure): context beside the measured peaks
 NOMINAL_HBM_GBS = 8000.0
 
-# DRAM bytes (read + write) per decode-kernel launch and listed sequence, from an ncu capture of the GPT-2-shaped
-# stack at 4096 cached tokens (batch 8, scaled by the batch: a launch's traffic is its sequences' latent rows)
-NCU_TRAFFIC = {"c5": {"bytes_per_sequence": 54.23e6 / 8, "captured_on": "c5_gpt2s_12l_L4096_b8",
-                      "profile": "profiles/decode_pair_kernel_c5.md"}}
+# DRAM bytes (read + write) of a decode_latent_kernel launch over its algorithmic bytes (the latent rows of its sources),
+# from an ncu capture of the GPT-2-shaped stack at 4096 cached tokens, batch 8: 89.64 MB for 83.89 MB of rows
+NCU_TRAFFIC = {"c5": {"over_algorithmic": 89.64 / 83.89, "captured_on": "c5_gpt2s_12l_L4096_b8",
+                      "profile": "profiles/decode_latent_kernel.md"}}
 
 
 def roofline_of(flops, byts, seconds, peaks, launches):
@@ -641,13 +641,14 @@ def measure(w, args, torch, B, steps, warmup, uncompressed, flush, peaks, fused=
     torch.cuda.synchronize()
     sess.ctx.sync_status(stream)
     plain_flops = sum(sess.ctx.layer_work_per_token(l)[1] * L * w.batch for (l, L, _, _) in kev)
-    flops = sum(sess.ctx.layer_work_absorbed(l, both) * L * w.batch for (l, L, _, _) in kev) if absorbed else plain_flops
+    # operations of the form that runs: every kernel but the restoring one applies the last decoder layer outside the tiles
+    own_form = args.kernel != "generic" and not uncompressed
+    flops = sum(sess.ctx.layer_work_absorbed(l, True) * L * w.batch for (l, L, _, _) in kev) if own_form else plain_flops
     byts = sum(sess.ctx.layer_work_per_token(l)[0] * L * w.batch for (l, L, _, _) in kev)
     kern_s = sum(a_.elapsed_time(b_) for (_, _, a_, b_) in kev) / 1e3
     roof = roofline_of(flops, byts, kern_s, peaks, len(kev))
-    if absorbed:   # the plain form's operations over the same time: what the absorbed form is worth as plain-form throughput
-        roof["form"] = ("absorbed K and V sides (KVCAR_ABSORBED | KVCAR_ABSORBED_V)" if both else
-                        "absorbed K scores (KVCAR_ABSORBED)") + ": achieved and frac count this form's own operations"
+    if own_form:   # the restoring form's operations over the same time: what the form that runs is worth as its throughput
+        roof["form"] = "last decoder layer outside the tiles: achieved and frac count this form's own operations"
         roof["plain_form_flops_per_launch"] = plain_flops / len(kev)
         roof["plain_form_equivalent_frac"] = plain_flops / kern_s / 1e12 / roof["peak"] if roof.get("bound") == "tensor" else None
     comp, full = sess.ctx.cache_bytes_per_token()
@@ -714,9 +715,9 @@ def main():
     cfg_key = args.workload
     if not args.uncompressed and args.kernel == "auto" and cfg_key in NCU_TRAFFIC:
         t = NCU_TRAFFIC[cfg_key]
-        roof["traffic"] = t["bytes_per_sequence"] * w.batch
-        roof["traffic_source"] = (f"ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch on {t['captured_on']}, "
-                                  f"scaled by the batch; {t['profile']}")
+        roof["traffic"] = t["over_algorithmic"] * roof["algorithmic_bytes_per_launch"]
+        roof["traffic_source"] = (f"algorithmic bytes x {t['over_algorithmic']:.3f}, the ratio of ncu dram__bytes_read.sum + "
+                                  f"dram__bytes_write.sum to them in one launch on {t['captured_on']}; {t['profile']}")
     sess, src, aes, k, v, q, out = head.pop("session")
     seqs = list(range(w.batch))
     stream = sess.stream()
@@ -811,16 +812,6 @@ def main():
                     row["raw_twin"] = {"tokens_per_s": u["tokens_per_s"], "us_per_launch": ru["avg_launch_us"],
                                        "bound": ru["bound"], "frac": ru["frac"], "achieved_gbs": ru["achieved"],
                                        "cache_bytes_per_token": u["cache_bytes_per_token"]}
-                # the headline workload once more with the K side in the absorbed form (same results up to rounding)
-                if wc.name == w.name and wc.storage == "bf16" and not args.absorbed and not args.uncompressed:
-                    class A2: pass
-                    for key, both_ in (("absorbed_k", False), ("absorbed_kv", True)):
-                        a2 = A2(); a2.kernel = args.kernel; a2.absorbed = True; a2.absorbed_v = both_
-                        ab = measure(wc, a2, torch, B, st_, 3, False, flush, peaks)
-                        ra = ab["roofline"]
-                        row[key] = {"tokens_per_s": ab["tokens_per_s"], "us_per_launch": ra["avg_launch_us"],
-                                    "frac_on_own_operation_count": ra["frac"],
-                                    "frac_if_credited_with_the_plain_form": ra.get("plain_form_equivalent_frac")}
             except Exception as ex:      # a configuration that does not fit or fails is reported, not fatal
                 row["error"] = str(ex)[:200]
             configs.append(row)
