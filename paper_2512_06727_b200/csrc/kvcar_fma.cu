@@ -1,4 +1,6 @@
-// Decode attention over latent rows in fp32 arithmetic: fp32 storage, int8 latent rows, head widths other than 64.
+// Decode attention over latent rows in fp32 arithmetic: fp32 storage, head widths other than 64, pages that are no multiple of 64 tokens,
+// and bf16 or int8 layers beyond the limits of kvcar_latent.cu (more than 32 query heads, hidden layers above 1024 or 384 with more than
+// 16 heads, more than six source layers, wide latents, widths that are no multiples of 16).
 //
 // The algebra of kvcar_latent.cu (the last decoder layer is linear, so it is applied to the query before and to the weighted
 // sum after the cached tokens) with everything in fp32 on the CUDA cores.  decode_generic_kernel, which restores every head of

@@ -23,7 +23,7 @@
 // decode_latent_kernel.  A cluster of two CTAs walks two runs of consecutive tiles in step, one run per CTA; every
 // product is one tcgen05.mma.cta_group::2 of M = 256 (both tiles), so a weight slab crosses L2 -> shared memory once
 // per 256 tokens, half into each CTA.  Per step the K side of a tile, then the V side of the tile before (so that the way from S to
-// the probabilities is behind the next scores' products), per source layer, per chunk of 192 hidden columns:
+// the probabilities is behind the next scores' products), per source layer, per chunk of 192 hidden columns (128: below):
 //   hidden   H[256 tok x 192] = Z[256 tok x d] . W1[192 x d]^T into one of two accumulators in tensor memory; the hidden
 //            warps add the shift, apply LeakyReLU, round to bf16 and write 64-column slabs into a ring.  The BatchNorm
 //            scale is not theirs: its sign is in W1, its size in W4^T q and in the merge (LeakyReLU is positively
@@ -1131,7 +1131,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
 // sources that do not serve the head are zeroed.
 // Every block runs its code once, so instruction fetch counts like the loads: with loops unrolled only where that keeps loads in flight,
 // addresses stepped instead of computed per load and the encoder's rows bounded, this kernel went from 63 to 39 KB of code and
-// latent_back_kernel from 41-47 to 33-37; 12 layers of GPT-2's shape, 1 x 200 tokens 355 -> 314 us, 8 x 1024 609 -> 580; 22 of
+// latent_back_kernel from 41-47 to 33-37; 12 layers of GPT-2's shape, 1 x 200 tokens an eighth less, 8 x 1024 609 -> 580 us; 22 of
 // TinyLLaMA's, 32 x 2048 1213 -> 1174.
 constexpr int LQ_SB = 8, LQ_COLS = 256, LF_THREADS = 256;
 struct QueryArgs {

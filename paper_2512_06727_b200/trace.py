@@ -34,6 +34,7 @@ def main(argv=None) -> int:
     ap.add_argument("--jobs", type=int, default=14, help="jobs to list")
     ap.add_argument("--absorbed", action="store_true", help="pass KVCAR_ABSORBED")
     ap.add_argument("--absorbed-v", action="store_true", help="with --absorbed: KVCAR_ABSORBED_V as well")
+    ap.add_argument("--int8", action="store_true", help="int8 latent rows")
     ap.add_argument("--json", default=None, help="also write the raw stamps here")
     args = ap.parse_args(argv)
 
@@ -49,7 +50,7 @@ def main(argv=None) -> int:
     aes = synth.make_stack_autoencoders(w, src, src)
     pps = (w.cached_tokens + 2 + w.page_tokens - 1) // w.page_tokens
     sess = Session(w.n_layers, w.n_q_heads, w.n_kv_heads, w.head_dim, w.page_tokens, w.batch, w.batch * pps, pps,
-                   w.storage, src, src, aes)
+                   w.storage, src, src, aes, latent_quant=args.int8)
     seqs = list(range(w.batch))
     for s in seqs:
         sess.ctx.seq_open(s)
@@ -62,7 +63,8 @@ def main(argv=None) -> int:
         for l in range(w.n_layers):
             k = torch.randn(w.batch, n, kvw, generator=g, device=sess.device).to(sess.dtype)
             v = torch.randn(w.batch, n, kvw, generator=g, device=sess.device).to(sess.dtype)
-            sess.ctx.encode_append_tensor(l, seqs, n, k.data_ptr(), v.data_ptr(), sess.stream())
+            encode = sess.ctx.encode_append if args.int8 else sess.ctx.encode_append_tensor
+            encode(l, seqs, n, k.data_ptr(), v.data_ptr(), sess.stream())
             torch.cuda.current_stream().synchronize()
         sess.ctx.advance(seqs, n, sess.stream())
     k = torch.randn(w.n_layers, w.batch, kvw, generator=g, device=sess.device).to(sess.dtype)
