@@ -827,15 +827,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
                         for (int u = 0; u < 4; ++u) {  // 32 columns (u / 2) x 16 of the warp's 32 rows (u % 2)
                             const int half = u >> 1, f = u & 1;
                             if (half < halves) {
-                                uint32_t r[16];
-                                tmem_ld_frag_x4(acc + (uint32_t)f * (16u << 16) + (uint32_t)(col0 + 32 * half), r);
                                 if (u == 2) {
                                     ta = __ldg(t4 + 8);
                                     tb = __ldg(t4 + 9);
                                 }
                                 const float2 t[4] = {make_float2(ta.x, ta.y), make_float2(ta.z, ta.w), make_float2(tb.x, tb.y),
                                                      make_float2(tb.z, tb.w)};
-                                tmem_ld_wait();
+                                uint32_t r[16];
+                                tmem_ld_frag_x4(acc + (uint32_t)f * (16u << 16) + (uint32_t)(col0 + 32 * half), r);
+                                tmem_ld_wait(r);
                                 if (f == 1 && half + 1 == halves) {
                                     tc_fence_before();
                                     __syncwarp();
@@ -962,7 +962,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
             float r[16];
             tmem_ld8(addr, r);
             tmem_ld8(NQ <= 16 ? addr + NQ : addr + 8u, r + 8);
-            tmem_ld_wait();
+            tmem_ld_wait(r);
             tc_fence_before();
             __syncwarp();
             if (elect_one()) mbar_arrive_remote(empty_leader + 8 * ob);

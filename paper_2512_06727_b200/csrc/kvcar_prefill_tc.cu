@@ -298,7 +298,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PF_THREADS, 1)
                     if (32 * g >= nt) break;  // warp-uniform
                     float *vh = v + (SPLIT ? 32 * hg : 0);
                     tmem_ld32(acc + ((uint32_t)(32 * q) << 16) + 32u * g, vh);
-                    tmem_ld_wait();
+                    tmem_ld_wait32(vh);
 #pragma unroll
                     for (int c8 = 0; c8 < 4; ++c8) {
                         const int c = 32 * g + 8 * c8;

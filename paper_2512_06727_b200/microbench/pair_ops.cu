@@ -435,7 +435,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(384, 1) bg_kernel(co
                 }
             } else if (P.mode >= 3) {
                 tmem_ld32(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 64u + 32u * (it & 3), v);
-                tmem_ld_wait();
+                tmem_ld_wait32(v);
                 const int reps = P.mode == 3 ? 0 : P.mode == 4 ? 2 : 64;
                 for (int rr = 0; rr < reps; ++rr)
 #pragma unroll

@@ -301,3 +301,23 @@ def test_status_codes_of_the_header_match_the_binding():
     body = body[:body.index("}")]
     codes = {int(v): k for k, v in re.findall(r"KVCAR_(?:ERR_)?([A-Z_]+)\s*=\s*(\d+)", body)}
     assert codes == B.STATUS_NAMES, (codes, B.STATUS_NAMES)
+
+
+@pytest.mark.parametrize("change,needs", [({}, False), (dict(latent_full=576, reuse_frac=0.0), False), (dict(page_tokens=48), True),
+                                          (dict(n_q_heads=36), True), (dict(latent_full=576), True)])
+def test_workspace_of_the_fp32_kernels_only_where_a_layer_needs_them(change, needs):
+    """Their operands and partial results (here more than 50 MB) are set aside in contexts with a layer that the tensor-core kernels do
+    not take: pages that are no multiple of 64 tokens, more than 32 query heads, hidden widths that are no multiple of 16 (latent 576
+    with nine stored heads).  One sequence of one page, so that nothing else of that size is in the workspace but the bulk encoder's
+    scratch."""
+    w = synth.scaled(synth.CONFIGS["c2"], n_layers=2, batch=1, **change)
+    src = synth.make_reuse_map(w.n_layers, w.n_kv_heads, w.reuse_frac, w.seed)
+    c = B.Context(w.n_layers, w.n_q_heads, w.n_kv_heads, w.head_dim, w.page_tokens, 1, 1, 1, B.BF16)
+    c.set_reuse_map(src, src)
+    widest = 0
+    for (l, which), ae in synth.make_stack_autoencoders(w, src, src).items():
+        c.set_autoencoder(l, which, ae)
+        widest = max(widest, ae["hidden"])
+    scratch = 2 * 32768 * ((widest + 63) // 64 * 64) * 2
+    rest = c.required_bytes()[2] - scratch
+    assert (rest > 50e6) == needs, rest
