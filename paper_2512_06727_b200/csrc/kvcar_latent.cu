@@ -29,8 +29,9 @@
 //            scale is not theirs: its sign is in W1, its size in W4^T q and in the merge (LeakyReLU is positively
 //            homogeneous; a slope above 1 is turned round on the host).  The accumulator is read in matrix-fragment layout: a lane needs eight shifts instead of 32
 //            (scale and shift fetched per column took 750-900 of a slab's 1 300 cycles) and stores with stmatrix.
-//   K side   S[256 tok x 2R] += slab . (W4^T q rows)^T, over all sources: rows of heads that another source serves are
-//            zero, so the sources simply add up.  Columns R r .. belong to CTA r (its own sequence's queries)
+//   K side   S[256 tok x 2R] += slab . (W4^T q rows)^T, over the columns of a source; the output warps take of it the heads that the
+//            source serves (a stray NaN in one source's rows stays with its heads).  Columns R r .. belong to CTA r (its own
+//            sequence's queries)
 //   V side   per two slabs: U[256 x 2R] = (slab pair)^T [128 features] . P^T over the tile's 128 tokens.  Each CTA supplies
 //            its own hidden slabs and its own probabilities, so in its accumulator its own R columns are its tile's
 // S and the U blocks share two 64-column accumulators in turn; the output warps turn S into probabilities and keep the
@@ -570,57 +571,55 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
             const bool two = NQ > 16 && a.two_terms_k;
 #pragma unroll 1
             for (int it = 0; it < n_steps; ++it) {
-                if (side_lo == 0 && on(it, 0)) {  // S
+#pragma unroll 1
+                for (int s = 0; s < (side_lo == 0 && on(it, 0) ? list_of(0).n : 0); ++s) {  // S
                     const uint32_t ob = o & 1u, acc = tmem + TM_OUT + 64u * ob;
                     mbar_wait(o_empty + 8 * ob, ((o >> 1) & 1u) ^ 1u, a.status, &abort_flag, 0x605);
                     TR(TR_OUT_ISSUE, 0x13);
                     bool begin = true;
+                    const int m = list_of(0).src[s].m, ksm = (m + 63) >> 6, nk_last = ((m - 1) & 63) / 16 + 1;
+                    if constexpr (TERMS == 2) {
 #pragma unroll 1
-                    for (int s = 0; s < list_of(0).n; ++s) {
-                        const int m = list_of(0).src[s].m, ksm = (m + 63) >> 6, nk_last = ((m - 1) & 63) / 16 + 1;
-                        if constexpr (TERMS == 2) {
+                        for (int sl0 = 0; sl0 < ksm; sl0 += CSLABS) {
+                            const int n_sl = min(CSLABS, ksm - sl0);
+                            uint32_t qs = qslot, qp = qphase;
 #pragma unroll 1
-                            for (int sl0 = 0; sl0 < ksm; sl0 += CSLABS) {
-                                const int n_sl = min(CSLABS, ksm - sl0);
-                                uint32_t qs = qslot, qp = qphase;
+                            for (int term = 0; term < TERMS; ++term) {  // both terms meet the same query slabs
+                                hslot += hslot & 1u;
+                                if (hslot == (uint32_t)a.nh) hslot = 0;
+                                mbar_wait(h_ready + 8 * (h & 7u), (h >> 3) & 1u, a.status, &abort_flag, 0x604);
+                                tc_fence_after();
+                                ++h;
+                                qs = qslot;
+                                qp = qphase;
 #pragma unroll 1
-                                for (int term = 0; term < TERMS; ++term) {  // both terms meet the same query slabs
-                                    hslot += hslot & 1u;
-                                    if (hslot == (uint32_t)a.nh) hslot = 0;
-                                    mbar_wait(h_ready + 8 * (h & 7u), (h >> 3) & 1u, a.status, &abort_flag, 0x604);
-                                    tc_fence_after();
-                                    ++h;
-                                    qs = qslot;
-                                    qp = qphase;
+                                for (int i = 0; i < n_sl; ++i) {
+                                    mbar_wait(q_full + 8 * qs, qp, a.status, &abort_flag, 0x60e);
+                                    TR(TR_OUT_ISSUE, 0x30);
+                                    const uint64_t da = h_desc + hslot * (SLAB >> 4), db = q_desc + qs * (QSLAB >> 4);
+                                    const int nk = sl0 + i + 1 < ksm ? 4 : nk_last;
+                                    if (begin)
+                                        umma_pair<0>(acc, da, db, idesc);
+                                    else
+                                        umma_pair<1>(acc, da, db, idesc);
+                                    begin = false;
 #pragma unroll 1
-                                    for (int i = 0; i < n_sl; ++i) {
-                                        mbar_wait(q_full + 8 * qs, qp, a.status, &abort_flag, 0x60e);
-                                        TR(TR_OUT_ISSUE, 0x30);
-                                        const uint64_t da = h_desc + hslot * (SLAB >> 4), db = q_desc + qs * (QSLAB >> 4);
-                                        const int nk = sl0 + i + 1 < ksm ? 4 : nk_last;
-                                        if (begin)
-                                            umma_pair<0>(acc, da, db, idesc);
-                                        else
-                                            umma_pair<1>(acc, da, db, idesc);
-                                        begin = false;
+                                    for (int t = 1; t < nk; ++t) umma_pair<1>(acc, da + 2u * t, db + 2u * t, idesc);
+                                    if (two && term == 0) {
 #pragma unroll 1
-                                        for (int t = 1; t < nk; ++t) umma_pair<1>(acc, da + 2u * t, db + 2u * t, idesc);
-                                        if (two && term == 0) {
-#pragma unroll 1
-                                            for (int t = 0; t < nk; ++t) umma_pair<1>(acc, da + 2u * t, db + (QSLAB / 2 >> 4) + 2u * t, idesc);
-                                        }
-                                        umma_commit_pair(h_free + 8 * hslot);
-                                        if (term + 1 == TERMS) umma_commit_pair(q_empty + 8 * qs);
-                                        TR(TR_OUT_ISSUE, 0x31);
-                                        if (++hslot == (uint32_t)a.nh) hslot = 0;
-                                        if (++qs == (uint32_t)a.nqs) { qs = 0; qp ^= 1u; }
+                                        for (int t = 0; t < nk; ++t) umma_pair<1>(acc, da + 2u * t, db + (QSLAB / 2 >> 4) + 2u * t, idesc);
                                     }
+                                    umma_commit_pair(h_free + 8 * hslot);
+                                    if (term + 1 == TERMS) umma_commit_pair(q_empty + 8 * qs);
+                                    TR(TR_OUT_ISSUE, 0x31);
+                                    if (++hslot == (uint32_t)a.nh) hslot = 0;
+                                    if (++qs == (uint32_t)a.nqs) { qs = 0; qp ^= 1u; }
                                 }
-                                qslot = qs;
-                                qphase = qp;
                             }
-                            continue;
+                            qslot = qs;
+                            qphase = qp;
                         }
+                    } else {
 #pragma unroll 1
                         for (int sl = 0, in_job = 0; sl < ksm; ++sl) {
                             if (in_job == 0) {  // the job's slabs, written by both CTAs
@@ -1031,7 +1030,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
         for (int it = 0; it <= n_it; ++it) {
             float s[NT];
             if (it < n_it && a.mode != MODE_V) {
-                fetch(s, 7);
+                // a source's columns count for the heads that it serves only
+#pragma unroll
+                for (int q = 0; q < NT; ++q) s[q] = 0.f;
+#pragma unroll 1
+                for (int si = 0; si < list_of(0).n; ++si) {
+                    const uint32_t mask = list_of(0).src[si].mask >> q0;
+                    float v[NT];
+                    fetch(v, 7);
+#pragma unroll
+                    for (int q = 0; q < NT; ++q)
+                        if ((mask >> q) & 1u) s[q] += v[q];
+                }
             } else if (it < n_it) {
                 if (it == 0) grid_dependency_wait();  // the launch before holds the scores
 #pragma unroll
@@ -1128,7 +1138,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
 // thread = two hidden columns and four of the sequences, all 64 rows of the head.  The query is scaled by 1/sqrt(head_dim) and by
 // log2(e): the tile kernel's exponentials are powers of two.  Bound by the latency of the weight loads at few sequences, so all
 // of them are in flight before the wait for the preceding kernels; everything else comes from the parameters.  Operand rows of
-// sources that do not serve the head are zeroed.
+// sources that do not serve the head are left as they are: nobody reads their scores.
 // Every block runs its code once, so instruction fetch counts like the loads: with loops unrolled only where that keeps loads in flight,
 // addresses stepped instead of computed per load and the encoder's rows bounded, this kernel went from 63 to 39 KB of code and
 // latent_back_kernel from 41-47 to 33-37; 12 layers of GPT-2's shape, 1 x 200 tokens an eighth less, 8 x 1024 609 -> 580 us; 22 of
@@ -1187,15 +1197,13 @@ __device__ __forceinline__ void query_block(const LatHeads &hp, const QueryArgs 
         lo[i] = a.two_terms ? pack_bf16(x[i] - __uint_as_float(hi[i] << 16), y[i] - __uint_as_float(hi[i] & 0xffff0000u)) : 0u;
     }
     const int64_t seq_step = (int64_t)rows * (a.m_pad >> 1), low = (int64_t)a.nq * (a.m_pad >> 1);
-    uint32_t *r = reinterpret_cast<uint32_t *>(a.wq) + (int64_t)(si0 + i0) * seq_step + (int64_t)qh * (a.m_pad >> 1) + j;
-#pragma unroll 1
-    for (int ss = 0; ss < hp.n_src[0]; ++ss, r += a.batch * seq_step) {
-        if (j >= (hp.src[0][ss].m >> 1)) continue;
+    uint32_t *r = reinterpret_cast<uint32_t *>(a.wq) + ((int64_t)s * a.batch + si0 + i0) * seq_step + (int64_t)qh * (a.m_pad >> 1) + j;
+    if (j < m2) {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
             if (i0 + i < n_here) {
-                r[i * seq_step] = ss == s ? hi[i] : 0u;
-                r[i * seq_step + low] = ss == s ? lo[i] : 0u;
+                r[i * seq_step] = hi[i];
+                r[i * seq_step + low] = lo[i];
             }
     }
     if (cb != 0) return;

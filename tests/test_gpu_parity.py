@@ -895,3 +895,35 @@ def test_runs_of_several_tiles_beyond(shape, int8, monkeypatch):
     assert p.s.ctx.layer_kernel(0) == B.KERNEL_TENSOR
     for step in range(2):
         _check_step(p.decode_step(seqs, step, fused=True), "bf16", f"{shape} int8 {int8} step {step}")
+
+
+@pytest.mark.parametrize("int8", [False, True], ids=["bf16", "int8"])
+@pytest.mark.parametrize("cfg,n", [("c2", 200), ("c2", 2300), ("c3", 200), ("c3", 2300)])
+def test_a_stray_value_stays_with_the_heads_that_read_its_source(cfg, n, int8):
+    """A NaN in one cached K row of layer 0: in layer 1, the heads that reuse layer 0's K read it, those that read layer 1's own rows
+    give the same bits as without it (small grids, where K and V are two launches, and blocks that walk several tiles)."""
+    w = synth.scaled(synth.CONFIGS[cfg], n_layers=2, batch=9, cached_tokens=0, decode_steps=1)
+    src = -np.ones((2, w.n_kv_heads), np.int32)
+    src[1, ::2] = np.arange(w.n_kv_heads)[::2]             # every other KV head of layer 1 reads layer 0's K
+    none = -np.ones(2 * w.n_kv_heads, np.int32)
+    pps = n // 64 + 2
+    p = Pair(w, max_seqs=9, max_pages=9 * pps, max_pages_per_seq=pps, src_k=src.reshape(-1), src_v=none, latent_quant=int8,
+             with_oracle=False)
+    seqs = list(range(9))
+    p.open(seqs)
+    p.prefill(seqs, n)
+    q = np.stack([synth.make_q(w, 1, s_, 3) for s_ in seqs])
+    clean, _, _ = p.attention(1, seqs, q, include_current=False)
+    row = p.s.ctx.debug_locate(4, 70)[1]
+    if int8:
+        p.s.pool_quant_params(0, 0)[row] = float("nan")
+    else:
+        p.s.pool_rows(0, 0)[row] = float("nan")
+    torch.cuda.synchronize()
+    got, _, _ = p.attention(1, seqs, q, include_current=False)
+    group = w.n_q_heads // w.n_kv_heads
+    reads = np.repeat(np.arange(w.n_kv_heads) % 2 == 0, group)
+    assert (got[4][reads] != clean[4][reads]).any(axis=-1).all()
+    assert np.array_equal(got[4][~reads], clean[4][~reads])
+    others = [s_ for s_ in seqs if s_ != 4]
+    assert np.array_equal(got[others], clean[others])
