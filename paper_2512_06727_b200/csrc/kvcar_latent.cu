@@ -1041,6 +1041,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(n_threads(CN), 1)
 #pragma unroll
                     for (int q = 0; q < NT; ++q)
                         if ((mask >> q) & 1u) s[q] += v[q];
+                    if (si + 1 < list_of(0).n) TR(TR_OUT, 0x73);
                 }
             } else if (it < n_it) {
                 if (it == 0) grid_dependency_wait();  // the launch before holds the scores
